@@ -25,6 +25,8 @@
 
 #include "ctx.cuh"
 #include "tc_gemm.cuh"
+#include "tc_ptx.cuh"
+#include "tc_slice.cuh"
 
 namespace adc {
 
@@ -32,124 +34,6 @@ namespace {
 
 constexpr int TC_BM = 128;
 constexpr int TC_BK = 64;
-constexpr uint64_t WAIT_NS = 2000000000ull;   // limit of every pipeline wait (default)
-constexpr uint64_t DRAIN_NS = 2000000000ull;  // limit of the waits that drain work in flight after an abort
-// limit of the pipeline waits in use; a diagnostic may lower it so that a
-// wait gives up on purpose (the drains keep DRAIN_NS)
-__device__ unsigned long long g_wait_ns = WAIT_NS;
-
-__device__ __forceinline__ uint32_t smem_u32(const void *p) {
-  return (uint32_t)__cvta_generic_to_shared(p);
-}
-__device__ __forceinline__ uint64_t gtimer() {
-  uint64_t t;
-  asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
-  return t;
-}
-__device__ __forceinline__ void mbar_init(uint32_t a, uint32_t count) {
-  asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(a), "r"(count) : "memory");
-}
-__device__ __forceinline__ void mbar_expect_tx(uint32_t a, uint32_t bytes) {
-  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(a), "r"(bytes) : "memory");
-}
-__device__ __forceinline__ bool mbar_try(uint32_t a, uint32_t parity) {
-  uint32_t ok;
-  asm volatile(
-      "{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
-      "selp.u32 %0, 1, 0, p;\n\t}\n"
-      : "=r"(ok)
-      : "r"(a), "r"(parity)
-      : "memory");
-  return ok != 0;
-}
-// bounded wait; false when it gave up or another role aborted
-__device__ __forceinline__ bool mbar_wait(uint32_t a, uint32_t parity, volatile int *abort_flag) {
-  const uint64_t t0 = gtimer();
-  const uint64_t lim = *(volatile unsigned long long *)&g_wait_ns;
-  while (!mbar_try(a, parity)) {
-    if (*abort_flag) return false;
-    if (gtimer() - t0 > lim) return false;
-  }
-  return true;
-}
-// wait for work already in flight (copies, MMAs) after an abort: fixed limit
-__device__ __forceinline__ void mbar_drain(uint32_t a, uint32_t parity) {
-  const uint64_t t0 = gtimer();
-  while (!mbar_try(a, parity) && gtimer() - t0 < DRAIN_NS) {
-  }
-}
-__device__ __forceinline__ void tma_load_2d(uint32_t dst, const CUtensorMap *map, int x, int y,
-                                            uint32_t mbar) {
-  asm volatile(
-      "cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];"
-      ::"r"(dst), "l"((uint64_t)map), "r"(x), "r"(y), "r"(mbar)
-      : "memory");
-}
-// the same with an L2 cache policy (createpolicy)
-__device__ __forceinline__ void tma_load_2d_hint(uint32_t dst, const CUtensorMap *map, int x, int y, uint32_t mbar,
-                                                 uint64_t policy) {
-  asm volatile(
-      "cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes.L2::cache_hint"
-      " [%0], [%1, {%2, %3}], [%4], %5;"
-      ::"r"(dst), "l"((uint64_t)map), "r"(x), "r"(y), "r"(mbar), "l"(policy)
-      : "memory");
-}
-__device__ __forceinline__ uint64_t policy_evict_last() {
-  uint64_t p;
-  asm volatile("createpolicy.fractional.L2::evict_last.b64 %0, 1.0;" : "=l"(p));
-  return p;
-}
-__device__ __forceinline__ uint64_t policy_evict_first() {
-  uint64_t p;
-  asm volatile("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(p));
-  return p;
-}
-__device__ __forceinline__ void fence_before() {
-  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-}
-__device__ __forceinline__ void fence_after() {
-  asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-}
-// shared-memory matrix descriptor: K-major operand, 128-byte swizzle, rows of
-// 128 bytes, 8-row groups 1024 bytes apart (SBO), descriptor version 1
-__device__ __forceinline__ uint64_t sdesc(uint32_t saddr) {
-  uint64_t d = 0;
-  d |= (uint64_t)((saddr >> 4) & 0x3FFFu);
-  d |= (uint64_t)1u << 16;
-  d |= (uint64_t)(1024u >> 4) << 32;
-  d |= (uint64_t)1u << 46;
-  d |= (uint64_t)2u << 61;
-  return d;
-}
-// instruction descriptor, kind::f16: D = F32, A = B = BF16, both K-major
-__host__ __device__ constexpr uint32_t idesc_bf16(int M, int N) {
-  return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(M >> 4) << 24);
-}
-__device__ __forceinline__ void mma_bf16(uint32_t tmem_d, uint64_t ad, uint64_t bd, uint32_t idesc,
-                                         uint32_t accum) {
-  asm volatile(
-      "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}\n"
-      ::"r"(tmem_d), "l"(ad), "l"(bd), "r"(idesc), "r"(accum));
-}
-__device__ __forceinline__ void mma_commit(uint32_t mbar) {
-  asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(mbar)
-               : "memory");
-}
-__device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t (&v)[32]) {
-  asm volatile(
-      "tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, "
-      "%13, %14, %15, %16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31}, "
-      "[%32];"
-      : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]),
-        "=r"(v[8]), "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]),
-        "=r"(v[15]), "=r"(v[16]), "=r"(v[17]), "=r"(v[18]), "=r"(v[19]), "=r"(v[20]), "=r"(v[21]),
-        "=r"(v[22]), "=r"(v[23]), "=r"(v[24]), "=r"(v[25]), "=r"(v[26]), "=r"(v[27]), "=r"(v[28]),
-        "=r"(v[29]), "=r"(v[30]), "=r"(v[31])
-      : "r"(taddr));
-  asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-}
-
 template <int BN, int ST>
 struct TcLayout {
   static constexpr int A_BYTES = TC_BM * TC_BK * 2;
@@ -406,14 +290,17 @@ __global__ void k_emb_B(BSrc src, int64_t Nc, int64_t K, int conj, int64_t kp, _
 
 PFN_cuTensorMapEncodeTiled_v12000 g_encode = nullptr;
 
+void load_encode() {
+  if (g_encode) return;
+  cudaDriverEntryPointQueryResult q;
+  void *fn = nullptr;
+  ADC_CUDA(cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &fn, 12000, cudaEnableDefault, &q));
+  ADC_REQUIRE(fn && q == cudaDriverEntryPointSuccess, ADC_ERR_CUDA, "cuTensorMapEncodeTiled unavailable");
+  g_encode = (PFN_cuTensorMapEncodeTiled_v12000)fn;
+}
+
 void make_map(CUtensorMap *map, const void *base, int64_t rows, int64_t kp2, int box_rows) {
-  if (!g_encode) {
-    cudaDriverEntryPointQueryResult q;
-    void *fn = nullptr;
-    ADC_CUDA(cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &fn, 12000, cudaEnableDefault, &q));
-    ADC_REQUIRE(fn && q == cudaDriverEntryPointSuccess, ADC_ERR_CUDA, "cuTensorMapEncodeTiled unavailable");
-    g_encode = (PFN_cuTensorMapEncodeTiled_v12000)fn;
-  }
+  load_encode();
   ADC_REQUIRE(((uintptr_t)base & 15) == 0 && (kp2 * 2) % 16 == 0, ADC_ERR_ARG, "TMA alignment");
   cuuint64_t dims[2] = {(cuuint64_t)kp2, (cuuint64_t)rows};
   cuuint64_t strides[1] = {(cuuint64_t)(kp2 * 2)};
@@ -424,7 +311,6 @@ void make_map(CUtensorMap *map, const void *base, int64_t rows, int64_t kp2, int
                         CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
   ADC_REQUIRE(r == CUDA_SUCCESS, ADC_ERR_CUDA, "cuTensorMapEncodeTiled failed: " + std::to_string((int)r));
 }
-
 
 template <int BN, int ST>
 void launch_tc(Exec &ex, const TcView &A, const TcView &B, int64_t M, int64_t N2, cplx alpha, cplx beta,
@@ -500,9 +386,6 @@ struct TgLayout {
 
 __device__ __forceinline__ void tensormap_acquire(const CUtensorMap *m) {
   asm volatile("fence.proxy.tensormap::generic.acquire.gpu [%0], 128;" ::"l"((uint64_t)m) : "memory");
-}
-__device__ __forceinline__ void mbar_arrive(uint32_t a) {
-  asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(a) : "memory");
 }
 
 struct TgTile {
@@ -771,6 +654,20 @@ k_tc_grouped(const TcJob *__restrict__ jobs, int njobs, int total_tiles, int *co
 
 }  // namespace
 
+void tc_make_map3(CUtensorMap *map, const void *base, int64_t rows, int64_t kp2, int64_t planes, int64_t plane_elems,
+                  int box_rows) {
+  load_encode();
+  ADC_REQUIRE(((uintptr_t)base & 15) == 0 && kp2 % TC_BK == 0 && plane_elems % 8 == 0, ADC_ERR_ARG, "TMA alignment");
+  cuuint64_t dims[3] = {(cuuint64_t)kp2, (cuuint64_t)rows, (cuuint64_t)planes};
+  cuuint64_t strides[2] = {(cuuint64_t)(kp2 * 2), (cuuint64_t)(plane_elems * 2)};
+  cuuint32_t box[3] = {(cuuint32_t)TC_BK, (cuuint32_t)box_rows, 1};
+  cuuint32_t estr[3] = {1, 1, 1};
+  CUresult r = g_encode(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void *>(base), dims, strides, box,
+                        estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
+                        CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+  ADC_REQUIRE(r == CUDA_SUCCESS, ADC_ERR_CUDA, "cuTensorMapEncodeTiled failed: " + std::to_string((int)r));
+}
+
 static void alloc_planes(Exec &ex, TcMat &dst, size_t bytes, int planes) {
   if (dst.hi.bytes < bytes || (planes == 3 && dst.lo2.bytes < bytes)) {
     dst.hi.reset(); dst.lo.reset(); dst.lo2.reset();
@@ -915,9 +812,7 @@ void tc_gemm_grouped(Exec &ex, const std::vector<TcJobDesc> &in, TcGroup &grp, i
   grp.flops = 0.0;
   for (int j = 0; j < nj; ++j) {
     const TcJobDesc &d = in[j];
-    ADC_REQUIRE(d.A && d.B && (d.out || d.out32), ADC_ERR_ARG, "tc_gemm_grouped: job operands");
-    ADC_REQUIRE(d.nseg == 3 || d.nseg == 1, ADC_ERR_ARG, "tc_gemm_grouped: products per tile");
-    ADC_REQUIRE(!d.out32 || d.kb_split > 0, ADC_ERR_ARG, "tc_gemm_grouped: raw output needs kb_split");
+    ADC_REQUIRE(d.A && d.B && d.out, ADC_ERR_ARG, "tc_gemm_grouped: job operands");
     ADC_REQUIRE(d.A->kp == d.B->kp, ADC_ERR_ARG, "tc_gemm_grouped: inner sizes differ");
     ADC_REQUIRE(d.A->rows >= d.M && d.B->rows >= 2 * d.N, ADC_ERR_ARG, "tc_gemm_grouped: operand rows");
     ADC_REQUIRE(d.M < (1ll << 31) && 2 * d.N < (1ll << 31), ADC_ERR_UNSUPPORTED, "tc_gemm_grouped: size");
@@ -930,7 +825,7 @@ void tc_gemm_grouped(Exec &ex, const std::vector<TcJobDesc> &in, TcGroup &grp, i
     if (p.bn <= 0) p.bn = bn_rule(p.N2);
     ADC_REQUIRE(p.bn >= 32 && p.bn <= TC_BNMAX && p.bn % 32 == 0, ADC_ERR_ARG, "tc_gemm_grouped: tile width");
     p.kps = (int)(2 * d.A->kp / TC_BK);
-    p.nseg = d.nseg;
+    p.nseg = 3;  // hi hi, hi lo, lo hi
     p.tiles_m = (int)((d.M + TC_BM - 1) / TC_BM);
     p.tiles_n = (int)((p.N2 + p.bn - 1) / p.bn);
     work += (double)p.tiles_m * p.tiles_n * (double)p.nseg * p.kps;
@@ -946,12 +841,6 @@ void tc_gemm_grouped(Exec &ex, const std::vector<TcJobDesc> &in, TcGroup &grp, i
   size_t part_need = 0;
   for (auto &p : pl) {
     const int total_kb = p.nseg * p.kps;
-    if (in[p.idx].out32) {
-      // raw output: the caller fixes the split (exact FP32 sums need short splits)
-      p.kbps = std::min(in[p.idx].kb_split, total_kb);
-      p.ksplit = (total_kb + p.kbps - 1) / p.kbps;
-      continue;
-    }
     int ks = 1;
     if (total_kb > target) ks = (int)std::min<double>(128.0, std::ceil(total_kb / target));
     p.kbps = (total_kb + ks - 1) / ks;
@@ -985,20 +874,15 @@ void tc_gemm_grouped(Exec &ex, const std::vector<TcJobDesc> &in, TcGroup &grp, i
     TcJob &J = grp.host[i];
     std::memset(&J, 0, sizeof(J));
     const int64_t kp2 = 2 * d.A->kp;
-    // one-product jobs read only the hi planes (a single-plane operand has no lo)
+    ADC_REQUIRE(d.A->lo.p && d.B->lo.p, ADC_ERR_ARG, "tc_gemm_grouped: three products need lo planes");
     make_map(&J.mAh, d.A->hi.p, d.A->rows, kp2, TC_BM);
-    make_map(&J.mAl, d.A->lo.p ? d.A->lo.p : d.A->hi.p, d.A->rows, kp2, TC_BM);
+    make_map(&J.mAl, d.A->lo.p, d.A->rows, kp2, TC_BM);
     make_map(&J.mBh, d.B->hi.p, d.B->rows, kp2, p.bn);
-    make_map(&J.mBl, d.B->lo.p ? d.B->lo.p : d.B->hi.p, d.B->rows, kp2, p.bn);
-    ADC_REQUIRE(p.nseg == 1 || (d.A->lo.p && d.B->lo.p), ADC_ERR_ARG, "tc_gemm_grouped: three products need lo planes");
+    make_map(&J.mBl, d.B->lo.p, d.B->rows, kp2, p.bn);
     J.out = d.out;
     J.nseg = p.nseg;
-    if (d.out32) {
-      J.part = d.out32;
-    } else {
-      J.part = p.ksplit > 1 ? (float *)grp.part.p + poff : nullptr;
-      if (p.ksplit > 1) poff += (size_t)p.ksplit * d.M * p.N2;
-    }
+    J.part = p.ksplit > 1 ? (float *)grp.part.p + poff : nullptr;
+    if (p.ksplit > 1) poff += (size_t)p.ksplit * d.M * p.N2;
     J.s_m = d.s_m;
     J.s_nh = d.s_nh;
     J.s_nl = d.s_nl;
@@ -1018,7 +902,7 @@ void tc_gemm_grouped(Exec &ex, const std::vector<TcJobDesc> &in, TcGroup &grp, i
       // B is re-read by every row block. When A is several times larger, the
       // tiles run in panels of B columns whose planes fit in about a third of
       // L2, loaded with an evict-last policy (A evict-first, streaming through)
-      const double planes_used = (p.nseg == 1) ? 1.0 : 2.0;
+      const double planes_used = 2.0;
       const double col_block = (double)p.bn * kp2 * 2.0 * planes_used;  // bytes of one column block of B
       const double bbytes = (double)std::min<int64_t>(d.B->rows, p.N2) * kp2 * 2.0 * planes_used;
       const double abytes = (double)std::min<int64_t>(d.A->rows, d.M) * kp2 * 2.0 * planes_used;
@@ -1039,16 +923,13 @@ void tc_gemm_grouped(Exec &ex, const std::vector<TcJobDesc> &in, TcGroup &grp, i
   }
   ADC_CUDA(cudaMemsetAsync(grp.counter.p, 0, sizeof(int), ex.stream));
   const int grid = (int)std::min<int64_t>(tiles, sms);
-  // one-product raw jobs are the digit pairs of the sliced product (tc_slice.cu)
-  bool raw = true;
-  for (const auto &d : in) raw = raw && d.out32 && d.nseg == 1;
-  int pr = ex.prof_begin(raw ? "tc_sliced_pairs" : "tc_grouped_bf16x3", grp.flops);
+  int pr = ex.prof_begin("tc_grouped_bf16x3", grp.flops);
   k_tc_grouped<<<grid, 192, TgLayout::SMEM, ex.stream>>>((const TcJob *)grp.jobs.p, np, (int)tiles,
                                                          (int *)grp.counter.p, err);
   ADC_CHECK_LAUNCH();
   for (int i = 0; i < np; ++i) {
     const TcJob &J = grp.host[i];
-    if (J.ksplit <= 1 || in[pl[i].idx].out32) continue;
+    if (J.ksplit <= 1) continue;
     k_tc_reduce<<<grid1d((int64_t)J.M * (J.N2 / 2), 256), 256, 0, ex.stream>>>(
         J.part, J.ksplit, J.M, J.N2, J.out, J.s_m, J.s_nh, J.s_nl, J.n_in, J.alpha, J.beta);
     ADC_CHECK_LAUNCH();
@@ -1059,6 +940,7 @@ void tc_gemm_grouped(Exec &ex, const std::vector<TcJobDesc> &in, TcGroup &grp, i
 void tc_set_wait_ns(uint64_t ns) {
   const unsigned long long v = ns ? (unsigned long long)ns : (unsigned long long)WAIT_NS;
   ADC_CUDA(cudaMemcpyToSymbol(g_wait_ns, &v, sizeof(v)));
+  sl_set_wait_ns(v);
 }
 
 int tc_autotune_bn(Exec &ex, const TcJobDesc &d, int *err) {

@@ -101,6 +101,10 @@ struct TcView {
   int64_t rows = 0, kp = 0, kreal = 0;
 };
 TcView tc_view(const TcMat &m, int64_t row0 = 0, int64_t rows = -1);
+// tensor map of BF16 planes [planes][rows][kp2] (planes plane_elems apart), boxes of
+// box_rows x 64 elements, 128-byte swizzle, rows past the end read as zero
+void tc_make_map3(CUtensorMap *map, const void *base, int64_t rows, int64_t kp2, int64_t planes, int64_t plane_elems,
+                  int box_rows);
 
 // A[m][k] = op(src[m*s_m + k*s_k]) (op = conj when conj is set); planes 2 or 3
 void tc_pack_A(Exec &ex, TcMat &dst, const cplx *src, int64_t M, int64_t K, int64_t s_m, int64_t s_k, bool conj,
@@ -145,14 +149,6 @@ struct TcJobDesc {
   cplx *out = nullptr;
   int64_t s_m = 0, s_nh = 0, s_nl = 0, n_in = 1;
   int bn = 0;
-  // products per tile: 3 (hi hi, hi lo, lo hi) or 1 (hi hi: one plane of each
-  // operand, e.g. one pair of slices of the sliced FP64 product)
-  int nseg = 3;
-  // raw mode: when set, the FP32 sums of each K split s are written to
-  // out32[s][M][2N] (real columns) and out/alpha/beta are unused; every split
-  // holds at most kb_split k-blocks of 64 (required in raw mode)
-  float *out32 = nullptr;
-  int kb_split = 0;
 };
 
 // device and pinned host state of a grouped launch. A captured graph copies

@@ -5,282 +5,668 @@
 // The operands use the real embedding of tc_gemm.cu (an A row is [Re | Im], a
 // complex B row n becomes [Re | -Im] and [Im | Re]). Every row of an operand
 // is scaled by a power of two, 2^E with max |row| < 2^E, and each scaled value
-// y (|y| < 1) is written as a sum of slices y = sum_i d_i 2^(-b i), i = 1..ns,
-// with integer digits d_i = rint((y - d_1 2^-b - ... - d_(i-1) 2^(-b (i-1))) 2^(b i)),
-// so |d_1| <= 2^b and |d_i| <= 2^(b-1) for i >= 2: integers of at most b + 1
-// bits, exact in BF16 for b <= 7. The product of slice i of A and slice j of B
-// over K2 embedded terms is a sum of integers whose partial sums stay below
-// K2 2^(2b); with K2 <= 2^(24 - 2b) (longer inner sizes are split) every
-// partial sum is an integer below 2^24 and the tensor cores' FP32 accumulator
-// holds it exactly. The pairs i + j <= ns + 1 run as one grouped tcgen05 launch
-// (tc_gemm_grouped, one product per tile, raw FP32 outputs) and a combine
-// kernel forms, in FP64, sum over pairs and splits of 2^(E_m + F_n - b (i + j)) P_ij.
-// The error comes only from the dropped slice digits and pairs, about 2^(-b ns)
+// y (|y| < 1), rounded to a multiple of 2^(-b ns), is written with ns signed
+// digits of b bits (seven, but see sl_digits), y = sum_i d_i 2^(-b i), |d_1| <= 2^b
+// and |d_i| <= 2^(b-1) after it: integers that BF16 holds exactly. A product of digit i of A and
+// digit j of B has weight 2^(-b (i + j)); the pairs of one weight form a class
+// c = i + j, and the classes 2 .. ns + 1 are kept. The error comes only from
+// the rounding of the operands and the dropped classes, about 2^(-b ns)
 // relative to the row and column maxima, whatever K is: an error-free
 // splitting of the products in the manner of Ozaki, Ogita, Oishi and Rump
 // ("Error-free transformations of matrix multiplication by using fast
 // routines of matrix multiplication", Numer. Algorithms 59, 2012), on BF16
 // tensor cores with integer digits.
+//
+// Exactness. All pairs of one class add into the same FP32 accumulator. Per
+// inner element a class of n pairs adds at most (n + 2) 2^(2b-2) in magnitude (two
+// of its pairs hold a first digit; the class of the pair (1, 1) alone at most
+// 2^(2b) = 4 * 2^(2b-2)), so a run of floor(2^(20-2b) / (n + 2)) blocks of 64 stays
+// within 2^24 and every partial sum is an integer that FP32 holds. After such a
+// run the accumulators are drained into 64-bit integers.
 #include <cuda_bf16.h>
 
+#include <algorithm>
 #include <cmath>
 
 #include "ctx.cuh"
 #include "tc_gemm.cuh"
+#include "tc_ptx.cuh"
 #include "tc_slice.cuh"
 
 namespace adc {
 
 namespace {
 
-constexpr int SL_MAXPAIRS = 160;
+// ---------------------------------------------------------------- row scales
+// The scale of a row is kept as its largest magnitude word: the high 31 bits
+// of |x| (the lowest bit set too when only the low word is nonzero), so that
+// an integer maximum finds it. 0: a row of zeros; exponent field 2047: the row
+// holds an infinity or a NaN.
+__device__ __forceinline__ unsigned mag_word(double x) {
+  const unsigned hi = (unsigned)__double2hiint(x) & 0x7fffffffu;
+  return hi | (__double2loint(x) != 0 ? 1u : 0u);
+}
+__device__ __forceinline__ unsigned mag_word(cplx x) { return max(mag_word(x.x), mag_word(x.y)); }
+__device__ __forceinline__ bool not_finite(unsigned w) { return (w >> 20) == 0x7ffu; }
+// E with every |x| of the row below 2^E
+__device__ __forceinline__ int scale_exp(unsigned w) { return (w >> 20) ? (int)(w >> 20) - 1022 : -1021; }
 
-__device__ __forceinline__ double amax2(cplx x) { return fmax(fabs(x.x), fabs(x.y)); }
+// round(x 2^(bits - E)) as an integer (|x| < 2^E, so at most 2^bits; ties to even)
+__device__ __forceinline__ long long fixed_of(double x, int E, int bits) {
+  const long long u = __double_as_longlong(x);
+  const int field = (int)((u >> 52) & 0x7ff);
+  long long m = u & 0xfffffffffffffll;
+  if (field) m |= 1ll << 52;
+  const int s = (field ? field : 1) - 1075 + bits - E;  // value = m 2^(s + E - bits); s <= bits - 53
+  long long r;
+  if (s >= 0) r = m << s;
+  else if (s >= -54) r = (m + ((1ll << (-s - 1)) - 1) + ((m >> -s) & 1)) >> -s;
+  else r = 0;
+  return u < 0 ? -r : r;
+}
 
-// block-wide maximum (blockDim.x a multiple of 32, at most 1024)
-__device__ double block_max(double v) {
-  __shared__ double red[32];
-  for (int off = 16; off > 0; off >>= 1) v = fmax(v, __shfl_down_sync(0xffffffffu, v, off));
-  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = v;
-  __syncthreads();
-  if (threadIdx.x < 32) {
-    v = (threadIdx.x < (blockDim.x >> 5)) ? red[threadIdx.x] : 0.0;
-    for (int off = 16; off > 0; off >>= 1) v = fmax(v, __shfl_down_sync(0xffffffffu, v, off));
+constexpr int PK_R = 32, PK_K = 64;    // tile of the packing kernels: rows x inner elements
+constexpr int PK_LD = PK_K + PK_K / 8;  // one element of padding per eight
+__device__ __forceinline__ int pk_at(int r, int k) { return r * PK_LD + k + (k >> 3); }
+
+// element (row n, inner k) of the operand rows a packing block handles: the
+// address arithmetic of BSrc split into a part per row and a part per k
+struct PkRow {
+  const cplx *p;
+  int b;
+};
+__device__ __forceinline__ PkRow pk_row(const BSrc &s, int64_t n) {
+  PkRow r;
+  if (s.mode == 0) {
+    const int64_t nh = n / s.n_in, nl = n - nh * s.n_in;
+    r.p = s.p + nh * s.s_nh + nl * s.s_nl;
+    r.b = 0;
+  } else {
+    const int64_t per = (s.mode == 1) ? s.v : s.o, vec = n / per;
+    r.p = s.p + s.n1 + vec * s.N;
+    r.b = (int)(n - vec * per);
   }
-  return v;  // valid in thread 0
+  return r;
+}
+__device__ __forceinline__ cplx pk_get(const BSrc &s, const PkRow &r, int64_t k, int kh, int kl) {
+  if (s.mode == 0) return r.p[k * s.s_k];
+  if (s.mode == 1) {  // (kh, kl) = (kk, c): X[kk][(c, b)]
+    if (kl == r.b) return cmake(0.0, 0.0);
+    const cplx x = kl < r.b ? r.p[kh * (s.v * (s.v - 1) / 2) + pair_index(kl, r.b, s.v)]
+                            : r.p[kh * (s.v * (s.v - 1) / 2) + pair_index(r.b, kl, s.v)];
+    return kl < r.b ? x : cmake(-x.x, -x.y);
+  }
+  // mode 2, (kh, kl) = (kq, b): X[(i, kq)][b]
+  if (kh == r.b) return cmake(0.0, 0.0);
+  const cplx x = r.b < kh ? r.p[pair_index(r.b, kh, s.o) * s.v + kl] : r.p[pair_index(kh, r.b, s.o) * s.v + kl];
+  return r.b < kh ? x : cmake(-x.x, -x.y);
 }
 
-// exponent E with max < 2^E (0 for an all-zero row)
-__device__ __forceinline__ int exp_above(double amax) {
-  if (!(amax > 0.0)) return 0;
-  int e;
-  frexp(amax, &e);  // amax = f 2^e, f in [0.5, 1)
-  return e;
+// loads rows [n0, n0 + 32) x [k0, k0 + 64) of the source, zero outside, calling
+// f(row, k, value); lanes run along whichever index is contiguous in memory
+template <class F>
+__device__ __forceinline__ void pk_load(const BSrc &src, int64_t n0, int64_t rows, int64_t k0, int64_t K, bool kfast,
+                                        const PkRow *row, F f) {
+#pragma unroll
+  for (int it = 0; it < PK_R * PK_K / 256; ++it) {
+    const int idx = threadIdx.x + 256 * it;
+    const int r = kfast ? idx >> 6 : idx & 31, kk = kfast ? idx & 63 : idx >> 5;
+    cplx x = cmake(0.0, 0.0);
+    const int64_t k = k0 + kk;
+    if (n0 + r < rows && k < K) {
+      int kh = 0, kl = 0;
+      if (src.mode != 0) { kh = (int)((unsigned)k / (unsigned)src.v); kl = (int)k - kh * (int)src.v; }
+      x = pk_get(src, row[r], k, kh, kl);
+    }
+    f(r, kk, x);
+  }
 }
 
-// E[m] for the rows of A (element (m, k) at src[m*s_m + k*s_k]), one block per row
-__global__ void k_sl_exp_A(const cplx *__restrict__ src, int64_t M, int64_t K, int64_t s_m, int64_t s_k, int *E) {
-  for (int64_t m = blockIdx.x; m < M; m += gridDim.x) {
-    double v = 0.0;
-    for (int64_t k = threadIdx.x; k < K; k += blockDim.x) v = fmax(v, amax2(src[m * s_m + k * s_k]));
-    v = block_max(v);
-    if (threadIdx.x == 0) E[m] = exp_above(v);
+// W[n] = max(W[n], largest magnitude word of row n over the inner range of this
+// block). Blocks: (row tiles, inner ranges); the maximum is exact in any order
+__global__ void __launch_bounds__(256)
+k_sl_scale(BSrc src, int64_t rows, int64_t K, int64_t krange, int kfast, unsigned *W) {
+  __shared__ PkRow row[PK_R];
+  __shared__ unsigned mx[PK_R];
+  const int64_t kb = (int64_t)blockIdx.y * krange, ke = min(K, kb + krange);
+  for (int64_t n0 = (int64_t)blockIdx.x * PK_R; n0 < rows; n0 += (int64_t)gridDim.x * PK_R) {
+    if (threadIdx.x < PK_R) {
+      row[threadIdx.x] = pk_row(src, min(n0 + (int64_t)threadIdx.x, rows - 1));
+      mx[threadIdx.x] = 0;
+    }
+    __syncthreads();
+    unsigned own = 0;  // lanes along the rows: one row per thread
+    for (int64_t k0 = kb; k0 < ke; k0 += PK_K)
+      pk_load(src, n0, rows, k0, ke, kfast != 0, row, [&](int r, int, cplx x) {
+        const unsigned w = mag_word(x);
+        if (kfast) {
+          const unsigned m = __reduce_max_sync(0xffffffffu, w);  // a warp covers half a row
+          if ((threadIdx.x & 31) == 0) atomicMax(&mx[r], m);
+        } else {
+          own = max(own, w);
+        }
+      });
+    if (!kfast) atomicMax(&mx[threadIdx.x & 31], own);
+    __syncthreads();
+    if (threadIdx.x < PK_R && n0 + threadIdx.x < rows) atomicMax(&W[n0 + threadIdx.x], mx[threadIdx.x]);
     __syncthreads();
   }
 }
 
-// F[n] for the complex rows of B, one block per row
-__global__ void k_sl_exp_B(BSrc src, int64_t Nc, int64_t K, int *F) {
-  for (int64_t n = blockIdx.x; n < Nc; n += gridDim.x) {
-    double v = 0.0;
-    for (int64_t k = threadIdx.x; k < K; k += blockDim.x) v = fmax(v, amax2(src.get(n, k)));
-    v = block_max(v);
-    if (threadIdx.x == 0) F[n] = exp_above(v);
+__device__ __forceinline__ uint32_t bf16x2_of(int a, int b) {
+  const __nv_bfloat162 h = __floats2bfloat162_rn((float)a, (float)b);  // exact: |a|, |b| <= 128
+  return *(const uint32_t *)&h;
+}
+
+// Bound by memory (16 bytes read, 4 ns or 8 ns written per element); the tile in
+// shared memory lets lanes run along whichever source index is contiguous.
+// Digits of a 32 x 64 tile staged in shared memory: every thread takes eight
+// consecutive inner elements of a row and stores 16 bytes per plane. EMB = 1:
+// an A row [Re | Im]; EMB = 2: the two rows of the B embedding.
+// The digits come from the top, each the remainder rounded to nearest, so that
+// they are centred on zero: digits cut from the bottom, in [-2^(b-1), 2^(b-1) - 1],
+// have a mean of -1/2, and the dropped classes would leave an error that grows with K.
+template <int EMB>
+__global__ void __launch_bounds__(256)
+k_sl_pack(BSrc src, int64_t rows, int64_t K, int conj, int64_t kp, int kfast, const unsigned *__restrict__ W, int b, int ns,
+          __nv_bfloat16 *base, int64_t pe) {
+  __shared__ cplx tile[PK_R * PK_LD];
+  __shared__ PkRow row[PK_R];
+  const int bits = b * ns;
+  for (int64_t n0 = (int64_t)blockIdx.x * PK_R; n0 < rows; n0 += (int64_t)gridDim.x * PK_R) {
+    if (threadIdx.x < PK_R) row[threadIdx.x] = pk_row(src, min(n0 + (int64_t)threadIdx.x, rows - 1));
     __syncthreads();
-  }
-}
-
-// Digits in integer arithmetic (the FP64 pipe is the scarce one): the value
-// y = x 2^-E (|y| < 1) as the integer R = round(y 2^(b ns)) (at most 61 bits),
-// then ns signed digits of b bits, each rounded to nearest with the remainder
-// carried to the next (|d_1| <= 2^b, |d_i| <= 2^(b-1) after it), so that
-// y = sum_i d_i 2^(-b i) to within 2^(-b ns - 1).
-__device__ __forceinline__ long long fixed_of(double x, int E, int bns) { return llrint(ldexp(x, bns - E)); }
-__device__ __forceinline__ int next_digit(long long &R, int sh) {
-  const long long d = (sh > 0) ? ((R + (1LL << (sh - 1))) >> sh) : R;
-  R -= d * (1LL << sh);
-  return (int)d;
-}
-
-// A rows [Re | Im] (conj negates Im), padded to kp with zeros. One thread per
-// 8 consecutive k of a row, 16-byte stores of every slice
-__global__ void k_sl_slice_A(const cplx *__restrict__ src, int64_t M, int64_t K, int64_t s_m, int64_t s_k, int conj,
-                             int64_t kp, const int *__restrict__ E, int ns, int b, __nv_bfloat16 *base, int64_t pe) {
-  const int64_t kq = kp >> 3;
-  const int64_t total = M * kq;
-  const int bns = b * ns;
-  for (int64_t idx = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; idx < total;
-       idx += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t m = idx / kq, k0 = (idx - m * kq) << 3;
-    const cplx *row = src + m * s_m;
-    const int e = E[m];
-    long long Rr[8], Ri[8];
+    for (int64_t k0 = (int64_t)blockIdx.y * PK_K; k0 < kp; k0 += (int64_t)gridDim.y * PK_K) {
+      pk_load(src, n0, rows, k0, K, kfast != 0, row, [&](int r, int kk, cplx x) { tile[pk_at(r, kk)] = x; });
+      __syncthreads();
+      const int r = threadIdx.x >> 3, oct = threadIdx.x & 7;
+      const int64_t n = n0 + r;
+      if (n < rows) {
+        const unsigned w = W[n];
+        const int e = scale_exp(w);
+        const bool dead = not_finite(w);
+        long long re[8], im[8];
 #pragma unroll
-    for (int j = 0; j < 8; ++j) {
-      const int64_t k = k0 + j;
-      cplx x = cmake(0.0, 0.0);
-      if (k < K) x = row[k * s_k];
-      Rr[j] = fixed_of(x.x, e, bns);
-      Ri[j] = fixed_of(conj ? -x.y : x.y, e, bns);
-    }
-    const int64_t r0 = m * 2 * kp + k0;
-    for (int i = 1; i <= ns; ++i) {
-      const int sh = b * (ns - i);
-      __align__(16) __nv_bfloat16 dr[8], di[8];
+        for (int j = 0; j < 8; ++j) {
+          const cplx x = tile[pk_at(r, 8 * oct + j)];
+          re[j] = dead ? 0 : fixed_of(x.x, e, bits);
+          im[j] = dead ? 0 : fixed_of(conj ? -x.y : x.y, e, bits);
+        }
+        for (int i = 0; i < ns; ++i) {
+          const int sh = b * (ns - 1 - i);
+          const long long rnd = (1ll << sh) >> 1;
+          int dr[8], di[8];
 #pragma unroll
-      for (int j = 0; j < 8; ++j) {
-        dr[j] = __int2bfloat16_rn(next_digit(Rr[j], sh));
-        di[j] = __int2bfloat16_rn(next_digit(Ri[j], sh));
+          for (int j = 0; j < 8; ++j) {
+            dr[j] = (int)((re[j] + rnd) >> sh);
+            di[j] = (int)((im[j] + rnd) >> sh);
+            re[j] -= (long long)dr[j] << sh;
+            im[j] -= (long long)di[j] << sh;
+          }
+          uint4 vr, vi;
+          vr.x = bf16x2_of(dr[0], dr[1]); vr.y = bf16x2_of(dr[2], dr[3]);
+          vr.z = bf16x2_of(dr[4], dr[5]); vr.w = bf16x2_of(dr[6], dr[7]);
+          vi.x = bf16x2_of(di[0], di[1]); vi.y = bf16x2_of(di[2], di[3]);
+          vi.z = bf16x2_of(di[4], di[5]); vi.w = bf16x2_of(di[6], di[7]);
+          __nv_bfloat16 *pl = base + (int64_t)i * pe + (int64_t)EMB * n * 2 * kp + k0 + 8 * oct;
+          *(uint4 *)pl = vr;
+          if (EMB == 1) {
+            *(uint4 *)(pl + kp) = vi;
+          } else {
+            uint4 vn;
+            vn.x = bf16x2_of(-di[0], -di[1]); vn.y = bf16x2_of(-di[2], -di[3]);
+            vn.z = bf16x2_of(-di[4], -di[5]); vn.w = bf16x2_of(-di[6], -di[7]);
+            *(uint4 *)(pl + kp) = vn;
+            *(uint4 *)(pl + 2 * kp) = vi;
+            *(uint4 *)(pl + 3 * kp) = vr;
+          }
+        }
       }
-      __nv_bfloat16 *pl = base + (int64_t)(i - 1) * pe;
-      *(uint4 *)(pl + r0) = *(const uint4 *)dr;
-      *(uint4 *)(pl + r0 + kp) = *(const uint4 *)di;
+      __syncthreads();
     }
   }
 }
 
-// B rows: row 2n = [Re | -Im], row 2n+1 = [Im | Re] (conj negates Im first).
-// One thread per 8 consecutive k of a row; every slice's digits of the 8
-// elements go out as 16-byte stores (the digits of -Im are the negated digits of Im)
-__global__ void k_sl_slice_B(BSrc src, int64_t Nc, int64_t K, int conj, int64_t kp, const int *__restrict__ F,
-                             int ns, int b, __nv_bfloat16 *base, int64_t pe) {
-  const int64_t kq = kp >> 3;
-  const int64_t total = Nc * kq;
-  const int bns = b * ns;
-  for (int64_t idx = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; idx < total;
-       idx += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t n = idx / kq, k0 = (idx - n * kq) << 3;
-    cplx x[8];
-    src.get8(n, k0, K, x);
-    const int e = F[n];
-    long long Rr[8], Ri[8];
-#pragma unroll
-    for (int j = 0; j < 8; ++j) {
-      Rr[j] = fixed_of(x[j].x, e, bns);
-      Ri[j] = fixed_of(conj ? -x[j].y : x[j].y, e, bns);
-    }
-    const int64_t r0 = (2 * n) * 2 * kp + k0, r1 = (2 * n + 1) * 2 * kp + k0;
-    for (int i = 1; i <= ns; ++i) {
-      const int sh = b * (ns - i);
-      __align__(16) __nv_bfloat16 dr[8], di[8], dn[8];
-#pragma unroll
-      for (int j = 0; j < 8; ++j) {
-        const int a = next_digit(Rr[j], sh), c = next_digit(Ri[j], sh);
-        dr[j] = __int2bfloat16_rn(a);
-        di[j] = __int2bfloat16_rn(c);
-        dn[j] = __int2bfloat16_rn(-c);
-      }
-      __nv_bfloat16 *pl = base + (int64_t)(i - 1) * pe;
-      *(uint4 *)(pl + r0) = *(const uint4 *)dr;
-      *(uint4 *)(pl + r0 + kp) = *(const uint4 *)dn;
-      *(uint4 *)(pl + r1) = *(const uint4 *)di;
-      *(uint4 *)(pl + r1 + kp) = *(const uint4 *)dr;
-    }
-  }
-}
-
-struct SlCombine {
-  int npair, ksplit;
-  int sh[SL_MAXPAIRS];     // b (i + j) of each pair; pairs ordered by i + j
-  double sc[SL_MAXPAIRS];  // 2^-sh (exact)
+// ---------------------------------------------------------------- the product
+// One CTA per SM, resident, takes output tiles of 128 rows by BN real columns.
+// Four classes c = hi, hi - 1, .. share a pass over K with one TMEM accumulator
+// each (4 x BN columns); stage i of an inner block holds digit i of A and digit
+// hi - i of B, and digit hi - i of B is multiplied with the digits i, i - 1, ..
+// of A, which are still in shared memory from the stages before. So a pass of
+// the classes 9..6 reads 16 operand blocks for 26 block products, where one
+// product at a time reads 52: a 128 x 128 x 64 block product takes 256 clocks
+// of the tensor core and 32 KB from L2, 128 bytes a clock for every SM, far
+// more than L2 delivers; shared, it is 39.
+// Warp 0 issues the TMA loads, warp 1 the MMAs, warps 2..9 drain the
+// accumulators (integer multiply-adds; the FP64 units would take longer than
+// the MMAs) and form the results from 128-bit integers, rounded once, while
+// the next tile's MMAs run. The passes run from the least significant classes
+// up; the first one's sums wait in a global buffer per CTA (L2).
+// What bounds it: the tensor cores (1.07 PFLOP/s of BF16 products at the first
+// two shapes below; N = 128 keeps shared memory busy with operand reads).
+// Measured (GB300, 40-bit digits ready, M x N x K complex), with every digit pair a
+// product of its own, FP32 sums through memory and a combining kernel, then now:
+// 19900 x 320 x 19900 48.1 -> 19.9 ms, 8000 x 1600 x 8000 25.0 -> 16.0 ms,
+// 4000 x 1000 x 200 1.63 -> 0.29 ms, 200 x 8 x 200000 2.12 -> 0.56 ms.
+struct SlArgs {
+  CUtensorMap mA, mB;
+  int M, N2, b, ns, kps, kb_per_split, ksplit, tiles_m, tiles_n, panel, items;
+  const unsigned *WA, *WB;
+  cplx *out;
+  int64_t s_m, s_nh, s_nl;
+  int n_in, amode, bmode;  // amode, bmode: 0 the factor is 1 (alpha) or 0 (beta), 1 real, 2 complex
+  cplx alpha, beta;
+  cplx *part;         // [ksplit][M][N2 / 2] partial products when ksplit > 1
+  long long *spill;   // [CTA][BN / H][32 * 4 H]
+  int *err;
 };
 
-// out[m][n] = alpha 2^(E_m + F_n) sum_p sum_s 2^-sh_p P[p][s][m][2n..2n+1] + beta out.
-// Every P is an integer below 2^24 held exactly in FP32; the pairs of one
-// shift (same i + j) and their K splits are summed exactly as 64-bit integers,
-// and only one FP64 conversion and product per shift remains (the FP64 pipe is
-// the scarce one).
-__global__ void k_sl_combine(const float *__restrict__ P, SlCombine cfg, int64_t M, int64_t N2,
-                             const int *__restrict__ E, const int *__restrict__ F, cplx alpha, cplx beta, cplx *out,
-                             int64_t s_m, int64_t s_nh, int64_t s_nl, int64_t n_in) {
-  const int64_t Nc = N2 / 2, total = M * Nc, per = M * N2;
+template <int BN>
+struct SlTile {
+  static constexpr int ABYTES = 128 * 64 * 2, BBYTES = BN * 64 * 2, STAGE = ABYTES + BBYTES;
+  static constexpr int ST = BN == 128 ? 7 : BN == 64 ? 9 : 11;
+  static constexpr int BAR_OFF = ST * STAGE;
+  static constexpr int SMEM = 1024 + BAR_OFF + 256;
+  static constexpr int H = BN >= 64 ? 2 : 1;  // column halves, four draining warps each
+  static constexpr int VALS = BN / H;         // values per draining thread
+  static constexpr uint32_t TMEM_COLS = 4 * BN;
+};
+
+struct SlItem {
+  int m0, n0, split, kb_beg, kb_end;
+};
+template <int BN>
+__device__ __forceinline__ SlItem sl_item(const SlArgs &a, int it) {
+  SlItem d;
+  const int tiles = a.tiles_m * a.tiles_n;
+  d.split = it / tiles;
+  const int t = it - d.split * tiles;
+  // panels of a.panel column tiles; row tiles inside a panel, columns fastest
+  const int full = (a.tiles_n / a.panel) * a.panel * a.tiles_m;
+  int w = a.panel, p = 0, r = t;
+  if (t < full) {
+    p = t / (a.panel * a.tiles_m);
+    r = t - p * (a.panel * a.tiles_m);
+  } else {
+    p = a.tiles_n / a.panel;
+    r = t - full;
+    w = a.tiles_n - p * a.panel;
+  }
+  const int tm = r / w;
+  d.m0 = tm * 128;
+  d.n0 = (p * a.panel + r - tm * w) * BN;
+  d.kb_beg = d.split * a.kb_per_split;
+  d.kb_end = min(a.kps, d.kb_beg + a.kb_per_split);
+  return d;
+}
+
+// highest class of a pass, classes of the pass, inner blocks per exact run
+__device__ __forceinline__ int pass_classes(int hi) { return min(4, hi - 1); }
+__device__ __forceinline__ int pass_run(int hi, int b) { return (1 << (20 - 2 * b)) / (hi == 2 ? 4 : hi + 1); }
+
+// (hi 2^sh + lo) 2^e rounded to nearest
+__device__ __forceinline__ double scaled_i128(long long hi, int sh, long long lo, int e) {
+  const __int128 t = ((__int128)hi << sh) + lo;
+  const bool neg = t < 0;
+  unsigned __int128 u = neg ? (unsigned __int128)(-t) : (unsigned __int128)t;
+  uint64_t h = (uint64_t)(u >> 64), l = (uint64_t)u;
+  if ((h | l) == 0) return 0.0;
+  int top = 127;
+  if (h == 0) { h = l; l = 0; top = 63; }
+  const int lz = __clzll((long long)h);
+  if (lz) { h = (h << lz) | (l >> (64 - lz)); l <<= lz; }
+  top -= lz;                       // value = 1.xxx 2^(top + e)
+  if (l) h |= 1;                   // sticky
+  uint64_t m = h >> 11;            // 53 bits, the leading one set
+  const uint32_t rem = (uint32_t)h & 0x7ffu;
+  if (rem > 0x400u || (rem == 0x400u && (m & 1))) ++m;
+  const int be = top + e + 1023;
+  double r;
+  if (be >= 1 && be <= 2045) {
+    r = __longlong_as_double((long long)(((uint64_t)(be - 1) << 52) + m));
+  } else {
+    r = ldexp((double)m, top + e - 52);
+  }
+  return neg ? -r : r;
+}
+
+__device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t (&v)[16]) {
+  asm volatile(
+      "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, "
+      "%13, %14, %15}, [%16];"
+      : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]),
+        "=r"(v[8]), "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]), "=r"(v[15])
+      : "r"(taddr));
+  asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+}
+
+// bounded wait that looks at the barrier before it reads the clock and the limit
+__device__ __forceinline__ bool sl_wait(uint32_t bar, uint32_t parity, volatile int *abort_flag) {
+  return mbar_try(bar, parity) || mbar_wait(bar, parity, abort_flag);
+}
+
+template <int BN>
+__global__ void __launch_bounds__(320, 1) k_sl_gemm(const __grid_constant__ SlArgs a) {
+  using L = SlTile<BN>;
+  extern __shared__ uint8_t smem_raw[];
+  uint8_t *smem = (uint8_t *)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
+  uint64_t *full = (uint64_t *)(smem + L::BAR_OFF);
+  uint64_t *empty = full + L::ST;
+  uint64_t *accf = empty + L::ST;  // a run's accumulators are complete (MMA -> draining warps)
+  uint64_t *acce = accf + 1;       // accumulator d drained (draining warps -> MMA)
+  uint64_t *fin = acce + 4;
+  uint32_t *tmem_slot = (uint32_t *)(fin + 1);
+  volatile int *abort_flag = (volatile int *)(tmem_slot + 1);
+
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  if (threadIdx.x == 0) {
+    for (int s = 0; s < L::ST; ++s) {
+      mbar_init(smem_u32(&full[s]), 1);
+      mbar_init(smem_u32(&empty[s]), 1);
+    }
+    mbar_init(smem_u32(accf), 1);
+    for (int d = 0; d < 4; ++d) mbar_init(smem_u32(&acce[d]), 4 * L::H);
+    mbar_init(smem_u32(fin), 1);
+    *abort_flag = 0;
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+  }
+  if (warp == 1) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)),
+                 "r"(L::TMEM_COLS)
+                 : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+  }
+  fence_before();
+  __syncthreads();
+  fence_after();
+  const uint32_t tmem = *tmem_slot;
+
+  if (warp == 0 && lane == 0) {
+    // ---------------- TMA producer
+    int s = 0, issued = 0, last_s = 0;
+    uint32_t par = 1;  // parity of the wait on empty[s]: the first round finds it free
+    bool stop = false;
+    for (int it = blockIdx.x; it < a.items && !stop; it += gridDim.x) {
+      const SlItem d = sl_item<BN>(a, it);
+      for (int hi = a.ns + 1; hi >= 2 && !stop; hi -= 4) {
+        for (int kb = d.kb_beg; kb < d.kb_end && !stop; ++kb) {
+          for (int i = 1; i < hi; ++i) {
+            if (!sl_wait(smem_u32(&empty[s]), par, abort_flag)) {
+              if (!*abort_flag) *(volatile int *)a.err = 21;
+              *abort_flag = 1;
+              stop = true;
+              break;
+            }
+            const uint32_t fb = smem_u32(&full[s]);
+            mbar_expect_tx(fb, L::STAGE);
+            uint8_t *sa = smem + s * L::STAGE;
+            tma_load_3d(smem_u32(sa), &a.mA, kb * 64, d.m0, i - 1, fb);
+            tma_load_3d(smem_u32(sa + L::ABYTES), &a.mB, kb * 64, d.n0, hi - i - 1, fb);
+            ++issued;
+            last_s = s;
+            if (++s == L::ST) { s = 0; par ^= 1; }
+          }
+        }
+      }
+    }
+    if (*abort_flag) {
+      // drain this CTA's copies in flight before shared memory is released: the
+      // last min(issued, ST) loads, each the (issued / ST)-th or so use of its stage
+      const int n = issued < L::ST ? issued : L::ST;
+      for (int j = 0; j < n; ++j) {
+        const int q = issued - 1 - j;  // global index of a load; its stage and use
+        int st = last_s - j;
+        if (st < 0) st += L::ST;
+        mbar_drain(smem_u32(&full[st]), (q / L::ST) & 1);
+      }
+    }
+  } else if (warp == 1 && lane == 0) {
+    // ---------------- MMA issuer
+    constexpr uint32_t idesc = idesc_bf16(128, BN);
+    int s = 0;
+    uint32_t par = 0, used = 0, epar = 0;  // used, epar: bit d: accumulator d was used, parity of its next wait
+    bool stop = false;
+    for (int it = blockIdx.x; it < a.items && !stop; it += gridDim.x) {
+      const SlItem d = sl_item<BN>(a, it);
+      for (int hi = a.ns + 1; hi >= 2 && !stop; hi -= 4) {
+        const int nd = pass_classes(hi), run = pass_run(hi, a.b);
+        for (int kb0 = d.kb_beg; kb0 < d.kb_end && !stop; kb0 += run) {
+          const int kb1 = min(d.kb_end, kb0 + run);
+          for (int kb = kb0; kb < kb1 && !stop; ++kb) {
+            for (int i = 1; i < hi; ++i) {
+              bool ok = sl_wait(smem_u32(&full[s]), par, abort_flag);
+              const int dn = min(nd, i);
+              if (ok && kb == kb0 && i <= nd && ((used >> (i - 1)) & 1u)) {
+                // first product into accumulator i - 1 of this run
+                ok = sl_wait(smem_u32(&acce[i - 1]), (epar >> (i - 1)) & 1u, abort_flag);
+                epar ^= 1u << (i - 1);
+              }
+              if (!ok) {
+                if (!*abort_flag) *(volatile int *)a.err = 22;
+                *abort_flag = 1;
+                stop = true;
+                break;
+              }
+              fence_after();
+              const uint32_t b0 = smem_u32(smem + s * L::STAGE + L::ABYTES);
+              for (int dd = 0; dd < dn; ++dd) {
+                int sa = s - dd;
+                if (sa < 0) sa += L::ST;
+                const uint32_t a0 = smem_u32(smem + sa * L::STAGE);
+                const uint32_t acc = tmem + (uint32_t)(dd * BN);
+                const bool first = (kb == kb0 && i == dd + 1);
+#pragma unroll
+                for (int k = 0; k < 4; ++k)
+                  mma_bf16(acc, sdesc(a0 + 32 * k), sdesc(b0 + 32 * k), idesc, (first && k == 0) ? 0u : 1u);
+              }
+              if (kb == kb0 && i <= nd) used |= 1u << (i - 1);
+              // digit i - nd + 1 of A has met its last partner; at the end of the block all have
+              if (i >= nd) {
+                int se = s - (nd - 1);
+                if (se < 0) se += L::ST;
+                mma_commit(smem_u32(&empty[se]));
+              }
+              if (i == hi - 1)
+                for (int e = nd - 2; e >= 0; --e) {
+                  int se = s - e;
+                  if (se < 0) se += L::ST;
+                  mma_commit(smem_u32(&empty[se]));
+                }
+              if (++s == L::ST) { s = 0; par ^= 1; }
+            }
+          }
+          if (!stop) mma_commit(smem_u32(accf));
+        }
+      }
+    }
+    // every MMA this thread issued has finished before TMEM is freed
+    mma_commit(smem_u32(fin));
+    mbar_drain(smem_u32(fin), 0);
+  } else if (warp >= 2 && warp < 2 + 4 * L::H) {
+    // ---------------- draining warps
+    const int q = warp & 3, half = (warp - 2) >> 2;
+    const int tid = (warp - 2) * 32 + lane;
+    constexpr int NT = 128 * L::H;
+    const uint32_t tbase = tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(half * L::VALS);
+    long long *sp = a.spill + (int64_t)blockIdx.x * L::VALS * NT + tid;
+    uint32_t par = 0;
+    bool ok = true;
+    for (int it = blockIdx.x; it < a.items; it += gridDim.x) {
+      const SlItem d = sl_item<BN>(a, it);
+      long long acc[L::VALS];
+      int sh = 0;  // the pass's weight against the first one's: 4 b bits per pass
+      for (int hi = a.ns + 1; hi >= 2 && ok; hi -= 4) {
+        const int nd = pass_classes(hi), run = pass_run(hi, a.b);
+#pragma unroll
+        for (int j = 0; j < L::VALS; ++j) acc[j] = 0;
+        for (int kb0 = d.kb_beg; kb0 < d.kb_end; kb0 += run) {
+          ok = __all_sync(0xffffffffu, sl_wait(smem_u32(accf), par, abort_flag));
+          if (!ok) {
+            if (lane == 0 && !*abort_flag) { *(volatile int *)a.err = 23; *abort_flag = 1; }
+            break;
+          }
+          par ^= 1;
+          fence_after();
+          for (int dd = 0; dd < nd; ++dd) {
+            const int w = 1 << (a.b * dd);
+#pragma unroll
+            for (int c0 = 0; c0 < L::VALS; c0 += 16) {
+              uint32_t v[16];
+              tmem_ld16(tbase + (uint32_t)(dd * BN + c0), v);
+#pragma unroll
+              for (int j = 0; j < 16; ++j) acc[c0 + j] += (long long)__float2int_rn(__uint_as_float(v[j])) * w;
+            }
+            fence_before();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(smem_u32(&acce[dd]));
+          }
+        }
+        if (ok && hi > 5) {  // another pass follows: the sums so far, in units of the first pass, wait
+          if (sh == 0) {
+#pragma unroll
+            for (int j = 0; j < L::VALS; ++j) sp[(int64_t)j * NT] = acc[j];
+          } else {
+#pragma unroll
+            for (int j = 0; j < L::VALS; ++j) sp[(int64_t)j * NT] += acc[j] << sh;
+          }
+          sh += 4 * a.b;
+        }
+      }
+      // ---- results, in units of 2^(-b (ns + 1))
+      const int64_t m = (int64_t)d.m0 + q * 32 + lane;
+      if (m >= a.M) continue;
+      const unsigned wa = a.WA[m];
+      const int n_beg = (d.n0 + half * L::VALS) >> 1;
+      const int Nc = a.N2 >> 1;
+      int nh = n_beg / a.n_in, nl = n_beg - nh * a.n_in;
+#pragma unroll
+      for (int j = 0; j < L::VALS / 2; ++j) {
+        const int n = n_beg + j;
+        if (n < Nc) {
+          const unsigned wb = a.WB[n];
+          cplx val;
+          if (!ok || not_finite(wa) || not_finite(wb)) {
+            // (after a wait that gave up the tile holds no result)
+            val = cmake(__longlong_as_double(0x7ff8000000000000ll), __longlong_as_double(0x7ff8000000000000ll));
+          } else {
+            const int e = scale_exp(wa) + scale_exp(wb) - a.b * (a.ns + 1);
+            const long long lr = sh ? sp[(int64_t)(2 * j) * NT] : 0, li = sh ? sp[(int64_t)(2 * j + 1) * NT] : 0;
+            val = cmake(scaled_i128(acc[2 * j], sh, lr, e), scaled_i128(acc[2 * j + 1], sh, li, e));
+          }
+          if (a.part) {
+            a.part[((int64_t)d.split * a.M + m) * Nc + n] = val;
+          } else {
+            cplx *dst = a.out + m * a.s_m + nh * a.s_nh + nl * a.s_nl;
+            if (a.amode == 1) val = cscale(val, a.alpha.x);
+            else if (a.amode == 2) val = cmul(a.alpha, val);
+            if (a.bmode == 1) { const cplx o = *dst; val = cmake(val.x + a.beta.x * o.x, val.y + a.beta.x * o.y); }
+            else if (a.bmode == 2) val = cadd(val, cmul(a.beta, *dst));
+            *dst = val;
+          }
+        }
+        if (++nl == a.n_in) { nl = 0; ++nh; }
+      }
+    }
+  }
+  fence_before();
+  __syncthreads();
+  if (warp == 1) {
+    __syncwarp();
+    fence_after();
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(L::TMEM_COLS) : "memory");
+  }
+}
+
+// out = alpha sum_s part[s] + beta out, the splits in order
+__global__ void k_sl_reduce(const cplx *__restrict__ part, int ksplit, int64_t M, int64_t Nc, cplx *out, int64_t s_m,
+                            int64_t s_nh, int64_t s_nl, int64_t n_in, cplx alpha, cplx beta) {
+  const int64_t total = M * Nc;
   const bool use_beta = (beta.x != 0.0 || beta.y != 0.0);
   for (int64_t idx = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; idx < total;
        idx += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t n = idx % Nc, m = idx / Nc;
-    const float *base = P + m * N2 + 2 * n;
-    double re = 0.0, im = 0.0;
-    long long ar = 0, ai = 0;
-    for (int p = cfg.npair - 1; p >= 0; --p) {  // smallest terms first
-      for (int s = 0; s < cfg.ksplit; ++s) {
-        const float2 v = *(const float2 *)(base + ((int64_t)p * cfg.ksplit + s) * per);
-        ar += __float2int_rn(v.x);
-        ai += __float2int_rn(v.y);
-      }
-      if (p == 0 || cfg.sh[p - 1] != cfg.sh[p]) {  // last pair of this shift
-        re = fma((double)ar, cfg.sc[p], re);
-        im = fma((double)ai, cfg.sc[p], im);
-        ar = 0;
-        ai = 0;
-      }
-    }
-    const int e = E[m] + F[n];
-    const cplx val0 = cmake(ldexp(re, e), ldexp(im, e));
+    const int64_t m = idx / Nc, n = idx - m * Nc;
+    cplx v = cmake(0.0, 0.0);
+    for (int s = 0; s < ksplit; ++s) v = cadd(v, part[(int64_t)s * total + idx]);
     const int64_t nh = n / n_in, nl = n - nh * n_in;
     cplx *dst = out + m * s_m + nh * s_nh + nl * s_nl;
-    cplx val = cmul(alpha, val0);
-    if (use_beta) val = cadd(val, cmul(beta, *dst));
-    *dst = val;
+    v = cmul(alpha, v);
+    if (use_beta) v = cadd(v, cmul(beta, *dst));
+    *dst = v;
   }
 }
 
-int ceil_log2(int64_t x) {
-  int l = 0;
-  while ((1ll << l) < x) ++l;
-  return l;
-}
-
-void set_views(SlMat &d) {
-  const int64_t pe = d.rows * 2 * d.kp;
-  d.s.resize(d.ns);
-  for (int i = 0; i < d.ns; ++i) {
-    TcMat &t = d.s[i];
-    t.hi.ex = nullptr;  // a view into d.planes
-    t.hi.p = (__nv_bfloat16 *)d.planes.p + (int64_t)i * pe;
-    t.hi.bytes = (size_t)pe * sizeof(__nv_bfloat16);
-    t.planes = 1;
-    t.rows = d.rows;
-    t.kp = d.kp;
-    t.kreal = d.kreal;
-  }
-}
-
-void alloc_sl(Exec &ex, SlMat &d, int64_t rows, int64_t expn) {
+void alloc_sl(Exec &ex, SlMat &d, int64_t rows, int64_t nscale) {
   const size_t bytes = (size_t)d.ns * rows * 2 * d.kp * sizeof(__nv_bfloat16);
   if (d.planes.bytes < bytes) {
-    d.s.clear();
     d.planes.reset();
     d.planes = DBuf(ex, bytes);
   }
-  if (d.exps.bytes < (size_t)expn * sizeof(int)) {
+  if (d.exps.bytes < (size_t)nscale * sizeof(unsigned)) {
     d.exps.reset();
-    d.exps = DBuf(ex, (size_t)std::max<int64_t>(expn, 1) * sizeof(int));
+    d.exps = DBuf(ex, (size_t)std::max<int64_t>(nscale, 1) * sizeof(unsigned));
   }
   d.rows = rows;
-  set_views(d);
+}
+
+// scales and digits of `rows` complex rows (emb 1: A rows, 2: B rows)
+void pack_rows(Exec &ex, SlMat &d, const BSrc &s, int64_t rows, int64_t K, bool conj, int emb) {
+  alloc_sl(ex, d, emb * rows, rows);
+  if (rows <= 0) return;
+  ADC_REQUIRE(s.mode == 0 || K < (1ll << 31), ADC_ERR_UNSUPPORTED, "sliced product: ring size");
+  const int kfast = (s.mode != 0 || s.s_k == 1 || s.s_nl != 1) ? 1 : 0;
+  const int64_t rt = (rows + PK_R - 1) / PK_R;
+  const unsigned gx = (unsigned)std::min<int64_t>(rt, 1 << 20);
+  unsigned *W = (unsigned *)d.exps.p;
+  fill_zero(ex, W, rows * sizeof(unsigned));
+  // inner ranges: enough blocks to fill the GPU, each at least 512 elements long
+  const int64_t want = 8ll * device_sm_count();
+  const int64_t parts = std::max<int64_t>(1, std::min<int64_t>((K + 511) / 512, (want + rt - 1) / rt));
+  int64_t krange = (std::max<int64_t>(K, 1) + parts - 1) / parts;
+  krange = (krange + PK_K - 1) / PK_K * PK_K;
+  const unsigned gy = (unsigned)((std::max<int64_t>(K, 1) + krange - 1) / krange);
+  int pr = ex.prof_begin("sl_pack", 0.0, (double)rows * (16.0 * K + 4.0 * emb * d.ns * d.kp));
+  k_sl_scale<<<dim3(gx, gy), 256, 0, ex.stream>>>(s, rows, K, krange, kfast, W);
+  ADC_CHECK_LAUNCH();
+  const dim3 grid(gx, (unsigned)std::min<int64_t>(d.kp / PK_K, 65535));
+  const int64_t pe = (int64_t)emb * rows * 2 * d.kp;
+  if (emb == 1)
+    k_sl_pack<1><<<grid, 256, 0, ex.stream>>>(s, rows, K, conj ? 1 : 0, d.kp, kfast, W, d.b, d.ns,
+                                              (__nv_bfloat16 *)d.planes.p, pe);
+  else
+    k_sl_pack<2><<<grid, 256, 0, ex.stream>>>(s, rows, K, conj ? 1 : 0, d.kp, kfast, W, d.b, d.ns,
+                                              (__nv_bfloat16 *)d.planes.p, pe);
+  ADC_CHECK_LAUNCH();
+  ex.prof_end(pr);
+}
+
+template <int BN>
+void launch_sl(Exec &ex, SlArgs &g, SlWork &w, int grid) {
+  using L = SlTile<BN>;
+  set_smem_limit((const void *)k_sl_gemm<BN>, L::SMEM);
+  const size_t need = (size_t)grid * L::VALS * 128 * L::H * sizeof(long long);
+  if (g.ns > 4 && w.spill.bytes < need) {
+    w.spill.reset();
+    w.spill = DBuf(ex, need);
+  }
+  g.spill = (long long *)w.spill.p;
+  k_sl_gemm<BN><<<grid, 320, L::SMEM, ex.stream>>>(g);
+  ADC_CHECK_LAUNCH();
 }
 
 }  // namespace
 
-SlParams sl_params(int64_t K, int bits) {
-  SlParams p;
-  p.kp = (K + 63) / 64 * 64;
-  if (p.kp == 0) p.kp = 64;
-  const int64_t K2 = 2 * p.kp;
-  int b = (24 - ceil_log2(K2)) / 2;
-  b = std::max(4, std::min(7, b));
-  p.b = b;
-  p.ns = (bits + b - 1) / b;
-  p.kb_split = (int)((1ll << (24 - 2 * b)) / 64);
-  return p;
-}
+void sl_set_wait_ns(unsigned long long ns) { ADC_CUDA(cudaMemcpyToSymbol(g_wait_ns, &ns, sizeof(ns))); }
 
 void sl_pack_A(Exec &ex, SlMat &dst, const cplx *src, int64_t M, int64_t K, int64_t s_m, int64_t s_k, bool conj,
                int bits) {
-  const SlParams p = sl_params(K, bits);
-  dst.kp = p.kp;
+  const SlDigits dg = sl_digits(K, bits);
+  dst.kp = sl_kp(K);
   dst.kreal = K;
-  dst.ns = p.ns;
-  dst.bits = p.b;
-  dst.kb_split = p.kb_split;
-  alloc_sl(ex, dst, M, M);
-  if (M <= 0) return;
-  k_sl_exp_A<<<(unsigned)std::min<int64_t>(M, 65535), 256, 0, ex.stream>>>(src, M, K, s_m, s_k, (int *)dst.exps.p);
-  ADC_CHECK_LAUNCH();
-  k_sl_slice_A<<<grid1d(M * (dst.kp / 8), 256), 256, 0, ex.stream>>>(src, M, K, s_m, s_k, conj ? 1 : 0, dst.kp,
-                                                               (const int *)dst.exps.p, dst.ns, dst.bits,
-                                                               (__nv_bfloat16 *)dst.planes.p, M * 2 * dst.kp);
-  ADC_CHECK_LAUNCH();
+  dst.b = dg.b;
+  dst.ns = dg.ns;
+  const BSrc s{src, 0, 0, s_m, std::max<int64_t>(M, 1), s_k, 0, 0, 0, 0};
+  pack_rows(ex, dst, s, M, K, conj, 1);
 }
 
 static void sl_pack_B_impl(Exec &ex, SlMat &dst, const BSrc &s, int64_t Nc, int64_t K, bool conj, const SlMat &like,
@@ -288,24 +674,18 @@ static void sl_pack_B_impl(Exec &ex, SlMat &dst, const BSrc &s, int64_t Nc, int6
   ADC_REQUIRE(like.kreal == K, ADC_ERR_ARG, "sl_pack_B: inner size differs from the A operand");
   dst.kp = like.kp;
   dst.kreal = K;
-  // fewer significant bits: the leading digits of the same width (the product
-  // then runs over the common leading slices of both operands)
-  dst.ns = bits > 0 ? std::min(like.ns, (bits + like.bits - 1) / like.bits) : like.ns;
-  dst.bits = like.bits;
-  dst.kb_split = like.kb_split;
-  alloc_sl(ex, dst, 2 * Nc, Nc);
-  if (Nc <= 0) return;
-  k_sl_exp_B<<<(unsigned)std::min<int64_t>(Nc, 65535), 256, 0, ex.stream>>>(s, Nc, K, (int *)dst.exps.p);
-  ADC_CHECK_LAUNCH();
-  k_sl_slice_B<<<grid1d(Nc * (dst.kp / 8), 256), 256, 0, ex.stream>>>(s, Nc, K, conj ? 1 : 0, dst.kp,
-                                                                (const int *)dst.exps.p, dst.ns, dst.bits,
-                                                                (__nv_bfloat16 *)dst.planes.p, 2 * Nc * 2 * dst.kp);
-  ADC_CHECK_LAUNCH();
+  // fewer significant bits: the leading digits (the product then runs over the
+  // common leading slices of both operands)
+  dst.b = like.b;
+  dst.ns = bits > 0 ? std::min(like.ns, (bits + like.b - 1) / like.b) : like.ns;
+  pack_rows(ex, dst, s, Nc, K, conj, 2);
 }
 
 void sl_pack_B(Exec &ex, SlMat &dst, const cplx *src, int64_t Nc, int64_t K, int64_t s_nh, int64_t s_nl,
                int64_t n_in, int64_t s_k, bool conj, const SlMat &like, int bits) {
   BSrc s{src, 0, s_nh, s_nl, n_in, s_k, 0, 0, 0, 0};
+  // one row index: strides as an A operand, so that the packing sees which index is contiguous
+  if (n_in == 1) { s.n_in = std::max<int64_t>(Nc, 1); s.s_nl = s_nh; s.s_nh = 0; }
   sl_pack_B_impl(ex, dst, s, Nc, K, conj, like, bits);
 }
 
@@ -317,130 +697,180 @@ void sl_pack_B_ring(Exec &ex, SlMat &dst, const adc_ctx *c, const cplx *X, int64
 
 void sl_gemm(Exec &ex, const SlMat &A, const SlMat &B, int64_t M, int64_t N, cplx alpha, cplx beta, cplx *out,
              int64_t s_m, int64_t s_nh, int64_t s_nl, int64_t n_in, int *err, SlWork &w) {
-  ADC_REQUIRE(A.kp == B.kp && A.bits == B.bits, ADC_ERR_ARG, "sl_gemm: operands sliced differently");
-  const int ns = std::min(A.ns, B.ns);  // the common leading slices
+  ADC_REQUIRE(A.kp == B.kp && A.b == B.b, ADC_ERR_ARG, "sl_gemm: operands sliced differently");
   ADC_REQUIRE(A.rows >= M && B.rows >= 2 * N, ADC_ERR_ARG, "sl_gemm: operand rows");
   if (M <= 0 || N <= 0) return;
+  ADC_REQUIRE(M < (1ll << 31) && 2 * N < (1ll << 31), ADC_ERR_UNSUPPORTED, "sl_gemm: size");
   if (n_in <= 0) n_in = 1;
-  const int64_t N2 = 2 * N;
-  const int kps = (int)(2 * A.kp / 64);
-  const int kbs = std::min(A.kb_split, kps);
-  const int ksplit = (kps + kbs - 1) / kbs;
-  SlCombine cfg{};
-  std::vector<std::pair<int, int>> pairs;
-  for (int g = 2; g <= ns + 1; ++g)
-    for (int i = 1; i < g; ++i)
-      if (i <= ns && g - i <= ns) pairs.push_back({i, g - i});
-  ADC_REQUIRE((int)pairs.size() <= SL_MAXPAIRS, ADC_ERR_UNSUPPORTED, "sl_gemm: too many slice pairs");
-  cfg.npair = (int)pairs.size();
-  cfg.ksplit = ksplit;
-  for (size_t q = 0; q < pairs.size(); ++q) {
-    cfg.sh[q] = A.bits * (pairs[q].first + pairs[q].second);
-    cfg.sc[q] = std::ldexp(1.0, -cfg.sh[q]);
+  const int sms = device_sm_count();
+  SlArgs g{};
+  g.b = A.b;
+  g.ns = std::min(A.ns, B.ns);  // the common leading slices
+  const int64_t N2 = 2 * N, kp2 = 2 * A.kp;
+  const int bn = N2 <= 32 ? 32 : N2 <= 64 ? 64 : 128;
+  tc_make_map3(&g.mA, A.planes.p, A.rows, kp2, A.ns, A.rows * kp2, 128);
+  tc_make_map3(&g.mB, B.planes.p, B.rows, kp2, B.ns, B.rows * kp2, bn);
+  g.M = (int)M;
+  g.N2 = (int)N2;
+  g.kps = (int)(kp2 / 64);
+  g.tiles_m = (int)((M + 127) / 128);
+  g.tiles_n = (int)((N2 + bn - 1) / bn);
+  g.panel = std::min(g.tiles_n, 8);
+  g.WA = (const unsigned *)A.exps.p;
+  g.WB = (const unsigned *)B.exps.p;
+  g.out = out;
+  g.s_m = s_m; g.s_nh = s_nh; g.s_nl = s_nl;
+  // one column group covers every column when n_in reaches past them
+  g.n_in = (int)std::min<int64_t>(n_in, N);
+  g.alpha = alpha;
+  g.beta = beta;
+  g.amode = alpha.y != 0.0 ? 2 : alpha.x != 1.0 ? 1 : 0;
+  g.bmode = beta.y != 0.0 ? 2 : beta.x != 0.0 ? 1 : 0;
+  g.err = err;
+  // inner splits: the count that leaves the fewest rounds of work, in units of
+  // inner blocks, a tile's fixed cost being that of about three blocks; at
+  // least eight blocks per split, partial products within 1 GiB
+  const int64_t tiles = (int64_t)g.tiles_m * g.tiles_n;
+  int best = 1;
+  double cost = 1e300;
+  for (int s = 1; s <= 64 && (s == 1 || g.kps / s >= 8); ++s) {
+    if (s > 1 && (double)s * M * N * sizeof(cplx) > (double)(1ll << 30)) break;
+    const double c = (double)((tiles * s + sms - 1) / sms) * ((g.kps + s - 1) / s + 3.0) * (s > 1 ? 1.05 : 1.0);
+    if (c < cost) { cost = c; best = s; }
   }
-  // output rows in chunks whose FP32 pair products stay within about 2 GiB
-  const size_t per_row = (size_t)ksplit * N2 * pairs.size() * sizeof(float);
-  const size_t budget = (size_t)2 << 30;
-  int64_t mc = M;
-  if ((size_t)M * per_row > budget) mc = std::max<int64_t>(128, (int64_t)(budget / per_row) / 128 * 128);
-  const size_t need = per_row * (size_t)std::min(mc, M);
-  if (w.part.bytes < need) {
-    w.part.reset();
-    w.part = DBuf(ex, need);
+  g.kb_per_split = (g.kps + best - 1) / best;
+  g.ksplit = (g.kps + g.kb_per_split - 1) / g.kb_per_split;
+  ADC_REQUIRE(tiles * g.ksplit < (1ll << 31), ADC_ERR_UNSUPPORTED, "sl_gemm: too many tiles");
+  g.items = (int)(tiles * g.ksplit);
+  if (g.ksplit > 1) {
+    const size_t need = (size_t)g.ksplit * M * N * sizeof(cplx);
+    if (w.part.bytes < need) {
+      w.part.reset();
+      try {
+        w.part = DBuf(ex, need);
+      } catch (const Error &e) {
+        if (e.code != ADC_ERR_OOM) throw;
+        g.ksplit = 1;  // no room for partial products: whole inner sums
+        g.kb_per_split = g.kps;
+        g.items = (int)tiles;
+      }
+    }
+    if (g.ksplit > 1) g.part = w.part.c();
   }
-  const int bn = N2 <= 32 ? 32 : N2 <= 64 ? 64 : N2 <= 128 ? 128 : 256;
-  std::vector<TcMat> av(ns);
-  for (int64_t m0 = 0; m0 < M; m0 += mc) {
-    const int64_t mm = std::min(mc, M - m0);
-    const size_t per = (size_t)ksplit * mm * N2;
-    for (int i = 0; i < ns; ++i) {  // views of rows m0 .. m0 + mm of the A slices used
-      TcMat &t = av[i];
-      t.hi.ex = nullptr;
-      t.hi.p = (__nv_bfloat16 *)A.s[i].hi.p + m0 * 2 * A.kp;
-      t.hi.bytes = (size_t)mm * 2 * A.kp * sizeof(__nv_bfloat16);
-      t.planes = 1;
-      t.rows = mm;
-      t.kp = A.kp;
-      t.kreal = A.kreal;
-    }
-    std::vector<TcJobDesc> jobs(pairs.size());
-    for (size_t q = 0; q < pairs.size(); ++q) {
-      TcJobDesc &d = jobs[q];
-      d.A = &av[pairs[q].first - 1];
-      d.B = &B.s[pairs[q].second - 1];
-      d.M = mm;
-      d.N = N;
-      d.nseg = 1;
-      d.out32 = (float *)w.part.p + q * per;
-      d.kb_split = kbs;
-      d.bn = bn;
-    }
-    tc_gemm_grouped(ex, jobs, w.grp, err, false);
-    int pr = ex.prof_begin("sl_combine", 0.0);
-    k_sl_combine<<<grid1d(mm * N, 256), 256, 0, ex.stream>>>((const float *)w.part.p, cfg, mm, N2,
-                                                             (const int *)A.exps.p + m0, (const int *)B.exps.p,
-                                                             alpha, beta, out + m0 * s_m, s_m, s_nh, s_nl, n_in);
+  const int grid = (int)std::min<int64_t>(g.items, sms);
+  int pr = ex.prof_begin("tc_sliced", 8.0 * (double)M * (double)N * (double)A.kreal);
+  if (bn == 32) launch_sl<32>(ex, g, w, grid);
+  else if (bn == 64) launch_sl<64>(ex, g, w, grid);
+  else launch_sl<128>(ex, g, w, grid);
+  if (g.ksplit > 1) {
+    k_sl_reduce<<<grid1d(M * N, 256), 256, 0, ex.stream>>>(g.part, g.ksplit, M, N, out, s_m, s_nh, s_nl, g.n_in,
+                                                           alpha, beta);
     ADC_CHECK_LAUNCH();
-    ex.prof_end(pr);
-    for (auto &t : av) { t.hi.p = nullptr; t.hi.bytes = 0; }
   }
-  for (auto &t : av) { t.hi.p = nullptr; t.hi.bytes = 0; }
+  ex.prof_end(pr);
 }
 
-// zgemm's operands and output (element strides, conj flags, batch) through
-// the sliced product: used for large contractions when Exec::sliced_bits > 0
+// ---------------------------------------------------------------- zgemm through the digits
 // > 0: fixed bytes per operand chunk of zgemm_sliced instead of the free-memory rule (test hook)
 static size_t g_sliced_cap = 0;
 void set_sliced_cap_bytes(size_t bytes) { g_sliced_cap = bytes; }
 
-void zgemm_sliced(Exec &ex, int64_t M, int64_t N, int64_t K, int64_t batch, cplx alpha, const cplx *A, int64_t sAb,
-                  int64_t sAm, int64_t sAk, bool conjA, const cplx *B, int64_t sBb, int64_t sBk, int64_t sBn,
-                  bool conjB, cplx beta, cplx *C, int64_t sCb, int64_t sCm, int64_t sCn) {
-  SlMat Sa, Sb;
-  SlWork w;
-  DBuf err(ex, sizeof(int));
-  fill_zero(ex, err.p, sizeof(int));
-  // the digit planes take 4 ns kp bytes per row of A and 8 ns kp per column
-  // of B (ns slices of the real embedding): rows and columns in chunks whose
-  // planes stay within an eighth of the free device memory per operand
-  // (between 1 and 16 GiB), so that B is sliced once where it fits. When even
-  // one 128-row tile of A or 64 columns of B would exceed that, the inner
-  // index is split as well: the partial products (each FP64-accurate) add up
-  // in the output.
-  size_t fr = 0, tot = 0;
-  if (cudaMemGetInfo(&fr, &tot) != cudaSuccess) {
-    cudaGetLastError();
-    fr = (size_t)32 << 30;
-  }
-  const size_t cap =
-      g_sliced_cap ? g_sliced_cap : std::min<size_t>((size_t)16 << 30, std::max<size_t>((size_t)1 << 30, fr / 8));
+namespace {
+
+// One batch entry (or a batch folded into the column index: columns n of B at
+// (n / n_in) sBh + (n % n_in) sBn, of C at (n / n_in) sCh + (n % n_in) sCn) in
+// chunks. The digit planes take 4 ns kp bytes per row of A and 8 ns kp per
+// column of B (ns slices of the real embedding): rows and columns in chunks
+// whose planes stay within `cap` bytes per operand, so that B is sliced once
+// where it fits. When even one 128-row tile of A or 64 columns of B would
+// exceed that, the inner index is split as well: the partial products (each
+// FP64-accurate) add up in the output. `begun` is set once C may have changed.
+void digit_product(Exec &ex, int64_t M, int64_t N, int64_t K, cplx alpha, const cplx *A, int64_t sAm, int64_t sAk,
+                   bool conjA, const cplx *B, int64_t sBk, int64_t sBh, int64_t sBn, int64_t n_in, bool conjB,
+                   cplx beta, cplx *C, int64_t sCm, int64_t sCh, int64_t sCn, int bits, size_t cap, int *err,
+                   SlMat &Sa, SlMat &Sb, SlWork &w, bool &begun) {
+  const size_t ns = (size_t)sl_digits(K, bits).ns;
   int64_t kc = K;
   {
-    const SlParams sp = sl_params(K, ex.sliced_bits);
-    const size_t per = (size_t)4 * sp.ns * sp.kp * 128;  // one A row tile (B: 64 columns, the same bytes)
+    const size_t per = 4 * ns * (size_t)sl_kp(K) * 128;  // one A row tile (B: 64 columns, the same bytes)
     if (per > cap) kc = std::max<int64_t>(512, (int64_t)((double)K * (double)cap / (double)per) / 64 * 64);
   }
   for (int64_t k0 = 0; k0 < K; k0 += kc) {
     const int64_t kk = std::min(kc, K - k0);
     const cplx beta_k = (k0 == 0) ? beta : C1();
-    const SlParams sp = sl_params(kk, ex.sliced_bits);
-    const int64_t mc = std::min<int64_t>(M, std::max<int64_t>(128, (int64_t)(cap / ((size_t)4 * sp.ns * sp.kp))));
-    const int64_t nc = std::min<int64_t>(N, std::max<int64_t>(64, (int64_t)(cap / ((size_t)8 * sp.ns * sp.kp))));
-    for (int64_t b = 0; b < batch; ++b) {
-      const cplx *Ab = A + b * sAb + k0 * sAk, *Bb = B + b * sBb + k0 * sBk;
-      for (int64_t m0 = 0; m0 < M; m0 += mc) {
-        const int64_t mm = std::min(mc, M - m0);
-        sl_pack_A(ex, Sa, Ab + m0 * sAm, mm, kk, sAm, sAk, conjA, ex.sliced_bits);
-        for (int64_t n0 = 0; n0 < N; n0 += nc) {
-          const int64_t nn = std::min(nc, N - n0);
-          // B once per batch entry and inner chunk when it fits in one chunk
-          if (nc < N || m0 == 0) sl_pack_B(ex, Sb, Bb + n0 * sBn, nn, kk, sBn, 0, 1, sBk, conjB, Sa);
-          sl_gemm(ex, Sa, Sb, mm, nn, alpha, beta_k, C + b * sCb + m0 * sCm + n0 * sCn, sCm, sCn, 0, 1,
-                  (int *)err.p, w);
-        }
+    const size_t kp = (size_t)sl_kp(kk), ns = (size_t)sl_digits(kk, bits).ns;
+    const int64_t mc = std::min<int64_t>(M, std::max<int64_t>(128, (int64_t)(cap / (4 * ns * kp))));
+    int64_t nc = std::min<int64_t>(N, std::max<int64_t>(64, (int64_t)(cap / (8 * ns * kp))));
+    if (nc < N && n_in < N) nc = std::max<int64_t>(1, nc / n_in) * n_in;  // whole column groups
+    for (int64_t m0 = 0; m0 < M; m0 += mc) {
+      const int64_t mm = std::min(mc, M - m0);
+      sl_pack_A(ex, Sa, A + m0 * sAm + k0 * sAk, mm, kk, sAm, sAk, conjA, bits);
+      for (int64_t n0 = 0; n0 < N; n0 += nc) {
+        const int64_t nn = std::min(nc, N - n0);
+        const int64_t bo = (n_in < N) ? n0 / n_in * sBh : n0 * sBn, co = (n_in < N) ? n0 / n_in * sCh : n0 * sCn;
+        // B once per inner chunk when it fits in one chunk
+        if (nc < N || m0 == 0) sl_pack_B(ex, Sb, B + bo + k0 * sBk, nn, kk, sBh, sBn, n_in, sBk, conjB, Sa);
+        sl_gemm(ex, Sa, Sb, mm, nn, alpha, beta_k, C + m0 * sCm + co, sCm, sCh, sCn, n_in, err, w);
+        begun = true;
       }
     }
   }
+}
+
+// bytes per operand chunk: an eighth of the free device memory, between 1 and 16 GiB (need:
+// the larger operand's planes; the free memory is looked up only when they exceed 1 GiB)
+size_t digit_cap(double need) {
+  if (g_sliced_cap) return g_sliced_cap;
+  if (need <= (double)(1ll << 30)) return (size_t)1 << 30;
+  size_t fr = 0, tot = 0;
+  if (cudaMemGetInfo(&fr, &tot) != cudaSuccess) {
+    cudaGetLastError();
+    fr = (size_t)32 << 30;
+  }
+  return std::min<size_t>((size_t)16 << 30, std::max<size_t>((size_t)1 << 30, fr / 8));
+}
+
+// zgemm's operands and output (element strides, conj flags, batch). The larger
+// of M and N becomes the A side (half the bytes per digit); a batch whose A
+// (or, with the roles exchanged, B) is shared becomes a longer column index.
+void digit_zgemm(Exec &ex, int64_t M, int64_t N, int64_t K, int64_t batch, cplx alpha, const cplx *A, int64_t sAb,
+                 int64_t sAm, int64_t sAk, bool conjA, const cplx *B, int64_t sBb, int64_t sBk, int64_t sBn,
+                 bool conjB, cplx beta, cplx *C, int64_t sCb, int64_t sCm, int64_t sCn, int bits, int *err,
+                 bool &begun) {
+  const bool fold = batch > 1 && (sAb == 0 || sBb == 0);
+  if (fold ? sAb != 0 : N > M) {
+    std::swap(M, N);
+    std::swap(A, B);
+    std::swap(sAb, sBb);
+    std::swap(sAm, sBn);
+    std::swap(sAk, sBk);
+    std::swap(conjA, conjB);
+    std::swap(sCm, sCn);
+  }
+  SlMat Sa, Sb;
+  SlWork w;
+  const size_t cap = digit_cap(4.0 * sl_digits(K, bits).ns * (double)sl_kp(K) * std::max<double>(M, 2.0 * N * (fold ? batch : 1)));
+  if (fold) {
+    digit_product(ex, M, N * batch, K, alpha, A, sAm, sAk, conjA, B, sBk, sBb, sBn, N, conjB, beta, C, sCm, sCb, sCn,
+                  bits, cap, err, Sa, Sb, w, begun);
+    return;
+  }
+  for (int64_t b = 0; b < batch; ++b)
+    digit_product(ex, M, N, K, alpha, A + b * sAb, sAm, sAk, conjA, B + b * sBb, sBk, 0, sBn, N, conjB, beta,
+                  C + b * sCb, sCm, 0, sCn, bits, cap, err, Sa, Sb, w, begun);
+}
+
+}  // namespace
+
+// zgemm as the sliced product: large contractions when Exec::sliced_bits > 0
+void zgemm_sliced(Exec &ex, int64_t M, int64_t N, int64_t K, int64_t batch, cplx alpha, const cplx *A, int64_t sAb,
+                  int64_t sAm, int64_t sAk, bool conjA, const cplx *B, int64_t sBb, int64_t sBk, int64_t sBn,
+                  bool conjB, cplx beta, cplx *C, int64_t sCb, int64_t sCm, int64_t sCn) {
+  DBuf err(ex, sizeof(int));
+  fill_zero(ex, err.p, sizeof(int));
+  bool begun = false;
+  digit_zgemm(ex, M, N, K, batch, alpha, A, sAb, sAm, sAk, conjA, B, sBb, sBk, sBn, conjB, beta, C, sCb, sCm, sCn,
+              ex.sliced_bits, (int *)err.p, begun);
   int h = 0;
   ADC_CUDA(cudaMemcpyAsync(&h, err.p, sizeof(int), cudaMemcpyDeviceToHost, ex.stream));
   ADC_CUDA(cudaStreamSynchronize(ex.stream));

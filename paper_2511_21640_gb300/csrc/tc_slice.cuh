@@ -7,28 +7,42 @@
 
 namespace adc {
 
-// slicing of an inner size K: padded kp, digit width b (4..7 bits), slices ns
-// for about `bits` significant bits, k-blocks of 64 per exact FP32 split
-struct SlParams {
-  int64_t kp = 0;
-  int b = 0, ns = 0, kb_split = 0;
+// digits of an operand: ns of b bits
+struct SlDigits {
+  int b, ns;
 };
-SlParams sl_params(int64_t K, int bits);
+// Seven-bit digits, the widest whose products FP32 sums exactly over useful runs (eight-bit
+// ones drain four times as often): 4 and 6 of them for about 24 and 40 bits.
+// The setup's 48-bit products take digits whose whole inner sum fits FP32 (b = 7 .. 4
+// as the inner size grows): which bits of the operators they keep depends on the
+// digits, and the BF16 split of an operator must not change with how it was computed.
+inline SlDigits sl_digits(int64_t K, int bits) {
+  int b = 7;
+  if (bits > 40) {
+    const int64_t K2 = K <= 0 ? 128 : (K + 63) / 64 * 128;
+    int l = 0;
+    while ((1ll << l) < K2) ++l;
+    b = (24 - l) / 2;
+    b = b < 4 ? 4 : b > 7 ? 7 : b;
+  }
+  return {b, (bits + b - 1) / b};
+}
+// inner size as stored: padded to whole blocks of 64
+inline int64_t sl_kp(int64_t K) { return K <= 0 ? 64 : (K + 63) / 64 * 64; }
 
 // An operand as ns BF16 planes of integer digits, [rows][2*kp] each, and one
-// power-of-two exponent per row (A: per row; B: per complex row, shared by its
-// two embedded rows).
+// scale per row (A: per row; B: per complex row, shared by its two embedded
+// rows): the largest magnitude's leading word, see tc_slice.cu.
 struct SlMat {
   DBuf planes, exps;
-  std::vector<TcMat> s;  // views of the planes (one hi plane each)
-  int ns = 0, bits = 0, kb_split = 0;
+  int b = 0, ns = 0;
   int64_t rows = 0, kp = 0, kreal = 0;
 };
 
-// scratch of sl_gemm: raw FP32 products of the slice pairs and the grouped launch state
+// scratch of sl_gemm: the per-CTA spill of the less significant classes and
+// the partial products of a split inner index
 struct SlWork {
-  DBuf part;
-  TcGroup grp;
+  DBuf spill, part;
 };
 
 // sliced copies of a context's static operators (built on first use) and the per-call B operand
@@ -59,6 +73,8 @@ void zgemm_sliced(Exec &ex, int64_t M, int64_t N, int64_t K, int64_t batch, cplx
 void sl_gemm(Exec &ex, const SlMat &A, const SlMat &B, int64_t M, int64_t N, cplx alpha, cplx beta, cplx *out,
              int64_t s_m, int64_t s_nh, int64_t s_nl, int64_t n_in, int *err, SlWork &w);
 
+// pipeline wait limit of this file's kernels (tc_set_wait_ns sets both files')
+void sl_set_wait_ns(unsigned long long ns);
 // test hook: bytes per operand chunk of zgemm_sliced (0 restores the free-memory rule)
 void set_sliced_cap_bytes(size_t bytes);
 

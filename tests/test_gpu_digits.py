@@ -1,0 +1,43 @@
+"""The digit products on the tensor cores (tc_slice.cu) at the edges of their tiles.
+
+Seeded uniform operands against the FP64 units (``adc_diag_gemm``): 5 the
+sliced product (42 bits), 6 the setup's (48 bits, digits whose width follows
+the inner size).
+
+Tolerances, relative to the Frobenius norm. Rounding an operand to `bits` bits
+below its row maximum leaves an error uniform in +-2^(-bits-1), that is
+2^(-bits) of the operands' RMS for uniform values (max = sqrt(3) RMS), sqrt(2)
+of that for both operands; the dropped digit classes add less than as much
+again: 2^(1.5 - bits), and a factor of two in hand. The FP64 reference
+(three products per complex multiply-add) carries at most 2^-50 sqrt(K) of its own.
+"""
+import math
+
+import pytest
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+BITS = {5: 42, 6: 48}
+
+
+@pytest.fixture(scope="module")
+def gpu():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from conftest import build_library
+    build_library()
+    import paper_2511_21640_gb300 as m
+    return m
+
+
+# tile widths 32, 64 and 128 real columns with one column more and less; row
+# tiles of 128; inner sizes around a block of 64, around the exact runs of both
+# passes, split over the SMs, and (48 bits) of every digit width
+@pytest.mark.parametrize("M,N,K", [
+    (1, 1, 1), (127, 16, 63), (128, 17, 64), (129, 32, 65), (257, 33, 193), (130, 64, 320), (128, 65, 384),
+    (300, 129, 385), (64, 5, 30000), (1100, 140, 700), (90, 70, 2100), (40, 33, 9000)])
+@pytest.mark.parametrize("which", [5, 6])
+def test_digit_product_edges(gpu, which, M, N, K):
+    err, _ = gpu.diag_gemm(which, M, N, K, seed=3 + M, reps=1)
+    assert err < 2.0 ** (2.5 - BITS[which]) + 2.0 ** -50 * math.sqrt(K), err
