@@ -52,7 +52,9 @@ typedef struct adc_ctx adc_ctx;
 enum { ADC_IP = 0, ADC_EA = 1, ADC_EE = 2 };
 
 /* Arithmetic of a sigma product.
- * ADC_PREC_FP64:   every operation in FP64 (CUDA cores).
+ * ADC_PREC_FP64:   FP64 throughout: small contractions on the CUDA cores, large
+ *   ones on the tensor cores from 56-bit integer digits (below), whose error
+ *   against exact sums is no larger than that of FP64 multiply-adds.
  * ADC_PREC_BF16X3: the dense contractions on the tensor cores (tcgen05) with
  *   each FP64 operand split into two BF16 parts (hi + lo) and the three
  *   products hi*hi + hi*lo + lo*hi accumulated in FP32; complex arithmetic by

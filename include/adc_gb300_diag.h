@@ -25,8 +25,9 @@ typedef struct adc_ctx adc_ctx_opaque;
  * the three), 4 = the six-product (BF16x6) tensor-core GEMM, 5 = the sliced
  * FP64-accurate tensor-core product of ADC_PREC_SLICED, including the slicing
  * of both operands, 6 = the setup's route: zgemm as the sliced product with
- * about 48 bits, in operand chunks (adc_diag_set_sliced_cap)) and compared with
- * the FP64 GEMM. Outputs: rel_err = ||C - C_fp64||_F / ||C_fp64||_F,
+ * about 48 bits, in operand chunks (adc_diag_set_sliced_cap), 7 = zgemm's FP64
+ * product from 56-bit digits on the tensor cores, whatever the size) and
+ * compared with the FP64 GEMM on the CUDA cores. Outputs: rel_err = ||C - C_fp64||_F / ||C_fp64||_F,
  * ms = average time of one launch sequence over `reps` repetitions (CUDA
  * events, after one warm-up). Allocates and frees its own device memory.
  * Returns ADC_OK or a negative ADC_ERR_* code. */

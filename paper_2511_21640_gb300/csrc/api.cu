@@ -92,6 +92,12 @@ int fail(adc_ctx *c, const std::exception &e, int code) {
   return code;
 }
 
+// the stream drained, and no FP64 product's wait given up since the last check
+void sync_check(adc_ctx *c) {
+  ADC_CUDA(cudaStreamSynchronize(c->ex.stream));
+  c->ex.check_digits();
+}
+
 #define ADC_API_TRY try {
 #define ADC_API_CATCH(ctxp)                                           \
   }                                                                   \
@@ -109,6 +115,7 @@ adc_ctx::~adc_ctx() {
   B.reset(); eo.reset(); ev.reset();
   if (ex.stream) cudaStreamSynchronize(ex.stream);
   if (own_stream && ex.stream) cudaStreamDestroy(ex.stream);
+  if (ex.digit_err) cudaFreeHost(ex.digit_err);
 }
 
 extern "C" {
@@ -202,6 +209,7 @@ int adc_init(adc_ctx **out, const adc_c128 *B, int64_t naux, const double *eps_o
     }
     // the setup's large contractions as the sliced tensor-core product when asked for
     c->ex.sliced_bits = (c->opts.setup == ADC_PREC_SLICED) ? 48 : 0;
+    c->ex.digits = 1;
     c->ex.n_sliced = c->ex.n_fp64 = 0;
     c->ex.flops_sliced = c->ex.flops_fp64 = 0.0;
     {
@@ -210,6 +218,7 @@ int adc_init(adc_ctx **out, const adc_c128 *B, int64_t naux, const double *eps_o
       else setup_operators(c);
     }
     c->ex.sliced_bits = 0;
+    c->ex.check_digits();
     c->setup_n[0] = c->ex.n_sliced;
     c->setup_n[1] = c->ex.n_fp64;
     c->setup_flops[0] = c->ex.flops_sliced;
@@ -251,7 +260,7 @@ int adc_sigma(adc_ctx *c, const adc_c128 *X, adc_c128 *S, int64_t k, int precisi
   DevOut sout(c->ex, S, bytes);
   sigma(c, (const cplx *)xin.p, (cplx *)sout.p, k, precision);
   sout.finish(c->ex);
-  if (sout.host || xin.buf.p) ADC_CUDA(cudaStreamSynchronize(c->ex.stream));
+  if (sout.host || xin.buf.p) sync_check(c);
   return ADC_OK;
   ADC_API_CATCH(c)
 }
@@ -271,7 +280,7 @@ int adc_sigma_share(adc_ctx *c, const adc_c128 *X, adc_c128 *S, int64_t k, int64
   DevOut sout(c->ex, S, (size_t)k * ls * sizeof(cplx));
   sigma_fp64_share(c, (const cplx *)xin.p, (cplx *)sout.p, k, i0, i1, with_main != 0);
   sout.finish(c->ex);
-  if (sout.host || xin.buf.p) ADC_CUDA(cudaStreamSynchronize(c->ex.stream));
+  if (sout.host || xin.buf.p) sync_check(c);
   return ADC_OK;
   ADC_API_CATCH(c)
 }
@@ -281,7 +290,7 @@ int adc_diagonal(adc_ctx *c, double *diag) {
   if (!diag) return ADC_ERR_ARG;
   ADC_API_TRY
   ADC_CUDA(cudaMemcpyAsync(diag, c->diag.p, c->N * sizeof(double), cudaMemcpyDefault, c->ex.stream));
-  ADC_CUDA(cudaStreamSynchronize(c->ex.stream));
+  sync_check(c);
   return ADC_OK;
   ADC_API_CATCH(c)
 }
@@ -291,7 +300,7 @@ int adc_main_block(adc_ctx *c, adc_c128 *M11) {
   if (!M11) return ADC_ERR_ARG;
   ADC_API_TRY
   ADC_CUDA(cudaMemcpyAsync(M11, c->M11.p, c->n1 * c->n1 * sizeof(cplx), cudaMemcpyDefault, c->ex.stream));
-  ADC_CUDA(cudaStreamSynchronize(c->ex.stream));
+  sync_check(c);
   return ADC_OK;
   ADC_API_CATCH(c)
 }
@@ -310,7 +319,7 @@ int adc_davidson(adc_ctx *c, int nroots, double tol, int max_iter, int precision
   yout.finish(c->ex);
   ADC_CUDA(cudaMemcpyAsync(omega, om.data(), nroots * sizeof(double), cudaMemcpyDefault, c->ex.stream));
   if (err64) ADC_CUDA(cudaMemcpyAsync(err64, er.data(), nroots * sizeof(double), cudaMemcpyDefault, c->ex.stream));
-  ADC_CUDA(cudaStreamSynchronize(c->ex.stream));
+  sync_check(c);
   if (rc == ADC_ERR_NOCONV) c->err = "Davidson did not converge within max_iter";
   return rc;
   ADC_API_CATCH(c)
@@ -332,7 +341,7 @@ int adc_fns_density(adc_ctx *c, adc_c128 *D, double *eta, adc_c128 *V, double et
   int64_t nk = 0;
   fns_run(c, (cplx *)dD.p, (double *)dE.p, (cplx *)dV.p, eta_crit, &nk, (cplx *)dU.p, (double *)dN.p);
   dD.finish(c->ex); dE.finish(c->ex); dV.finish(c->ex); dU.finish(c->ex); dN.finish(c->ex);
-  ADC_CUDA(cudaStreamSynchronize(c->ex.stream));
+  sync_check(c);
   *n_keep = nk;
   return ADC_OK;
   ADC_API_CATCH(c)
@@ -347,7 +356,7 @@ int adc_fns_transform(adc_ctx *c, const adc_c128 *U, int64_t ldu, int64_t n_keep
   DevOut bout(c->ex, Bout, (size_t)c->Q * n2 * n2 * sizeof(cplx));
   fns_transform(c, (const cplx *)uin.p, ldu, n_keep, (cplx *)bout.p);
   bout.finish(c->ex);
-  ADC_CUDA(cudaStreamSynchronize(c->ex.stream));
+  sync_check(c);
   return ADC_OK;
   ADC_API_CATCH(c)
 }
@@ -362,7 +371,7 @@ int adc_state_density(adc_ctx *c, const adc_c128 *y, adc_c128 *D) {
   DevOut dD(c->ex, D, (size_t)v * v * sizeof(cplx));
   state_density(c, (const cplx *)yin.p, (cplx *)dD.p);
   dD.finish(c->ex);
-  ADC_CUDA(cudaStreamSynchronize(c->ex.stream));
+  sync_check(c);
   return ADC_OK;
   ADC_API_CATCH(c)
 }
@@ -386,7 +395,7 @@ int adc_ssfns_density(adc_ctx *c, const adc_c128 *y, double eta_crit, adc_c128 *
   int64_t nk = 0;
   fns_run(c, (cplx *)dD.p, (double *)dE.p, nullptr, eta_crit, &nk, (cplx *)dU.p, (double *)dN.p, Dst.c());
   dD.finish(c->ex); dE.finish(c->ex); dU.finish(c->ex); dN.finish(c->ex);
-  ADC_CUDA(cudaStreamSynchronize(c->ex.stream));
+  sync_check(c);
   *n_keep = nk;
   return ADC_OK;
   ADC_API_CATCH(c)
@@ -402,7 +411,7 @@ int adc_fns_vector(adc_ctx *c, const adc_c128 *y, const adc_c128 *U, int64_t ldu
   DevOut gout(c->ex, g, (size_t)fns_dim(c->kind, c->o, n_keep) * sizeof(cplx));
   to_fns_basis(c, (const cplx *)yin.p, (const cplx *)uin.p, ldu, n_keep, (cplx *)gout.p);
   gout.finish(c->ex);
-  ADC_CUDA(cudaStreamSynchronize(c->ex.stream));
+  sync_check(c);
   return ADC_OK;
   ADC_API_CATCH(c)
 }
@@ -419,7 +428,7 @@ int adc_davidson_follow(adc_ctx *c, const adc_c128 *guess, double tol, int max_i
   int rc = davidson_run(c, 1, tol, max_iter, precision, (const cplx *)gin.p, 1, omega, (cplx *)yout.p, &e, st,
                         true);
   yout.finish(c->ex);
-  ADC_CUDA(cudaStreamSynchronize(c->ex.stream));
+  sync_check(c);
   if (err64) *err64 = e;
   if (rc == ADC_ERR_NOCONV) {
     c->err = "davidson: not converged within max_iter";
@@ -459,7 +468,7 @@ int adc_transition_density(adc_ctx *c, const adc_c128 *Y, int64_t k, adc_c128 *r
   DevOut rout(c->ex, rho, (size_t)k * c->nmo * c->nmo * sizeof(cplx));
   transition_density(c, (const cplx *)yin.p, k, (cplx *)rout.p);
   rout.finish(c->ex);
-  ADC_CUDA(cudaStreamSynchronize(c->ex.stream));
+  sync_check(c);
   return ADC_OK;
   ADC_API_CATCH(c)
 }
@@ -473,7 +482,7 @@ int adc_state_pair_density(adc_ctx *c, const adc_c128 *YK, const adc_c128 *YL, i
   DevOut rout(c->ex, rho, (size_t)k * c->nmo * c->nmo * sizeof(cplx));
   state_pair_density(c, (const cplx *)kin.p, (const cplx *)lin.p, k, (cplx *)rout.p);
   rout.finish(c->ex);
-  ADC_CUDA(cudaStreamSynchronize(c->ex.stream));
+  sync_check(c);
   return ADC_OK;
   ADC_API_CATCH(c)
 }
@@ -487,7 +496,7 @@ int adc_spectroscopic_amplitudes(adc_ctx *c, const adc_c128 *Y, int64_t k, adc_c
   DevOut xout(c->ex, x, (size_t)k * c->nmo * sizeof(cplx));
   spectroscopic_amplitudes(c, (const cplx *)yin.p, k, (cplx *)xout.p);
   xout.finish(c->ex);
-  ADC_CUDA(cudaStreamSynchronize(c->ex.stream));
+  sync_check(c);
   return ADC_OK;
   ADC_API_CATCH(c)
 }
@@ -500,7 +509,7 @@ int adc_excited_density(adc_ctx *c, const adc_c128 *Y, int64_t k, adc_c128 *rho)
   DevOut rout(c->ex, rho, (size_t)k * c->nmo * c->nmo * sizeof(cplx));
   excited_density(c, (const cplx *)yin.p, k, (cplx *)rout.p);
   rout.finish(c->ex);
-  ADC_CUDA(cudaStreamSynchronize(c->ex.stream));
+  sync_check(c);
   return ADC_OK;
   ADC_API_CATCH(c)
 }
@@ -583,7 +592,7 @@ int adc_sigma_adjoint(adc_ctx *c, const adc_c128 *Y, const double *gomega, int64
   gbo.finish(c->ex);
   geo.finish(c->ex);
   gev.finish(c->ex);
-  ADC_CUDA(cudaStreamSynchronize(c->ex.stream));
+  sync_check(c);
   *gx = gxh;
   return ADC_OK;
   ADC_API_CATCH(c)
@@ -596,7 +605,10 @@ int adc_sync(adc_ctx *c) {
     c->err = cudaGetErrorString(e);
     return ADC_ERR_CUDA;
   }
+  ADC_API_TRY
+  c->ex.check_digits();
   return ADC_OK;
+  ADC_API_CATCH(c)
 }
 
 void adc_free(adc_ctx *c) { delete c; }

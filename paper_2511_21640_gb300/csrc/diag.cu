@@ -117,7 +117,7 @@ int diag_grouped(int64_t M, int64_t N, int64_t K, uint64_t seed, int reps, doubl
 
 extern "C" int adc_diag_gemm(int which, int64_t M, int64_t N, int64_t K, uint64_t seed, int reps,
                              double *rel_err, double *ms) {
-  if (M <= 0 || N <= 0 || K <= 0 || reps < 1 || which < 0 || which > 6) return ADC_ERR_ARG;
+  if (M <= 0 || N <= 0 || K <= 0 || reps < 1 || which < 0 || which > 7) return ADC_ERR_ARG;
   if (which == 3) return diag_grouped(M, N, K, seed, reps, rel_err, ms);
   Exec ex;
   try {
@@ -142,7 +142,9 @@ extern "C" int adc_diag_gemm(int which, int64_t M, int64_t N, int64_t K, uint64_
           ex.sliced_bits = 48;
           zgemm(ex, M, N, K, 1, C1(), A.c(), 0, K, 1, false, B.c(), 0, 1, K, false, C0(), C.c(), 0, N, 1);
           ex.sliced_bits = 0;
-        } else if (which == 0) {
+        } else if (which == 0 || which == 7) {
+          // FP64: the FP64 units, or the 56-bit digits whatever the size
+          ex.digits = which == 7 ? 2 : 0;
           zgemm(ex, M, N, K, 1, C1(), A.c(), 0, K, 1, false, B.c(), 0, 1, K, false, C0(), C.c(), 0, N, 1);
         } else if (which == 1 || which == 4) {
           tc_gemm(ex, Ta, Tb, M, N, C1(), C0(), C.c(), N, 1, 0, 1, (int *)err.p, which == 4 ? 6 : 3);
@@ -155,7 +157,7 @@ extern "C" int adc_diag_gemm(int which, int64_t M, int64_t N, int64_t K, uint64_
       if (which == 5) {
         sl_pack_A(ex, Sa, A.c(), M, K, K, 1, false, 40);
         sl_pack_B(ex, Sb, B.c(), N, K, K, 0, 1, 1, false, Sa);
-      } else if (which >= 1 && which != 6) {
+      } else if (which >= 1 && which < 6) {
         const int planes = which == 4 ? 3 : 2;
         tc_pack_A(ex, Ta, A.c(), M, K, K, 1, false, planes);
         tc_pack_B(ex, Tb, B.c(), N, K, K, 0, 1, 1, false, planes);
@@ -183,12 +185,15 @@ extern "C" int adc_diag_gemm(int which, int64_t M, int64_t N, int64_t K, uint64_
       ADC_CUDA(cudaStreamSynchronize(ex.stream));
       if (rel_err) *rel_err = std::sqrt(h[0] / std::max(h[1], 1e-300));
       if (he) throw Error(ADC_ERR_TIMEOUT, "tensor-core GEMM wait gave up");
+      ex.check_digits();
     }
     cudaStreamSynchronize(ex.stream);
     cudaStreamDestroy(ex.stream);
+    if (ex.digit_err) cudaFreeHost(ex.digit_err);
     return ADC_OK;
   } catch (const Error &e) {
     if (ex.stream) { cudaStreamSynchronize(ex.stream); cudaStreamDestroy(ex.stream); }
+    if (ex.digit_err) cudaFreeHost(ex.digit_err);
     fprintf(stderr, "adc_diag_gemm: %s\n", e.what());
     return e.code;
   }

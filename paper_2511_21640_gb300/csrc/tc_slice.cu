@@ -877,4 +877,37 @@ void zgemm_sliced(Exec &ex, int64_t M, int64_t N, int64_t K, int64_t batch, cplx
   ADC_REQUIRE(h == 0, ADC_ERR_TIMEOUT, "sliced GEMM: a tensor-core wait gave up (code " + std::to_string(h) + ")");
 }
 
+// FP64 products that leave the FP64 units (1.26 TFLOP/s) for the digits: from 2^27
+// flops on, inner sizes of at least one block. Measured (GB300, M x N x K, FP64 units /
+// digits, slicing included): 256^3 (2^27) 124 / 171 us, 384^3 326 / 215 us,
+// 512^3 783 / 192 us, 200 x 8 x 20000 1.71 / 0.27 ms,
+// 1000 x 1000 x 64 449 / 108 us; below 2^27 the square shapes lose (192^3: 66 / 147 us).
+static bool digits_pay(int64_t M, int64_t N, int64_t K, int64_t batch) {
+  return K >= 64 && 8.0 * (double)M * (double)N * (double)K * (double)batch >= (double)(1 << 27);
+}
+
+bool zgemm_fp64_digits(Exec &ex, int64_t M, int64_t N, int64_t K, int64_t batch, cplx alpha, const cplx *A,
+                       int64_t sAb, int64_t sAm, int64_t sAk, bool conjA, const cplx *B, int64_t sBb, int64_t sBk,
+                       int64_t sBn, bool conjB, cplx beta, cplx *C, int64_t sCb, int64_t sCm, int64_t sCn) {
+  const int64_t grouped = (batch > 1 && (sAb == 0 || sBb == 0)) ? batch : 1;
+  if (ex.digits == 0 || K <= 0 || (ex.digits == 1 && !digits_pay(M, N, K, grouped))) return false;
+  cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+  ADC_CUDA(cudaStreamIsCapturing(ex.stream, &cs));
+  if (cs != cudaStreamCaptureStatusNone) return false;
+  if (!ex.digit_err) {
+    ADC_CUDA(cudaHostAlloc((void **)&ex.digit_err, sizeof(int), cudaHostAllocMapped));
+    *ex.digit_err = 0;
+  }
+  bool begun = false;
+  try {
+    digit_zgemm(ex, M, N, K, batch, alpha, A, sAb, sAm, sAk, conjA, B, sBb, sBk, sBn, conjB, beta, C, sCb, sCm, sCn,
+                kDigitFp64Bits, ex.digit_err, begun);
+  } catch (const Error &e) {
+    // no room for the digit planes: the FP64 units need none
+    if (e.code != ADC_ERR_OOM || begun) throw;
+    return false;
+  }
+  return true;
+}
+
 }  // namespace adc

@@ -7,18 +7,22 @@
 
 namespace adc {
 
+// significant bits of an FP64 product (eight digits): operand rounding 2^-57 and dropped
+// classes of about 2^-58 of the row and column maxima
+constexpr int kDigitFp64Bits = 56;
+
 // digits of an operand: ns of b bits
 struct SlDigits {
   int b, ns;
 };
 // Seven-bit digits, the widest whose products FP32 sums exactly over useful runs (eight-bit
-// ones drain four times as often): 4 and 6 of them for about 24 and 40 bits.
+// ones drain four times as often): 4, 6 and 8 of them for about 24, 40 and 56 bits.
 // The setup's 48-bit products take digits whose whole inner sum fits FP32 (b = 7 .. 4
 // as the inner size grows): which bits of the operators they keep depends on the
 // digits, and the BF16 split of an operator must not change with how it was computed.
 inline SlDigits sl_digits(int64_t K, int bits) {
   int b = 7;
-  if (bits > 40) {
+  if (bits > 40 && bits < kDigitFp64Bits) {
     const int64_t K2 = K <= 0 ? 128 : (K + 63) / 64 * 128;
     int l = 0;
     while ((1ll << l) < K2) ++l;
@@ -69,6 +73,12 @@ void sl_pack_B_ring(Exec &ex, SlMat &dst, const adc_ctx *c, const cplx *X, int64
 void zgemm_sliced(Exec &ex, int64_t M, int64_t N, int64_t K, int64_t batch, cplx alpha, const cplx *A, int64_t sAb,
                   int64_t sAm, int64_t sAk, bool conjA, const cplx *B, int64_t sBb, int64_t sBk, int64_t sBn,
                   bool conjB, cplx beta, cplx *C, int64_t sCb, int64_t sCm, int64_t sCn);
+// zgemm's FP64 product of a large shape from 56-bit digits, asynchronous; false when it
+// is left to the FP64 units (small, under stream capture, no room for the digit planes).
+// A wait that gave up leaves NaN in the output and its code in *ex.digit_err
+bool zgemm_fp64_digits(Exec &ex, int64_t M, int64_t N, int64_t K, int64_t batch, cplx alpha, const cplx *A,
+                       int64_t sAb, int64_t sAm, int64_t sAk, bool conjA, const cplx *B, int64_t sBb, int64_t sBk,
+                       int64_t sBn, bool conjB, cplx beta, cplx *C, int64_t sCb, int64_t sCm, int64_t sCn);
 // out = alpha A B^T + beta out, addressing as tc_gemm
 void sl_gemm(Exec &ex, const SlMat &A, const SlMat &B, int64_t M, int64_t N, cplx alpha, cplx beta, cplx *out,
              int64_t s_m, int64_t s_nh, int64_t s_nl, int64_t n_in, int *err, SlWork &w);

@@ -43,6 +43,13 @@ void Exec::release(void *p, size_t bytes) {
 
 long long g_launches = 0;
 
+void Exec::check_digits() {
+  if (!digit_err) return;
+  const int h = *(volatile int *)digit_err;
+  *digit_err = 0;
+  if (h) throw Error(ADC_ERR_TIMEOUT, "FP64 product: a tensor-core wait gave up (code " + std::to_string(h) + ")");
+}
+
 cudaEvent_t Exec::event() {
   if (!event_pool.empty()) {
     cudaEvent_t e = event_pool.back();
@@ -274,6 +281,9 @@ void zgemm(Exec &ex, int64_t M, int64_t N, int64_t K, int64_t batch, cplx alpha,
   }
   ex.n_fp64 += 1;
   ex.flops_fp64 += 8.0 * (double)M * N * K * batch;
+  if (zgemm_fp64_digits(ex, M, N, K, batch, alpha, A, sAb, sAm, sAk, conjA, B, sBb, sBk, sBn, conjB, beta, C, sCb,
+                        sCm, sCn))
+    return;
   zgemm_attr();
   const int64_t mt_ = (M + BM - 1) / BM, nt_ = (N + BN - 1) / BN;
   const int mfast = (nt_ <= 65535) ? 1 : 0;

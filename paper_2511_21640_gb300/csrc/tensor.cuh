@@ -22,6 +22,13 @@ struct Exec {
   // 512) as the sliced tensor-core product with about this many significant
   // bits (tc_slice.cu)
   int sliced_bits = 0;
+  // FP64 zgemm on the tensor cores (tc_slice.cu): 0 never (the FP64 units alone),
+  // 1 products large enough to pay, 2 every product (a diagnostic's choice)
+  int digits = 0;
+  // pinned word in which such a product records a wait that gave up; the host
+  // looks at it after the next synchronisation (check_digits)
+  int *digit_err = nullptr;
+  void check_digits();
   // complex GEMMs issued through zgemm since the counters were cleared: how
   // many took the sliced tensor-core route and how many the FP64 kernel, with
   // their algorithmic flops (host-side counts)

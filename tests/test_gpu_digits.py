@@ -2,7 +2,7 @@
 
 Seeded uniform operands against the FP64 units (``adc_diag_gemm``): 5 the
 sliced product (42 bits), 6 the setup's (48 bits, digits whose width follows
-the inner size).
+the inner size), 7 the FP64 product (56 bits).
 
 Tolerances, relative to the Frobenius norm. Rounding an operand to `bits` bits
 below its row maximum leaves an error uniform in +-2^(-bits-1), that is
@@ -18,7 +18,7 @@ import pytest
 torch = pytest.importorskip("torch")
 pytestmark = pytest.mark.gpu
 
-BITS = {5: 42, 6: 48}
+BITS = {5: 42, 6: 48, 7: 56}
 
 
 @pytest.fixture(scope="module")
@@ -37,7 +37,7 @@ def gpu():
 @pytest.mark.parametrize("M,N,K", [
     (1, 1, 1), (127, 16, 63), (128, 17, 64), (129, 32, 65), (257, 33, 193), (130, 64, 320), (128, 65, 384),
     (300, 129, 385), (64, 5, 30000), (1100, 140, 700), (90, 70, 2100), (40, 33, 9000)])
-@pytest.mark.parametrize("which", [5, 6])
+@pytest.mark.parametrize("which", [5, 6, 7])
 def test_digit_product_edges(gpu, which, M, N, K):
     err, _ = gpu.diag_gemm(which, M, N, K, seed=3 + M, reps=1)
     assert err < 2.0 ** (2.5 - BITS[which]) + 2.0 ** -50 * math.sqrt(K), err
