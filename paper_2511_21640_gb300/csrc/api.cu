@@ -113,6 +113,8 @@ adc_ctx::~adc_ctx() {
   scratch.reset();
   t1.reset(); W.reset(); Glad.reset(); Lvv.reset(); diag.reset(); d2.reset(); Cpl.reset(); M11.reset();
   B.reset(); eo.reset(); ev.reset();
+  ex.release(ex.zcount.p, ex.zcount.bytes);
+  ex.release(ex.zpart.p, ex.zpart.bytes);
   if (ex.stream) cudaStreamSynchronize(ex.stream);
   if (own_stream && ex.stream) cudaStreamDestroy(ex.stream);
   if (ex.digit_err) cudaFreeHost(ex.digit_err);
@@ -210,6 +212,11 @@ int adc_init(adc_ctx **out, const adc_c128 *B, int64_t naux, const double *eps_o
     // the setup's large contractions as the sliced tensor-core product when asked for
     c->ex.sliced_bits = (c->opts.setup == ADC_PREC_SLICED) ? 48 : 0;
     c->ex.digits = 1;
+    ex.zcount.p = ex.alloc(4096 * sizeof(unsigned));
+    ex.zcount.bytes = 4096 * sizeof(unsigned);
+    fill_zero(ex, ex.zcount.p, ex.zcount.bytes);
+    ex.zpart.p = ex.alloc((size_t)4 << 20);
+    ex.zpart.bytes = (size_t)4 << 20;
     c->ex.n_sliced = c->ex.n_fp64 = 0;
     c->ex.flops_sliced = c->ex.flops_fp64 = 0.0;
     {

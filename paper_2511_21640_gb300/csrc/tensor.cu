@@ -91,84 +91,121 @@ void fill_zero(Exec &ex, void *p, size_t bytes) {
 }
 
 // ------------------------------------------------------------------ GEMM
-// 64x64 output tile per CTA, 256 threads (16x16), 4x4 complex outputs per
-// thread, K staged 16 at a time through shared memory. FP64 FMA throughput
-// bounds it on GB300, so the loads only need to be coalesced along whichever
-// operand index has unit stride.
+// FP64 units (two multiply-adds a clock and SM on GB300) bound every product
+// here, so what counts is to give them no padding and to use every SM: the
+// output tile is chosen by shape from 64 x 64 down to strips of four rows or
+// columns (the k trial vectors of a product), and the inner index is split
+// over CTAs, each CTA's partial tile going to a buffer that the tile's last
+// CTA sums in the splits' order. The loads only need to be coalesced along
+// whichever operand index has unit stride; K is staged 16 at a time, the next
+// stage's elements loaded while the current one is used.
+// Measured (GB300, M x N x K, one 64 x 64 tile for every shape before / now): 16^3
+// 55 / 6 us, 64^3 63 / 12 us, 128^3 66 / 25 us, 4 x 672 x 8 57 / 6 us, 200 x 8 x 20000
+// 1.71 / 0.21 ms, 20000 x 8 x 200 1.94 / 0.22 ms (0.15 at the FP64 units' rate),
+// 4 x 1156 x 1156 511 / 59 us, 512^3 0.78 / 0.76 ms (0.64).
 namespace {
-constexpr int BM = 64, BN = 64, BKK = 16;
-constexpr int ZG_SMEM = (2 * BKK * (BM + 1) + 2 * BKK * (BN + 1) + BKK * (BM + 1) + BKK * (BN + 1)) * 8;
+constexpr int BKK = 16;
 
-__global__ void __launch_bounds__(256)
-k_zgemm(int64_t M, int64_t N, int64_t K, const cplx *__restrict__ A, int64_t sAb, int64_t sAm,
-        int64_t sAk, int conjA, int a_kfast, const cplx *__restrict__ B, int64_t sBb,
-        int64_t sBk, int64_t sBn, int conjB, int b_nfast, cplx *C, int64_t sCb, int64_t sCm,
-        int64_t sCn, cplx alpha, cplx beta, int64_t batch0, int ksplit, int64_t kchunk,
-        cplx *part, int64_t nbatch, int mfast) {
+struct ZArgs {
+  int64_t M, N, K;
+  const cplx *A;
+  int64_t sAb, sAm, sAk;
+  const cplx *B;
+  int64_t sBb, sBk, sBn;
+  cplx *C;
+  int64_t sCb, sCm, sCn;
+  cplx alpha, beta;
+  int64_t batch0, kchunk, nbatch;
+  int conjA, a_kfast, conjB, b_nfast, ksplit, mfast;
+  cplx *part;     // [ksplit][nbatch][M][N] partial products (ksplit > 1)
+  unsigned *cnt;  // a counter per output tile (zero between launches), or null: k_splitk_reduce follows
+};
+
+template <int BM, int BN, int TM, int TN>
+__global__ void __launch_bounds__((BM / TM) * (BN / TN)) k_zgemm(const ZArgs z) {
   // 3M products: (ar + i ai)(br + i bi) = T1 - T2 + i (T3 - T1 - T2) with
   // T1 = ar br, T2 = ai bi, T3 = (ar + ai)(br + bi): three FP64 FMAs per
   // complex MAC instead of four. The sums are formed once per staged element.
+  constexpr int RM = BM / TM, RN = BN / TN, NT = RM * RN;
+  constexpr int LA = (BM * BKK + NT - 1) / NT, LB = (BN * BKK + NT - 1) / NT;
   extern __shared__ double zsm[];
   cplx(*As)[BM + 1] = reinterpret_cast<cplx(*)[BM + 1]>(zsm);
   cplx(*Bs)[BN + 1] = reinterpret_cast<cplx(*)[BN + 1]>(zsm + 2 * BKK * (BM + 1));
   double(*Ass)[BM + 1] = reinterpret_cast<double(*)[BM + 1]>(zsm + 2 * BKK * (BM + 1) + 2 * BKK * (BN + 1));
   double(*Bss)[BN + 1] = reinterpret_cast<double(*)[BN + 1]>(zsm + 3 * BKK * (BM + 1) + 2 * BKK * (BN + 1));
   const int tid = threadIdx.x;
-  const int tx = tid & 15, ty = tid >> 4;
+  const int tx = tid % RN, ty = tid / RN;
   const int64_t zl = blockIdx.z;
-  const int64_t split = zl % ksplit;
-  const int64_t bl = zl / ksplit;
-  const int64_t b = bl + batch0;
+  const int64_t split = zl % z.ksplit;
+  const int64_t bl = zl / z.ksplit;
+  const int64_t b = bl + z.batch0;
   // with mfast the row tiles vary fastest, so the CTAs that read one column
   // tile of B (the large operand of the skinny shapes) run together and share it in L2
-  const int64_t m0 = (int64_t)(mfast ? blockIdx.x : blockIdx.y) * BM;
-  const int64_t n0 = (int64_t)(mfast ? blockIdx.y : blockIdx.x) * BN;
-  const int64_t kbeg = split * kchunk;
-  const int64_t kend = (kbeg + kchunk < K) ? kbeg + kchunk : K;
-  const cplx *Ab = A + b * sAb;
-  const cplx *Bb = B + b * sBb;
-  double t1[4][4], t2[4][4], t3[4][4];
+  const int64_t m0 = (int64_t)(z.mfast ? blockIdx.x : blockIdx.y) * BM;
+  const int64_t n0 = (int64_t)(z.mfast ? blockIdx.y : blockIdx.x) * BN;
+  const int64_t kbeg = split * z.kchunk;
+  const int64_t kend = (kbeg + z.kchunk < z.K) ? kbeg + z.kchunk : z.K;
+  const cplx *Ab = z.A + b * z.sAb;
+  const cplx *Bb = z.B + b * z.sBb;
+  double t1[TM][TN], t2[TM][TN], t3[TM][TN];
 #pragma unroll
-  for (int i = 0; i < 4; ++i)
+  for (int i = 0; i < TM; ++i)
 #pragma unroll
-    for (int j = 0; j < 4; ++j) t1[i][j] = t2[i][j] = t3[i][j] = 0.0;
-  const double sa = conjA ? -1.0 : 1.0, sb = conjB ? -1.0 : 1.0;
+    for (int j = 0; j < TN; ++j) t1[i][j] = t2[i][j] = t3[i][j] = 0.0;
+  const double sa = z.conjA ? -1.0 : 1.0, sb = z.conjB ? -1.0 : 1.0;
+  cplx ra[LA], rb[LB];
+  auto load = [&](int64_t k0) {
+#pragma unroll
+    for (int r = 0; r < LA; ++r) {
+      const int idx = tid + NT * r;
+      const int kk = z.a_kfast ? idx % BKK : idx / BM, mm = z.a_kfast ? idx / BKK : idx % BM;
+      const int64_t gm = m0 + mm, gk = k0 + kk;
+      ra[r] = (idx < BM * BKK && gm < z.M && gk < kend) ? Ab[gm * z.sAm + gk * z.sAk] : cmake(0.0, 0.0);
+    }
+#pragma unroll
+    for (int r = 0; r < LB; ++r) {
+      const int idx = tid + NT * r;
+      const int kk = z.b_nfast ? idx / BN : idx % BKK, nn = z.b_nfast ? idx % BN : idx / BKK;
+      const int64_t gn = n0 + nn, gk = k0 + kk;
+      rb[r] = (idx < BN * BKK && gn < z.N && gk < kend) ? Bb[gk * z.sBk + gn * z.sBn] : cmake(0.0, 0.0);
+    }
+  };
+  load(kbeg);
   for (int64_t k0 = kbeg; k0 < kend; k0 += BKK) {
 #pragma unroll
-    for (int r = 0; r < 4; ++r) {
-      int kk, mm;
-      if (a_kfast) { kk = tid & 15; mm = (tid >> 4) + 16 * r; }
-      else { mm = tid & 63; kk = (tid >> 6) + 4 * r; }
-      int64_t gm = m0 + mm, gk = k0 + kk;
-      cplx val = cmake(0.0, 0.0);
-      if (gm < M && gk < kend) { val = Ab[gm * sAm + gk * sAk]; val.y *= sa; }
-      As[kk][mm] = val;
-      Ass[kk][mm] = val.x + val.y;
+    for (int r = 0; r < LA; ++r) {
+      const int idx = tid + NT * r;
+      const int kk = z.a_kfast ? idx % BKK : idx / BM, mm = z.a_kfast ? idx / BKK : idx % BM;
+      if (BM * BKK % NT != 0 && idx >= BM * BKK) continue;
+      const cplx v = cmake(ra[r].x, ra[r].y * sa);
+      As[kk][mm] = v;
+      Ass[kk][mm] = v.x + v.y;
     }
 #pragma unroll
-    for (int r = 0; r < 4; ++r) {
-      int kk, nn;
-      if (b_nfast) { nn = tid & 63; kk = (tid >> 6) + 4 * r; }
-      else { kk = tid & 15; nn = (tid >> 4) + 16 * r; }
-      int64_t gn = n0 + nn, gk = k0 + kk;
-      cplx val = cmake(0.0, 0.0);
-      if (gn < N && gk < kend) { val = Bb[gk * sBk + gn * sBn]; val.y *= sb; }
-      Bs[kk][nn] = val;
-      Bss[kk][nn] = val.x + val.y;
+    for (int r = 0; r < LB; ++r) {
+      const int idx = tid + NT * r;
+      const int kk = z.b_nfast ? idx / BN : idx % BKK, nn = z.b_nfast ? idx % BN : idx / BKK;
+      if (BN * BKK % NT != 0 && idx >= BN * BKK) continue;
+      const cplx v = cmake(rb[r].x, rb[r].y * sb);
+      Bs[kk][nn] = v;
+      Bss[kk][nn] = v.x + v.y;
     }
     __syncthreads();
+    if (k0 + BKK < kend) load(k0 + BKK);
+    // (the last stage holds only the elements there are: the FP64 units do no padding)
+    const int kn = (int)(kend - k0 < BKK ? kend - k0 : BKK);
 #pragma unroll 4
-    for (int kk = 0; kk < BKK; ++kk) {
-      cplx a[4], bv[4];
-      double as[4], bs[4];
+    for (int kk = 0; kk < kn; ++kk) {
+      cplx a[TM], bv[TN];
+      double as[TM], bs[TN];
 #pragma unroll
-      for (int i = 0; i < 4; ++i) { a[i] = As[kk][ty + 16 * i]; as[i] = Ass[kk][ty + 16 * i]; }
+      for (int i = 0; i < TM; ++i) { a[i] = As[kk][ty + RM * i]; as[i] = Ass[kk][ty + RM * i]; }
 #pragma unroll
-      for (int j = 0; j < 4; ++j) { bv[j] = Bs[kk][tx + 16 * j]; bs[j] = Bss[kk][tx + 16 * j]; }
+      for (int j = 0; j < TN; ++j) { bv[j] = Bs[kk][tx + RN * j]; bs[j] = Bss[kk][tx + RN * j]; }
 #pragma unroll
-      for (int i = 0; i < 4; ++i)
+      for (int i = 0; i < TM; ++i)
 #pragma unroll
-        for (int j = 0; j < 4; ++j) {
+        for (int j = 0; j < TN; ++j) {
           t1[i][j] = fma(a[i].x, bv[j].x, t1[i][j]);
           t2[i][j] = fma(a[i].y, bv[j].y, t2[i][j]);
           t3[i][j] = fma(as[i], bs[j], t3[i][j]);
@@ -176,39 +213,64 @@ k_zgemm(int64_t M, int64_t N, int64_t K, const cplx *__restrict__ A, int64_t sAb
     }
     __syncthreads();
   }
-  cplx acc[4][4];
+  cplx acc[TM][TN];
 #pragma unroll
-  for (int i = 0; i < 4; ++i)
+  for (int i = 0; i < TM; ++i)
 #pragma unroll
-    for (int j = 0; j < 4; ++j) acc[i][j] = cmake(t1[i][j] - t2[i][j], t3[i][j] - t1[i][j] - t2[i][j]);
-  if (part) {
+    for (int j = 0; j < TN; ++j) acc[i][j] = cmake(t1[i][j] - t2[i][j], t3[i][j] - t1[i][j] - t2[i][j]);
+  if (z.ksplit > 1) {
     // split-K partial tile, unscaled: part[split][bl][m][n]
-    cplx *P = part + ((int64_t)split * nbatch + bl) * M * N;
+    const int64_t step = z.nbatch * z.M * z.N;
+    cplx *P = z.part + bl * z.M * z.N;
 #pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      int64_t gm = m0 + ty + 16 * i;
-      if (gm >= M) continue;
+    for (int i = 0; i < TM; ++i) {
+      const int64_t gm = m0 + ty + RM * i;
 #pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        int64_t gn = n0 + tx + 16 * j;
-        if (gn < N) P[gm * N + gn] = acc[i][j];
+      for (int j = 0; j < TN; ++j) {
+        const int64_t gn = n0 + tx + RN * j;
+        if (gm < z.M && gn < z.N) P[split * step + gm * z.N + gn] = acc[i][j];
       }
     }
-    return;
+    if (!z.cnt) return;
+    // the CTA that finds every other split's tile written sums them, in order
+    __shared__ unsigned seen;
+    __threadfence();
+    __syncthreads();
+    unsigned *cnt = z.cnt + ((int64_t)bl * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x;
+    if (tid == 0) seen = atomicAdd(cnt, 1u);
+    __syncthreads();
+    if (seen != (unsigned)z.ksplit - 1) return;
+    __threadfence();
+    if (tid == 0) *cnt = 0;
+#pragma unroll
+    for (int i = 0; i < TM; ++i) {
+      const int64_t gm = m0 + ty + RM * i;
+#pragma unroll
+      for (int j = 0; j < TN; ++j) {
+        const int64_t gn = n0 + tx + RN * j;
+        cplx s = cmake(0.0, 0.0);
+        if (gm < z.M && gn < z.N) {
+          const cplx *p = P + gm * z.N + gn;
+#pragma unroll 8
+          for (int k = 0; k < z.ksplit; ++k) s = cadd(s, __ldcg(p + k * step));
+        }
+        acc[i][j] = s;
+      }
+    }
   }
-  cplx *Cb = C + b * sCb;
-  const bool use_beta = (beta.x != 0.0 || beta.y != 0.0);
+  cplx *Cb = z.C + b * z.sCb;
+  const bool use_beta = (z.beta.x != 0.0 || z.beta.y != 0.0);
 #pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    int64_t gm = m0 + ty + 16 * i;
-    if (gm >= M) continue;
+  for (int i = 0; i < TM; ++i) {
+    int64_t gm = m0 + ty + RM * i;
+    if (gm >= z.M) continue;
 #pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      int64_t gn = n0 + tx + 16 * j;
-      if (gn >= N) continue;
-      cplx *dst = Cb + gm * sCm + gn * sCn;
-      cplx r = cmul(alpha, acc[i][j]);
-      if (use_beta) r = cadd(r, cmul(beta, *dst));
+    for (int j = 0; j < TN; ++j) {
+      int64_t gn = n0 + tx + RN * j;
+      if (gn >= z.N) continue;
+      cplx *dst = Cb + gm * z.sCm + gn * z.sCn;
+      cplx r = cmul(z.alpha, acc[i][j]);
+      if (use_beta) r = cadd(r, cmul(z.beta, *dst));
       *dst = r;
     }
   }
@@ -261,8 +323,90 @@ void set_smem_limit(const void *kernel, int bytes) {
   g_smem_set.insert(key);
 }
 
-static void zgemm_attr() { set_smem_limit((const void *)k_zgemm, ZG_SMEM); }
 static int num_sms() { return device_sm_count(); }
+
+namespace {
+// output tiles of the FP64 kernel
+struct ZTile {
+  int bm, bn;
+  void (*kernel)(const ZArgs);
+  int threads;
+};
+const ZTile kZTiles[] = {
+    {64, 64, k_zgemm<64, 64, 4, 4>, 256}, {32, 32, k_zgemm<32, 32, 2, 2>, 256}, {16, 16, k_zgemm<16, 16, 2, 2>, 64},
+    {8, 32, k_zgemm<8, 32, 2, 2>, 64},    {32, 8, k_zgemm<32, 8, 2, 2>, 64},    {4, 64, k_zgemm<4, 64, 2, 2>, 64},
+    {64, 4, k_zgemm<64, 4, 2, 2>, 64},    {8, 8, k_zgemm<8, 8, 1, 1>, 64}};
+
+// Tile and inner split of the least estimated time, in clocks: the SM with the
+// most CTAs runs ceil(CTAs / SMs) tiles at two multiply-adds a clock (three per
+// complex one, and the staging adds), half a one per scheduler, so that fewer
+// than four warps on an SM leave part of it idle; each stage of a CTA costs a
+// load latency that the SM's other CTAs hide; a split's partial sums cost a pass
+// through L2 by the tile's last CTA (or a second kernel).
+// max_split: 1 without a workspace; the partial products stay within max_part elements.
+struct ZPlan {
+  const ZTile *t = nullptr;
+  int ksplit = 1;
+  double clocks = 0.0;
+};
+ZPlan z_plan(int64_t M, int64_t N, int64_t K, int64_t batch, int max_split, int64_t max_part, bool fused) {
+  static const int kSplits[] = {1, 2, 3, 4, 6, 8, 12, 16, 24, 32, 48, 64};
+  const double sms = num_sms();
+  ZPlan best;
+  best.clocks = 1e300;
+  for (const ZTile &t : kZTiles) {
+    const int64_t tm = (M + t.bm - 1) / t.bm, tn = (N + t.bn - 1) / t.bn;
+    if (std::min(tm, tn) > 65535) continue;
+    const double tiles = (double)tm * (double)tn * (double)batch;
+    for (int s : kSplits) {
+      if (s > max_split) break;
+      if (s > 1 && (s > (K + BKK - 1) / BKK || (double)s * M * N * batch > (double)max_part)) break;
+      const double stages = std::ceil((double)((K + s - 1) / s) / BKK);
+      const double per = std::ceil(tiles * s / sms);
+      const double kk = std::min<double>(stages * BKK, std::max<double>(K, 1));
+      const double work = per * (1.5 * t.bm * t.bn + 0.5 * (t.bm + t.bn)) * kk * std::max(1.0, 4.0 / (per * t.threads / 32));
+      const double lat = stages * 1100.0 * std::ceil(per * t.threads / 512.0);
+      const double red = s == 1 ? 0.0 : fused ? 2500.0 + 80.0 * s : 8000.0 + 20.0 * s;
+      const double c = std::max(work, lat) + 0.3 * std::min(work, lat) + red;
+      if (c < best.clocks) { best.clocks = c; best.t = &t; best.ksplit = s; }
+      if (tiles * s > 8.0 * sms) break;
+    }
+  }
+  return best;
+}
+
+// one FP64 product with the tile and split of p, in batch slices; part: room for
+// ksplit partial products of a slice of at most slice(batch) entries; cnt as ZArgs::cnt
+void z_launch(Exec &ex, const ZPlan &p, ZArgs z, int64_t batch, cplx *part, unsigned *cnt) {
+  const int64_t mt = (z.M + p.t->bm - 1) / p.t->bm, nt = (z.N + p.t->bn - 1) / p.t->bn;
+  z.mfast = (nt <= 65535) ? 1 : 0;
+  ADC_REQUIRE(z.mfast || mt <= 65535, ADC_ERR_UNSUPPORTED, "zgemm: shape too large");
+  z.a_kfast = (z.sAk == 1) ? 1 : 0;
+  z.b_nfast = (z.sBn == 1) ? 1 : 0;
+  z.ksplit = p.ksplit;
+  z.kchunk = (z.K + p.ksplit - 1) / p.ksplit;
+  if (p.ksplit > 1) z.kchunk = (z.kchunk + BKK - 1) / BKK * BKK;
+  z.part = part;
+  z.cnt = cnt;
+  const int64_t bmax = 65535 / p.ksplit;
+  const int smem = 3 * BKK * (p.t->bm + 1 + p.t->bn + 1) * (int)sizeof(double);
+  if (smem > 48 * 1024 - 64) set_smem_limit((const void *)p.t->kernel, smem);
+  for (int64_t b0 = 0; b0 < batch; b0 += bmax) {
+    z.nbatch = std::min<int64_t>(bmax, batch - b0);
+    z.batch0 = b0;
+    const dim3 grid(z.mfast ? (unsigned)mt : (unsigned)nt, z.mfast ? (unsigned)nt : (unsigned)mt,
+                    (unsigned)(z.nbatch * p.ksplit));
+    p.t->kernel<<<grid, p.t->threads, smem, ex.stream>>>(z);
+    ADC_CHECK_LAUNCH();
+    if (p.ksplit > 1 && !cnt) {
+      k_splitk_reduce<<<grid1d(z.nbatch * z.M * z.N, 256), 256, 0, ex.stream>>>(
+          part, p.ksplit, z.nbatch, z.M, z.N, z.C, z.sCb, z.sCm, z.sCn, z.alpha, z.beta, b0);
+      ADC_CHECK_LAUNCH();
+    }
+  }
+}
+constexpr int64_t kMaxPart = (int64_t)1 << 26;  // elements of a call's partial products
+}  // namespace
 
 void zgemm(Exec &ex, int64_t M, int64_t N, int64_t K, int64_t batch, cplx alpha, const cplx *A,
            int64_t sAb, int64_t sAm, int64_t sAk, bool conjA, const cplx *B, int64_t sBb,
@@ -284,50 +428,24 @@ void zgemm(Exec &ex, int64_t M, int64_t N, int64_t K, int64_t batch, cplx alpha,
   if (zgemm_fp64_digits(ex, M, N, K, batch, alpha, A, sAb, sAm, sAk, conjA, B, sBb, sBk, sBn, conjB, beta, C, sCb,
                         sCm, sCn))
     return;
-  zgemm_attr();
-  const int64_t mt_ = (M + BM - 1) / BM, nt_ = (N + BN - 1) / BN;
-  const int mfast = (nt_ <= 65535) ? 1 : 0;
-  ADC_REQUIRE(mfast || mt_ <= 65535, ADC_ERR_UNSUPPORTED, "zgemm: shape too large");
-  int a_kfast = (sAk == 1) ? 1 : 0;
-  int b_nfast = (sBn == 1) ? 1 : 0;
-  dim3 block(256);
-  const int64_t tiles = ((N + BN - 1) / BN) * ((M + BM - 1) / BM);
-  // split K when the output tiles alone cannot fill the GPU (down to chunks of
-  // 16: on GB300's FP64 units a few CTAs over a short K still take far longer
-  // than the partial sums cost), the partial buffer within 2^26 elements
-  int ksplit = 1;
-  const int64_t want = 2 * (int64_t)num_sms();
-  if (tiles * batch < want && K >= 32) {
-    int64_t s = (want + tiles * batch - 1) / (tiles * batch);
-    s = std::min<int64_t>(s, (K + BKK - 1) / BKK);
-    s = std::min<int64_t>(s, 256);
-    s = std::min<int64_t>(s, std::max<int64_t>(1, ((int64_t)1 << 26) / std::max<int64_t>(1, M * N * batch)));
-    ksplit = (int)std::max<int64_t>(1, s);
+  const ZArgs z{M, N, K, A, sAb, sAm, sAk, B, sBb, sBk, sBn, C, sCb, sCm, sCn, alpha, beta, 0, 0, 0,
+                conjA ? 1 : 0, 0, conjB ? 1 : 0, 0, 1, 0, nullptr, nullptr};
+  ZPlan p = z_plan(M, N, K, batch, 64, kMaxPart, ex.zcount.p != nullptr);
+  ADC_REQUIRE(p.t, ADC_ERR_UNSUPPORTED, "zgemm: shape too large");
+  DBuf part;
+  unsigned *cnt = nullptr;
+  cplx *pp = nullptr;
+  if (p.ksplit > 1) {
+    const int64_t slice = std::min<int64_t>(batch, 65535 / p.ksplit);
+    const int64_t tiles = (M + p.t->bm - 1) / p.t->bm * ((N + p.t->bn - 1) / p.t->bn) * slice;
+    if (tiles <= (int64_t)(ex.zcount.bytes / sizeof(unsigned))) cnt = (unsigned *)ex.zcount.p;
+    // the partial products: the context's own small buffer, or one of the call
+    if (cnt && (size_t)p.ksplit * slice * M * N * sizeof(cplx) <= ex.zpart.bytes) pp = (cplx *)ex.zpart.p;
+    else { part = cbuf(ex, (int64_t)p.ksplit * slice * M * N); pp = part.c(); }
   }
-  const int64_t bmax = 65535 / ksplit;
   int pr = ex.prof_begin("zgemm_fp64", 8.0 * (double)M * N * K * batch,
                          16.0 * (double)batch * ((double)M * K + (double)K * N + (double)M * N));
-  for (int64_t b0 = 0; b0 < batch; b0 += bmax) {
-    int64_t nb = std::min<int64_t>(bmax, batch - b0);
-    dim3 grid(mfast ? (unsigned)mt_ : (unsigned)nt_, mfast ? (unsigned)nt_ : (unsigned)mt_, (unsigned)(nb * ksplit));
-    if (ksplit == 1) {
-      k_zgemm<<<grid, block, ZG_SMEM, ex.stream>>>(M, N, K, A, sAb, sAm, sAk, conjA ? 1 : 0, a_kfast, B,
-                                             sBb, sBk, sBn, conjB ? 1 : 0, b_nfast, C, sCb, sCm,
-                                             sCn, alpha, beta, b0, 1, K, nullptr, nb, mfast);
-      ADC_CHECK_LAUNCH();
-    } else {
-      int64_t kchunk = (K + ksplit - 1) / ksplit;
-      kchunk = (kchunk + BKK - 1) / BKK * BKK;
-      DBuf part = cbuf(ex, (int64_t)ksplit * nb * M * N);
-      k_zgemm<<<grid, block, ZG_SMEM, ex.stream>>>(M, N, K, A, sAb, sAm, sAk, conjA ? 1 : 0, a_kfast, B,
-                                             sBb, sBk, sBn, conjB ? 1 : 0, b_nfast, C, sCb, sCm,
-                                             sCn, alpha, beta, b0, ksplit, kchunk, part.c(), nb, mfast);
-      ADC_CHECK_LAUNCH();
-      k_splitk_reduce<<<grid1d(nb * M * N, 256), 256, 0, ex.stream>>>(
-          part.c(), ksplit, nb, M, N, C, sCb, sCm, sCn, alpha, beta, b0);
-      ADC_CHECK_LAUNCH();
-    }
-  }
+  z_launch(ex, p, z, batch, pp, cnt);
   ex.prof_end(pr);
 }
 
@@ -337,47 +455,12 @@ void zgemm_ws(Exec &ex, int64_t M, int64_t N, int64_t K, int64_t batch, cplx alp
               int64_t ws_elems) {
   if (M <= 0 || N <= 0 || batch <= 0) return;
   if (K < 0) K = 0;
-  zgemm_attr();
-  const int64_t mt_ = (M + BM - 1) / BM, nt_ = (N + BN - 1) / BN;
-  const int mfast = (nt_ <= 65535) ? 1 : 0;
-  ADC_REQUIRE(mfast || mt_ <= 65535, ADC_ERR_UNSUPPORTED, "zgemm: shape too large");
-  int a_kfast = (sAk == 1) ? 1 : 0;
-  int b_nfast = (sBn == 1) ? 1 : 0;
-  dim3 block(256);
-  const int64_t tiles = ((N + BN - 1) / BN) * ((M + BM - 1) / BM);
-  // same split-K choice as zgemm, capped by the workspace the caller provides
-  int ksplit = 1;
-  const int64_t want = 2 * (int64_t)num_sms();
-  if (tiles * batch < want && K > 2048) {
-    int64_t s = (want + tiles * batch - 1) / (tiles * batch);
-    s = std::min<int64_t>(s, K / 1024);
-    s = std::min<int64_t>(s, 256);
-    ksplit = (int)std::max<int64_t>(1, s);
-  }
-  const int64_t bmax = 65535 / ksplit;
-  for (int64_t b0 = 0; b0 < batch; b0 += bmax) {
-    int64_t nb = std::min<int64_t>(bmax, batch - b0);
-    int ks = ksplit;
-    if (ks > 1 && ws) ks = (int)std::max<int64_t>(1, std::min<int64_t>(ks, ws_elems / std::max<int64_t>(1, nb * M * N)));
-    if (!ws) ks = 1;
-    dim3 grid(mfast ? (unsigned)mt_ : (unsigned)nt_, mfast ? (unsigned)nt_ : (unsigned)mt_, (unsigned)(nb * ks));
-    if (ks == 1) {
-      k_zgemm<<<grid, block, ZG_SMEM, ex.stream>>>(M, N, K, A, sAb, sAm, sAk, conjA ? 1 : 0, a_kfast, B, sBb, sBk, sBn,
-                                             conjB ? 1 : 0, b_nfast, C, sCb, sCm, sCn, alpha, beta, b0, 1, K,
-                                             nullptr, nb, mfast);
-      ADC_CHECK_LAUNCH();
-    } else {
-      int64_t kchunk = (K + ks - 1) / ks;
-      kchunk = (kchunk + BKK - 1) / BKK * BKK;
-      k_zgemm<<<grid, block, ZG_SMEM, ex.stream>>>(M, N, K, A, sAb, sAm, sAk, conjA ? 1 : 0, a_kfast, B, sBb, sBk, sBn,
-                                             conjB ? 1 : 0, b_nfast, C, sCb, sCm, sCn, alpha, beta, b0, ks, kchunk,
-                                             ws, nb, mfast);
-      ADC_CHECK_LAUNCH();
-      k_splitk_reduce<<<grid1d(nb * M * N, 256), 256, 0, ex.stream>>>(ws, ks, nb, M, N, C, sCb, sCm, sCn, alpha,
-                                                                      beta, b0);
-      ADC_CHECK_LAUNCH();
-    }
-  }
+  const ZArgs z{M, N, K, A, sAb, sAm, sAk, B, sBb, sBk, sBn, C, sCb, sCm, sCn, alpha, beta, 0, 0, 0,
+                conjA ? 1 : 0, 0, conjB ? 1 : 0, 0, 1, 0, nullptr, nullptr};
+  // the splits are capped by the workspace the caller provides
+  const ZPlan p = z_plan(M, N, K, batch, ws ? 64 : 1, ws_elems, false);
+  ADC_REQUIRE(p.t, ADC_ERR_UNSUPPORTED, "zgemm: shape too large");
+  z_launch(ex, p, z, batch, ws, nullptr);
 }
 
 // ------------------------------------------------------------------ permute

@@ -28,6 +28,13 @@ struct Exec {
   // pinned word in which such a product records a wait that gave up; the host
   // looks at it after the next synchronisation (check_digits)
   int *digit_err = nullptr;
+  // the FP64 kernel's inner splits: tile counters (zero between launches) and a small
+  // buffer of partial products. Held by a context for its life, on its one stream; null
+  // elsewhere: a second kernel then sums the splits
+  struct Held {
+    void *p = nullptr;
+    size_t bytes = 0;
+  } zcount, zpart;
   void check_digits();
   // complex GEMMs issued through zgemm since the counters were cleared: how
   // many took the sliced tensor-core route and how many the FP64 kernel, with

@@ -36,7 +36,9 @@ def gpu():
 # passes, split over the SMs, and (48 bits) of every digit width
 @pytest.mark.parametrize("M,N,K", [
     (1, 1, 1), (127, 16, 63), (128, 17, 64), (129, 32, 65), (257, 33, 193), (130, 64, 320), (128, 65, 384),
-    (300, 129, 385), (64, 5, 30000), (1100, 140, 700), (90, 70, 2100), (40, 33, 9000)])
+    (300, 129, 385), (64, 5, 30000), (1100, 140, 700), (90, 70, 2100), (40, 33, 9000),
+    # the FP64 units' tiles (strips of 4 and 8 rows or columns, 8, 16, 32 and 64 square), whole and split
+    (3, 300, 50), (300, 3, 50), (7, 90, 1000), (90, 7, 1000), (9, 9, 20), (20, 20, 400), (70, 50, 40), (700, 650, 33)])
 @pytest.mark.parametrize("which", [5, 6, 7])
 def test_digit_product_edges(gpu, which, M, N, K):
     err, _ = gpu.diag_gemm(which, M, N, K, seed=3 + M, reps=1)
