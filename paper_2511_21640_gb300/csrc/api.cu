@@ -118,6 +118,7 @@ adc_ctx::~adc_ctx() {
   if (ex.stream) cudaStreamSynchronize(ex.stream);
   if (own_stream && ex.stream) cudaStreamDestroy(ex.stream);
   if (ex.digit_err) cudaFreeHost(ex.digit_err);
+  if (pooled) pool_release(dev);
 }
 
 extern "C" {
@@ -169,6 +170,8 @@ int adc_init(adc_ctx **out, const adc_c128 *B, int64_t naux, const double *eps_o
     c->N = c->n1 + c->n2;
     c->ex.mem_limit = c->opts.mem_limit;
     ADC_CUDA(cudaGetDevice(&c->dev));
+    pool_retain(c->dev);
+    c->pooled = true;
     if (c->opts.stream) {
       c->ex.stream = (cudaStream_t)c->opts.stream;
     } else {

@@ -608,9 +608,11 @@ int adc_batch_solve(int n, const adc_problem *p, int nroots, double tol, int max
   if (cudaGetDevice(&dev) != cudaSuccess) return bfail(nullptr, "adc_batch_solve: no device", ADC_ERR_CUDA);
   int64_t budget = o.mem_budget;
   if (budget <= 0) {
-    size_t fr = 0, tot = 0;
-    if (cudaMemGetInfo(&fr, &tot) != cudaSuccess) return bfail(nullptr, "adc_batch_solve: cudaMemGetInfo", ADC_ERR_CUDA);
-    budget = (int64_t)(0.85 * (double)fr);
+    try {
+      budget = (int64_t)(0.85 * (double)free_device_memory());
+    } catch (const Error &e) {
+      return bfail(nullptr, e.what(), e.code);
+    }
   }
   std::vector<int> order(n), wave(n);
   int nw = plan_waves(n, p, nroots, budget, order.data(), wave.data(), nullptr, nullptr, o.refine == ADC_PREC_SLICED);

@@ -15,6 +15,7 @@ struct BatchCoord;  // cross-problem sigma batching (batch.cu)
 struct adc_ctx {
   adc::Exec ex;
   bool own_stream = false;
+  bool pooled = false;  // counted by the device's memory pool
   int dev = -1;  // CUDA device that was current at adc_init (holds every buffer)
   // zgemm routes taken by adc_init: products (sliced, FP64) and their algorithmic flops
   int64_t setup_n[2] = {0, 0};
@@ -139,6 +140,12 @@ void sigma_fp64(adc_ctx *c, const cplx *X, cplx *S, int64_t k);
 void sigma_fp64_share(adc_ctx *c, const cplx *X, cplx *S, int64_t k, int64_t i0, int64_t i1, bool with_main);
 // split-precision sigma on the tensor cores: nseg = 3 (BF16x3) or 6 (BF16x6) products
 void sigma_split(adc_ctx *c, const cplx *X, cplx *S, int64_t k, int nseg);
+// one term of the FP64 sigma from the kept digits of a static operator (sigma_tc.cu; which: SL_*);
+// false when the term is left to zgemm. fp64_ops_prepare builds the digits ahead of a solve
+bool fp64_op_product(adc_ctx *c, int which, bool ring, const cplx *X, int64_t k, const cplx *Bsrc, int64_t Nc,
+                     int64_t b_nh, int64_t b_nl, int64_t b_in, int64_t b_k, cplx alpha, cplx beta, cplx *out,
+                     int64_t s_m, int64_t s_nh, int64_t s_nl, int64_t n_in);
+void fp64_ops_prepare(adc_ctx *c, int64_t k);
 // FP64-accurate sigma with the dense contractions as sliced tensor-core products (IP/EA)
 void sigma_sliced(adc_ctx *c, const cplx *X, cplx *S, int64_t k, int bits = kSlicedBits);
 // estimate of the largest device scratch one sigma call of k vectors allocates (bytes)

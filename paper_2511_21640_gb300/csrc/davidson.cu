@@ -460,10 +460,9 @@ int davidson_run(adc_ctx *c, int nroots, double tol, int max_iter, int precision
     if (c->kind == ADC_EE && c->ee)
       ee_prepare(c, precision == ADC_PREC_FP64 ? 0 : (mixed == ADC_PREC_BF16X6 ? 3 : 2),
                  c->opts.refine == ADC_PREC_SLICED);
+    if (precision == ADC_PREC_FP64 || c->opts.refine == ADC_PREC_FP64) fp64_ops_prepare(c, kb);
     ADC_CUDA(cudaStreamSynchronize(c->ex.stream));
-    size_t fr = 0, tot = 0;
-    ADC_CUDA(cudaMemGetInfo(&fr, &tot));
-    double avail = (double)fr;
+    double avail = (double)free_device_memory();
     if (c->ex.mem_limit > 0) avail = std::min(avail, (double)(c->ex.mem_limit - c->ex.mem_used));
     const double vec = (double)N * sizeof(cplx);
     const double scratch = sigma_scratch_bytes(c, kb);

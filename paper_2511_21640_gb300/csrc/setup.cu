@@ -282,9 +282,7 @@ void setup_operators(adc_ctx *c) {
     if (c->opts.ladder == 1) {
       c->direct_ladder = true;
     } else if (c->opts.ladder == 0) {
-      size_t fr = 0, tot = 0;
-      ADC_CUDA(cudaMemGetInfo(&fr, &tot));
-      c->direct_ladder = (double)pv * (double)pv * sizeof(cplx) > 0.25 * (double)fr;
+      c->direct_ladder = (double)pv * (double)pv * sizeof(cplx) > 0.25 * (double)free_device_memory();
     }
   }
   StageScope stage(ex, "first_order_amplitudes");

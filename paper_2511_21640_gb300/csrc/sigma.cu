@@ -11,6 +11,7 @@
 // (Sec. 2.1 Eqs. 10-12; integrals from Eq. 43.) The satellite terms of
 // first order are the ladder (packed GEMM) and the ring (GEMM over (k,c)).
 #include "ctx.cuh"
+#include "tc_slice.cuh"
 
 namespace adc {
 
@@ -45,9 +46,11 @@ void sigma_fp64(adc_ctx *c, const cplx *X, cplx *S, int64_t k) {
   zgemm(ex, k, n1, n1, 1, C1(), X, 0, N, 1, false, c->M11.c(), 0, 1, n1, false, C0(), S, 0, N, 1);
   // S1 += X2 Cpl^T
   ex.tag = "coupling";
-  zgemm(ex, k, n1, n2, 1, C1(), X + n1, 0, N, 1, false, c->Cpl.c(), 0, 1, n2, false, C1(), S, 0, N, 1);
+  if (!fp64_op_product(c, SL_CPL, false, X, k, X + n1, k, N, 0, 1, 1, C1(), C1(), S, 1, N, 0, 1))
+    zgemm(ex, k, n1, n2, 1, C1(), X + n1, 0, N, 1, false, c->Cpl.c(), 0, 1, n2, false, C1(), S, 0, N, 1);
   // S2 = X1 conj(Cpl)
-  zgemm(ex, k, n2, n1, 1, C1(), X, 0, N, 1, false, c->Cpl.c(), 0, n2, 1, true, C0(), S + n1, 0, N, 1);
+  if (!fp64_op_product(c, SL_CPLT, false, X, k, X, k, N, 0, 1, 1, C1(), C0(), S + n1, 1, N, 0, 1))
+    zgemm(ex, k, n2, n1, 1, C1(), X, 0, N, 1, false, c->Cpl.c(), 0, n2, 1, true, C0(), S + n1, 0, N, 1);
   // S2 += d2 * X2
   diag_mul_add(ex, k, n2, c->d2.d(), X + n1, N, S + n1, N, 1.0);
   if (!sat) return;
@@ -55,20 +58,26 @@ void sigma_fp64(adc_ctx *c, const cplx *X, cplx *S, int64_t k) {
     const int64_t pv = npairs(v);
     // ladder: S2[r][j][(ab)] += x sum_(cd) X2[r][j][(cd)] Glad[(ab)][(cd)], one GEMM over all (r, j)
     ex.tag = "ladder";
-    cplx *Xf = scratch(c, 2 * k * o * v * v + 2 * k * o * pv);
-    cplx *T = Xf + k * o * v * v;
-    cplx *Xg = T + k * o * v * v, *Og = Xg + k * o * pv;
     if (c->direct_ladder) {
       ladder_direct(c, X + n1, N, o, S + n1, N, k, x, ADC_LADDER_FP64, nullptr);
-    } else {
+    } else if (!fp64_op_product(c, SL_GLAD, false, X, k, X + n1, k * o, N, pv, o, 1, CR(x), C1(), S + n1, 1, N, pv,
+                                o)) {
+      cplx *Xg = scratch(c, 2 * k * o * pv), *Og = Xg + k * o * pv;
       ADC_CUDA(cudaMemcpy2DAsync(Xg, o * pv * sizeof(cplx), X + n1, N * sizeof(cplx), o * pv * sizeof(cplx), k,
                                  cudaMemcpyDeviceToDevice, ex.stream));
       zgemm(ex, k * o, pv, pv, 1, C1(), Xg, 0, pv, 1, false, c->Glad.c(), 0, 1, pv, false, C0(), Og, 0, pv, 1);
       k_rows_axpy<<<grid1d(k * o * pv, 256), 256, 0, ex.stream>>>(k, o * pv, CR(x), Og, o * pv, S + n1, N);
       ADC_CHECK_LAUNCH();
     }
-    // ring: Xf[r][k][c][b] (antisymmetric in c,b); T[(j,a)][(r,b)] = sum_(kc) W[(j,a)][(kc)] Xt[(kc)][(r,b)]
+    // ring: R[(j,a)][(r,b)] = sum_(kc) W[(j,a)][(kc)] Xf[r][k][c][b], Xf antisymmetric in (c, b)
     ex.tag = "ring";
+    cplx *R = scratch(c, 2 * k * o * v * v);
+    if (fp64_op_product(c, SL_W, true, X, k, nullptr, k * v, 0, 0, 1, 0, C1(), C0(), R, v, o * v * v, 1, v)) {
+      // R[r][j][a][b]; S2[r][j][(a<b)] -= x (R[r][j][a][b] - R[r][j][b][a])
+      pair_pack(ex, R, o * v * v, v * v, v, 1, 0, 1.0, k, o, v, 1, S + n1, N, pv, CR(-x), C1());
+      return;
+    }
+    cplx *Xf = R, *T = Xf + k * o * v * v;
     pair_unpack(ex, X + n1, k, o, N, pv, v, 1, Xf);
     // Xt[(kc)][r][b] = Xf[r][(kc)][b]
     permute(ex, Xf, {o * v, k, v}, {v, o * v * v, 1}, false, T, C1(), C0());
@@ -80,15 +89,18 @@ void sigma_fp64(adc_ctx *c, const cplx *X, cplx *S, int64_t k) {
     const int64_t po = npairs(o);
     // ladder: S2[r][(ij)][a] += x sum_(kl) Glad[(ij)][(kl)] X2[r][(kl)][a]
     ex.tag = "ladder";
-    zgemm(ex, po, v, po, k, CR(x), c->Glad.c(), 0, po, 1, false, X + n1, N, v, 1, false, C1(),
-          S + n1, N, v, 1);
+    if (!fp64_op_product(c, SL_GLAD, false, X, k, X + n1, k * v, N, 1, v, v, CR(x), C1(), S + n1, v, N, 1, v))
+      zgemm(ex, po, v, po, k, CR(x), c->Glad.c(), 0, po, 1, false, X + n1, N, v, 1, false, C1(),
+            S + n1, N, v, 1);
     // ring: Xf[r][i][k][b]; T[r][(j,a)][i] = -sum_(kb) W[(j,a)][(kb)] Xf[r][i][(kb)]
     ex.tag = "ring";
     cplx *Xf = scratch(c, 2 * k * o * o * v);
     cplx *T = Xf + k * o * o * v;
-    pair_unpack(ex, X + n1, k, 1, N, 0, o, v, Xf);
-    zgemm(ex, o * v, o, o * v, k, CR(-1.0), c->W.c(), 0, o * v, 1, false, Xf, o * o * v, 1, o * v,
-          false, C0(), T, o * v * o, o, 1);
+    if (!fp64_op_product(c, SL_W, true, X, k, nullptr, k * o, 0, 0, 1, 0, CR(-1.0), C0(), T, o, o * v * o, 1, o)) {
+      pair_unpack(ex, X + n1, k, 1, N, 0, o, v, Xf);
+      zgemm(ex, o * v, o, o * v, k, CR(-1.0), c->W.c(), 0, o * v, 1, false, Xf, o * o * v, 1, o * v,
+            false, C0(), T, o * v * o, o, 1);
+    }
     // S2[r][(i<j)][a] += x (T[r][j][a][i] - T[r][i][a][j]); view T'(p=i, q=j, in=a) = T[q][in][p]
     pair_pack(ex, T, o * v * o, 0, 1, v * o, o, 1.0, k, 1, o, v, S + n1, N, 0, CR(x), C1());
   }

@@ -207,34 +207,42 @@ void sigma_split(adc_ctx *c, const cplx *X, cplx *S, int64_t k, int nseg) {
   }
 }
 
-// ---- FP64-accurate sigma: the same contractions as sliced tensor-core products.
-// The operators are sliced once for kSlicedBits; a product with fewer bits
-// (the intermediate refinement step) slices only the leading digits of the
-// trial vectors and pairs them with the same leading slices of the operators.
-static void build_sl(adc_ctx *c) {
+// ---- products from digits: the same contractions as sliced tensor-core products.
+static SlCache &sl_cache(adc_ctx *c) {
+  if (!c->sl) c->sl.reset(new SlCache());
+  return *c->sl;
+}
+
+// The digits of a static operator, built when first asked for and rebuilt with
+// more digits when asked for more; a product with fewer bits uses the leading
+// digits of the trial vectors and the same leading digits of the operator.
+static const SlMat &sl_op(adc_ctx *c, int which, int bits) {
   Exec &ex = c->ex;
-  c->sl.reset(new SlCache());
-  SlCache &sl = *c->sl;
-  const int64_t o = c->o, v = c->v, n1 = c->n1, n2 = c->n2;
-  sl.bits = kSlicedBits;
-  sl_pack_A(ex, sl.Cpl, c->Cpl.c(), n1, n2, n2, 1, false, sl.bits);
-  sl_pack_A(ex, sl.CplT, c->Cpl.c(), n2, n1, 1, n2, true, sl.bits);
-  if (c->order == 3 && c->x != 0.0) {
-    const int64_t P = (c->kind == ADC_EA) ? npairs(v) : npairs(o);
-    if (!(c->kind == ADC_EA && c->direct_ladder)) sl_pack_A(ex, sl.Glad, c->Glad.c(), P, P, P, 1, false, sl.bits);
-    sl_pack_A(ex, sl.W, c->W.c(), o * v, o * v, o * v, 1, false, sl.bits);
-  }
-  sl.err = DBuf(ex, sizeof(int));
-  fill_zero(ex, sl.err.p, sizeof(int));
-  sl.ready = true;
+  SlMat &m = sl_cache(c).op[which];
+  if (m.ns * m.b >= bits) return m;
+  const int64_t o = c->o, v = c->v, n1 = c->n1, n2 = c->n2, P = (c->kind == ADC_EA) ? npairs(v) : npairs(o);
+  m.ns = 0;  // nothing usable until the packing is enqueued
+  SlMat t;
+  std::swap(t.planes, m.planes);
+  std::swap(t.exps, m.exps);
+  if (which == SL_CPL) sl_pack_A(ex, t, c->Cpl.c(), n1, n2, n2, 1, false, bits);
+  else if (which == SL_CPLT) sl_pack_A(ex, t, c->Cpl.c(), n2, n1, 1, n2, true, bits);
+  else if (which == SL_GLAD) sl_pack_A(ex, t, c->Glad.c(), P, P, P, 1, false, bits);
+  else sl_pack_A(ex, t, c->W.c(), o * v, o * v, o * v, 1, false, bits);
+  m = std::move(t);
+  return m;
 }
 
 void sigma_sliced(adc_ctx *c, const cplx *X, cplx *S, int64_t k, int bits) {
   ADC_REQUIRE(c->kind != ADC_EE, ADC_ERR_ARG, "sigma_sliced: IP and EA (EE goes through sigma_ee_split)");
   Exec &ex = c->ex;
-  if (!c->sl || !c->sl->ready) build_sl(c);
-  SlCache &sl = *c->sl;
+  SlCache &sl = sl_cache(c);
+  if (!sl.err.p) {
+    sl.err = DBuf(ex, sizeof(int));
+    fill_zero(ex, sl.err.p, sizeof(int));
+  }
   int *err = (int *)sl.err.p;
+  auto op = [&](int which) -> const SlMat & { return sl_op(c, which, kSlicedBits); };
   const int64_t o = c->o, v = c->v, n1 = c->n1, n2 = c->n2, N = c->N;
   const bool sat = (c->order == 3 && c->x != 0.0);
   const double x = sat ? c->x : 0.0;
@@ -243,10 +251,11 @@ void sigma_sliced(adc_ctx *c, const cplx *X, cplx *S, int64_t k, int bits) {
   zgemm(ex, k, n1, n1, 1, C1(), X, 0, N, 1, false, c->M11.c(), 0, 1, n1, false, C0(), S, 0, N, 1);
   // S1 += Cpl X2, S2 = Cpl^H X1
   ex.tag = "coupling";
-  sl_pack_B(ex, sl.Bx, X + n1, k, n2, N, 0, 1, 1, false, sl.Cpl, bits);
-  sl_gemm(ex, sl.Cpl, sl.Bx, n1, k, C1(), C1(), S, 1, N, 0, 1, err, sl.w);
-  sl_pack_B(ex, sl.Bx, X, k, n1, N, 0, 1, 1, false, sl.CplT, bits);
-  sl_gemm(ex, sl.CplT, sl.Bx, n2, k, C1(), C0(), S + n1, 1, N, 0, 1, err, sl.w);
+  const SlMat &cpl = op(SL_CPL), &cplt = op(SL_CPLT);
+  sl_pack_B(ex, sl.Bx, X + n1, k, n2, N, 0, 1, 1, false, cpl, bits);
+  sl_gemm(ex, cpl, sl.Bx, n1, k, C1(), C1(), S, 1, N, 0, 1, err, sl.w);
+  sl_pack_B(ex, sl.Bx, X, k, n1, N, 0, 1, 1, false, cplt, bits);
+  sl_gemm(ex, cplt, sl.Bx, n2, k, C1(), C0(), S + n1, 1, N, 0, 1, err, sl.w);
   diag_mul_add(ex, k, n2, c->d2.d(), X + n1, N, S + n1, N, 1.0);
   if (sat) {
     if (c->kind == ADC_EA) {
@@ -255,23 +264,27 @@ void sigma_sliced(adc_ctx *c, const cplx *X, cplx *S, int64_t k, int bits) {
       if (c->direct_ladder) {
         ladder_direct(c, X + n1, N, o, S + n1, N, k, x, ADC_LADDER_SLICED, err);
       } else {
-        sl_pack_B(ex, sl.Bx, X + n1, k * o, pv, N, pv, o, 1, false, sl.Glad, bits);
-        sl_gemm(ex, sl.Glad, sl.Bx, pv, k * o, CR(x), C1(), S + n1, 1, N, pv, o, err, sl.w);
+        const SlMat &g = op(SL_GLAD);
+        sl_pack_B(ex, sl.Bx, X + n1, k * o, pv, N, pv, o, 1, false, g, bits);
+        sl_gemm(ex, g, sl.Bx, pv, k * o, CR(x), C1(), S + n1, 1, N, pv, o, err, sl.w);
       }
       ex.tag = "ring";
       cplx *T = scratch(c, k * o * v * v);
-      sl_pack_B_ring(ex, sl.Bx, c, X, k, sl.W, bits);
-      sl_gemm(ex, sl.W, sl.Bx, o * v, k * v, C1(), C0(), T, v, o * v * v, 1, v, err, sl.w);
+      const SlMat &w = op(SL_W);
+      sl_pack_B_ring(ex, sl.Bx, c, X, k, w, bits);
+      sl_gemm(ex, w, sl.Bx, o * v, k * v, C1(), C0(), T, v, o * v * v, 1, v, err, sl.w);
       pair_pack(ex, T, o * v * v, v * v, v, 1, 0, 1.0, k, o, v, 1, S + n1, N, pv, CR(-x), C1());
     } else {
       const int64_t po = npairs(o);
       ex.tag = "ladder";
-      sl_pack_B(ex, sl.Bx, X + n1, k * v, po, N, 1, v, v, false, sl.Glad, bits);
-      sl_gemm(ex, sl.Glad, sl.Bx, po, k * v, CR(x), C1(), S + n1, v, N, 1, v, err, sl.w);
+      const SlMat &g = op(SL_GLAD);
+      sl_pack_B(ex, sl.Bx, X + n1, k * v, po, N, 1, v, v, false, g, bits);
+      sl_gemm(ex, g, sl.Bx, po, k * v, CR(x), C1(), S + n1, v, N, 1, v, err, sl.w);
       ex.tag = "ring";
       cplx *T = scratch(c, k * o * v * o);
-      sl_pack_B_ring(ex, sl.Bx, c, X, k, sl.W, bits);
-      sl_gemm(ex, sl.W, sl.Bx, o * v, k * o, CR(-1.0), C0(), T, o, o * v * o, 1, o, err, sl.w);
+      const SlMat &w = op(SL_W);
+      sl_pack_B_ring(ex, sl.Bx, c, X, k, w, bits);
+      sl_gemm(ex, w, sl.Bx, o * v, k * o, CR(-1.0), C0(), T, o, o * v * o, 1, o, err, sl.w);
       pair_pack(ex, T, o * v * o, 0, 1, v * o, o, 1.0, k, 1, o, v, S + n1, N, 0, CR(x), C1());
     }
   }
@@ -281,6 +294,73 @@ void sigma_sliced(adc_ctx *c, const cplx *X, cplx *S, int64_t k, int bits) {
   if (h != 0) {
     fill_zero(ex, err, sizeof(int));
     throw Error(ADC_ERR_TIMEOUT, "tensor-core GEMM wait gave up (code " + std::to_string(h) + ")");
+  }
+}
+
+// ---- one term of the FP64 product with the kept digits of its operator:
+// out = alpha op B^T + beta out as tc_gemm addresses it, B by its strides or (ring)
+// gathered from X2. Slicing the operator again in every product took 6.9 of the
+// 23.6 ms of device time of an EA product at o = 30, v = 150, 8 vectors, and 4.0 of
+// 7.0 ms at second order (o = 25, v = 180, 6 vectors). False (nothing enqueued to out):
+// the term is small, the stream is capturing, or the digits do not fit (they may
+// take a quarter of the free device memory).
+bool fp64_op_product(adc_ctx *c, int which, bool ring, const cplx *X, int64_t k, const cplx *Bsrc, int64_t Nc,
+                     int64_t b_nh, int64_t b_nl, int64_t b_in, int64_t b_k, cplx alpha, cplx beta, cplx *out,
+                     int64_t s_m, int64_t s_nh, int64_t s_nl, int64_t n_in) {
+  Exec &ex = c->ex;
+  const int64_t o = c->o, v = c->v, n1 = c->n1, n2 = c->n2, P = (c->kind == ADC_EA) ? npairs(v) : npairs(o);
+  const int64_t M = which == SL_CPL ? n1 : which == SL_CPLT ? n2 : which == SL_GLAD ? P : o * v;
+  const int64_t K = which == SL_CPL ? n2 : which == SL_CPLT ? n1 : M;
+  if (!fp64_digits_usable(ex, M, Nc, K)) return false;
+  SlCache &sl = sl_cache(c);
+  SlMat &m = sl.op[which];
+  if (sl.no_room[which]) return false;
+  if (m.ns * m.b < kDigitFp64Bits) {
+    const double need = 4.0 * sl_digits(K, kDigitFp64Bits).ns * (double)M * (double)sl_kp(K);
+    double room = 0.25 * (double)free_device_memory();
+    if (ex.mem_limit > 0) room = std::min(room, (double)(ex.mem_limit - ex.mem_used));
+    if (need > room) {
+      sl.no_room[which] = true;
+      return false;
+    }
+  }
+  try {
+    const SlMat &A = sl_op(c, which, kDigitFp64Bits);
+    if (ring) sl_pack_B_ring(ex, sl.Bx, c, X, k, A, kDigitFp64Bits);
+    else sl_pack_B(ex, sl.Bx, Bsrc, Nc, K, b_nh, b_nl, b_in, b_k, false, A, kDigitFp64Bits);
+    sl_gemm(ex, A, sl.Bx, M, Nc, alpha, beta, out, s_m, s_nh, s_nl, n_in, ex.digit_err, sl.w);
+  } catch (const Error &e) {
+    if (e.code != ADC_ERR_OOM) throw;
+    sl.no_room[which] = true;
+    return false;
+  }
+  return true;
+}
+
+// the operators' digits that an FP64 product of k vectors will use, built ahead
+// of a solve that takes the memory left (a term too small to use them builds none)
+void fp64_ops_prepare(adc_ctx *c, int64_t k) {
+  if (c->kind == ADC_EE) return;
+  const int64_t o = c->o, v = c->v, n1 = c->n1, n2 = c->n2, P = (c->kind == ADC_EA) ? npairs(v) : npairs(o);
+  const bool ea = (c->kind == ADC_EA), sat = (c->order == 3 && c->x != 0.0);
+  const int64_t M[SL_NOPS] = {n1, n2, P, o * v}, K[SL_NOPS] = {n2, n1, P, o * v};
+  const int64_t Nc[SL_NOPS] = {k, k, k * (ea ? o : v), k * (ea ? v : o)};
+  for (int w = 0; w < SL_NOPS; ++w) {
+    if (w >= SL_GLAD && !sat) continue;
+    if (w == SL_GLAD && ea && c->direct_ladder) continue;
+    if (!fp64_digits_usable(c->ex, M[w], Nc[w], K[w])) continue;
+    SlCache &sl = sl_cache(c);
+    const double need = 4.0 * sl_digits(K[w], kDigitFp64Bits).ns * (double)M[w] * (double)sl_kp(K[w]);
+    double room = 0.25 * (double)free_device_memory();
+    if (c->ex.mem_limit > 0) room = std::min(room, (double)(c->ex.mem_limit - c->ex.mem_used));
+    if (sl.op[w].ns * sl.op[w].b >= kDigitFp64Bits || sl.no_room[w]) continue;
+    if (need > room) { sl.no_room[w] = true; continue; }
+    try {
+      sl_op(c, w, kDigitFp64Bits);
+    } catch (const Error &e) {
+      if (e.code != ADC_ERR_OOM) throw;
+      sl.no_room[w] = true;
+    }
   }
 }
 

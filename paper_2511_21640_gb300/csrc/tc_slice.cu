@@ -822,11 +822,7 @@ void digit_product(Exec &ex, int64_t M, int64_t N, int64_t K, cplx alpha, const 
 size_t digit_cap(double need) {
   if (g_sliced_cap) return g_sliced_cap;
   if (need <= (double)(1ll << 30)) return (size_t)1 << 30;
-  size_t fr = 0, tot = 0;
-  if (cudaMemGetInfo(&fr, &tot) != cudaSuccess) {
-    cudaGetLastError();
-    fr = (size_t)32 << 30;
-  }
+  const size_t fr = free_device_memory();
   return std::min<size_t>((size_t)16 << 30, std::max<size_t>((size_t)1 << 30, fr / 8));
 }
 
@@ -886,11 +882,8 @@ static bool digits_pay(int64_t M, int64_t N, int64_t K, int64_t batch) {
   return K >= 64 && 8.0 * (double)M * (double)N * (double)K * (double)batch >= (double)(1 << 27);
 }
 
-bool zgemm_fp64_digits(Exec &ex, int64_t M, int64_t N, int64_t K, int64_t batch, cplx alpha, const cplx *A,
-                       int64_t sAb, int64_t sAm, int64_t sAk, bool conjA, const cplx *B, int64_t sBb, int64_t sBk,
-                       int64_t sBn, bool conjB, cplx beta, cplx *C, int64_t sCb, int64_t sCm, int64_t sCn) {
-  const int64_t grouped = (batch > 1 && (sAb == 0 || sBb == 0)) ? batch : 1;
-  if (ex.digits == 0 || K <= 0 || (ex.digits == 1 && !digits_pay(M, N, K, grouped))) return false;
+// a stream under capture keeps the FP64 units (the digit route allocates and may look up free memory)
+static bool digits_ready(Exec &ex) {
   cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
   ADC_CUDA(cudaStreamIsCapturing(ex.stream, &cs));
   if (cs != cudaStreamCaptureStatusNone) return false;
@@ -898,6 +891,18 @@ bool zgemm_fp64_digits(Exec &ex, int64_t M, int64_t N, int64_t K, int64_t batch,
     ADC_CUDA(cudaHostAlloc((void **)&ex.digit_err, sizeof(int), cudaHostAllocMapped));
     *ex.digit_err = 0;
   }
+  return true;
+}
+
+bool fp64_digits_usable(Exec &ex, int64_t M, int64_t N, int64_t K) {
+  return ex.digits != 0 && digits_pay(M, N, K, 1) && digits_ready(ex);
+}
+
+bool zgemm_fp64_digits(Exec &ex, int64_t M, int64_t N, int64_t K, int64_t batch, cplx alpha, const cplx *A,
+                       int64_t sAb, int64_t sAm, int64_t sAk, bool conjA, const cplx *B, int64_t sBb, int64_t sBk,
+                       int64_t sBn, bool conjB, cplx beta, cplx *C, int64_t sCb, int64_t sCm, int64_t sCn) {
+  const int64_t grouped = (batch > 1 && (sAb == 0 || sBb == 0)) ? batch : 1;
+  if (ex.digits == 0 || K <= 0 || (ex.digits == 1 && !digits_pay(M, N, K, grouped)) || !digits_ready(ex)) return false;
   bool begun = false;
   try {
     digit_zgemm(ex, M, N, K, batch, alpha, A, sAb, sAm, sAk, conjA, B, sBb, sBk, sBn, conjB, beta, C, sCb, sCm, sCn,

@@ -49,13 +49,15 @@ struct SlWork {
   DBuf spill, part;
 };
 
-// sliced copies of a context's static operators (built on first use) and the per-call B operand
+// digits of a context's static operators (A side), each built when a product first needs
+// it, and the per-call B operand: shared by the sliced products (their leading digits) and
+// the FP64 ones
+enum { SL_CPL = 0, SL_CPLT = 1, SL_GLAD = 2, SL_W = 3, SL_NOPS = 4 };
 struct SlCache {
-  int bits = 0;
-  SlMat Glad, W, Cpl, CplT, Bx;
+  SlMat op[SL_NOPS], Bx;
+  bool no_room[SL_NOPS] = {};  // FP64 products: the operator's digits did not fit
   SlWork w;
   DBuf err;
-  bool ready = false;
 };
 
 // A[m][k] = op(src[m*s_m + k*s_k]); digits for about `bits` significant bits
@@ -79,6 +81,8 @@ void zgemm_sliced(Exec &ex, int64_t M, int64_t N, int64_t K, int64_t batch, cplx
 bool zgemm_fp64_digits(Exec &ex, int64_t M, int64_t N, int64_t K, int64_t batch, cplx alpha, const cplx *A,
                        int64_t sAb, int64_t sAm, int64_t sAk, bool conjA, const cplx *B, int64_t sBb, int64_t sBk,
                        int64_t sBn, bool conjB, cplx beta, cplx *C, int64_t sCb, int64_t sCm, int64_t sCn);
+// whether an FP64 product of this shape would run from digits now (size, not under capture)
+bool fp64_digits_usable(Exec &ex, int64_t M, int64_t N, int64_t K);
 // out = alpha A B^T + beta out, addressing as tc_gemm
 void sl_gemm(Exec &ex, const SlMat &A, const SlMat &B, int64_t M, int64_t N, cplx alpha, cplx beta, cplx *out,
              int64_t s_m, int64_t s_nh, int64_t s_nl, int64_t n_in, int *err, SlWork &w);

@@ -55,9 +55,15 @@ struct Exec {
   void prof_end(int r);
   void prof_clear();
 
-  void *alloc(size_t bytes);           // cudaMallocAsync on the stream, counted
+  void *alloc(size_t bytes);           // from the device's pool on the stream, counted
   void release(void *p, size_t bytes);  // cudaFreeAsync on the stream
 };
+
+// the device's memory pool keeps freed memory while contexts exist on it (tensor.cu)
+void pool_retain(int dev);
+void pool_release(int dev);
+// free memory of the current device, what the pool holds unused included
+size_t free_device_memory();
 
 // RAII device buffer counted against the context budget.
 struct DBuf {
