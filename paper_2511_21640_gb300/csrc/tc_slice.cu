@@ -330,6 +330,7 @@ __device__ __forceinline__ double scaled_i128(long long hi, int sh, long long lo
   return neg ? -r : r;
 }
 
+// (16 columns at a time: with 32 the registers of the sums spill)
 __device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t (&v)[16]) {
   asm volatile(
       "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, "
@@ -421,9 +422,14 @@ __global__ void __launch_bounds__(320, 1) k_sl_gemm(const __grid_constant__ SlAr
         mbar_drain(smem_u32(&full[st]), (q / L::ST) & 1);
       }
     }
-  } else if (warp == 1 && lane == 0) {
-    // ---------------- MMA issuer
+  } else if (warp == 1) {
+    // ---------------- MMA issuer: the warp walks the schedule as one (so that descriptors
+    // stay in uniform registers), one elected lane issues
     constexpr uint32_t idesc = idesc_bf16(128, BN);
+    const bool lead = elect_one();
+    const uint32_t smem0 = __shfl_sync(0xffffffffu, smem_u32(smem), 0);
+    const uint32_t acc0 = __shfl_sync(0xffffffffu, tmem, 0);
+    const uint32_t desc0 = sdesc_lo(smem0);
     int s = 0;
     uint32_t par = 0, used = 0, epar = 0;  // used, epar: bit d: accumulator d was used, parity of its next wait
     bool stop = false;
@@ -437,51 +443,49 @@ __global__ void __launch_bounds__(320, 1) k_sl_gemm(const __grid_constant__ SlAr
             for (int i = 1; i < hi; ++i) {
               bool ok = sl_wait(smem_u32(&full[s]), par, abort_flag);
               const int dn = min(nd, i);
-              if (ok && kb == kb0 && i <= nd && ((used >> (i - 1)) & 1u)) {
-                // first product into accumulator i - 1 of this run
+              const bool fresh = kb == kb0 && i <= nd;  // the first product into accumulator i - 1 of this run
+              if (ok && fresh && ((used >> (i - 1)) & 1u)) {
                 ok = sl_wait(smem_u32(&acce[i - 1]), (epar >> (i - 1)) & 1u, abort_flag);
                 epar ^= 1u << (i - 1);
               }
-              if (!ok) {
-                if (!*abort_flag) *(volatile int *)a.err = 22;
-                *abort_flag = 1;
+              if (!__all_sync(0xffffffffu, ok)) {
+                if (lane == 0) {
+                  if (!*abort_flag) *(volatile int *)a.err = 22;
+                  *abort_flag = 1;
+                }
                 stop = true;
                 break;
               }
               fence_after();
-              const uint32_t b0 = smem_u32(smem + s * L::STAGE + L::ABYTES);
-              for (int dd = 0; dd < dn; ++dd) {
-                int sa = s - dd;
-                if (sa < 0) sa += L::ST;
-                const uint32_t a0 = smem_u32(smem + sa * L::STAGE);
-                const uint32_t acc = tmem + (uint32_t)(dd * BN);
-                const bool first = (kb == kb0 && i == dd + 1);
+              const uint32_t db = desc0 + (uint32_t)((s * L::STAGE + L::ABYTES) >> 4);
+              if (lead) {
+                for (int dd = 0; dd < dn; ++dd) {
+                  const int sa = s - dd + (s < dd ? L::ST : 0);
+                  const uint32_t da = desc0 + (uint32_t)((sa * L::STAGE) >> 4);
+                  const uint32_t acc = acc0 + (uint32_t)(dd * BN);
+                  const uint32_t keep = (fresh && dd == i - 1) ? 0u : 1u;
+                  mma_bf16_lo(acc, da, db, idesc, keep);
 #pragma unroll
-                for (int k = 0; k < 4; ++k)
-                  mma_bf16(acc, sdesc(a0 + 32 * k), sdesc(b0 + 32 * k), idesc, (first && k == 0) ? 0u : 1u);
-              }
-              if (kb == kb0 && i <= nd) used |= 1u << (i - 1);
-              // digit i - nd + 1 of A has met its last partner; at the end of the block all have
-              if (i >= nd) {
-                int se = s - (nd - 1);
-                if (se < 0) se += L::ST;
-                mma_commit(smem_u32(&empty[se]));
-              }
-              if (i == hi - 1)
-                for (int e = nd - 2; e >= 0; --e) {
-                  int se = s - e;
-                  if (se < 0) se += L::ST;
-                  mma_commit(smem_u32(&empty[se]));
+                  for (int k = 1; k < 4; ++k) mma_bf16_lo(acc, da + 2 * k, db + 2 * k, idesc, 1u);
                 }
+                // digit i - nd + 1 of A has met its last partner; at the end of the block all have
+                if (i >= nd) mma_commit(smem_u32(&empty[s - (nd - 1) + (s < nd - 1 ? L::ST : 0)]));
+                if (i == hi - 1)
+                  for (int e = nd - 2; e >= 0; --e) mma_commit(smem_u32(&empty[s - e + (s < e ? L::ST : 0)]));
+              }
+              __syncwarp();
+              if (fresh) used |= 1u << (i - 1);
               if (++s == L::ST) { s = 0; par ^= 1; }
             }
           }
-          if (!stop) mma_commit(smem_u32(accf));
+          if (!stop && lead) mma_commit(smem_u32(accf));
+          __syncwarp();
         }
       }
     }
-    // every MMA this thread issued has finished before TMEM is freed
-    mma_commit(smem_u32(fin));
+    // every MMA this warp issued has finished before TMEM is freed
+    if (lead) mma_commit(smem_u32(fin));
+    __syncwarp();
     mbar_drain(smem_u32(fin), 0);
   } else if (warp >= 2 && warp < 2 + 4 * L::H) {
     // ---------------- draining warps
