@@ -68,18 +68,32 @@ __device__ inline void atomic_max_nonneg(double *addr, double v) {
   atomicMax((unsigned long long *)addr, (unsigned long long)__double_as_longlong(v));
 }
 
-__global__ void k_herm_check(const cplx *B, int64_t Q, int64_t n, double *out) {
-  const int64_t total = Q * n * n;
+// out[0] = max |B_pq - conj(B_qp)| (1e300 when an element is not finite), out[1] = max |B_pq|.
+// A block takes a 32 x 32 tile of one B[Q] and its mirror image through shared
+// memory, so that both are read along rows (column reads took 1.34 ms for 540 vectors
+// of 108 spinors, 101 MB)
+__global__ void __launch_bounds__(256) k_herm_check(const cplx *B, int64_t Q, int64_t n, double *out) {
+  __shared__ cplx mir[32][33];
+  const int64_t nt = (n + 31) / 32, total = Q * nt * nt;
+  const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
   double dev = 0.0, mag = 0.0;
   bool bad = false;
-  for (int64_t idx = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; idx < total;
-       idx += (int64_t)gridDim.x * blockDim.x) {
-    int64_t q = idx % n, r = idx / n;
-    int64_t p = r % n, Qi = r / n;
-    cplx a = B[idx], b = B[(Qi * n + q) * n + p];
-    if (!isfinite(a.x) || !isfinite(a.y)) bad = true;
-    dev = fmax(dev, fmax(fabs(a.x - b.x), fabs(a.y + b.y)));
-    mag = fmax(mag, fmax(fabs(a.x), fabs(a.y)));
+  for (int64_t t = blockIdx.x; t < total; t += gridDim.x) {
+    const int64_t Qi = t / (nt * nt), r = t - Qi * nt * nt;
+    const int64_t p0 = r / nt * 32, q0 = (r - r / nt * nt) * 32;
+    if (q0 < p0) continue;  // the tile below the diagonal is the mirror image of one above
+    const cplx *Bq = B + Qi * n * n;
+    __syncthreads();
+    for (int i = ty; i < 32; i += 8)
+      if (q0 + i < n && p0 + tx < n) mir[i][tx] = Bq[(q0 + i) * n + p0 + tx];
+    __syncthreads();
+    for (int i = ty; i < 32; i += 8)
+      if (p0 + i < n && q0 + tx < n) {
+        const cplx a = Bq[(p0 + i) * n + q0 + tx], b = mir[tx][i];
+        if (!isfinite(a.x) || !isfinite(a.y) || !isfinite(b.x) || !isfinite(b.y)) bad = true;
+        dev = fmax(dev, fmax(fabs(a.x - b.x), fabs(a.y + b.y)));
+        mag = fmax(mag, fmax(fmax(fabs(a.x), fabs(a.y)), fmax(fabs(b.x), fabs(b.y))));
+      }
   }
   if (bad) dev = 1e300;
   atomic_max_nonneg(out, dev);

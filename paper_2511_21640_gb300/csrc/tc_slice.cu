@@ -304,41 +304,39 @@ __device__ __forceinline__ SlItem sl_item(const SlArgs &a, int it) {
 __device__ __forceinline__ int pass_classes(int hi) { return min(4, hi - 1); }
 __device__ __forceinline__ int pass_run(int hi, int b) { return (1 << (20 - 2 * b)) / (hi == 2 ? 4 : hi + 1); }
 
-// (hi 2^sh + lo) 2^e rounded to nearest
-__device__ __forceinline__ double scaled_i128(long long hi, int sh, long long lo, int e) {
-  const __int128 t = ((__int128)hi << sh) + lo;
-  const bool neg = t < 0;
-  unsigned __int128 u = neg ? (unsigned __int128)(-t) : (unsigned __int128)t;
-  uint64_t h = (uint64_t)(u >> 64), l = (uint64_t)u;
-  if ((h | l) == 0) return 0.0;
-  int top = 127;
-  if (h == 0) { h = l; l = 0; top = 63; }
-  const int lz = __clzll((long long)h);
-  if (lz) { h = (h << lz) | (l >> (64 - lz)); l <<= lz; }
-  top -= lz;                       // value = 1.xxx 2^(top + e)
-  if (l) h |= 1;                   // sticky
-  uint64_t m = h >> 11;            // 53 bits, the leading one set
-  const uint32_t rem = (uint32_t)h & 0x7ffu;
-  if (rem > 0x400u || (rem == 0x400u && (m & 1))) ++m;
-  const int be = top + e + 1023;
-  double r;
-  if (be >= 1 && be <= 2045) {
-    r = __longlong_as_double((long long)(((uint64_t)(be - 1) << 52) + m));
-  } else {
-    r = ldexp((double)m, top + e - 52);
+// (hi 2^sh + lo) 2^e rounded to nearest: hi is shifted up as far as 64 bits allow (62 bits
+// of the sum at least are kept), the sum normalised and packed with integer instructions
+// (an FP64 conversion takes 64 clocks of a scheduler's FP64 unit per warp)
+__device__ __forceinline__ double scaled_sum(long long hi, int sh, long long lo, int e) {
+  const int room = max(0, __clzll(hi < 0 ? -hi : hi) - 2);
+  const int up = min(sh, room);
+  const long long v = (long long)((unsigned long long)hi << up) + (lo >> (sh - up));
+  unsigned long long u = (unsigned long long)(v < 0 ? -v : v);
+  if (u == 0) return 0.0;
+  const int lz = __clzll((long long)u);
+  u <<= lz;
+  const unsigned long long m = (u >> 11) + ((u >> 10) & 1);  // 53 bits, the leading one set (or 2^53)
+  const int be = 63 - lz + (sh - up) + e + 1023;
+  if (be < 1 || be > 2045) {
+    const double r = ldexp((double)m, be - 1075);
+    return v < 0 ? -r : r;
   }
-  return neg ? -r : r;
+  return __longlong_as_double((long long)((((unsigned long long)(be - 1) << 52) + m) |
+                                          ((unsigned long long)v & 0x8000000000000000ull)));
 }
 
-// (16 columns at a time: with 32 the registers of the sums spill)
-__device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t (&v)[16]) {
-  asm volatile(
-      "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, "
-      "%13, %14, %15}, [%16];"
-      : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]),
-        "=r"(v[8]), "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]), "=r"(v[15])
-      : "r"(taddr));
-  asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+// eight columns of an accumulator into registers, and the wait that makes them readable (the
+// registers pass through it, so that no use moves before it); with 16 the sums' registers spill
+__device__ __forceinline__ void tmem_ld8(uint32_t taddr, uint32_t (&v)[8]) {
+  asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+               : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7])
+               : "r"(taddr));
+}
+__device__ __forceinline__ void tmem_wait8(uint32_t (&v)[8]) {
+  asm volatile("tcgen05.wait::ld.sync.aligned;"
+               : "+r"(v[0]), "+r"(v[1]), "+r"(v[2]), "+r"(v[3]), "+r"(v[4]), "+r"(v[5]), "+r"(v[6]), "+r"(v[7])
+               :
+               : "memory");
 }
 
 // bounded wait that looks at the barrier before it reads the clock and the limit
@@ -459,7 +457,9 @@ __global__ void __launch_bounds__(320, 1) k_sl_gemm(const __grid_constant__ SlAr
               fence_after();
               const uint32_t db = desc0 + (uint32_t)((s * L::STAGE + L::ABYTES) >> 4);
               if (lead) {
-                for (int dd = 0; dd < dn; ++dd) {
+#pragma unroll
+                for (int dd = 0; dd < 4; ++dd) {
+                  if (dd >= dn) break;
                   const int sa = s - dd + (s < dd ? L::ST : 0);
                   const uint32_t da = desc0 + (uint32_t)((sa * L::STAGE) >> 4);
                   const uint32_t acc = acc0 + (uint32_t)(dd * BN);
@@ -512,18 +512,27 @@ __global__ void __launch_bounds__(320, 1) k_sl_gemm(const __grid_constant__ SlAr
           }
           par ^= 1;
           fence_after();
+          // the next eight columns load while the current ones are added; an accumulator is
+          // handed back as soon as its last columns are in registers
+          constexpr int CH = L::VALS / 8;
+          uint32_t v[2][8];
+          tmem_ld8(tbase, v[0]);
           for (int dd = 0; dd < nd; ++dd) {
             const int w = 1 << (a.b * dd);
 #pragma unroll
-            for (int c0 = 0; c0 < L::VALS; c0 += 16) {
-              uint32_t v[16];
-              tmem_ld16(tbase + (uint32_t)(dd * BN + c0), v);
+            for (int c = 0; c < CH; ++c) {
+              tmem_wait8(v[c & 1]);
+              if (c + 1 < CH) {
+                tmem_ld8(tbase + (uint32_t)(dd * BN + 8 * (c + 1)), v[(c + 1) & 1]);
+              } else {
+                fence_before();
+                __syncwarp();
+                if (lane == 0) mbar_arrive(smem_u32(&acce[dd]));
+                if (dd + 1 < nd) tmem_ld8(tbase + (uint32_t)((dd + 1) * BN), v[0]);
+              }
 #pragma unroll
-              for (int j = 0; j < 16; ++j) acc[c0 + j] += (long long)__float2int_rn(__uint_as_float(v[j])) * w;
+              for (int j = 0; j < 8; ++j) acc[8 * c + j] += (long long)__float2int_rn(__uint_as_float(v[c & 1][j])) * w;
             }
-            fence_before();
-            __syncwarp();
-            if (lane == 0) mbar_arrive(smem_u32(&acce[dd]));
           }
         }
         if (ok && hi > 5) {  // another pass follows: the sums so far, in units of the first pass, wait
@@ -556,7 +565,7 @@ __global__ void __launch_bounds__(320, 1) k_sl_gemm(const __grid_constant__ SlAr
           } else {
             const int e = scale_exp(wa) + scale_exp(wb) - a.b * (a.ns + 1);
             const long long lr = sh ? sp[(int64_t)(2 * j) * NT] : 0, li = sh ? sp[(int64_t)(2 * j + 1) * NT] : 0;
-            val = cmake(scaled_i128(acc[2 * j], sh, lr, e), scaled_i128(acc[2 * j + 1], sh, li, e));
+            val = cmake(scaled_sum(acc[2 * j], sh, lr, e), scaled_sum(acc[2 * j + 1], sh, li, e));
           }
           if (a.part) {
             a.part[((int64_t)d.split * a.M + m) * Nc + n] = val;
@@ -623,9 +632,10 @@ void pack_rows(Exec &ex, SlMat &d, const BSrc &s, int64_t rows, int64_t K, bool 
   const unsigned gx = (unsigned)std::min<int64_t>(rt, 1 << 20);
   unsigned *W = (unsigned *)d.exps.p;
   fill_zero(ex, W, rows * sizeof(unsigned));
-  // inner ranges: enough blocks to fill the GPU, each at least 512 elements long
+  // inner ranges: enough blocks to fill the GPU (a step of 64 elements takes a few
+  // microseconds whatever its neighbours do: 16 blocks over 500 elements took 31 us)
   const int64_t want = 8ll * device_sm_count();
-  const int64_t parts = std::max<int64_t>(1, std::min<int64_t>((K + 511) / 512, (want + rt - 1) / rt));
+  const int64_t parts = std::max<int64_t>(1, std::min<int64_t>((K + PK_K - 1) / PK_K, (want + rt - 1) / rt));
   int64_t krange = (std::max<int64_t>(K, 1) + parts - 1) / parts;
   krange = (krange + PK_K - 1) / PK_K * PK_K;
   const unsigned gy = (unsigned)((std::max<int64_t>(K, 1) + krange - 1) / krange);
@@ -699,6 +709,36 @@ void sl_pack_B_ring(Exec &ex, SlMat &dst, const adc_ctx *c, const cplx *X, int64
   sl_pack_B_impl(ex, dst, s, Nc, c->o * c->v, false, like, bits);
 }
 
+// Tile width and inner split of a product: the ones that leave the SM with the most
+// work the least of it, in units of an inner block of a 128-column tile (ns (ns + 1) / 2
+// block products of 256 clocks). A 64-column block takes 0.75 and a 32-column one 0.6
+// of that (the A operand's reads bound them); a tile's fill, drains and results cost
+// about 28 k, 16 k and 16 k clocks; a split costs its partial products, about 10 us
+// with the summing kernel's launch.
+struct SlPlan {
+  int bn = 128, ksplit = 1;
+  double clocks = 0.0;
+};
+static SlPlan sl_plan(int64_t M, int64_t N, int64_t kps, int ns) {
+  const double sms = device_sm_count(), block = 128.0 * ns * (ns + 1);
+  const int64_t N2 = 2 * N, tm = (M + 127) / 128;
+  SlPlan best;
+  best.clocks = 1e300;
+  for (int bn = 128; bn >= 32; bn /= 2) {
+    if (bn > 32 && bn / 2 >= N2) continue;  // a narrower tile holds every column
+    const int64_t tiles = tm * ((N2 + bn - 1) / bn);
+    const double per = block * (bn == 128 ? 1.0 : bn == 64 ? 0.75 : 0.6), fixed = bn == 128 ? 28e3 : 16e3;
+    for (int s = 1; s <= 64 && (s == 1 || kps / s >= 2); ++s) {
+      // partial products within 1 GiB
+      if (s > 1 && (double)s * M * N * sizeof(cplx) > (double)(1ll << 30)) break;
+      const double red = s > 1 ? 2e4 + (double)(s + 1) * M * N * 0.01 : 0.0;
+      const double c = std::ceil(tiles * s / sms) * ((double)((kps + s - 1) / s) * per + fixed) + red;
+      if (c < best.clocks) { best.clocks = c; best.bn = bn; best.ksplit = s; }
+    }
+  }
+  return best;
+}
+
 void sl_gemm(Exec &ex, const SlMat &A, const SlMat &B, int64_t M, int64_t N, cplx alpha, cplx beta, cplx *out,
              int64_t s_m, int64_t s_nh, int64_t s_nl, int64_t n_in, int *err, SlWork &w) {
   ADC_REQUIRE(A.kp == B.kp && A.b == B.b, ADC_ERR_ARG, "sl_gemm: operands sliced differently");
@@ -711,7 +751,8 @@ void sl_gemm(Exec &ex, const SlMat &A, const SlMat &B, int64_t M, int64_t N, cpl
   g.b = A.b;
   g.ns = std::min(A.ns, B.ns);  // the common leading slices
   const int64_t N2 = 2 * N, kp2 = 2 * A.kp;
-  const int bn = N2 <= 32 ? 32 : N2 <= 64 ? 64 : 128;
+  const SlPlan plan = sl_plan(M, N, kp2 / 64, g.ns);
+  const int bn = plan.bn;
   tc_make_map3(&g.mA, A.planes.p, A.rows, kp2, A.ns, A.rows * kp2, 128);
   tc_make_map3(&g.mB, B.planes.p, B.rows, kp2, B.ns, B.rows * kp2, bn);
   g.M = (int)M;
@@ -731,18 +772,8 @@ void sl_gemm(Exec &ex, const SlMat &A, const SlMat &B, int64_t M, int64_t N, cpl
   g.amode = alpha.y != 0.0 ? 2 : alpha.x != 1.0 ? 1 : 0;
   g.bmode = beta.y != 0.0 ? 2 : beta.x != 0.0 ? 1 : 0;
   g.err = err;
-  // inner splits: the count that leaves the fewest rounds of work, in units of
-  // inner blocks, a tile's fixed cost being that of about three blocks; at
-  // least eight blocks per split, partial products within 1 GiB
   const int64_t tiles = (int64_t)g.tiles_m * g.tiles_n;
-  int best = 1;
-  double cost = 1e300;
-  for (int s = 1; s <= 64 && (s == 1 || g.kps / s >= 8); ++s) {
-    if (s > 1 && (double)s * M * N * sizeof(cplx) > (double)(1ll << 30)) break;
-    const double c = (double)((tiles * s + sms - 1) / sms) * ((g.kps + s - 1) / s + 3.0) * (s > 1 ? 1.05 : 1.0);
-    if (c < cost) { cost = c; best = s; }
-  }
-  g.kb_per_split = (g.kps + best - 1) / best;
+  g.kb_per_split = (g.kps + plan.ksplit - 1) / plan.ksplit;
   g.ksplit = (g.kps + g.kb_per_split - 1) / g.kb_per_split;
   ADC_REQUIRE(tiles * g.ksplit < (1ll << 31), ADC_ERR_UNSUPPORTED, "sl_gemm: too many tiles");
   g.items = (int)(tiles * g.ksplit);
@@ -877,13 +908,23 @@ void zgemm_sliced(Exec &ex, int64_t M, int64_t N, int64_t K, int64_t batch, cplx
   ADC_REQUIRE(h == 0, ADC_ERR_TIMEOUT, "sliced GEMM: a tensor-core wait gave up (code " + std::to_string(h) + ")");
 }
 
-// FP64 products that leave the FP64 units (1.26 TFLOP/s) for the digits: from 2^27
-// flops on, inner sizes of at least one block. Measured (GB300, M x N x K, FP64 units /
-// digits, slicing included): 256^3 (2^27) 124 / 171 us, 384^3 326 / 215 us,
-// 512^3 783 / 192 us, 200 x 8 x 20000 1.71 / 0.27 ms,
-// 1000 x 1000 x 64 449 / 108 us; below 2^27 the square shapes lose (192^3: 66 / 147 us).
-static bool digits_pay(int64_t M, int64_t N, int64_t K, int64_t batch) {
-  return K >= 64 && 8.0 * (double)M * (double)N * (double)K * (double)batch >= (double)(1 << 27);
+// FP64 products that leave the FP64 units (1.26 TFLOP/s) for the digits: those whose
+// estimated time is shorter there. The digits' estimate is their launches (about 45 us
+// with both operands' slicing, 25 us with the larger one's digits at hand), the slicing's
+// passes over memory at 3 TB/s and the tensor-core kernel's plan; the FP64 units' is their
+// kernel's plan. Measured (GB300, M x N x K, FP64 units / digits, slicing included):
+// 256^3 110 / 150 us, 384^3 320 / 200 us, 200 x 8 x 20000 213 / 250 us,
+// 1000 x 1000 x 64 391 / 104 us, 2500 x 2500 x 40 1760 / 400 us.
+static bool digits_pay(int64_t M, int64_t N, int64_t K, int64_t batch, bool kept) {
+  if (8.0 * (double)M * (double)N * (double)K * (double)batch < (double)(1 << 24)) return false;
+  const double fp64 = zgemm_fp64_clocks(M, N, K, batch);
+  N *= batch;  // a shared operand: the batch becomes a longer column index
+  if (N > M && !kept) std::swap(M, N);
+  constexpr int ns = kDigitFp64Bits / SL_DIGIT;
+  const double kp = (double)sl_kp(K);
+  const double bytes = (kept ? 0.0 : (double)M * (32.0 * K + 4.0 * ns * kp)) + (double)N * (32.0 * K + 8.0 * ns * kp);
+  const double digits = (kept ? 25.0 : 45.0) * 1920.0 + bytes / 3e12 * 1.92e9 + sl_plan(M, N, 2 * sl_kp(K) / 64, ns).clocks;
+  return digits < fp64;
 }
 
 // a stream under capture keeps the FP64 units (the digit route allocates and may look up free memory)
@@ -899,14 +940,14 @@ static bool digits_ready(Exec &ex) {
 }
 
 bool fp64_digits_usable(Exec &ex, int64_t M, int64_t N, int64_t K) {
-  return ex.digits != 0 && digits_pay(M, N, K, 1) && digits_ready(ex);
+  return ex.digits != 0 && digits_pay(M, N, K, 1, true) && digits_ready(ex);
 }
 
 bool zgemm_fp64_digits(Exec &ex, int64_t M, int64_t N, int64_t K, int64_t batch, cplx alpha, const cplx *A,
                        int64_t sAb, int64_t sAm, int64_t sAk, bool conjA, const cplx *B, int64_t sBb, int64_t sBk,
                        int64_t sBn, bool conjB, cplx beta, cplx *C, int64_t sCb, int64_t sCm, int64_t sCn) {
   const int64_t grouped = (batch > 1 && (sAb == 0 || sBb == 0)) ? batch : 1;
-  if (ex.digits == 0 || K <= 0 || (ex.digits == 1 && !digits_pay(M, N, K, grouped)) || !digits_ready(ex)) return false;
+  if (ex.digits == 0 || K <= 0 || (ex.digits == 1 && !digits_pay(M, N, K, grouped, false)) || !digits_ready(ex)) return false;
   bool begun = false;
   try {
     digit_zgemm(ex, M, N, K, batch, alpha, A, sAb, sAm, sAk, conjA, B, sBb, sBk, sBn, conjB, beta, C, sCb, sCm, sCn,

@@ -11,6 +11,7 @@ namespace adc {
 // classes of about 2^-58 of the row and column maxima
 constexpr int kDigitFp64Bits = 56;
 
+constexpr int SL_DIGIT = 7;  // bits of a digit, but for the setup's products (sl_digits)
 // digits of an operand: ns of b bits
 struct SlDigits {
   int b, ns;
@@ -21,7 +22,7 @@ struct SlDigits {
 // as the inner size grows): which bits of the operators they keep depends on the
 // digits, and the BF16 split of an operator must not change with how it was computed.
 inline SlDigits sl_digits(int64_t K, int bits) {
-  int b = 7;
+  int b = SL_DIGIT;
   if (bits > 40 && bits < kDigitFp64Bits) {
     const int64_t K2 = K <= 0 ? 128 : (K + 63) / 64 * 128;
     int l = 0;

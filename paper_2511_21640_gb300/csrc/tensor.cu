@@ -484,6 +484,10 @@ void z_launch(Exec &ex, const ZPlan &p, ZArgs z, int64_t batch, cplx *part, unsi
 constexpr int64_t kMaxPart = (int64_t)1 << 26;  // elements of a call's partial products
 }  // namespace
 
+double zgemm_fp64_clocks(int64_t M, int64_t N, int64_t K, int64_t batch) {
+  return z_plan(M, N, K, batch, 64, kMaxPart, true).clocks;
+}
+
 void zgemm(Exec &ex, int64_t M, int64_t N, int64_t K, int64_t batch, cplx alpha, const cplx *A,
            int64_t sAb, int64_t sAm, int64_t sAk, bool conjA, const cplx *B, int64_t sBb,
            int64_t sBk, int64_t sBn, bool conjB, cplx beta, cplx *C, int64_t sCb, int64_t sCm,
@@ -715,17 +719,24 @@ __global__ void k_add_diag(cplx *M, const double *e, int64_t n, double s) {
   int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (p < n) M[p * n + p].x += s * e[p];
 }
-__global__ void k_antisym_diag(const cplx *B, int64_t Q, int64_t nmo, double *g) {
-  int64_t idx = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (idx >= nmo * nmo) return;
-  int64_t q = idx % nmo, p = idx / nmo;
+// g[p][q] = Re sum_Q (B_pp B_qq - B_pq B_qp): 32 columns q per block, the Cholesky index
+// over eight rows of threads, summed in a fixed order
+__global__ void __launch_bounds__(256)
+k_antisym_diag(const cplx *B, int64_t Q, int64_t nmo, double *g) {
+  __shared__ double red[8][33];
+  const int64_t p = blockIdx.y, q = (int64_t)blockIdx.x * 32 + threadIdx.x;
   double acc = 0.0;
-  for (int64_t Qi = 0; Qi < Q; ++Qi) {
-    const cplx *Bq = B + Qi * nmo * nmo;
-    cplx pp = Bq[p * nmo + p], qq = Bq[q * nmo + q], pq = Bq[p * nmo + q], qp = Bq[q * nmo + p];
-    acc += (pp.x * qq.x - pp.y * qq.y) - (pq.x * qp.x - pq.y * qp.y);
-  }
-  g[idx] = acc;
+  if (q < nmo)
+    for (int64_t Qi = threadIdx.y; Qi < Q; Qi += 8) {
+      const cplx *Bq = B + Qi * nmo * nmo;
+      const cplx pp = Bq[p * nmo + p], qq = Bq[q * nmo + q], pq = Bq[p * nmo + q], qp = Bq[q * nmo + p];
+      acc += (pp.x * qq.x - pp.y * qq.y) - (pq.x * qp.x - pq.y * qp.y);
+    }
+  red[threadIdx.y][threadIdx.x] = acc;
+  __syncthreads();
+  if (threadIdx.y || q >= nmo) return;
+  for (int r = 1; r < 8; ++r) acc += red[r][threadIdx.x];
+  g[p * nmo + q] = acc;
 }
 __global__ void k_zaxpby(int64_t n, cplx a, const cplx *x, cplx b, cplx *y) {
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
@@ -776,7 +787,8 @@ void add_diag(Exec &ex, cplx *M, const double *e, int64_t n, double s) {
   ADC_CHECK_LAUNCH();
 }
 void antisym_diag(Exec &ex, const cplx *B, int64_t Q, int64_t nmo, double *g) {
-  k_antisym_diag<<<grid1d(nmo * nmo, 256), 256, 0, ex.stream>>>(B, Q, nmo, g);
+  // one grid row per spinor: memory ends far below 65535 of them (68 GB per Cholesky vector)
+  k_antisym_diag<<<dim3((unsigned)((nmo + 31) / 32), (unsigned)nmo), dim3(32, 8), 0, ex.stream>>>(B, Q, nmo, g);
   ADC_CHECK_LAUNCH();
 }
 void zaxpby(Exec &ex, int64_t n, cplx a, const cplx *x, cplx b, cplx *y) {

@@ -151,6 +151,9 @@ void zgemm(Exec &ex, int64_t M, int64_t N, int64_t K, int64_t batch, cplx alpha,
            const cplx *B, int64_t sBb, int64_t sBk, int64_t sBn, bool conjB, cplx beta,
            cplx *C, int64_t sCb, int64_t sCm, int64_t sCn);
 
+// estimated clocks of this product on the FP64 units
+double zgemm_fp64_clocks(int64_t M, int64_t N, int64_t K, int64_t batch);
+
 // zgemm without any allocation: split-K partial sums go to ws (ws_elems complex
 // elements; fewer splits when it is small, none when ws is NULL)
 void zgemm_ws(Exec &ex, int64_t M, int64_t N, int64_t K, int64_t batch, cplx alpha,
