@@ -69,9 +69,9 @@ __device__ inline void atomic_max_nonneg(double *addr, double v) {
 }
 
 // out[0] = max |B_pq - conj(B_qp)| (1e300 when an element is not finite), out[1] = max |B_pq|.
-// A block takes a 32 x 32 tile of one B[Q] and its mirror image through shared
-// memory, so that both are read along rows (column reads took 1.34 ms for 540 vectors
-// of 108 spinors, 101 MB)
+// One pair of atomics per warp (one per thread, on two addresses, took 1.34 ms
+// for 540 vectors of 108 spinors, 101 MB); a block takes a 32 x 32 tile of one B[Q] and
+// its mirror image through shared memory, so that both are read along rows
 __global__ void __launch_bounds__(256) k_herm_check(const cplx *B, int64_t Q, int64_t n, double *out) {
   __shared__ cplx mir[32][33];
   const int64_t nt = (n + 31) / 32, total = Q * nt * nt;
@@ -96,6 +96,11 @@ __global__ void __launch_bounds__(256) k_herm_check(const cplx *B, int64_t Q, in
       }
   }
   if (bad) dev = 1e300;
+  for (int off = 16; off > 0; off >>= 1) {
+    dev = fmax(dev, __shfl_xor_sync(0xffffffffu, dev, off));
+    mag = fmax(mag, __shfl_xor_sync(0xffffffffu, mag, off));
+  }
+  if (tx) return;
   atomic_max_nonneg(out, dev);
   atomic_max_nonneg(out + 1, mag);
 }

@@ -117,11 +117,12 @@ DBuf build_vvvv_packed(adc_ctx *c) {
   DBuf L = cbuf(c->ex, v * v * Q);
   permute(c->ex, c->B.c() + c->o * c->nmo + c->o, {v, v, Q}, {c->nmo, 1, c->nmo * c->nmo}, false,
           L.c(), C1(), C0());
-  // a blocks sized so that J stays below ~1 GiB, and at least eight of them: a block
-  // computes b >= a0, so eight do 56% of the square's work and one all of it (EA, v = 90,
-  // naux = 540: one block took 11.4 ms of a 57 ms setup)
+  // a blocks sized so that J stays below ~1 GiB, and eight of them while each keeps 512 rows:
+  // a block computes b >= a0, so eight do 56% of the square's work and one all of it (EA,
+  // v = 90, naux = 540: one block took 11.4 ms of a 57 ms setup)
   int64_t ca = std::max<int64_t>(1, (int64_t)(1ll << 26) / (v * v * v));
-  ca = std::min(ca, std::max<int64_t>((v + 7) / 8, 1));
+  ca = std::min(ca, std::max((v + 7) / 8, (512 + v - 1) / v));
+  ca = std::min(ca, v);
   DBuf J = cbuf(c->ex, ca * v * v * v);
   for (int64_t a0 = 0; a0 < v - 1; a0 += ca) {
     int64_t na = std::min(ca, v - a0);

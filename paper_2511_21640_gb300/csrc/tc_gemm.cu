@@ -120,25 +120,37 @@ k_tc_gemm(const __grid_constant__ CUtensorMap mAh, const __grid_constant__ CUten
         mbar_drain(smem_u32(&full[s]), r & 1);
       }
     }
-  } else if (warp == 1 && lane == 0) {
-    // ---------------- MMA issuer
+  } else if (warp == 1) {
+    // ---------------- MMA issuer: the warp walks the stages as one, so that descriptors stay
+    // in uniform registers (formed in one thread's they take longer than the MMAs), and an
+    // elected lane issues
     constexpr uint32_t idesc = idesc_bf16(TC_BM, BN);
+    const bool lead = elect_one();
+    const uint32_t acc = __shfl_sync(0xffffffffu, tmem, 0);
+    const uint32_t desc0 = sdesc_lo(__shfl_sync(0xffffffffu, smem_u32(smem), 0));
     for (int i = 0; i < nkb; ++i) {
       const int s = i % ST, r = i / ST;
-      if (!mbar_wait(smem_u32(&full[s]), r & 1, abort_flag)) {
-        if (!*abort_flag) atomicExch(err, 2);
-        *abort_flag = 1;
+      if (!__all_sync(0xffffffffu, mbar_try(smem_u32(&full[s]), r & 1) ||
+                                       mbar_wait(smem_u32(&full[s]), r & 1, abort_flag))) {
+        if (lane == 0) {
+          if (!*abort_flag) atomicExch(err, 2);
+          *abort_flag = 1;
+        }
+        __syncwarp();
         break;
       }
       fence_after();
-      const uint32_t a0 = smem_u32(smem + s * L::STAGE);
-      const uint32_t b0 = a0 + L::A_BYTES;
+      const uint32_t da = desc0 + (uint32_t)((s * L::STAGE) >> 4), db = da + (uint32_t)(L::A_BYTES >> 4);
+      if (lead) {
+        mma_bf16_lo(acc, da, db, idesc, i > 0 ? 1u : 0u);
 #pragma unroll
-      for (int k = 0; k < TC_BK / 16; ++k)
-        mma_bf16(tmem, sdesc(a0 + 32 * k), sdesc(b0 + 32 * k), idesc, (i > 0 || k > 0) ? 1u : 0u);
-      mma_commit(smem_u32(&empty[s]));
+        for (int k = 1; k < TC_BK / 16; ++k) mma_bf16_lo(acc, da + 2 * k, db + 2 * k, idesc, 1u);
+        mma_commit(smem_u32(&empty[s]));
+      }
+      __syncwarp();
     }
-    mma_commit(smem_u32(accum));
+    if (lead) mma_commit(smem_u32(accum));
+    __syncwarp();
     // after an abort the MMAs already issued finish before TMEM is freed
     if (*abort_flag) mbar_drain(smem_u32(accum), 0);
   } else if (warp >= 2) {
@@ -388,6 +400,17 @@ __device__ __forceinline__ void tensormap_acquire(const CUtensorMap *m) {
   asm volatile("fence.proxy.tensormap::generic.acquire.gpu [%0], 128;" ::"l"((uint64_t)m) : "memory");
 }
 
+// The wide launches' shared memory: rings of A blocks (16 KB) and B blocks (up to 32 KB).
+// The plain loop loads both operands of every product, six blocks for the three
+// products of an inner block; here the four blocks hi and lo of A and B are
+// loaded once and serve all three.
+struct TwLayout {
+  static constexpr int A_BYTES = TC_BM * TC_BK * 2, B_BYTES = TC_BNMAX * TC_BK * 2;
+  static constexpr int SA = 4, SB = 5;
+  static constexpr int B_OFF = SA * A_BYTES, BAR_OFF = B_OFF + SB * B_BYTES;
+  static constexpr int SMEM = 1024 + BAR_OFF + 512;
+};
+
 struct TgTile {
   const TcJob *J;
   int m0, n0, bn, split, kb_beg, nkb;
@@ -429,13 +452,18 @@ __device__ __forceinline__ TgTile tg_decode(const TcJob *__restrict__ jobs, int 
   return d;
 }
 
+// WIDE: the loop for launches dominated by wide tiles (TwLayout); the products of a tile
+// run in the same order in both, so that their sums are the same to the last bit
+template <bool WIDE>
 __global__ void __launch_bounds__(192, 1)
 k_tc_grouped(const TcJob *__restrict__ jobs, int njobs, int total_tiles, int *counter, int *err) {
   extern __shared__ uint8_t smem_raw[];
   uint8_t *smem = (uint8_t *)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
-  uint64_t *full = (uint64_t *)(smem + TgLayout::BAR_OFF);
-  uint64_t *empty = full + TG_ST;
-  uint64_t *accf = empty + TG_ST;   // accumulator b holds a finished tile (MMA -> epilogue)
+  // plain: full, empty per stage; wide: full and empty of A blocks, then of B blocks
+  constexpr int RING = WIDE ? TwLayout::SA + TwLayout::SB : TG_ST;
+  uint64_t *full = (uint64_t *)(smem + (WIDE ? TwLayout::BAR_OFF : TgLayout::BAR_OFF));
+  uint64_t *empty = full + RING;
+  uint64_t *accf = empty + RING;   // accumulator b holds a finished tile (MMA -> epilogue)
   uint64_t *acce = accf + 2;        // accumulator b drained (epilogue -> MMA)
   uint64_t *tfull = acce + 2;       // tile number published (producer -> consumers)
   uint64_t *tempty = tfull + TG_TQ;  // tile number read by the MMA warp and the 4 epilogue warps
@@ -446,7 +474,7 @@ k_tc_grouped(const TcJob *__restrict__ jobs, int njobs, int total_tiles, int *co
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   if (threadIdx.x == 0) {
-    for (int s = 0; s < TG_ST; ++s) {
+    for (int s = 0; s < RING; ++s) {
       mbar_init(smem_u32(&full[s]), 1);
       mbar_init(smem_u32(&empty[s]), 1);
     }
@@ -476,7 +504,7 @@ k_tc_grouped(const TcJob *__restrict__ jobs, int njobs, int total_tiles, int *co
 
   if (warp == 0 && lane == 0) {
     // ---------------- tile scheduler and TMA producer
-    uint32_t g = 0, g_issued = 0;
+    uint32_t g = 0, gB = 0, g_issued = 0;  // wide: A and B blocks loaded
     const uint64_t pol_last = policy_evict_last(), pol_first = policy_evict_first();
     for (uint32_t q = 0;; ++q) {
       const int slot = (int)(q % TG_TQ);
@@ -496,8 +524,39 @@ k_tc_grouped(const TcJob *__restrict__ jobs, int njobs, int total_tiles, int *co
       tensormap_acquire(&J.mAl);
       tensormap_acquire(&J.mBh);
       tensormap_acquire(&J.mBl);
-      const uint32_t bytes = (uint32_t)(TgLayout::A_BYTES + d.bn * TC_BK * 2);
       bool stop = false;
+      if constexpr (WIDE) {
+        // blocks in the order of their use: A hi, B hi, B lo, A lo
+        const uint32_t bb = (uint32_t)(d.bn * TC_BK * 2);
+        auto load = [&](bool isA, const CUtensorMap *map, int kx, int y) {
+          uint32_t &n = isA ? g : gB;
+          constexpr uint32_t SA = TwLayout::SA, SB = TwLayout::SB;
+          const uint32_t s = isA ? n % SA : n % SB, use = isA ? n / SA : n / SB;
+          const uint32_t bar = isA ? s : SA + s;
+          if (use > 0 && !mbar_wait(smem_u32(&empty[bar]), (use - 1) & 1, abort_flag)) return false;
+          const uint32_t fb = smem_u32(&full[bar]);
+          mbar_expect_tx(fb, isA ? (uint32_t)TwLayout::A_BYTES : bb);
+          const uint32_t dst =
+              smem_u32(smem + (isA ? s * TwLayout::A_BYTES : TwLayout::B_OFF + s * TwLayout::B_BYTES));
+          if (J.l2keepB) tma_load_2d_hint(dst, map, kx, y, fb, isA ? pol_first : pol_last);
+          else tma_load_2d(dst, map, kx, y, fb);
+          ++n;
+          return true;
+        };
+        for (int q = d.kb_beg / 3; q <= (d.kb_beg + d.nkb - 1) / 3; ++q) {
+          const int kx = q * TC_BK;
+          if (!load(true, &J.mAh, kx, d.m0) || !load(false, &J.mBh, kx, d.n0) || !load(false, &J.mBl, kx, d.n0) ||
+              !load(true, &J.mAl, kx, d.m0)) {
+            if (!*abort_flag) atomicExch(err, 11);
+            *abort_flag = 1;
+            stop = true;
+            break;
+          }
+        }
+        if (stop) break;
+        continue;
+      }
+      const uint32_t bytes = (uint32_t)(TgLayout::A_BYTES + d.bn * TC_BK * 2);
       for (int i = 0; i < d.nkb; ++i) {
         const uint32_t gi = g + (uint32_t)i;
         const int s = (int)(gi % TG_ST);
@@ -530,12 +589,91 @@ k_tc_grouped(const TcJob *__restrict__ jobs, int njobs, int total_tiles, int *co
     }
     if (*abort_flag) {
       // drain this CTA's copies in flight before shared memory is released
+      if constexpr (WIDE) {
+        constexpr uint32_t SA = TwLayout::SA, SB = TwLayout::SB;
+        for (uint32_t q = (g > SA ? g - SA : 0); q < g; ++q) mbar_drain(smem_u32(&full[q % SA]), (q / SA) & 1);
+        for (uint32_t q = (gB > SB ? gB - SB : 0); q < gB; ++q)
+          mbar_drain(smem_u32(&full[SA + q % SB]), (q / SB) & 1);
+      }
       for (uint32_t gj = (g_issued > TG_ST ? g_issued - TG_ST : 0); gj < g_issued; ++gj) {
         const int s = (int)(gj % TG_ST);
         mbar_drain(smem_u32(&full[s]), (gj / TG_ST) & 1);
       }
     }
-  } else if (warp == 1 && lane == 0) {
+  } else if (WIDE && warp == 1) {
+    // ---------------- MMA issuer of the wide loop: the warp walks the tiles as one
+    // (descriptors in uniform registers), an elected lane issues
+    constexpr uint32_t SA = TwLayout::SA, SB = TwLayout::SB;
+    const bool lead = elect_one();
+    const uint32_t acc0 = __shfl_sync(0xffffffffu, tmem, 0);
+    const uint32_t desc0 = sdesc_lo(__shfl_sync(0xffffffffu, smem_u32(smem), 0));
+    uint32_t nA = 0, nB = 0;  // blocks consumed
+    auto wait_all = [&](uint64_t *bar, uint32_t parity, int code) {
+      if (__all_sync(0xffffffffu, mbar_try(smem_u32(bar), parity) || mbar_wait(smem_u32(bar), parity, abort_flag)))
+        return true;
+      if (lane == 0) {
+        if (!*abort_flag) atomicExch(err, code);
+        *abort_flag = 1;
+      }
+      __syncwarp();
+      return false;
+    };
+    for (uint32_t q = 0;; ++q) {
+      const int slot = (int)(q % TG_TQ);
+      if (!wait_all(&tfull[slot], (q / TG_TQ) & 1, 15)) break;
+      const int t = __shfl_sync(0xffffffffu, (int)ring[slot], 0);
+      __syncwarp();
+      if (lane == 0) mbar_arrive(smem_u32(&tempty[slot]));
+      if (t >= total_tiles) break;
+      const TgTile d = tg_decode(jobs, njobs, t);
+      const uint32_t b = q & 1u, use = q >> 1;
+      if (use > 0 && !wait_all(&acce[b], (use - 1) & 1, 16)) break;
+      fence_after();
+      const uint32_t dacc = acc0 + b * (uint32_t)TC_BNMAX;
+      const uint32_t idesc = idesc_bf16(TC_BM, __shfl_sync(0xffffffffu, d.bn, 0));
+      const int kb_beg = __shfl_sync(0xffffffffu, d.kb_beg, 0), kb_end = kb_beg + __shfl_sync(0xffffffffu, d.nkb, 0);
+      auto product = [&](uint32_t a, uint32_t bb, uint32_t keep) {
+        const uint32_t da = desc0 + ((a * TwLayout::A_BYTES) >> 4);
+        const uint32_t db = desc0 + ((TwLayout::B_OFF + bb * TwLayout::B_BYTES) >> 4);
+        mma_bf16_lo(dacc, da, db, idesc, keep);
+#pragma unroll
+        for (int k = 1; k < TC_BK / 16; ++k) mma_bf16_lo(dacc, da + 2 * k, db + 2 * k, idesc, 1u);
+      };
+      bool stop = false;
+      for (int kq = kb_beg / 3; kq <= (kb_end - 1) / 3; ++kq) {
+        // a split may begin or end inside the three products of a block
+        const int lo = max(0, kb_beg - 3 * kq), hi = min(3, kb_end - 3 * kq);
+        const uint32_t ah = nA % SA, al = (nA + 1) % SA, bh = nB % SB, bl = (nB + 1) % SB;
+        if (!wait_all(&full[ah], (nA / SA) & 1, 12) || !wait_all(&full[SA + bh], (nB / SB) & 1, 12)) { stop = true; break; }
+        fence_after();
+        if (lead && lo == 0) product(ah, bh, 3 * kq > kb_beg ? 1u : 0u);
+        if (!wait_all(&full[SA + bl], ((nB + 1) / SB) & 1, 12)) { stop = true; break; }
+        fence_after();
+        if (lead) {
+          if (lo <= 1 && hi > 1) product(ah, bl, 3 * kq + 1 > kb_beg ? 1u : 0u);
+          mma_commit(smem_u32(&empty[ah]));
+          mma_commit(smem_u32(&empty[SA + bl]));
+        }
+        __syncwarp();
+        if (!wait_all(&full[al], ((nA + 1) / SA) & 1, 12)) { stop = true; break; }
+        fence_after();
+        if (lead) {
+          if (hi > 2) product(al, bh, 3 * kq + 2 > kb_beg ? 1u : 0u);
+          mma_commit(smem_u32(&empty[al]));
+          mma_commit(smem_u32(&empty[SA + bh]));
+        }
+        __syncwarp();
+        nA += 2;
+        nB += 2;
+      }
+      if (stop) break;
+      if (lead) mma_commit(smem_u32(&accf[b]));
+      __syncwarp();
+    }
+    if (lead) mma_commit(smem_u32(fin));
+    __syncwarp();
+    mbar_drain(smem_u32(fin), 0);
+  } else if (!WIDE && warp == 1 && lane == 0) {
     // ---------------- MMA issuer, accumulators alternating
     uint32_t g = 0;
     for (uint32_t q = 0;; ++q) {
@@ -795,10 +933,11 @@ static int cached_bn(const TcJobDesc &d) {
   return it == g_tuned.end() ? 0 : it->second;
 }
 
-void tc_gemm_grouped(Exec &ex, const std::vector<TcJobDesc> &in, TcGroup &grp, int *err, bool may_tune) {
+void tc_gemm_grouped(Exec &ex, const std::vector<TcJobDesc> &in, TcGroup &grp, int *err, bool may_tune, bool timing) {
   const int nj = (int)in.size();
   if (nj == 0) return;
-  set_smem_limit((const void *)k_tc_grouped, TgLayout::SMEM);
+  set_smem_limit((const void *)k_tc_grouped<false>, TgLayout::SMEM);
+  set_smem_limit((const void *)k_tc_grouped<true>, TwLayout::SMEM);
   cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
   ADC_CUDA(cudaStreamIsCapturing(ex.stream, &cs));
   const bool capturing = (cs != cudaStreamCaptureStatusNone);
@@ -808,7 +947,7 @@ void tc_gemm_grouped(Exec &ex, const std::vector<TcJobDesc> &in, TcGroup &grp, i
     int64_t N2;
   };
   std::vector<Plan> pl;
-  double work = 0.0;
+  double work = 0.0, cols = 0.0, wide_cols = 0.0;
   grp.flops = 0.0;
   for (int j = 0; j < nj; ++j) {
     const TcJobDesc &d = in[j];
@@ -828,7 +967,10 @@ void tc_gemm_grouped(Exec &ex, const std::vector<TcJobDesc> &in, TcGroup &grp, i
     p.nseg = 3;  // hi hi, hi lo, lo hi
     p.tiles_m = (int)((d.M + TC_BM - 1) / TC_BM);
     p.tiles_n = (int)((p.N2 + p.bn - 1) / p.bn);
-    work += (double)p.tiles_m * p.tiles_n * (double)p.nseg * p.kps;
+    const double job_work = (double)p.tiles_m * p.tiles_n * (double)p.nseg * p.kps;
+    work += job_work;
+    cols += job_work * p.bn;
+    if (p.bn >= 192) wide_cols += job_work * p.bn;
     const int64_t Kc = d.A->kreal > 0 ? d.A->kreal : d.A->kp;
     grp.flops += 8.0 * (double)d.M * (double)d.N * (double)Kc;
     pl.push_back(p);
@@ -924,8 +1066,18 @@ void tc_gemm_grouped(Exec &ex, const std::vector<TcJobDesc> &in, TcGroup &grp, i
   ADC_CUDA(cudaMemsetAsync(grp.counter.p, 0, sizeof(int), ex.stream));
   const int grid = (int)std::min<int64_t>(tiles, sms);
   int pr = ex.prof_begin("tc_grouped_bf16x3", grp.flops);
-  k_tc_grouped<<<grid, 192, TgLayout::SMEM, ex.stream>>>((const TcJob *)grp.jobs.p, np, (int)tiles,
-                                                         (int *)grp.counter.p, err);
+  // The wide loop where tiles of 192 columns and more hold nine tenths of the work and every
+  // SM has a thousand 256-column block products to do (fewer, and the plain loop's lighter stages do as
+  // well). Measured (GB300, EA o = 40, v = 200, 8 vectors: 5.6 PFLOP in one launch) plain 5.17,
+  // wide 4.34 ms. The autotuner always times the plain loop: the width it picks also
+  // decides how inner sums are split, which must not depend on the loop that runs.
+  const bool wide = !timing && wide_cols >= 0.9 * cols && cols >= 256e3 * sms;
+  if (wide)
+    k_tc_grouped<true><<<grid, 192, TwLayout::SMEM, ex.stream>>>((const TcJob *)grp.jobs.p, np, (int)tiles,
+                                                                 (int *)grp.counter.p, err);
+  else
+    k_tc_grouped<false><<<grid, 192, TgLayout::SMEM, ex.stream>>>((const TcJob *)grp.jobs.p, np, (int)tiles,
+                                                                  (int *)grp.counter.p, err);
   ADC_CHECK_LAUNCH();
   for (int i = 0; i < np; ++i) {
     const TcJob &J = grp.host[i];
@@ -982,9 +1134,9 @@ int tc_autotune_bn(Exec &ex, const TcJobDesc &d, int *err) {
       t.alpha = C1();
       t.beta = C0();
       std::vector<TcJobDesc> one{t};
-      tc_gemm_grouped(ex, one, g, err, false);
+      tc_gemm_grouped(ex, one, g, err, false, true);
       ADC_CUDA(cudaEventRecord(e0, ex.stream));
-      for (int r = 0; r < 2; ++r) tc_gemm_grouped(ex, one, g, err, false);
+      for (int r = 0; r < 2; ++r) tc_gemm_grouped(ex, one, g, err, false, true);
       ADC_CUDA(cudaEventRecord(e1, ex.stream));
       ADC_CUDA(cudaEventSynchronize(e1));
       float ms = 0.f;

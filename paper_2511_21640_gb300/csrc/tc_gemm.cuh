@@ -170,7 +170,9 @@ struct TcGroup {
 // enqueue all jobs as one persistent launch (plus split-K reductions). With
 // may_tune, jobs with bn == 0 get the autotuned tile width (timing runs need a
 // stream that is not being captured); otherwise a size rule picks it.
-void tc_gemm_grouped(Exec &ex, const std::vector<TcJobDesc> &jobs, TcGroup &grp, int *err, bool may_tune);
+// (timing: one of the autotuner's own launches)
+void tc_gemm_grouped(Exec &ex, const std::vector<TcJobDesc> &jobs, TcGroup &grp, int *err, bool may_tune,
+                     bool timing = false);
 // tile width chosen by timing every candidate once per (M, N, K) shape; cached
 int tc_autotune_bn(Exec &ex, const TcJobDesc &d, int *err);
 // table of tuned shapes: (M, N2, kp, bn); returns the number of entries

@@ -43,3 +43,13 @@ def gpu():
 def test_digit_product_edges(gpu, which, M, N, K):
     err, _ = gpu.diag_gemm(which, M, N, K, seed=3 + M, reps=1)
     assert err < 2.0 ** (2.5 - BITS[which]) + 2.0 ** -50 * math.sqrt(K), err
+
+
+@pytest.mark.parametrize("which,M,N,K", [(2, 6000, 1300, 3300), (3, 6000, 1300, 3300)])
+def test_wide_grouped_launch(gpu, which, M, N, K):
+    """A grouped BF16x3 launch large enough for the wide loop, one job and three (one of them
+    narrow, its inner sums split inside a block's three products). Each operand keeps 16 bits
+    (2^-17 relative, 2^-16.5 for both) and the FP32 sums of K random terms lose at most 2^-24
+    sqrt(2 K) of the largest: 2^-14 covers both."""
+    err, _ = gpu.diag_gemm(which, M, N, K, seed=21, reps=1)
+    assert err < 2.0 ** -14, err
