@@ -188,6 +188,8 @@ k_combine(const cplx *__restrict__ C, int64_t ldc, int m, int nr, const cplx *__
     }
     __syncthreads();
     if (k < n) {
+      // (eight rows' loads in flight)
+#pragma unroll 8
       for (int i = 0; i < ni; ++i) {
         const cplx v = V[(int64_t)(i0 + i) * ldv + k];
         const double vs = v.x + v.y;
@@ -245,7 +247,8 @@ void gram(Exec &ex, const cplx *A, int64_t lda, int na, const cplx *B, int64_t l
   const int gy = (np + best->ga - 1) / best->ga, gz = (nr + best->gb - 1) / best->gb;
   // enough CTAs for four per SM, each chunk at least four staged steps
   int64_t nchunk = std::max<int64_t>(1, (4 * (int64_t)sm_count() + gy * gz - 1) / (gy * gz));
-  nchunk = std::min<int64_t>(nchunk, std::max<int64_t>(1, n / (4 * best->gk)));
+  // (short vectors: down to one step, so that more than a few SMs take part)
+  nchunk = std::min<int64_t>(nchunk, std::max<int64_t>(1, n / (n < 65536 ? best->gk : 4 * best->gk)));
   int64_t chunk = (n + nchunk - 1) / nchunk;
   chunk = (chunk + best->gk - 1) / best->gk * best->gk;
   nchunk = std::max<int64_t>(1, (n + chunk - 1) / chunk);
@@ -263,10 +266,13 @@ void gram(Exec &ex, const cplx *A, int64_t lda, int na, const cplx *B, int64_t l
 void combine(Exec &ex, const cplx *C, int64_t ldc, int m, int nr, const cplx *V, int64_t ldv, int64_t n,
              cplx alpha, cplx beta, cplx *Y, int64_t ldy) {
   if (nr <= 0 || n <= 0) return;
-  const int64_t gx = (n + 255) / 256;
   // rows per CTA: the smallest group that covers nr in as few padded rows as
-  // possible (16 for more than 8)
-  const int RR = nr >= 9 ? 16 : nr >= 5 ? 8 : nr >= 3 ? 4 : nr;
+  // possible (16 for more than 8). Short vectors, whose CTAs would leave most SMs
+  // idle, one row and 64 threads (680 elements, 40 rows into 4: 20 us on three SMs)
+  const bool small = (n + 255) / 256 * ((nr + 3) / 4) < sm_count();
+  const int threads = small ? 64 : 256;
+  const int64_t gx = (n + threads - 1) / threads;
+  const int RR = small ? 1 : nr >= 9 ? 16 : nr >= 5 ? 8 : nr >= 3 ? 4 : nr;
   const int gy = (nr + RR - 1) / RR;
   ADC_REQUIRE(gx < (1ll << 31) && gy <= 65535, ADC_ERR_UNSUPPORTED, "combine: shape");
   const bool rd = (beta.x != 0.0 || beta.y != 0.0);
@@ -274,11 +280,11 @@ void combine(Exec &ex, const cplx *C, int64_t ldc, int m, int nr, const cplx *V,
                          16.0 * ((double)m + (rd ? 2.0 : 1.0) * nr) * (double)n);
   const dim3 grid((unsigned)gx, gy);
   switch (RR) {
-    case 1: k_combine<1><<<grid, 256, 0, ex.stream>>>(C, ldc, m, nr, V, ldv, n, alpha, beta, Y, ldy); break;
-    case 2: k_combine<2><<<grid, 256, 0, ex.stream>>>(C, ldc, m, nr, V, ldv, n, alpha, beta, Y, ldy); break;
-    case 4: k_combine<4><<<grid, 256, 0, ex.stream>>>(C, ldc, m, nr, V, ldv, n, alpha, beta, Y, ldy); break;
-    case 8: k_combine<8><<<grid, 256, 0, ex.stream>>>(C, ldc, m, nr, V, ldv, n, alpha, beta, Y, ldy); break;
-    default: k_combine<16><<<grid, 256, 0, ex.stream>>>(C, ldc, m, nr, V, ldv, n, alpha, beta, Y, ldy); break;
+    case 1: k_combine<1><<<grid, threads, 0, ex.stream>>>(C, ldc, m, nr, V, ldv, n, alpha, beta, Y, ldy); break;
+    case 2: k_combine<2><<<grid, threads, 0, ex.stream>>>(C, ldc, m, nr, V, ldv, n, alpha, beta, Y, ldy); break;
+    case 4: k_combine<4><<<grid, threads, 0, ex.stream>>>(C, ldc, m, nr, V, ldv, n, alpha, beta, Y, ldy); break;
+    case 8: k_combine<8><<<grid, threads, 0, ex.stream>>>(C, ldc, m, nr, V, ldv, n, alpha, beta, Y, ldy); break;
+    default: k_combine<16><<<grid, threads, 0, ex.stream>>>(C, ldc, m, nr, V, ldv, n, alpha, beta, Y, ldy); break;
   }
   ADC_CHECK_LAUNCH();
   ex.prof_end(pr);

@@ -60,6 +60,38 @@ __host__ __device__ inline void cfma(cplx &acc, cplx a, cplx b) {
   acc.y = fma(a.y, b.x, acc.y);
 }
 
+// A factor by kind: 0 zero, 1 one, 2 real, 3 complex. The element-wise kernels take the
+// kind, because a complex multiply by 1 or by a real factor costs four FP64 operations of
+// which none or two are needed, and at two a clock and SM they, not memory, bound such kernels.
+inline int factor_kind(cplx a) { return a.y != 0.0 ? 3 : a.x == 1.0 ? 1 : a.x == 0.0 ? 0 : 2; }
+__device__ __forceinline__ cplx scaled(int kind, cplx a, cplx v) {
+  if (kind == 1) return v;
+  if (kind == 3) return cmul(a, v);
+  return make_double2(a.x * v.x, a.x * v.y);
+}
+// alpha v + beta *old
+__device__ __forceinline__ cplx axpby(int ka, cplx alpha, cplx v, int kb, cplx beta, const cplx *old) {
+  cplx r = scaled(ka, alpha, v);
+  if (kb) {
+    const cplx o = scaled(kb, beta, *old);
+    r = make_double2(r.x + o.x, r.y + o.y);
+  }
+  return r;
+}
+
+// Division of n < 2^31 by a constant found at run time: two multiplies' worth instead of
+// the tens of instructions of an integer division
+struct FastDiv {
+  uint32_t d, mul, sh;
+};
+inline FastDiv fast_div(uint32_t d) {
+  FastDiv f{d, 1, 0};
+  while ((1ull << f.sh) < d) ++f.sh;
+  f.mul = (uint32_t)((((1ull << f.sh) - d) << 32) / d + 1);
+  return f;
+}
+__device__ __forceinline__ uint32_t fdiv(uint32_t n, FastDiv f) { return (__umulhi(n, f.mul) + n) >> f.sh; }
+
 // index of the pair (p < q) among the n(n-1)/2 pairs, row-major upper triangle
 __host__ __device__ inline int64_t pair_index(int64_t p, int64_t q, int64_t n) {
   return p * n - p * (p + 1) / 2 + (q - p - 1);

@@ -23,8 +23,11 @@
 #include <cuda_bf16.h>
 #include <cudaTypedefs.h>
 
+#include <algorithm>
+
 #include "ctx.cuh"
 #include "tc_gemm.cuh"
+#include "tc_pack.cuh"
 #include "tc_ptx.cuh"
 #include "tc_slice.cuh"
 
@@ -200,23 +203,25 @@ k_tc_gemm(const __grid_constant__ CUtensorMap mAh, const __grid_constant__ CUten
 }
 
 __global__ void k_tc_reduce(const float *__restrict__ part, int ksplit, int64_t M, int64_t N2, cplx *out,
-                            int64_t s_m, int64_t s_nh, int64_t s_nl, int64_t n_in, cplx alpha, cplx beta) {
+                            int64_t s_m, int64_t s_nh, int64_t s_nl, int64_t n_in, cplx alpha, int ka, cplx beta,
+                            int kb) {
   const int64_t total = M * (N2 / 2);
-  const bool use_beta = (beta.x != 0.0 || beta.y != 0.0);
   for (int64_t idx = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; idx < total;
        idx += (int64_t)gridDim.x * blockDim.x) {
     const int64_t n = idx % (N2 / 2), m = idx / (N2 / 2);
     double re = 0.0, im = 0.0;
+    const float *pp = part + m * N2 + 2 * n;
+    const int64_t step = M * N2;
+    // (eight splits' loads in flight: few outputs and many splits leave little else to hide them)
+#pragma unroll 8
     for (int s = 0; s < ksplit; ++s) {
-      const float *pp = part + ((int64_t)s * M + m) * N2 + 2 * n;
-      re += (double)pp[0];
-      im += (double)pp[1];
+      const float2 v = *(const float2 *)(pp + s * step);
+      re += (double)v.x;
+      im += (double)v.y;
     }
     const int64_t nh = n / n_in, nl = n - nh * n_in;
     cplx *dst = out + m * s_m + nh * s_nh + nl * s_nl;
-    cplx val = cmul(alpha, cmake(re, im));
-    if (use_beta) val = cadd(val, cmul(beta, *dst));
-    *dst = val;
+    *dst = axpby(ka, alpha, cmake(re, im), kb, beta, dst);
   }
 }
 
@@ -231,72 +236,103 @@ __device__ __forceinline__ void split_store(double x, __nv_bfloat16 *hi, __nv_bf
   if (lo2) *lo2 = __double2bfloat16(r - (double)__bfloat162float(l));
 }
 
-// A rows: [Re | Im] (conj negates Im); element (m, k) at src[m*s_m + k*s_k]
-__global__ void k_emb_A(const cplx *__restrict__ src, int64_t M, int64_t K, int64_t s_m, int64_t s_k,
-                        int conj, int64_t kp, __nv_bfloat16 *hi, __nv_bfloat16 *lo, __nv_bfloat16 *lo2) {
-  // one thread per 8 consecutive k of a row, 16-byte stores of every plane
-  const int64_t kq = kp >> 3;
-  const int64_t total = M * kq;
-  for (int64_t idx = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; idx < total;
-       idx += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t m = idx / kq, k0 = (idx - m * kq) << 3;
-    const cplx *row = src + m * s_m;
-    __align__(16) __nv_bfloat16 rh[8], rl[8], rl2[8], ih[8], il[8], il2[8];
-#pragma unroll
-    for (int j = 0; j < 8; ++j) {
-      const int64_t k = k0 + j;
-      cplx x = cmake(0.0, 0.0);
-      if (k < K) x = row[k * s_k];
-      split_store(x.x, &rh[j], &rl[j], &rl2[j]);
-      split_store(conj ? -x.y : x.y, &ih[j], &il[j], &il2[j]);
-    }
-    const int64_t base = m * 2 * kp + k0;
-    *(uint4 *)(hi + base) = *(const uint4 *)rh;
-    *(uint4 *)(hi + base + kp) = *(const uint4 *)ih;
-    *(uint4 *)(lo + base) = *(const uint4 *)rl;
-    *(uint4 *)(lo + base + kp) = *(const uint4 *)il;
-    if (lo2) {
-      *(uint4 *)(lo2 + base) = *(const uint4 *)rl2;
-      *(uint4 *)(lo2 + base + kp) = *(const uint4 *)il2;
-    }
+// The same split from the bits of x: hi is the leading 8 bits rounded to even, what is left
+// (exact, at most 46 bits) is normalised and rounded in turn. FP64 conversions and
+// subtractions took most of the packing's time (two lanes a clock and SM). Values whose
+// parts could leave BF16's normal range, infinities and NaN go to split_store.
+template <bool P3>
+__device__ __forceinline__ void split_bits(double x, uint16_t &h, uint16_t &l, uint16_t &l2) {
+  const long long u = __double_as_longlong(x);
+  const int ef = (int)((u >> 52) & 0x7ff);
+  if ((unsigned long long)u << 1 == 0) {  // (the antisymmetric operands and the padding hold many)
+    h = (uint16_t)((unsigned long long)u >> 48);
+    l = l2 = 0;
+    return;
   }
+  if (ef < 1023 - 50 || ef > 1023 + 125) {
+    __nv_bfloat16 a, b, c;
+    split_store(x, &a, &b, P3 ? &c : nullptr);
+    h = __bfloat16_as_ushort(a);
+    l = __bfloat16_as_ushort(b);
+    if (P3) l2 = __bfloat16_as_ushort(c);
+    return;
+  }
+  // rounds r 2^(e - 52) (r > 0) to 8 bits; r becomes the signed rest
+  auto part = [](long long &r, int e, unsigned sign) -> uint16_t {
+    const bool neg = r < 0;
+    unsigned long long a = (unsigned long long)(neg ? -r : r);
+    if (a == 0) return 0;
+    const int top = 63 - __clzll((long long)a);  // value in [2^top, 2^(top + 1))
+    const int sh = top - 7;
+    unsigned long long q = a;
+    if (sh > 0) q = (a + ((1ull << (sh - 1)) - 1) + ((a >> sh) & 1)) >> sh;
+    else q = a << -sh;
+    const long long back = sh > 0 ? (long long)(q << sh) : (long long)a;
+    r = neg ? back - (long long)a : (long long)a - back;
+    // q in [128, 256]: 256 carries into the exponent by itself
+    const unsigned bits = ((unsigned)(e - 52 + top + 127) << 7) + (unsigned)(q - 128);
+    return (uint16_t)(bits | ((sign ^ (neg ? 1u : 0u)) << 15));
+  };
+  const unsigned sign = (unsigned)((unsigned long long)u >> 63);
+  long long r = (u & 0xfffffffffffffll) | (1ll << 52);
+  const int e = ef - 1023;
+  h = part(r, e, sign);
+  l = part(r, e, sign);
+  if (P3) l2 = part(r, e, sign);
 }
 
+__device__ __forceinline__ uint4 pack8(const uint16_t (&v)[8]) {
+  return make_uint4(v[0] | (uint32_t)v[1] << 16, v[2] | (uint32_t)v[3] << 16, v[4] | (uint32_t)v[5] << 16,
+                    v[6] | (uint32_t)v[7] << 16);
+}
+__device__ __forceinline__ uint4 neg8(uint4 v) {
+  return make_uint4(v.x ^ 0x80008000u, v.y ^ 0x80008000u, v.z ^ 0x80008000u, v.w ^ 0x80008000u);
+}
 
-// B rows: row 2n = [Re | -Im], row 2n+1 = [Im | Re] (conj negates Im first).
-// One thread per 8 consecutive k of a row: one row index computation per
-// thread, 16-byte stores of every plane (the splits of -Im are the negated
-// splits of Im: round to nearest is symmetric)
-__global__ void k_emb_B(BSrc src, int64_t Nc, int64_t K, int conj, int64_t kp, __nv_bfloat16 *hi,
-                        __nv_bfloat16 *lo, __nv_bfloat16 *lo2) {
-  const int64_t kq = kp >> 3;
-  const int64_t total = Nc * kq;
-  for (int64_t idx = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; idx < total;
-       idx += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t n = idx / kq, k0 = (idx - n * kq) << 3;
-    cplx x[8];
-    src.get8(n, k0, K, x);
-    __align__(16) __nv_bfloat16 rh[8], rl[8], rl2[8], ih[8], il[8], il2[8], nh[8], nl[8], nl2[8];
+// BF16 planes of the rows of an operand, padded to kp with zeros. EMB = 1: A rows
+// [Re | Im]; EMB = 2: B rows 2n = [Re | -Im], 2n + 1 = [Im | Re] (conj negates Im
+// first; the split of -Im is the negated split of Im, round to nearest being
+// symmetric). Bound by the bytes written (16 or 32 per element and two planes); every
+// thread takes eight inner elements of a staged tile and stores 16 bytes at a time.
+template <int EMB, bool P3>
+__global__ void __launch_bounds__(256)
+k_emb(BSrc src, int64_t rows, int64_t K, int conj, int64_t kp, int kfast, __nv_bfloat16 *hi, __nv_bfloat16 *lo,
+      __nv_bfloat16 *lo2) {
+  __shared__ cplx tile[PK_R * PK_LD];
+  __shared__ PkRow row[PK_R];
+  for (int64_t n0 = (int64_t)blockIdx.x * PK_R; n0 < rows; n0 += (int64_t)gridDim.x * PK_R) {
+    if (threadIdx.x < PK_R) row[threadIdx.x] = pk_row(src, min(n0 + (int64_t)threadIdx.x, rows - 1));
+    __syncthreads();
+    for (int64_t k0 = (int64_t)blockIdx.y * PK_K; k0 < kp; k0 += (int64_t)gridDim.y * PK_K) {
+      pk_load(src, n0, rows, k0, K, kfast != 0, row, [&](int r, int kk, cplx x) { tile[pk_at(r, kk)] = x; });
+      __syncthreads();
+      const int r = threadIdx.x >> 3, oct = threadIdx.x & 7;
+      const int64_t n = n0 + r;
+      if (n < rows) {
+        uint16_t re[3][8], im[3][8];
 #pragma unroll
-    for (int j = 0; j < 8; ++j) {
-      const double im = conj ? -x[j].y : x[j].y;
-      split_store(x[j].x, &rh[j], &rl[j], &rl2[j]);
-      split_store(im, &ih[j], &il[j], &il2[j]);
-      nh[j] = __hneg(ih[j]);
-      nl[j] = __hneg(il[j]);
-      nl2[j] = __hneg(il2[j]);
+        for (int j = 0; j < 8; ++j) {
+          const cplx x = tile[pk_at(r, 8 * oct + j)];
+          split_bits<P3>(x.x, re[0][j], re[1][j], re[2][j]);
+          split_bits<P3>(conj ? -x.y : x.y, im[0][j], im[1][j], im[2][j]);
+        }
+        const int64_t at = (int64_t)EMB * n * 2 * kp + k0 + 8 * oct;
+#pragma unroll
+        for (int p = 0; p < (P3 ? 3 : 2); ++p) {
+          __nv_bfloat16 *pl = (p == 0 ? hi : p == 1 ? lo : lo2) + at;
+          const uint4 vr = pack8(re[p]), vi = pack8(im[p]);
+          *(uint4 *)pl = vr;
+          if (EMB == 1) {
+            *(uint4 *)(pl + kp) = vi;
+          } else {
+            *(uint4 *)(pl + kp) = neg8(vi);
+            *(uint4 *)(pl + 2 * kp) = vi;
+            *(uint4 *)(pl + 3 * kp) = vr;
+          }
+        }
+      }
+      __syncthreads();
     }
-    const int64_t r0 = (2 * n) * 2 * kp + k0, r1 = (2 * n + 1) * 2 * kp + k0;
-    auto put = [&](__nv_bfloat16 *plane, const __nv_bfloat16 (&re)[8], const __nv_bfloat16 (&imv)[8],
-                   const __nv_bfloat16 (&nim)[8]) {
-      *(uint4 *)(plane + r0) = *(const uint4 *)re;
-      *(uint4 *)(plane + r0 + kp) = *(const uint4 *)nim;
-      *(uint4 *)(plane + r1) = *(const uint4 *)imv;
-      *(uint4 *)(plane + r1 + kp) = *(const uint4 *)re;
-    };
-    put(hi, rh, ih, nh);
-    put(lo, rl, il, nl);
-    if (lo2) put(lo2, rl2, il2, nl2);
   }
 }
 
@@ -368,7 +404,8 @@ void launch_tc(Exec &ex, const TcView &A, const TcView &B, int64_t M, int64_t N2
   ADC_CHECK_LAUNCH();
   if (ksplit > 1) {
     k_tc_reduce<<<grid1d(M * (N2 / 2), 256), 256, 0, ex.stream>>>((const float *)part.p, ksplit, M, N2, out, s_m,
-                                                                  s_nh, s_nl, n_in, alpha, beta);
+                                                                  s_nh, s_nl, n_in, alpha, factor_kind(alpha), beta,
+                                                                  factor_kind(beta));
     ADC_CHECK_LAUNCH();
   }
   ex.prof_end(pr);
@@ -816,43 +853,41 @@ static void alloc_planes(Exec &ex, TcMat &dst, size_t bytes, int planes) {
   dst.planes = (planes == 3 && dst.lo2.p) ? 3 : 2;
 }
 
-void tc_pack_A(Exec &ex, TcMat &dst, const cplx *src, int64_t M, int64_t K, int64_t s_m, int64_t s_k, bool conj,
-               int planes) {
-  dst.rows = M;
+static void launch_emb(Exec &ex, TcMat &dst, const BSrc &s, int64_t rows, int64_t K, bool conj, int planes, int emb) {
+  dst.rows = emb * rows;
   dst.kreal = K;
   dst.kp = (K + TC_BK - 1) / TC_BK * TC_BK;
   if (dst.kp == 0) dst.kp = TC_BK;
-  const size_t bytes = (size_t)M * 2 * dst.kp * sizeof(__nv_bfloat16);
-  alloc_planes(ex, dst, bytes, planes);
-  k_emb_A<<<grid1d(M * (dst.kp / 8), 256), 256, 0, ex.stream>>>(src, M, K, s_m, s_k, conj ? 1 : 0, dst.kp,
-                                                          (__nv_bfloat16 *)dst.hi.p, (__nv_bfloat16 *)dst.lo.p,
-                                                          planes == 3 ? (__nv_bfloat16 *)dst.lo2.p : nullptr);
+  alloc_planes(ex, dst, (size_t)dst.rows * 2 * dst.kp * sizeof(__nv_bfloat16), planes);
+  if (rows <= 0) return;
+  ADC_REQUIRE(s.mode == 0 || K < (1ll << 31), ADC_ERR_UNSUPPORTED, "operand packing: ring size");
+  const dim3 grid((unsigned)std::min<int64_t>((rows + PK_R - 1) / PK_R, 1 << 20),
+                  (unsigned)std::min<int64_t>(dst.kp / PK_K, 65535));
+  __nv_bfloat16 *hi = (__nv_bfloat16 *)dst.hi.p, *lo = (__nv_bfloat16 *)dst.lo.p;
+  __nv_bfloat16 *lo2 = planes == 3 ? (__nv_bfloat16 *)dst.lo2.p : nullptr;
+  auto kernel = emb == 1 ? (lo2 ? k_emb<1, true> : k_emb<1, false>) : (lo2 ? k_emb<2, true> : k_emb<2, false>);
+  kernel<<<grid, 256, 0, ex.stream>>>(s, rows, K, conj ? 1 : 0, dst.kp, pk_kfast(s), hi, lo, lo2);
   ADC_CHECK_LAUNCH();
 }
 
-static void pack_B_impl(Exec &ex, TcMat &dst, const BSrc &s, int64_t Nc, int64_t K, bool conj, int planes) {
-  dst.rows = 2 * Nc;
-  dst.kreal = K;
-  dst.kp = (K + TC_BK - 1) / TC_BK * TC_BK;
-  if (dst.kp == 0) dst.kp = TC_BK;
-  const size_t bytes = (size_t)dst.rows * 2 * dst.kp * sizeof(__nv_bfloat16);
-  alloc_planes(ex, dst, bytes, planes);
-  k_emb_B<<<grid1d(Nc * (dst.kp / 8), 256), 256, 0, ex.stream>>>(s, Nc, K, conj ? 1 : 0, dst.kp,
-                                                           (__nv_bfloat16 *)dst.hi.p, (__nv_bfloat16 *)dst.lo.p,
-                                                           planes == 3 ? (__nv_bfloat16 *)dst.lo2.p : nullptr);
-  ADC_CHECK_LAUNCH();
+void tc_pack_A(Exec &ex, TcMat &dst, const cplx *src, int64_t M, int64_t K, int64_t s_m, int64_t s_k, bool conj,
+               int planes) {
+  const BSrc s{src, 0, 0, s_m, std::max<int64_t>(M, 1), s_k, 0, 0, 0, 0};
+  launch_emb(ex, dst, s, M, K, conj, planes, 1);
 }
 
 void tc_pack_B(Exec &ex, TcMat &dst, const cplx *src, int64_t Nc, int64_t K, int64_t s_nh, int64_t s_nl,
                int64_t n_in, int64_t s_k, bool conj, int planes) {
   BSrc s{src, 0, s_nh, s_nl, n_in, s_k, 0, 0, 0, 0};
-  pack_B_impl(ex, dst, s, Nc, K, conj, planes);
+  // one row index: strides as an A operand, so that the packing sees which index is contiguous
+  if (n_in == 1) { s.n_in = std::max<int64_t>(Nc, 1); s.s_nl = s_nh; s.s_nh = 0; }
+  launch_emb(ex, dst, s, Nc, K, conj, planes, 2);
 }
 
 void tc_pack_B_ring(Exec &ex, TcMat &dst, const adc_ctx *c, const cplx *X, int64_t k, int planes) {
   BSrc s{X, c->kind == ADC_EA ? 1 : 2, 0, 0, 1, 0, c->o, c->v, c->N, c->n1};
   const int64_t Nc = (c->kind == ADC_EA) ? k * c->v : k * c->o;
-  pack_B_impl(ex, dst, s, Nc, c->o * c->v, false, planes);
+  launch_emb(ex, dst, s, Nc, c->o * c->v, false, planes, 2);
 }
 
 TcView tc_view(const TcMat &m, int64_t row0, int64_t rows) {
@@ -1083,7 +1118,8 @@ void tc_gemm_grouped(Exec &ex, const std::vector<TcJobDesc> &in, TcGroup &grp, i
     const TcJob &J = grp.host[i];
     if (J.ksplit <= 1) continue;
     k_tc_reduce<<<grid1d((int64_t)J.M * (J.N2 / 2), 256), 256, 0, ex.stream>>>(
-        J.part, J.ksplit, J.M, J.N2, J.out, J.s_m, J.s_nh, J.s_nl, J.n_in, J.alpha, J.beta);
+        J.part, J.ksplit, J.M, J.N2, J.out, J.s_m, J.s_nh, J.s_nl, J.n_in, J.alpha, factor_kind(J.alpha), J.beta,
+        factor_kind(J.beta));
     ADC_CHECK_LAUNCH();
   }
   ex.prof_end(pr);
@@ -1122,8 +1158,7 @@ int tc_autotune_bn(Exec &ex, const TcJobDesc &d, int *err) {
     cudaEvent_t e0, e1;
     ADC_CUDA(cudaEventCreate(&e0));
     ADC_CUDA(cudaEventCreate(&e1));
-    double tbest = 1e300;
-    for (int bn : cand) {
+    auto time_of = [&](int bn, bool warm) {
       TcJobDesc t = d;
       t.bn = bn;
       t.out = scratch.c();
@@ -1134,14 +1169,26 @@ int tc_autotune_bn(Exec &ex, const TcJobDesc &d, int *err) {
       t.alpha = C1();
       t.beta = C0();
       std::vector<TcJobDesc> one{t};
-      tc_gemm_grouped(ex, one, g, err, false, true);
+      if (warm) tc_gemm_grouped(ex, one, g, err, false, true);
       ADC_CUDA(cudaEventRecord(e0, ex.stream));
       for (int r = 0; r < 2; ++r) tc_gemm_grouped(ex, one, g, err, false, true);
       ADC_CUDA(cudaEventRecord(e1, ex.stream));
       ADC_CUDA(cudaEventSynchronize(e1));
       float ms = 0.f;
       ADC_CUDA(cudaEventElapsedTime(&ms, e0, e1));
-      if (ms < tbest) { tbest = ms; best = bn; }
+      return ms;
+    };
+    std::vector<float> ms;
+    for (int bn : cand) ms.push_back(time_of(bn, true));
+    const float tbest = *std::min_element(ms.begin(), ms.end());
+    // Widths within 8% of the best are told apart by the best of five samples while these are
+    // short: one sample varies by a few per cent, and as the width also decides how inner sums
+    // are split, a choice that follows the noise changes the last FP32 digits from run to run
+    float least = 1e30f;
+    for (size_t c = 0; c < cand.size(); ++c) {
+      if (ms[c] > 1.08f * tbest) continue;
+      for (int extra = 0; extra < 4 && tbest < 1.0f; ++extra) ms[c] = std::min(ms[c], time_of(cand[c], false));
+      if (ms[c] < least) { least = ms[c]; best = cand[c]; }
     }
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);

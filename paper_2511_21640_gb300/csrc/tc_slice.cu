@@ -30,6 +30,7 @@
 
 #include "ctx.cuh"
 #include "tc_gemm.cuh"
+#include "tc_pack.cuh"
 #include "tc_ptx.cuh"
 #include "tc_slice.cuh"
 
@@ -63,63 +64,6 @@ __device__ __forceinline__ long long fixed_of(double x, int E, int bits) {
   else if (s >= -54) r = (m + ((1ll << (-s - 1)) - 1) + ((m >> -s) & 1)) >> -s;
   else r = 0;
   return u < 0 ? -r : r;
-}
-
-constexpr int PK_R = 32, PK_K = 64;    // tile of the packing kernels: rows x inner elements
-constexpr int PK_LD = PK_K + PK_K / 8;  // one element of padding per eight
-__device__ __forceinline__ int pk_at(int r, int k) { return r * PK_LD + k + (k >> 3); }
-
-// element (row n, inner k) of the operand rows a packing block handles: the
-// address arithmetic of BSrc split into a part per row and a part per k
-struct PkRow {
-  const cplx *p;
-  int b;
-};
-__device__ __forceinline__ PkRow pk_row(const BSrc &s, int64_t n) {
-  PkRow r;
-  if (s.mode == 0) {
-    const int64_t nh = n / s.n_in, nl = n - nh * s.n_in;
-    r.p = s.p + nh * s.s_nh + nl * s.s_nl;
-    r.b = 0;
-  } else {
-    const int64_t per = (s.mode == 1) ? s.v : s.o, vec = n / per;
-    r.p = s.p + s.n1 + vec * s.N;
-    r.b = (int)(n - vec * per);
-  }
-  return r;
-}
-__device__ __forceinline__ cplx pk_get(const BSrc &s, const PkRow &r, int64_t k, int kh, int kl) {
-  if (s.mode == 0) return r.p[k * s.s_k];
-  if (s.mode == 1) {  // (kh, kl) = (kk, c): X[kk][(c, b)]
-    if (kl == r.b) return cmake(0.0, 0.0);
-    const cplx x = kl < r.b ? r.p[kh * (s.v * (s.v - 1) / 2) + pair_index(kl, r.b, s.v)]
-                            : r.p[kh * (s.v * (s.v - 1) / 2) + pair_index(r.b, kl, s.v)];
-    return kl < r.b ? x : cmake(-x.x, -x.y);
-  }
-  // mode 2, (kh, kl) = (kq, b): X[(i, kq)][b]
-  if (kh == r.b) return cmake(0.0, 0.0);
-  const cplx x = r.b < kh ? r.p[pair_index(r.b, kh, s.o) * s.v + kl] : r.p[pair_index(kh, r.b, s.o) * s.v + kl];
-  return r.b < kh ? x : cmake(-x.x, -x.y);
-}
-
-// loads rows [n0, n0 + 32) x [k0, k0 + 64) of the source, zero outside, calling
-// f(row, k, value); lanes run along whichever index is contiguous in memory
-template <class F>
-__device__ __forceinline__ void pk_load(const BSrc &src, int64_t n0, int64_t rows, int64_t k0, int64_t K, bool kfast,
-                                        const PkRow *row, F f) {
-#pragma unroll
-  for (int it = 0; it < PK_R * PK_K / 256; ++it) {
-    const int idx = threadIdx.x + 256 * it;
-    const int r = kfast ? idx >> 6 : idx & 31, kk = kfast ? idx & 63 : idx >> 5;
-    cplx x = cmake(0.0, 0.0);
-    const int64_t k = k0 + kk;
-    if (n0 + r < rows && k < K) {
-      int kh = 0, kl = 0;
-      if (src.mode != 0) { kh = (int)((unsigned)k / (unsigned)src.v); kl = (int)k - kh * (int)src.v; }
-      x = pk_get(src, row[r], k, kh, kl);
-    }
-    f(r, kk, x);
-  }
 }
 
 // W[n] = max(W[n], largest magnitude word of row n over the inner range of this
@@ -593,19 +537,17 @@ __global__ void __launch_bounds__(320, 1) k_sl_gemm(const __grid_constant__ SlAr
 
 // out = alpha sum_s part[s] + beta out, the splits in order
 __global__ void k_sl_reduce(const cplx *__restrict__ part, int ksplit, int64_t M, int64_t Nc, cplx *out, int64_t s_m,
-                            int64_t s_nh, int64_t s_nl, int64_t n_in, cplx alpha, cplx beta) {
+                            int64_t s_nh, int64_t s_nl, int64_t n_in, cplx alpha, int ka, cplx beta, int kb) {
   const int64_t total = M * Nc;
-  const bool use_beta = (beta.x != 0.0 || beta.y != 0.0);
   for (int64_t idx = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; idx < total;
        idx += (int64_t)gridDim.x * blockDim.x) {
     const int64_t m = idx / Nc, n = idx - m * Nc;
     cplx v = cmake(0.0, 0.0);
+#pragma unroll 8
     for (int s = 0; s < ksplit; ++s) v = cadd(v, part[(int64_t)s * total + idx]);
     const int64_t nh = n / n_in, nl = n - nh * n_in;
     cplx *dst = out + m * s_m + nh * s_nh + nl * s_nl;
-    v = cmul(alpha, v);
-    if (use_beta) v = cadd(v, cmul(beta, *dst));
-    *dst = v;
+    *dst = axpby(ka, alpha, v, kb, beta, dst);
   }
 }
 
@@ -627,7 +569,7 @@ void pack_rows(Exec &ex, SlMat &d, const BSrc &s, int64_t rows, int64_t K, bool 
   alloc_sl(ex, d, emb * rows, rows);
   if (rows <= 0) return;
   ADC_REQUIRE(s.mode == 0 || K < (1ll << 31), ADC_ERR_UNSUPPORTED, "sliced product: ring size");
-  const int kfast = (s.mode != 0 || s.s_k == 1 || s.s_nl != 1) ? 1 : 0;
+  const int kfast = pk_kfast(s);
   const int64_t rt = (rows + PK_R - 1) / PK_R;
   const unsigned gx = (unsigned)std::min<int64_t>(rt, 1 << 20);
   unsigned *W = (unsigned *)d.exps.p;
@@ -799,7 +741,7 @@ void sl_gemm(Exec &ex, const SlMat &A, const SlMat &B, int64_t M, int64_t N, cpl
   else launch_sl<128>(ex, g, w, grid);
   if (g.ksplit > 1) {
     k_sl_reduce<<<grid1d(M * N, 256), 256, 0, ex.stream>>>(g.part, g.ksplit, M, N, out, s_m, s_nh, s_nl, g.n_in,
-                                                           alpha, beta);
+                                                           alpha, factor_kind(alpha), beta, factor_kind(beta));
     ADC_CHECK_LAUNCH();
   }
   ex.prof_end(pr);

@@ -552,26 +552,50 @@ struct PermArgs {
   int64_t ext[MAXD];
   int64_t sstr[MAXD];
   int64_t dstr[MAXD];
+  FastDiv fd[MAXD];
 };
 
-__global__ void k_permute(const cplx *__restrict__ src, PermArgs pa, int conj, cplx *dst,
-                          cplx alpha, cplx beta, int use_beta, int64_t total) {
+// (measured on 2.6 M elements of four axes: 36 us with 64-bit divisions and a complex factor)
+template <bool SMALL>
+__global__ void k_permute(const cplx *__restrict__ src, PermArgs pa, int conj, cplx *dst, cplx alpha, int ka,
+                          cplx beta, int kb, int64_t total) {
   for (int64_t idx = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; idx < total;
        idx += (int64_t)gridDim.x * blockDim.x) {
-    int64_t rem = idx, off = 0, doff = 0;
-    for (int d = pa.nd - 1; d >= 0; --d) {
-      int64_t i = rem % pa.ext[d];
-      rem /= pa.ext[d];
-      off += i * pa.sstr[d];
-      doff += i * pa.dstr[d];
+    int64_t off = 0, doff = 0;
+    if (SMALL) {  // fewer than 2^31 elements
+      uint32_t rem = (uint32_t)idx;
+      for (int d = pa.nd - 1; d >= 0; --d) {
+        const uint32_t q = fdiv(rem, pa.fd[d]), i = rem - q * pa.fd[d].d;
+        rem = q;
+        off += i * pa.sstr[d];
+        doff += i * pa.dstr[d];
+      }
+    } else {
+      int64_t rem = idx;
+      for (int d = pa.nd - 1; d >= 0; --d) {
+        int64_t i = rem % pa.ext[d];
+        rem /= pa.ext[d];
+        off += i * pa.sstr[d];
+        doff += i * pa.dstr[d];
+      }
     }
     if (!pa.strided_dst) doff = idx;
     cplx v = src[off];
     if (conj) v.y = -v.y;
-    cplx r = cmul(alpha, v);
-    if (use_beta) r = cadd(r, cmul(beta, dst[doff]));
-    dst[doff] = r;
+    dst[doff] = axpby(ka, alpha, v, kb, beta, dst + doff);
   }
+}
+
+void launch_permute(Exec &ex, const cplx *src, PermArgs &pa, bool conj, cplx *dst, cplx alpha, cplx beta,
+                    int64_t total) {
+  const int ka = factor_kind(alpha), kb = factor_kind(beta);
+  if (total < (1ll << 31)) {
+    for (int d = 0; d < pa.nd; ++d) pa.fd[d] = fast_div((uint32_t)pa.ext[d]);
+    k_permute<true><<<grid1d(total, 256), 256, 0, ex.stream>>>(src, pa, conj ? 1 : 0, dst, alpha, ka, beta, kb, total);
+  } else {
+    k_permute<false><<<grid1d(total, 256), 256, 0, ex.stream>>>(src, pa, conj ? 1 : 0, dst, alpha, ka, beta, kb, total);
+  }
+  ADC_CHECK_LAUNCH();
 }
 }  // namespace
 
@@ -590,9 +614,7 @@ void permute(Exec &ex, const cplx *src, const std::vector<int64_t> &ext, const s
     total *= ext[d];
   }
   if (total == 0) return;
-  const int use_beta = (beta.x != 0.0 || beta.y != 0.0) ? 1 : 0;
-  k_permute<<<grid1d(total, 256), 256, 0, ex.stream>>>(src, pa, conj ? 1 : 0, dst, alpha, beta, use_beta, total);
-  ADC_CHECK_LAUNCH();
+  launch_permute(ex, src, pa, conj, dst, alpha, beta, total);
 }
 
 void permute(Exec &ex, const cplx *src, const std::vector<int64_t> &ext,
@@ -604,10 +626,7 @@ void permute(Exec &ex, const cplx *src, const std::vector<int64_t> &ext,
   for (int d = 0; d < pa.nd; ++d) { pa.ext[d] = ext[d]; pa.sstr[d] = sstr[d]; total *= ext[d]; }
   if (pa.nd == 0) { pa.nd = 1; pa.ext[0] = 1; pa.sstr[0] = 0; }
   if (total == 0) return;
-  int use_beta = (beta.x != 0.0 || beta.y != 0.0) ? 1 : 0;
-  k_permute<<<grid1d(total, 256), 256, 0, ex.stream>>>(src, pa, conj ? 1 : 0, dst, alpha, beta,
-                                                       use_beta, total);
-  ADC_CHECK_LAUNCH();
+  launch_permute(ex, src, pa, conj, dst, alpha, beta, total);
 }
 
 // ------------------------------------------------------------------ pairs
@@ -628,10 +647,46 @@ __global__ void k_pair_unpack(const cplx *__restrict__ P, int64_t no1, int64_t n
   }
 }
 
+// The same for inner = 1 and one unit stride of T (sTq == 1, or sTp == 1 when qfast is 0):
+// a block takes the 32 x 32 tiles (p, q) and (q, p) of one outer index through shared
+// memory, so that T is read along its unit stride and P written along q
+__global__ void __launch_bounds__(256)
+k_pair_pack_tile(const cplx *__restrict__ T, int64_t sTo1, int64_t sTo0, int64_t ld, int qfast, double s, int64_t no0,
+                 int64_t n, cplx *P, int64_t sP1, int64_t sP0, cplx alpha, int ka, cplx beta, int kb) {
+  __shared__ cplx a[32][33], b[32][33];  // a[p][q] = T(p0 + p, q0 + q), b[q][p] = T(q0 + q, p0 + p)
+  // blockIdx.x counts the tile pairs pb <= qb row by row
+  const int nt = (int)((n + 31) / 32);
+  int pb = 0, r = blockIdx.x;
+  while (r >= nt - pb) { r -= nt - pb; ++pb; }
+  const int64_t p0 = 32 * pb, q0 = 32 * (pb + r);
+  const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
+  const int64_t o0 = blockIdx.y % no0, o1 = blockIdx.y / no0;
+  const cplx *Tb = T + o1 * sTo1 + o0 * sTo0;
+#pragma unroll
+  for (int i = ty; i < 32; i += 8) {
+    // rows of memory: qfast: T(p, .) at p ld, else T(., q) at q ld
+    const int64_t x = (qfast ? p0 : q0) + i, y = (qfast ? q0 : p0) + tx;
+    if (x < n && y < n) (qfast ? a[i][tx] : a[tx][i]) = Tb[x * ld + y];
+    const int64_t x2 = (qfast ? q0 : p0) + i, y2 = (qfast ? p0 : q0) + tx;
+    if (s != 0.0 && x2 < n && y2 < n) (qfast ? b[i][tx] : b[tx][i]) = Tb[x2 * ld + y2];
+  }
+  __syncthreads();
+  cplx *Pb = P + o1 * sP1 + o0 * sP0;
+#pragma unroll
+  for (int i = ty; i < 32; i += 8) {
+    const int64_t p = p0 + i, q = q0 + tx;
+    if (p >= q || q >= n) continue;
+    cplx v = a[i][tx];
+    if (s != 0.0) { const cplx w = b[tx][i]; v.x -= s * w.x; v.y -= s * w.y; }
+    cplx *dst = Pb + pair_index(p, q, n);
+    *dst = axpby(ka, alpha, v, kb, beta, dst);
+  }
+}
+
 __global__ void k_pair_pack(const cplx *__restrict__ T, int64_t sTo1, int64_t sTo0, int64_t sTp,
                             int64_t sTq, int64_t sTin, double s, int64_t no1, int64_t no0,
                             int64_t n, int64_t inner, cplx *P, int64_t sP1, int64_t sP0,
-                            cplx alpha, cplx beta, int use_beta, int64_t total) {
+                            cplx alpha, int ka, cplx beta, int kb, int64_t total) {
   // iterate over (o, p, q, in) with p < q encoded through the full square; half idle
   for (int64_t idx = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; idx < total;
        idx += (int64_t)gridDim.x * blockDim.x) {
@@ -645,9 +700,7 @@ __global__ void k_pair_pack(const cplx *__restrict__ T, int64_t sTo1, int64_t sT
     cplx v = Tb[p * sTp + q * sTq];
     if (s != 0.0) { cplx w = Tb[q * sTp + p * sTq]; v.x -= s * w.x; v.y -= s * w.y; }
     cplx *dst = P + o1 * sP1 + o0 * sP0 + pair_index(p, q, n) * inner + in;
-    cplx res = cmul(alpha, v);
-    if (use_beta) res = cadd(res, cmul(beta, *dst));
-    *dst = res;
+    *dst = axpby(ka, alpha, v, kb, beta, dst);
   }
 }
 }  // namespace
@@ -665,10 +718,17 @@ void pair_pack(Exec &ex, const cplx *T, int64_t sTo1, int64_t sTo0, int64_t sTp,
                cplx *P, int64_t sP1, int64_t sP0, cplx alpha, cplx beta) {
   int64_t total = no1 * no0 * n * n * inner;
   if (total == 0 || n < 2) return;
-  int use_beta = (beta.x != 0.0 || beta.y != 0.0) ? 1 : 0;
+  const int ka = factor_kind(alpha), kb = factor_kind(beta);
+  if (inner == 1 && (sTq == 1 || sTp == 1) && no1 * no0 <= 65535) {
+    const int64_t nt = (n + 31) / 32;
+    const int qfast = sTq == 1 ? 1 : 0;
+    k_pair_pack_tile<<<dim3((unsigned)(nt * (nt + 1) / 2), (unsigned)(no1 * no0)), 256, 0, ex.stream>>>(
+        T, sTo1, sTo0, qfast ? sTp : sTq, qfast, s, no0, n, P, sP1, sP0, alpha, ka, beta, kb);
+    ADC_CHECK_LAUNCH();
+    return;
+  }
   k_pair_pack<<<grid1d(total, 256), 256, 0, ex.stream>>>(T, sTo1, sTo0, sTp, sTq, sTin, s, no1,
-                                                         no0, n, inner, P, sP1, sP0, alpha, beta,
-                                                         use_beta, total);
+                                                         no0, n, inner, P, sP1, sP0, alpha, ka, beta, kb, total);
   ADC_CHECK_LAUNCH();
 }
 

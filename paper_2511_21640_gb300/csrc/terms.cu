@@ -40,19 +40,32 @@ constexpr int SA_MAXD = 10;
 struct SAArgs {
   int nd;
   int64_t ext[SA_MAXD], sstr[SA_MAXD], dstr[SA_MAXD];
+  FastDiv fd[SA_MAXD];
 };
 
-__global__ void k_strided_add(const cplx *__restrict__ src, SAArgs a, cplx alpha, cplx *dst, int64_t total) {
+template <bool SMALL>
+__global__ void k_strided_add(const cplx *__restrict__ src, SAArgs a, cplx alpha, int ka, cplx *dst, int64_t total) {
   for (int64_t idx = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; idx < total;
        idx += (int64_t)gridDim.x * blockDim.x) {
-    int64_t rem = idx, so = 0, dof = 0;
-    for (int d = a.nd - 1; d >= 0; --d) {
-      int64_t i = rem % a.ext[d];
-      rem /= a.ext[d];
-      so += i * a.sstr[d];
-      dof += i * a.dstr[d];
+    int64_t so = 0, dof = 0;
+    if (SMALL) {  // fewer than 2^31 elements
+      uint32_t rem = (uint32_t)idx;
+      for (int d = a.nd - 1; d >= 0; --d) {
+        const uint32_t q = fdiv(rem, a.fd[d]), i = rem - q * a.fd[d].d;
+        rem = q;
+        so += i * a.sstr[d];
+        dof += i * a.dstr[d];
+      }
+    } else {
+      int64_t rem = idx;
+      for (int d = a.nd - 1; d >= 0; --d) {
+        int64_t i = rem % a.ext[d];
+        rem /= a.ext[d];
+        so += i * a.sstr[d];
+        dof += i * a.dstr[d];
+      }
     }
-    dst[dof] = cadd(dst[dof], cmul(alpha, src[so]));
+    dst[dof] = cadd(dst[dof], scaled(ka, alpha, src[so]));
   }
 }
 
@@ -69,7 +82,13 @@ void strided_add(Exec &ex, const cplx *src, const std::vector<int64_t> &sstr, co
     total *= dst.ext[d];
   }
   if (!total) return;
-  k_strided_add<<<grid1d(total, 256), 256, 0, ex.stream>>>(src, a, alpha, dst.p, total);
+  const int ka = factor_kind(alpha);
+  if (total < (1ll << 31)) {
+    for (int d = 0; d < a.nd; ++d) a.fd[d] = fast_div((uint32_t)a.ext[d]);
+    k_strided_add<true><<<grid1d(total, 256), 256, 0, ex.stream>>>(src, a, alpha, ka, dst.p, total);
+  } else {
+    k_strided_add<false><<<grid1d(total, 256), 256, 0, ex.stream>>>(src, a, alpha, ka, dst.p, total);
+  }
   ADC_CHECK_LAUNCH();
 }
 
