@@ -110,6 +110,12 @@ class Clocks:
                 "reasons": reasons, "samples": len(self.samples)}
 
 
+def mma_per_flop(name):
+    """BF16 flops a tensor-core kernel executes per flop its profile entry counts: the sliced products
+    count their digit pairs, FP64 products from eight digits run 36 pairs, the splits 3 or 6 products."""
+    return 1.0 if name.startswith("tc_sliced") else 36.0 if name.startswith("tc_digits") else 6.0 if "bf16x6" in name else 3.0
+
+
 THREE_M = ("zgemm", "gram", "combine")  # FP64 kernels whose complex products take 3 real products
 # k_gram<32, 8, 4, 2, 32> on 32 x 8 vectors of n = 796200 (one launch, ncu): 510,109,184 B read +
 # 4,893,696 B written against (32 + 8) * 796200 * 16 + 32 * 8 * 16 = 509,572,096 algorithmic bytes
@@ -712,7 +718,7 @@ def run_ee(args, cfgname):
         avg = e["total_ms"] / e["launches"]
         alg = e["flops"] / e["launches"]
         if name.startswith("tc_"):
-            mma = (1.0 if name.startswith("tc_sliced") else 6.0 if "bf16x6" in name else 3.0) * alg
+            mma = mma_per_flop(name) * alg
             peak = pk.get("bf16_tflops_sustained", pk.get("bf16_tflops"))
             ach = mma / (avg * 1e-3) / 1e12
             return {"bound": "tensor", "kernel": name, "achieved": ach, "peak": peak, "unit": "TFLOP/s",
@@ -1016,7 +1022,7 @@ def main():
         if name.startswith("tc_"):
             # MMA work: the split products per complex product (3 or 6); the sliced digit
             # pairs are recorded as MMA work already
-            mma = (1.0 if name.startswith("tc_sliced") else 6.0 if "bf16x6" in name else 3.0) * alg
+            mma = mma_per_flop(name) * alg
             ach = mma / (avg_ms * 1e-3) / 1e12
             peak = pk.get("bf16_tflops_sustained", pk.get("bf16_tflops"))
             return {"bound": "tensor", "kernel": name, "achieved": ach, "peak": peak, "unit": "TFLOP/s",

@@ -186,12 +186,11 @@ k_sl_pack(BSrc src, int64_t rows, int64_t K, int conj, int64_t kp, int kfast, co
 // the MMAs) and form the results from 128-bit integers, rounded once, while
 // the next tile's MMAs run. The passes run from the least significant classes
 // up; the first one's sums wait in a global buffer per CTA (L2).
-// What bounds it: the tensor cores (1.07 PFLOP/s of BF16 products at the first
-// two shapes below; N = 128 keeps shared memory busy with operand reads).
+// What bounds it: the tensor cores, and at short inner sizes forming the results.
 // Measured (GB300, 40-bit digits ready, M x N x K complex), with every digit pair a
 // product of its own, FP32 sums through memory and a combining kernel, then now:
-// 19900 x 320 x 19900 48.1 -> 19.9 ms, 8000 x 1600 x 8000 25.0 -> 16.0 ms,
-// 4000 x 1000 x 200 1.63 -> 0.29 ms, 200 x 8 x 200000 2.12 -> 0.56 ms.
+// 19900 x 320 x 19900 48.1 -> 13.3 ms (1.60 PFLOP/s of BF16 products), 8100 x 8100 x 540
+// 4.9 ms (1.2 PFLOP/s: results and drains weigh more), 180 x 6 x 402752 0.62 ms.
 struct SlArgs {
   CUtensorMap mA, mB;
   int M, N2, b, ns, kps, kb_per_split, ksplit, tiles_m, tiles_n, panel, items;
@@ -250,7 +249,6 @@ __device__ __forceinline__ int pass_run(int hi, int b) { return (1 << (20 - 2 * 
 
 // (hi 2^sh + lo) 2^e rounded to nearest: hi is shifted up as far as 64 bits allow (62 bits
 // of the sum at least are kept), the sum normalised and packed with integer instructions
-// (an FP64 conversion takes 64 clocks of a scheduler's FP64 unit per warp)
 __device__ __forceinline__ double scaled_sum(long long hi, int sh, long long lo, int e) {
   const int room = max(0, __clzll(hi < 0 ? -hi : hi) - 2);
   const int up = min(sh, room);
@@ -267,6 +265,27 @@ __device__ __forceinline__ double scaled_sum(long long hi, int sh, long long lo,
   }
   return __longlong_as_double((long long)((((unsigned long long)(be - 1) << 52) + m) |
                                           ((unsigned long long)v & 0x8000000000000000ull)));
+}
+
+// The same in two FP64 operations where hi 2^sh + lo = H 2^sh + L with |H| < 2^51 and
+// 0 <= L < 2^sh: with H' = H - 2^(52 - sh), which the constant 1.5 2^52 turns into a double,
+// fma(H', 2^sh, 2^52 + L) is that sum rounded once (2^52 + L is L's bits under an exponent).
+// The power of two is added to the exponent. False (very large inner sizes, results
+// outside the normal range): scaled_sum.
+__device__ __forceinline__ bool quick_sum(long long hi, int sh, long long lo, double two_sh, int e, double &r) {
+  long long h = hi;
+  double low = 0.0;
+  if (sh) {
+    h += (lo >> sh) - (1ll << (52 - sh));
+    low = __longlong_as_double((lo & ((1ll << sh) - 1)) | 0x4330000000000000ll);
+  }
+  bool ok = (unsigned long long)(h + (1ll << 51)) < (1ull << 52);
+  double t = __longlong_as_double(h + 0x4338000000000000ll) - 6755399441055744.0;
+  if (sh) t = fma(t, two_sh, low);
+  const int top = __double2hiint(t), f = (top >> 20) & 0x7ff;
+  ok = ok && (f == 0 || (f + e >= 1 && f + e <= 2046));
+  r = f ? __hiloint2double(top + e * (1 << 20), __double2loint(t)) : 0.0;
+  return ok;
 }
 
 // eight columns of an accumulator into registers, and the wait that makes them readable (the
@@ -496,33 +515,50 @@ __global__ void __launch_bounds__(320, 1) k_sl_gemm(const __grid_constant__ SlAr
       const unsigned wa = a.WA[m];
       const int n_beg = (d.n0 + half * L::VALS) >> 1;
       const int Nc = a.N2 >> 1;
+      // The next column's spilled sums and scale load while the current one is formed (the
+      // sums' registers leave no room for more). Four columns per round, the sums moved
+      // down in between: unrolled over all of them the code outgrew the instruction cache
       int nh = n_beg / a.n_in, nl = n_beg - nh * a.n_in;
+      long long lr = 0, li = 0;
+      unsigned wb = a.WB[min(n_beg, Nc - 1)];
+      const double two_sh = __hiloint2double((sh + 1023) << 20, 0);
+      if (sh) { lr = sp[0]; li = sp[NT]; }
+#pragma unroll 1
+      for (int j0 = 0; j0 < L::VALS / 2; j0 += 4) {
 #pragma unroll
-      for (int j = 0; j < L::VALS / 2; ++j) {
-        const int n = n_beg + j;
-        if (n < Nc) {
-          const unsigned wb = a.WB[n];
-          cplx val;
-          if (!ok || not_finite(wa) || not_finite(wb)) {
-            // (after a wait that gave up the tile holds no result)
-            val = cmake(__longlong_as_double(0x7ff8000000000000ll), __longlong_as_double(0x7ff8000000000000ll));
-          } else {
-            const int e = scale_exp(wa) + scale_exp(wb) - a.b * (a.ns + 1);
-            const long long lr = sh ? sp[(int64_t)(2 * j) * NT] : 0, li = sh ? sp[(int64_t)(2 * j + 1) * NT] : 0;
-            val = cmake(scaled_sum(acc[2 * j], sh, lr, e), scaled_sum(acc[2 * j + 1], sh, li, e));
+        for (int jj = 0; jj < 4; ++jj) {
+          const int n = n_beg + j0 + jj;
+          const long long cr = lr, ci = li;
+          const unsigned cw = wb;
+          const int next = min(j0 + jj + 1, L::VALS / 2 - 1);
+          wb = a.WB[min(n_beg + next, Nc - 1)];
+          if (sh) { lr = sp[(int64_t)(2 * next) * NT]; li = sp[(int64_t)(2 * next + 1) * NT]; }
+          if (n < Nc) {
+            cplx val;
+            if (!ok || not_finite(wa) || not_finite(cw)) {
+              // (after a wait that gave up the tile holds no result)
+              val = cmake(__longlong_as_double(0x7ff8000000000000ll), __longlong_as_double(0x7ff8000000000000ll));
+            } else {
+              const int e = scale_exp(wa) + scale_exp(cw) - a.b * (a.ns + 1);
+              const bool qr = quick_sum(acc[2 * jj], sh, cr, two_sh, e, val.x);
+              const bool qi = quick_sum(acc[2 * jj + 1], sh, ci, two_sh, e, val.y);
+              if (!(qr && qi)) val = cmake(scaled_sum(acc[2 * jj], sh, cr, e), scaled_sum(acc[2 * jj + 1], sh, ci, e));
+            }
+            if (a.part) {
+              a.part[((int64_t)d.split * a.M + m) * Nc + n] = val;
+            } else {
+              cplx *dst = a.out + m * a.s_m + nh * a.s_nh + nl * a.s_nl;
+              if (a.amode == 1) val = cscale(val, a.alpha.x);
+              else if (a.amode == 2) val = cmul(a.alpha, val);
+              if (a.bmode == 1) { const cplx o = *dst; val = cmake(val.x + a.beta.x * o.x, val.y + a.beta.x * o.y); }
+              else if (a.bmode == 2) val = cadd(val, cmul(a.beta, *dst));
+              *dst = val;
+            }
           }
-          if (a.part) {
-            a.part[((int64_t)d.split * a.M + m) * Nc + n] = val;
-          } else {
-            cplx *dst = a.out + m * a.s_m + nh * a.s_nh + nl * a.s_nl;
-            if (a.amode == 1) val = cscale(val, a.alpha.x);
-            else if (a.amode == 2) val = cmul(a.alpha, val);
-            if (a.bmode == 1) { const cplx o = *dst; val = cmake(val.x + a.beta.x * o.x, val.y + a.beta.x * o.y); }
-            else if (a.bmode == 2) val = cadd(val, cmul(a.beta, *dst));
-            *dst = val;
-          }
+          if (++nl == a.n_in) { nl = 0; ++nh; }
         }
-        if (++nl == a.n_in) { nl = 0; ++nh; }
+#pragma unroll
+        for (int i = 0; i + 8 < L::VALS; ++i) acc[i] = acc[i + 8];
       }
     }
   }
@@ -735,7 +771,10 @@ void sl_gemm(Exec &ex, const SlMat &A, const SlMat &B, int64_t M, int64_t N, cpl
     if (g.ksplit > 1) g.part = w.part.c();
   }
   const int grid = (int)std::min<int64_t>(g.items, sms);
-  int pr = ex.prof_begin("tc_sliced", 8.0 * (double)M * (double)N * (double)A.kreal);
+  // the sliced products count their digit pairs as work, the FP64 ones the product they stand for
+  const double flops = 8.0 * (double)M * (double)N * (double)A.kreal;
+  const bool fp64 = g.ns * g.b >= kDigitFp64Bits;
+  int pr = ex.prof_begin(fp64 ? "tc_digits_fp64" : "tc_sliced_pairs", fp64 ? flops : flops * g.ns * (g.ns + 1) / 2);
   if (bn == 32) launch_sl<32>(ex, g, w, grid);
   else if (bn == 64) launch_sl<64>(ex, g, w, grid);
   else launch_sl<128>(ex, g, w, grid);
