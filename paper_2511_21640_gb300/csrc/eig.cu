@@ -199,6 +199,13 @@ constexpr double OA_ORTH = 1e-13;  // largest |X^H X - I| of an accepted decompo
 
 __device__ inline float2 f2mul(float2 a, float2 b) { return make_float2(a.x * b.x - a.y * b.y, a.x * b.y + a.y * b.x); }
 
+// (x, y) <- (cs x - sn e y, sn x + cs e y)
+__device__ inline void turn(float2 &x, float2 &y, float cs, float sn, float2 e) {
+  const float2 ey = f2mul(e, y);
+  y = make_float2(sn * x.x + cs * ey.x, sn * x.y + cs * ey.y);
+  x = make_float2(cs * x.x - sn * ey.x, cs * x.y - sn * ey.y);
+}
+
 __device__ inline float block_sum_f(float v, float *red) {
   for (int off = 16; off > 0; off >>= 1) v += __shfl_down_sync(0xffffffffu, v, off);
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
@@ -241,8 +248,14 @@ __host__ __device__ inline size_t jacobi32_head_bytes(int n) {
 
 // A (FP64, lda) -> FP32 A - sigma I in shared memory; cyclic Jacobi (round robin);
 // eigenvectors sorted by ascending eigenvalue into X (FP64, n x n, columns), sigma
-// into *shift. The eigenvector work array lives in shared memory, or in Vg
-// (n x n FP32 complex in global memory) when Vg is given.
+// into *shift. The eigenvector work array (transposed: one row per vector) lives in
+// shared memory, or in Vg (n x n FP32 complex in global memory) when Vg is given.
+// What bounds it: the chain of np - 1 steps per sweep, each a barrier, the angles, a
+// barrier and the rotations. Pairs are disjoint, so the 2 x 2 block of pair k's rows
+// and pair l's columns needs only its own four elements: one thread turns it from
+// both sides, in one pass over A and without the barrier between rows and columns.
+// A warp owns a pair k of A or of the vectors, so no index is divided.
+// Measured over the solves of an IP o=8 v=24 Davidson (n up to 48): 174 -> 122 us a call.
 __global__ void __launch_bounds__(1024)
 k_jacobi32(const cplx *__restrict__ Ag, int n, int lda, cplx *X, double *shift, int max_sweeps, float2 *Vg) {
   extern __shared__ float smf[];
@@ -257,6 +270,7 @@ k_jacobi32(const cplx *__restrict__ Ag, int n, int lda, cplx *X, double *shift, 
   float2 *V = Vg ? Vg : A + n * ld;
   __shared__ double dred[32];
   const int tid = threadIdx.x, nt = blockDim.x;
+  const int lane = tid & 31, wid = tid >> 5, nw = nt >> 5;
   // shift by the mean diagonal (FP64), then round
   double ds = 0.0;
   for (int i = tid; i < n; i += nt) ds += Ag[(int64_t)i * lda + i].x;
@@ -288,9 +302,9 @@ k_jacobi32(const cplx *__restrict__ Ag, int n, int lda, cplx *X, double *shift, 
   for (int sweep = 0; !done && sweep < max_sweeps; ++sweep) {
     for (int step = 0; step < np - 1; ++step) {
       for (int k = tid; k < npairs; k += nt) {
-        const int a = (k == 0) ? 0 : ((k - 1 + step) % (np - 1)) + 1;
-        const int kb = np - 1 - k;
-        const int b = ((kb - 1 + step) % (np - 1)) + 1;
+        const int m = np - 1, ka = k - 1 + step, kb = np - 2 - k + step;   // both below 2 m
+        const int a = (k == 0) ? 0 : (ka < m ? ka : ka - m) + 1;
+        const int b = (kb < m ? kb : kb - m) + 1;
         const int p = min(a, b), q = max(a, b);
         pp[k] = p;
         pq[k] = q;
@@ -311,26 +325,43 @@ k_jacobi32(const cplx *__restrict__ Ag, int n, int lda, cplx *X, double *shift, 
         rc[k] = cs; rs[k] = sn; rpr[k] = er; rpi[k] = ei;
       }
       __syncthreads();
-      for (int idx = tid; idx < npairs * n; idx += nt) {
-        const int k = idx / n, col = idx % n;
+      for (int task = wid; task < 2 * npairs; task += nw) {
+        const int k = task < npairs ? task : task - npairs;
         const int p = pp[k], q = pq[k];
-        if (q >= n) continue;
         const float cs = rc[k], sn = rs[k];
-        const float2 ap = A[p * ld + col], eaq = f2mul(make_float2(rpr[k], rpi[k]), A[q * ld + col]);
-        A[p * ld + col] = make_float2(cs * ap.x - sn * eaq.x, cs * ap.y - sn * eaq.y);
-        A[q * ld + col] = make_float2(sn * ap.x + cs * eaq.x, sn * ap.y + cs * eaq.y);
-      }
-      __syncthreads();
-      for (int idx = tid; idx < npairs * n * 2; idx += nt) {
-        const int which = idx / (npairs * n), rem = idx % (npairs * n);
-        const int k = rem / n, row = rem % n;
-        const int p = pp[k], q = pq[k];
-        if (q >= n) continue;
-        const float cs = rc[k], sn = rs[k];
-        float2 *M = which ? V : A;
-        const float2 xp = M[row * ld + p], exq = f2mul(make_float2(rpr[k], -rpi[k]), M[row * ld + q]);
-        M[row * ld + p] = make_float2(cs * xp.x - sn * exq.x, cs * xp.y - sn * exq.y);
-        M[row * ld + q] = make_float2(sn * xp.x + cs * exq.x, sn * xp.y + cs * exq.y);
+        const float2 e = make_float2(rpr[k], rpi[k]);
+        if (task >= npairs) {   // vectors p and q
+          if (q >= n) continue;
+          for (int c = lane; c < n; c += 32) {
+            float2 x = V[p * ld + c], y = V[q * ld + c];
+            turn(x, y, cs, sn, make_float2(e.x, -e.y));
+            V[p * ld + c] = x;
+            V[q * ld + c] = y;
+          }
+          continue;
+        }
+        for (int l = lane; l < npairs; l += 32) {
+          const int pl = pp[l], ql = pq[l];
+          const bool hq = q < n, hl = ql < n;
+          const float2 z = make_float2(0.f, 0.f);
+          float2 a00 = A[p * ld + pl], a01 = hl ? A[p * ld + ql] : z;
+          float2 a10 = hq ? A[q * ld + pl] : z, a11 = hq && hl ? A[q * ld + ql] : z;
+          if (hq) {
+            turn(a00, a10, cs, sn, e);
+            turn(a01, a11, cs, sn, e);
+          }
+          if (hl) {
+            const float2 ec = make_float2(rpr[l], -rpi[l]);
+            turn(a00, a01, rc[l], rs[l], ec);
+            turn(a10, a11, rc[l], rs[l], ec);
+            A[p * ld + ql] = a01;
+          }
+          A[p * ld + pl] = a00;
+          if (hq) {
+            A[q * ld + pl] = a10;
+            if (hl) A[q * ld + ql] = a11;
+          }
+        }
       }
       __syncthreads();
     }
@@ -352,50 +383,70 @@ k_jacobi32(const cplx *__restrict__ Ag, int n, int lda, cplx *X, double *shift, 
       const float dj = A[j * ld + j].x;
       if (dj < di || (dj == di && j < i)) ++rank;
     }
-    for (int r = 0; r < n; ++r) X[(int64_t)r * n + rank] = cmake((double)V[r * ld + i].x, (double)V[r * ld + i].y);
+    for (int r = 0; r < n; ++r) X[(int64_t)r * n + rank] = cmake((double)V[i * ld + r].x, (double)V[i * ld + r].y);
   }
   if (tid == 0) *shift = sigma;
 }
 
-// C = op(A) op(B) (n x n, FP64): 8 x 8 output tile per CTA, A rows and B
-// columns of the tile staged in shared memory; opA: 0 = A, 1 = A^H; B as is;
-// with shift, A - shift I is used for A (opA = 0). beta_one adds C0 (C = C0 + AB).
-constexpr int SG_T = 8;
-__global__ void __launch_bounds__(SG_T * SG_T)
-k_small_gemm(const cplx *__restrict__ A, int lda, int opA, const double *shift, const cplx *__restrict__ B, int ldb,
-             int n, const cplx *C0, cplx *C, int ldc) {
+// C = op(A) B (n x n, FP64): 8 x 8 output tile per CTA, A rows and B columns of the
+// tile staged in shared memory; opA: 0 = A, 1 = A^H; with shift, A - shift I is used
+// for A (opA = 0). herm: C is Hermitian, tiles below the diagonal are the conjugates
+// of those above. blockIdx.z picks one of two independent products. Two warps per half
+// of k: at 64 clocks per FP64 warp instruction of an SM's quarter, the four quarters
+// have to share a tile. With H and T in one launch and the
+// mirrored tiles, a step's products took 23 -> 14 us at n up to 48.
+constexpr int SG_T = 8, SG_THREADS = 2 * SG_T * SG_T;
+struct SgArgs {
+  const cplx *A;
+  int lda, opA;
+  const double *shift;
+  const cplx *B;
+  cplx *C;
+  int herm;
+};
+__global__ void __launch_bounds__(SG_THREADS)
+k_small_gemm(SgArgs g0, SgArgs g1, int n) {
   extern __shared__ double smg[];
+  __shared__ cplx half_sum[SG_T * SG_T];
+  const SgArgs g = blockIdx.z ? g1 : g0;
+  if (g.herm && blockIdx.x < blockIdx.y) return;
   cplx *sa = (cplx *)smg;            // [SG_T][n] rows i of op(A)
   cplx *sb = sa + SG_T * n;          // [n][SG_T] columns j of B
   const int i0 = blockIdx.y * SG_T, j0 = blockIdx.x * SG_T;
-  const double sh = shift ? *shift : 0.0;
-  for (int e = threadIdx.x; e < SG_T * n; e += blockDim.x) {
-    const int ii = e / n, k = e % n, i = i0 + ii;
+  const double sh = g.shift ? *g.shift : 0.0;
+  for (int e = threadIdx.x; e < SG_T * n; e += SG_THREADS) {
+    const int kt = e / SG_T, t = e % SG_T;
     cplx a = cmake(0.0, 0.0);
-    if (i < n) {
-      if (opA) { a = A[(int64_t)k * lda + i]; a.y = -a.y; }
-      else { a = A[(int64_t)i * lda + k]; if (k == i) a.x -= sh; }
+    if (g.opA) {
+      const int i = i0 + t;
+      if (i < n) { a = g.A[(int64_t)kt * g.lda + i]; a.y = -a.y; }
+      sa[t * n + kt] = a;
+    } else {
+      const int ii = e / n, k = e % n, i = i0 + ii;
+      if (i < n) { a = g.A[(int64_t)i * g.lda + k]; if (k == i) a.x -= sh; }
+      sa[e] = a;
     }
-    sa[ii * n + k] = a;
-    const int k2 = e / SG_T, jj = e % SG_T, j = j0 + jj;
-    sb[k2 * SG_T + jj] = (j < n) ? B[(int64_t)k2 * ldb + j] : cmake(0.0, 0.0);
+    sb[e] = (j0 + t < n) ? g.B[(int64_t)kt * n + j0 + t] : cmake(0.0, 0.0);
   }
   __syncthreads();
-  const int ii = threadIdx.x / SG_T, jj = threadIdx.x % SG_T;
+  const int half = threadIdx.x / (SG_T * SG_T), t = threadIdx.x % (SG_T * SG_T);
+  const int ii = t / SG_T, jj = t % SG_T;
   const int i = i0 + ii, j = j0 + jj;
   double re = 0.0, im = 0.0;
-  for (int k = 0; k < n; ++k) {
+  const int kh = (n + 1) / 2, k1 = half ? n : kh;
+  for (int k = half ? kh : 0; k < k1; ++k) {
     const cplx a = sa[ii * n + k], b = sb[k * SG_T + jj];
     re = fma(a.x, b.x, re);
     re = fma(-a.y, b.y, re);
     im = fma(a.x, b.y, im);
     im = fma(a.y, b.x, im);
   }
-  if (i < n && j < n) {
-    cplx r = cmake(re, im);
-    if (C0) r = cadd(r, C0[(int64_t)i * ldc + j]);
-    C[(int64_t)i * ldc + j] = r;
-  }
+  if (half) half_sum[t] = cmake(re, im);
+  __syncthreads();
+  if (half || i >= n || j >= n) return;
+  const cplx r = cadd(cmake(re, im), half_sum[t]);
+  g.C[(int64_t)i * n + j] = r;
+  if (g.herm && blockIdx.x > blockIdx.y) g.C[(int64_t)j * n + i] = cconj(r);
 }
 
 // Hermitian part of M (n x n) at (i, j)
@@ -404,221 +455,271 @@ __device__ inline cplx herm_at(const cplx *__restrict__ M, int n, int i, int j) 
   return cmake(0.5 * (a.x + b.x), 0.5 * (a.y - b.y));
 }
 
-// One refinement step: from H = X^H X and S = X^H (A - shift) X the estimates
-// lam, the clusters (label[i] = smallest column of i's cluster) and
-// F = I + correction. stat[0]: largest (|num_ij| - 1e-14 max|lam|) / |gap_ij|
-// over pairs in different clusters; stat[1]: clusters wider than CL_MAX.
-__global__ void __launch_bounds__(1024)
-k_oa_step(const cplx *__restrict__ H, const cplx *__restrict__ S, int n, double *lam, int *label, cplx *F,
-          double *stat) {
+// One refinement step: from H = X^H X and S = X^H (A - shift) X the estimates lam, the
+// clusters and F = I + correction, with every cluster's columns turned by its
+// eigenvectors. Some 40 FP64 operations per element: one SM's FP64 units (two fused
+// multiply-adds per clock) need longer for them than all SMs for the products, so four
+// launches spread them by rows; what a step needs of the whole matrix (norms, coupling
+// bits, labels) goes through a few kilobytes of scratch, and each CTA reads all of it.
+// Measured in the same Davidson: 75 -> 21 us a step, of which eight-column clusters
+// (one thread's Jacobi of 1.3 ms before) now at most 61 us. The whole eigensolver, random
+// spectrum: n = 32 0.60 -> 0.37 ms, 64 2.20 -> 1.04, 96 5.45 -> 2.60, 128 20.3 -> 6.9.
+constexpr int OA_W = EIG_NMAX / 32;
+constexpr int OA_PARTS = EIG_NMAX;    // one CTA per row
+struct OaArgs {
+  const cplx *H, *S;
+  int n;
+  double *rq;               // [n] Rayleigh quotients S_ii / H_ii
+  double *lam;              // [n] out: eigenvalue estimates
+  double *part;             // [2][OA_PARTS] per-row sums of |S_ij|^2 (i != j) and |R_ij|^2
+  unsigned *mask;           // [n][OA_W] coupling bits
+  cplx *U;                  // [n][CL_MAX] row j: j's row of its cluster's eigenvectors
+  int *label;               // [n] smallest column of the column's cluster
+  double *stat;             // [0]: largest (|num_ij| - 1e-14 max|lam|) / |gap_ij| over pairs
+                            // in different clusters; [1]: clusters wider than CL_MAX
+  cplx *F;
+};
+
+// row blockIdx.x: Rayleigh quotient and norms
+__global__ void __launch_bounds__(EIG_NMAX)
+k_oa_norms(OaArgs o) {
   __shared__ double red[32];
-  __shared__ unsigned int cmask[EIG_NMAX * (EIG_NMAX / 32)];
-  __shared__ int lab[EIG_NMAX];
-  __shared__ double sl[EIG_NMAX];
-  __shared__ int changed;
-  constexpr int W = EIG_NMAX / 32;
-  const int tid = threadIdx.x, nt = blockDim.x;
-  for (int i = tid; i < n; i += nt) {
-    sl[i] = S[(int64_t)i * n + i].x / H[(int64_t)i * n + i].x;
-    lab[i] = i;
-  }
-  for (int w = tid; w < n * W; w += nt) cmask[w] = 0u;
-  __syncthreads();
-  double so = 0.0, rr = 0.0, lm = 0.0;
-  for (int idx = tid; idx < n * n; idx += nt) {
-    const int i = idx / n, j = idx % n;
-    const cplx h = herm_at(H, n, i, j);
+  const int n = o.n, i = blockIdx.x, j = threadIdx.x;
+  double so = 0.0, rr = 0.0;
+  if (j < n) {
+    const cplx h = herm_at(o.H, n, i, j);
     const double rx = (i == j ? 1.0 : 0.0) - h.x, ry = -h.y;
-    rr += rx * rx + ry * ry;
+    rr = rx * rx + ry * ry;
     if (i != j) {
-      const cplx sv = herm_at(S, n, i, j);
-      so += sv.x * sv.x + sv.y * sv.y;
+      const cplx sv = herm_at(o.S, n, i, j);
+      so = sv.x * sv.x + sv.y * sv.y;
     }
   }
-  for (int i = tid; i < n; i += nt) lm = fmax(lm, fabs(sl[i]));
   so = block_sum(so, red);
   rr = block_sum(rr, red);
-  lm = block_max(lm, red);
-  const double thr = fmax(2.0 * (sqrt(so) + lm * sqrt(rr)), OA_TAU * lm);
-  for (int idx = tid; idx < n * n; idx += nt) {
-    const int i = idx / n, j = idx % n;
-    if (j <= i) continue;
-    const cplx h = herm_at(H, n, i, j), sv = herm_at(S, n, i, j);
-    const double gap = sl[j] - sl[i];
-    const double nx = sv.x - sl[j] * h.x, ny = sv.y - sl[j] * h.y;   // S_ij + lam_j R_ij
-    if (fabs(gap) <= thr || OA_ETA * fabs(gap) <= sqrt(nx * nx + ny * ny)) {
-      atomicOr(&cmask[i * W + (j >> 5)], 1u << (j & 31));
-      atomicOr(&cmask[j * W + (i >> 5)], 1u << (i & 31));
-    }
-  }
-  __syncthreads();
-  // connected components: every column takes the smallest label among its
-  // neighbours until nothing changes (labels only decrease)
-  for (int iter = 0; iter <= n; ++iter) {
-    if (tid == 0) changed = 0;
-    __syncthreads();
-    for (int i = tid; i < n; i += nt) {
-      int best = lab[i];
-      for (int w = 0; w < W; ++w) {
-        unsigned int m = cmask[i * W + w];
-        while (m) {
-          const int b = __ffs(m) - 1;
-          m &= m - 1u;
-          best = min(best, lab[w * 32 + b]);
-        }
-      }
-      if (best < lab[i]) { lab[i] = best; changed = 1; }
-    }
-    __syncthreads();
-    const int again = changed;
-    __syncthreads();
-    if (!again) break;
-  }
-  double fr = 0.0;
-  for (int idx = tid; idx < n * n; idx += nt) {
-    const int i = idx / n, j = idx % n;
-    const cplx h = herm_at(H, n, i, j);
-    const double rx = (i == j ? 1.0 : 0.0) - h.x, ry = -h.y;
-    cplx f;
-    if (i == j) {
-      f = cmake(1.0 + 0.5 * rx, 0.0);
-    } else if (lab[i] == lab[j]) {
-      f = cmake(0.5 * rx, 0.5 * ry);
-    } else {
-      const cplx sv = herm_at(S, n, i, j);
-      const double gap = sl[j] - sl[i];
-      const double nx = sv.x + sl[j] * rx, ny = sv.y + sl[j] * ry;
-      f = cmake(nx / gap, ny / gap);
-      fr = fmax(fr, (sqrt(nx * nx + ny * ny) - 1e-14 * lm) / fabs(gap));
-    }
-    F[idx] = f;
-  }
-  fr = block_max(fr, red);
-  int big = 0;
-  for (int i = tid; i < n; i += nt) {
-    lam[i] = sl[i];
-    label[i] = lab[i];
-    if (lab[i] == i) {
-      int cnt = 0;
-      for (int j = i; j < n; ++j) cnt += (lab[j] == i);
-      big += (cnt > CL_MAX);
-    }
-  }
-  const double bigd = block_sum((double)big, red);
-  if (tid == 0) {
-    stat[0] = fr;
-    stat[1] = bigd;
+  if (j == 0) {
+    o.part[i] = so;
+    o.part[OA_PARTS + i] = rr;
+    o.rq[i] = o.S[(int64_t)i * n + i].x / o.H[(int64_t)i * n + i].x;
+    if (i == 0) o.stat[0] = 0.0;
   }
 }
 
-// Each cluster of 2..CL_MAX columns (label from k_oa_step) is diagonalised
-// exactly: U, w = eig(P^H S_c P), P = I + R_c / 2; its columns of F become
-// F[:, c] U and its lam the eigenvalues w. Other columns of F are copied.
-__global__ void __launch_bounds__(1024)
-k_cluster_rotate(const cplx *__restrict__ F, const cplx *__restrict__ H, const cplx *__restrict__ S,
-                 const int *__restrict__ label, int n, double *lam, cplx *Fout) {
-  __shared__ cplx U[EIG_NMAX * CL_MAX];    // row j: j's row of its cluster's U
-  __shared__ int mem[EIG_NMAX * CL_MAX];   // members of the cluster rooted at i, ascending
-  __shared__ int csize[EIG_NMAX], pos[EIG_NMAX], lab[EIG_NMAX];
-  const int tid = threadIdx.x, nt = blockDim.x;
-  for (int j = tid; j < n; j += nt) lab[j] = label[j];
-  __syncthreads();
-  for (int j = tid; j < n; j += nt) {
-    const int root = lab[j];
-    int before = 0, total = 0;
-    for (int k = 0; k < n; ++k) {
-      const int in = (lab[k] == root);
-      total += in;
-      before += in && k < j;
-    }
-    pos[j] = before;
-    csize[j] = total;
-    if (before < CL_MAX) mem[root * CL_MAX + before] = j;
+// row blockIdx.x of the coupling bits
+__global__ void __launch_bounds__(EIG_NMAX)
+k_oa_couple(OaArgs o) {
+  __shared__ double red[32];
+  const int n = o.n, i = blockIdx.x, j = threadIdx.x;
+  const double so = block_sum(j < n ? o.part[j] : 0.0, red);
+  const double rr = block_sum(j < n ? o.part[OA_PARTS + j] : 0.0, red);
+  const double lm = block_max(j < n ? fabs(o.rq[j]) : 0.0, red);
+  const double thr = fmax(2.0 * (sqrt(so) + lm * sqrt(rr)), OA_TAU * lm);
+  bool couple = false;
+  if (j < n && j != i) {
+    const int a = min(i, j), b = max(i, j);
+    const cplx h = herm_at(o.H, n, a, b), sv = herm_at(o.S, n, a, b);
+    const double lb = o.rq[b], gap = lb - o.rq[a];
+    const double nx = sv.x - lb * h.x, ny = sv.y - lb * h.y;   // S_ab + lam_b R_ab
+    couple = fabs(gap) <= thr || OA_ETA * fabs(gap) <= sqrt(nx * nx + ny * ny);
   }
+  const unsigned bits = __ballot_sync(0xffffffffu, couple);
+  if ((j & 31) == 0) o.mask[i * OA_W + (j >> 5)] = bits;
+}
+
+// connected components of the coupling: every column takes the smallest label among
+// its neighbours until nothing changes (labels only decrease). One thread per column.
+__device__ inline void oa_labels(const unsigned *mask, int n, int *lab) {
+  const int j = threadIdx.x;
+  unsigned m[OA_W];
+  for (int w = 0; w < OA_W; ++w) m[w] = j < n ? mask[j * OA_W + w] : 0u;
+  lab[j] = j;
   __syncthreads();
-  for (int i = tid; i < n; i += nt) {
-    if (lab[i] != i) continue;
-    const int sc = csize[i];
-    if (sc < 2 || sc > CL_MAX) continue;
-    const int *mi = mem + i * CL_MAX;
-    cplx a[CL_MAX][CL_MAX], u[CL_MAX][CL_MAX], t[CL_MAX][CL_MAX];
-    // t = S_c P, a = P^H t with P = I + R_c / 2 (R = I - H)
-    for (int r = 0; r < sc; ++r)
-      for (int c = 0; c < sc; ++c) {
-        cplx acc = cmake(0.0, 0.0);
-        for (int l = 0; l < sc; ++l) {
-          const cplx hl = herm_at(H, n, mi[l], mi[c]);
-          const cplx p = cmake((l == c ? 1.5 : 0.0) - 0.5 * hl.x, -0.5 * hl.y);
-          acc = cadd(acc, cmul(herm_at(S, n, mi[r], mi[l]), p));
-        }
-        t[r][c] = acc;
-      }
-    for (int r = 0; r < sc; ++r)
-      for (int c = 0; c < sc; ++c) {
-        cplx acc = cmake(0.0, 0.0);
-        for (int l = 0; l < sc; ++l) {
-          const cplx hl = herm_at(H, n, mi[l], mi[r]);
-          const cplx pc = cmake((l == r ? 1.5 : 0.0) - 0.5 * hl.x, 0.5 * hl.y);   // conj(P[l][r])
-          acc = cadd(acc, cmul(pc, t[l][c]));
-        }
-        a[r][c] = acc;
-        u[r][c] = cmake(r == c ? 1.0 : 0.0, 0.0);
-      }
-    for (int r = 0; r < sc; ++r)
-      for (int c = r + 1; c < sc; ++c) {   // exact Hermitian symmetry for the Jacobi sweeps
-        const cplx m = cmake(0.5 * (a[r][c].x + a[c][r].x), 0.5 * (a[r][c].y - a[c][r].y));
-        a[r][c] = m;
-        a[c][r] = cconj(m);
-      }
-    for (int sweep = 0; sweep < 12; ++sweep) {
-      double off = 0.0, dia = 0.0;
-      for (int r = 0; r < sc; ++r)
-        for (int c = 0; c < sc; ++c) {
-          const double m2 = a[r][c].x * a[r][c].x + a[r][c].y * a[r][c].y;
-          if (r == c) dia += m2; else off += m2;
-        }
-      if (off <= 1e-32 * dia || off == 0.0) break;
-      for (int p = 0; p < sc - 1; ++p)
-        for (int q = p + 1; q < sc; ++q) {
-          const cplx apq = a[p][q];
-          const double mag = sqrt(apq.x * apq.x + apq.y * apq.y);
-          if (mag <= 1e-300) continue;
-          const cplx e = cmake(apq.x / mag, apq.y / mag), ec = cconj(e);
+  for (int iter = 0; iter <= n; ++iter) {
+    int best = lab[j];
+    for (int w = 0; w < OA_W; ++w)
+      for (unsigned b = m[w]; b; b &= b - 1u) best = min(best, lab[w * 32 + __ffs(b) - 1]);
+    const int less = best < lab[j];
+    const int again = __syncthreads_or(less);   // every neighbour is read before a label changes
+    if (less) lab[j] = best;
+    __syncthreads();
+    if (!again) break;
+  }
+}
+
+// Each cluster of 2..CL_MAX columns is diagonalised exactly: U, w = eig(P^H S_c P),
+// P = I + R_c / 2, by one warp: Jacobi rounds of up to four disjoint pairs, a lane per
+// pair for the angles and per pair and element for the rotations. The warp of a cluster
+// is that of its smallest column, four columns per CTA.
+constexpr int CLU_WARPS = EIG_NMAX / 32;
+__global__ void __launch_bounds__(EIG_NMAX)
+k_oa_cluster(OaArgs o) {
+  __shared__ int lab[EIG_NMAX];
+  __shared__ cplx sa[CLU_WARPS][CL_MAX][CL_MAX], su[CLU_WARPS][CL_MAX][CL_MAX], st[CLU_WARPS][CL_MAX][CL_MAX];
+  __shared__ int smem_mem[CLU_WARPS][CL_MAX];
+  const int n = o.n, lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  oa_labels(o.mask, n, lab);
+  const int i = blockIdx.x * CLU_WARPS + wid;
+  int sc = 0;                           // the size of the cluster that starts at column i
+  if (i < n && lab[i] == i)
+    for (int w = 0; w < OA_W; ++w) {
+      const int j = w * 32 + lane, in = j < n && lab[j] == i;
+      const unsigned bits = __ballot_sync(0xffffffffu, in);
+      const int at = sc + __popc(bits & ((1u << lane) - 1u));
+      if (in && at < CL_MAX) smem_mem[wid][at] = j;
+      sc += __popc(bits);
+    }
+  if (i < n && lane == 0) o.label[i] = lab[i];
+  if (blockIdx.x == 0) {
+    int big = 0;
+    for (int j = lane; j < n && wid == 0; j += 32) {
+      if (lab[j] != j) continue;
+      int cnt = 0;
+      for (int k = j; k < n; ++k) cnt += (lab[k] == j);
+      big += cnt > CL_MAX;
+    }
+    for (int off = 16; off > 0; off >>= 1) big += __shfl_down_sync(0xffffffffu, big, off);
+    if (threadIdx.x == 0) o.stat[1] = (double)big;
+  }
+  __syncwarp();
+  if (sc == 0) return;
+  if (sc == 1 || sc > CL_MAX) {         // a wide cluster keeps its columns as they are
+    for (int j = i + lane; j < n; j += 32)
+      if (lab[j] == i) o.lam[j] = o.rq[j];
+    return;
+  }
+  cplx(*a)[CL_MAX] = sa[wid], (*u)[CL_MAX] = su[wid], (*t)[CL_MAX] = st[wid];
+  const int *mi = smem_mem[wid];
+  // t = S_c P, a = P^H t with P = I + R_c / 2 (R = I - H)
+  for (int e = lane; e < sc * sc; e += 32) {
+    const int r = e / sc, c = e % sc;
+    cplx acc = cmake(0.0, 0.0);
+    for (int l = 0; l < sc; ++l) {
+      const cplx hl = herm_at(o.H, n, mi[l], mi[c]);
+      const cplx p = cmake((l == c ? 1.5 : 0.0) - 0.5 * hl.x, -0.5 * hl.y);
+      acc = cadd(acc, cmul(herm_at(o.S, n, mi[r], mi[l]), p));
+    }
+    t[r][c] = acc;
+  }
+  __syncwarp();
+  for (int e = lane; e < sc * sc; e += 32) {
+    const int r = e / sc, c = e % sc;
+    cplx acc = cmake(0.0, 0.0);
+    for (int l = 0; l < sc; ++l) {
+      const cplx hl = herm_at(o.H, n, mi[l], mi[r]);
+      const cplx pc = cmake((l == r ? 1.5 : 0.0) - 0.5 * hl.x, 0.5 * hl.y);   // conj(P[l][r])
+      acc = cadd(acc, cmul(pc, t[l][c]));
+    }
+    a[r][c] = acc;
+    u[r][c] = cmake(r == c ? 1.0 : 0.0, 0.0);
+  }
+  __syncwarp();
+  for (int e = lane; e < sc * sc; e += 32) {   // exact Hermitian symmetry for the Jacobi sweeps
+    const int r = e / sc, c = e % sc;
+    if (r >= c) continue;
+    const cplx m = cmake(0.5 * (a[r][c].x + a[c][r].x), 0.5 * (a[r][c].y - a[c][r].y));
+    a[r][c] = m;
+    a[c][r] = cconj(m);
+  }
+  __syncwarp();
+  const int np = sc + (sc & 1), pairs = np / 2, m = np - 1;
+  const int k = lane / CL_MAX, x = lane % CL_MAX;   // pair and element of this lane
+  for (int sweep = 0; sweep < 12; ++sweep) {
+    double off = 0.0, dia = 0.0;
+    for (int e = lane; e < sc * sc; e += 32) {
+      const cplx v = a[e / sc][e % sc];
+      const double m2 = v.x * v.x + v.y * v.y;
+      if (e / sc == e % sc) dia += m2; else off += m2;
+    }
+    for (int s = 16; s > 0; s >>= 1) {
+      off += __shfl_xor_sync(0xffffffffu, off, s);
+      dia += __shfl_xor_sync(0xffffffffu, dia, s);
+    }
+    if (off <= 1e-32 * dia || off == 0.0) break;
+    for (int step = 0; step < m; ++step) {
+      const int ka = k - 1 + step, kb = np - 2 - k + step;
+      const int pa = (k == 0) ? 0 : (ka < m ? ka : ka - m) + 1, pb = (kb < m ? kb : kb - m) + 1;
+      const int p = min(pa, pb), q = max(pa, pb);
+      bool act = k < pairs && q < sc;
+      double cs = 1.0, sn = 0.0;
+      cplx e = cmake(1.0, 0.0);
+      if (act) {
+        const cplx apq = a[p][q];
+        const double mag = sqrt(apq.x * apq.x + apq.y * apq.y);
+        act = mag > 1e-300;
+        if (act) {
+          e = cmake(apq.x / mag, apq.y / mag);
           const double tau = (a[q][q].x - a[p][p].x) / (2.0 * mag);
           const double tt = (tau >= 0.0 ? 1.0 : -1.0) / (fabs(tau) + sqrt(1.0 + tau * tau));
-          const double cs = 1.0 / sqrt(1.0 + tt * tt), sn = tt * cs;
-          for (int c = 0; c < sc; ++c) {   // rows p, q
-            const cplx ap = a[p][c], eaq = cmul(e, a[q][c]);
-            a[p][c] = cmake(cs * ap.x - sn * eaq.x, cs * ap.y - sn * eaq.y);
-            a[q][c] = cmake(sn * ap.x + cs * eaq.x, sn * ap.y + cs * eaq.y);
-          }
-          for (int r = 0; r < sc; ++r) {   // columns p, q of a and u
-            const cplx xp = a[r][p], exq = cmul(ec, a[r][q]);
-            a[r][p] = cmake(cs * xp.x - sn * exq.x, cs * xp.y - sn * exq.y);
-            a[r][q] = cmake(sn * xp.x + cs * exq.x, sn * xp.y + cs * exq.y);
-            const cplx up = u[r][p], euq = cmul(ec, u[r][q]);
-            u[r][p] = cmake(cs * up.x - sn * euq.x, cs * up.y - sn * euq.y);
-            u[r][q] = cmake(sn * up.x + cs * euq.x, sn * up.y + cs * euq.y);
-          }
+          cs = 1.0 / sqrt(1.0 + tt * tt);
+          sn = tt * cs;
         }
+      }
+      act = act && x < sc;
+      __syncwarp();
+      if (act) {   // rows p, q
+        const cplx ap = a[p][x], eaq = cmul(e, a[q][x]);
+        a[p][x] = cmake(cs * ap.x - sn * eaq.x, cs * ap.y - sn * eaq.y);
+        a[q][x] = cmake(sn * ap.x + cs * eaq.x, sn * ap.y + cs * eaq.y);
+      }
+      __syncwarp();
+      if (act) {   // columns p, q of a and u
+        const cplx ec = cconj(e);
+        const cplx xp = a[x][p], exq = cmul(ec, a[x][q]);
+        a[x][p] = cmake(cs * xp.x - sn * exq.x, cs * xp.y - sn * exq.y);
+        a[x][q] = cmake(sn * xp.x + cs * exq.x, sn * xp.y + cs * exq.y);
+        const cplx up = u[x][p], euq = cmul(ec, u[x][q]);
+        u[x][p] = cmake(cs * up.x - sn * euq.x, cs * up.y - sn * euq.y);
+        u[x][q] = cmake(sn * up.x + cs * euq.x, sn * up.y + cs * euq.y);
+      }
+      __syncwarp();
     }
-    for (int r = 0; r < sc; ++r)
-      for (int c = 0; c < sc; ++c) U[mi[r] * CL_MAX + c] = u[r][c];
-    for (int c = 0; c < sc; ++c) lam[mi[c]] = a[c][c].x;
   }
-  __syncthreads();
-  for (int idx = tid; idx < n * n; idx += nt) {
-    const int r = idx / n, j = idx % n;
-    const int sc = csize[j];
-    if (sc < 2 || sc > CL_MAX) {
-      Fout[idx] = F[idx];
-      continue;
+  for (int e = lane; e < sc * sc; e += 32) o.U[mi[e / sc] * CL_MAX + e % sc] = u[e / sc][e % sc];
+  if (lane < sc) o.lam[mi[lane]] = a[lane][lane].x;
+}
+
+// row blockIdx.x of F, its columns of each cluster of 2..CL_MAX times the cluster's U
+__global__ void __launch_bounds__(EIG_NMAX)
+k_oa_form(OaArgs o) {
+  __shared__ double red[32];
+  __shared__ cplx f[EIG_NMAX];
+  __shared__ int lab[EIG_NMAX];
+  const int n = o.n, i = blockIdx.x, j = threadIdx.x;
+  if (j < n) lab[j] = o.label[j];
+  const double lm = block_max(j < n ? fabs(o.rq[j]) : 0.0, red);
+  double fr = 0.0;
+  if (j < n) {
+    const cplx h = herm_at(o.H, n, i, j);
+    const double rx = (i == j ? 1.0 : 0.0) - h.x, ry = -h.y;
+    if (i == j) {
+      f[j] = cmake(1.0 + 0.5 * rx, 0.0);
+    } else if (lab[i] == lab[j]) {
+      f[j] = cmake(0.5 * rx, 0.5 * ry);
+    } else {
+      const cplx sv = herm_at(o.S, n, i, j);
+      const double lj = o.rq[j], gap = lj - o.rq[i];
+      const double nx = sv.x + lj * rx, ny = sv.y + lj * ry;
+      f[j] = cmake(nx / gap, ny / gap);
+      fr = fmax(fr, (sqrt(nx * nx + ny * ny) - 1e-14 * lm) / fabs(gap));
     }
-    const int *mj = mem + lab[j] * CL_MAX, jj = pos[j];
-    cplx acc = cmake(0.0, 0.0);
-    for (int l = 0; l < sc; ++l) acc = cadd(acc, cmul(F[(int64_t)r * n + mj[l]], U[mj[l] * CL_MAX + jj]));
-    Fout[idx] = acc;
   }
+  fr = block_max(fr, red);              // at least 0: its bits order like the number
+  if (j == 0) atomicMax((unsigned long long *)o.stat, (unsigned long long)__double_as_longlong(fr));
+  if (j >= n) return;
+  const int root = lab[j];
+  int sc = 0, pos = 0;
+  for (int k = root; k < n; ++k) {
+    const int in = lab[k] == root;
+    pos += in && k < j;
+    sc += in;
+  }
+  cplx r = f[j];
+  if (sc >= 2 && sc <= CL_MAX) {
+    r = cmake(0.0, 0.0);
+    for (int k = root; k < n; ++k)
+      if (lab[k] == root) r = cadd(r, cmul(f[k], o.U[k * CL_MAX + pos]));
+  }
+  o.F[(int64_t)i * n + j] = r;
 }
 
 // eigenvalues lam + shift sorted ascending into w, the columns of X likewise into V (ldv)
@@ -681,32 +782,40 @@ void eigh_refined(Exec &ex, const cplx *A, int n, int lda, double *w, cplx *V, i
   set_smem_limit((const void *)k_small_gemm, 64 * 1024);
   DBuf X0 = cbuf(ex, nn), X1 = cbuf(ex, nn), T = cbuf(ex, nn), H = cbuf(ex, nn), S = cbuf(ex, nn), F = cbuf(ex, nn);
   DBuf lam(ex, n * sizeof(double)), sc(ex, 4 * sizeof(double)), lab(ex, n * sizeof(int));
+  DBuf oas(ex, (EIG_NMAX + 2 * OA_PARTS) * sizeof(double) + EIG_NMAX * OA_W * sizeof(unsigned));
+  DBuf U = cbuf(ex, (int64_t)EIG_NMAX * CL_MAX);
   k_jacobi32<<<1, 1024, smem, ex.stream>>>(A, n, lda, X0.c(), sc.d(), 30, (float2 *)vg.p);
   ADC_CHECK_LAUNCH();
-  const dim3 g((n + SG_T - 1) / SG_T, (n + SG_T - 1) / SG_T);
+  const int gt = (n + SG_T - 1) / SG_T;
   const size_t gs = 2 * (size_t)SG_T * n * sizeof(cplx);
+  auto product = [&](const SgArgs &g0, const SgArgs *g1) {
+    k_small_gemm<<<dim3(gt, gt, g1 ? 2 : 1), SG_THREADS, gs, ex.stream>>>(g0, g1 ? *g1 : g0, n);
+    ADC_CHECK_LAUNCH();
+  };
+  double *part = oas.d() + EIG_NMAX;
+  OaArgs oa{H.c(), S.c(), n, oas.d(), lam.d(), part, (unsigned *)(part + 2 * OA_PARTS), U.c(), (int *)lab.p,
+            sc.d() + 1, F.c()};
   cplx *X = X0.c(), *Xn = X1.c();
   bool ok = false;
   for (int it = 0; it < nsteps + 3; ++it) {
-    // T = (A - shift) X, S = X^H T, H = X^H X
-    k_small_gemm<<<g, SG_T * SG_T, gs, ex.stream>>>(A, lda, 0, sc.d(), X, n, n, nullptr, T.c(), n);
+    // T = (A - shift) X and H = X^H X, then S = X^H T
+    const SgArgs gH{X, n, 1, nullptr, X, H.c(), 1};
+    product(SgArgs{A, lda, 0, sc.d(), X, T.c(), 0}, &gH);
+    product(SgArgs{X, n, 1, nullptr, T.c(), S.c(), 1}, nullptr);
+    k_oa_norms<<<n, EIG_NMAX, 0, ex.stream>>>(oa);
     ADC_CHECK_LAUNCH();
-    k_small_gemm<<<g, SG_T * SG_T, gs, ex.stream>>>(X, n, 1, nullptr, T.c(), n, n, nullptr, S.c(), n);
+    k_oa_couple<<<n, EIG_NMAX, 0, ex.stream>>>(oa);
     ADC_CHECK_LAUNCH();
-    k_small_gemm<<<g, SG_T * SG_T, gs, ex.stream>>>(X, n, 1, nullptr, X, n, n, nullptr, H.c(), n);
+    k_oa_cluster<<<(n + CLU_WARPS - 1) / CLU_WARPS, EIG_NMAX, 0, ex.stream>>>(oa);
     ADC_CHECK_LAUNCH();
-    k_oa_step<<<1, 1024, 0, ex.stream>>>(H.c(), S.c(), n, lam.d(), (int *)lab.p, F.c(), sc.d() + 1);
+    k_oa_form<<<n, EIG_NMAX, 0, ex.stream>>>(oa);
     ADC_CHECK_LAUNCH();
-    k_cluster_rotate<<<1, 1024, 0, ex.stream>>>(F.c(), H.c(), S.c(), (const int *)lab.p, n, lam.d(), T.c());
-    ADC_CHECK_LAUNCH();
-    // X <- X (I + F) blockdiag(U)
-    k_small_gemm<<<g, SG_T * SG_T, gs, ex.stream>>>(X, n, 0, nullptr, T.c(), n, n, nullptr, Xn, n);
-    ADC_CHECK_LAUNCH();
+    // X <- X F, F = (I + correction) blockdiag(U)
+    product(SgArgs{X, n, 0, nullptr, F.c(), Xn, 0}, nullptr);
     std::swap(X, Xn);
     if (it + 1 >= nsteps) {
       // orthonormality of the updated vectors
-      k_small_gemm<<<g, SG_T * SG_T, gs, ex.stream>>>(X, n, 1, nullptr, X, n, n, nullptr, H.c(), n);
-      ADC_CHECK_LAUNCH();
+      product(SgArgs{X, n, 1, nullptr, X, H.c(), 1}, nullptr);
       k_orth_err<<<1, 1024, 0, ex.stream>>>(H.c(), n, sc.d() + 3);
       ADC_CHECK_LAUNCH();
       double st[3];
