@@ -53,8 +53,9 @@ enum { ADC_IP = 0, ADC_EA = 1, ADC_EE = 2 };
 
 /* Arithmetic of a sigma product.
  * ADC_PREC_FP64:   FP64 throughout: small contractions on the CUDA cores, large
- *   ones on the tensor cores from 56-bit integer digits (below), whose error
- *   against exact sums is no larger than that of FP64 multiply-adds.
+ *   ones on the tensor cores from 56-bit integer digits (below): 56 bits
+ *   relative to the row and column maxima, measured no further from exact sums
+ *   than FP64 multiply-adds.
  * ADC_PREC_BF16X3: the dense contractions on the tensor cores (tcgen05) with
  *   each FP64 operand split into two BF16 parts (hi + lo) and the three
  *   products hi*hi + hi*lo + lo*hi accumulated in FP32; complex arithmetic by
@@ -67,9 +68,9 @@ enum { ADC_IP = 0, ADC_EA = 1, ADC_EE = 2 };
  *   more accurate. Batches (adc_batch_*) use BF16X3.
  * ADC_PREC_SLICED: FP64-accurate products on the tensor cores.
  *   Each operand row is scaled by a power of two and written as a sum of
- *   integer BF16 digits of 4 to 7 bits; every digit product is summed exactly
+ *   integer BF16 digits of seven bits; every digit product is summed exactly
  *   in the FP32 accumulator (the inner size is split so that the sums stay
- *   below 2^24) and the pair products are combined in FP64, for about 40
+ *   below 2^24) and then in integers, rounded once, for about 40
  *   significant bits relative to the row and column maxima (about 1e-11
  *   relative to the largest output). Used for the refinement products of the
  *   mixed Davidson when opts.refine selects it.

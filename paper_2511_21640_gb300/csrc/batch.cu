@@ -642,7 +642,10 @@ int adc_batch_solve(int n, const adc_problem *p, int nroots, double tol, int max
           op.setup = o.setup;
           op.refine = o.refine;
           irc[j] = adc_init(&ctxs[j], q.B, q.naux, q.eps_occ, q.nocc, q.eps_vir, q.nvir, q.kind, q.order, q.x, &op);
-          if (irc[j] == ADC_OK) irc[j] = adc_sync(ctxs[j]);
+          if (irc[j] == ADC_OK) {
+            ctxs[j]->keep_digits = false;  // the plan's memory has no room for them
+            irc[j] = adc_sync(ctxs[j]);
+          }
         }
       });
     }

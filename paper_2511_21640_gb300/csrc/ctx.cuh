@@ -47,6 +47,7 @@ struct adc_ctx {
   // split-precision copies for the tensor-core sigma
   std::unique_ptr<adc::TcCache> tc;
   // integer-digit slices for the FP64-accurate tensor-core sigma
+  bool keep_digits = true;  // FP64 products may keep their operators' digits
   std::unique_ptr<adc::SlCache> sl;
 
   // EE-ADC operators (kind == ADC_EE)

@@ -263,8 +263,8 @@ k_jacobi32(const cplx *__restrict__ Ag, int n, int lda, cplx *X, double *shift, 
   float *rc = smf, *rs = rc + npairs, *rpr = rs + npairs, *rpi = rpr + npairs;
   int *pp = (int *)(rpi + npairs), *pq = pp + npairs;
   float *red = (float *)(pq + npairs);
-  // rows padded to n + 1 elements: the column rotations walk down a column
-  // with consecutive lanes on consecutive rows, free of bank conflicts
+  // rows padded to n + 1 elements: reads down a column (the last pass over V) are free
+  // of bank conflicts
   const int ld = n + 1;
   float2 *A = (float2 *)(((uintptr_t)(red + 64) + 15) & ~(uintptr_t)15);
   float2 *V = Vg ? Vg : A + n * ld;

@@ -3,6 +3,8 @@
 // (sigma_sliced, tc_slice.cu). Same terms as sigma.cu (Sec. 2.1 Eqs. 10-12);
 // the coupling, ladder and ring contractions run on the tensor cores, the main
 // block (n1 x n1) and the zeroth-order diagonal stay FP64.
+#include <atomic>
+
 #include "ctx.cuh"
 #include "tc_gemm.cuh"
 #include "tc_slice.cuh"
@@ -208,10 +210,45 @@ void sigma_split(adc_ctx *c, const cplx *X, cplx *S, int64_t k, int nseg) {
 }
 
 // ---- products from digits: the same contractions as sliced tensor-core products.
+// Digits kept for FP64 products, all contexts of a device together: at most an
+// eighth of its memory (an EA problem at o = 40, v = 200 keeps 25 GB).
+static std::atomic<int64_t> sl_kept_total[64];
+SlCache::~SlCache() { sl_kept_total[dev] -= kept; }
+
+// The digits kept for FP64 products alone go back when the context runs short of
+// memory, and are not kept again: what fits without them still fits.
+static bool sl_give_back(void *ctx) {
+  SlCache *sl = ((adc_ctx *)ctx)->sl.get();
+  if (!sl || sl->busy) return false;
+  bool any = false;
+  for (int w = 0; w < SL_NOPS; ++w) {
+    if (sl->op[w].ns * sl->op[w].b < kDigitFp64Bits) continue;
+    sl->op[w] = SlMat();
+    sl->no_room[w] = true;
+    any = true;
+  }
+  sl_kept_total[sl->dev] -= sl->kept;
+  sl->kept = 0;
+  sl->Bx = SlMat();
+  sl->w.part.reset();
+  return any;
+}
+
 static SlCache &sl_cache(adc_ctx *c) {
-  if (!c->sl) c->sl.reset(new SlCache());
+  if (!c->sl) {
+    c->sl.reset(new SlCache());
+    c->sl->dev = std::max(0, c->dev) % 64;
+    c->ex.give_back = sl_give_back;
+    c->ex.give_back_of = c;
+  }
   return *c->sl;
 }
+
+struct SlUse {
+  SlCache &sl;
+  explicit SlUse(SlCache &s) : sl(s) { ++sl.busy; }
+  ~SlUse() { --sl.busy; }
+};
 
 // The digits of a static operator, built when first asked for and rebuilt with
 // more digits when asked for more; a product with fewer bits uses the leading
@@ -237,6 +274,7 @@ void sigma_sliced(adc_ctx *c, const cplx *X, cplx *S, int64_t k, int bits) {
   ADC_REQUIRE(c->kind != ADC_EE, ADC_ERR_ARG, "sigma_sliced: IP and EA (EE goes through sigma_ee_split)");
   Exec &ex = c->ex;
   SlCache &sl = sl_cache(c);
+  const SlUse use(sl);
   if (!sl.err.p) {
     sl.err = DBuf(ex, sizeof(int));
     fill_zero(ex, sl.err.p, sizeof(int));
@@ -297,6 +335,25 @@ void sigma_sliced(adc_ctx *c, const cplx *X, cplx *S, int64_t k, int bits) {
   }
 }
 
+// whether the FP64 digits of an operator are kept, or may be: within a quarter of the
+// context's free memory and the device's share
+static bool sl_keep(adc_ctx *c, SlCache &sl, int which, int64_t M, int64_t K) {
+  if (sl.no_room[which]) return false;
+  if (sl.op[which].ns * sl.op[which].b >= kDigitFp64Bits) return true;
+  const double need = 4.0 * sl_digits(K, kDigitFp64Bits).ns * (double)M * (double)sl_kp(K);
+  double room = (double)free_device_memory();
+  if (c->ex.mem_limit > 0) room = std::min(room, (double)(c->ex.mem_limit - c->ex.mem_used));
+  size_t fr = 0, tot = 0;
+  ADC_CUDA(cudaMemGetInfo(&fr, &tot));
+  if (!c->keep_digits || need > 0.25 * room || (double)sl_kept_total[sl.dev] + need > 0.125 * (double)tot) {
+    sl.no_room[which] = true;
+    return false;
+  }
+  sl_kept_total[sl.dev] += (int64_t)need;
+  sl.kept += (int64_t)need;
+  return true;
+}
+
 // ---- one term of the FP64 product with the kept digits of its operator:
 // out = alpha op B^T + beta out as tc_gemm addresses it, B by its strides or (ring)
 // gathered from X2. Slicing the operator again in every product took 6.9 of the
@@ -313,17 +370,8 @@ bool fp64_op_product(adc_ctx *c, int which, bool ring, const cplx *X, int64_t k,
   const int64_t K = which == SL_CPL ? n2 : which == SL_CPLT ? n1 : M;
   if (!fp64_digits_usable(ex, M, Nc, K)) return false;
   SlCache &sl = sl_cache(c);
-  SlMat &m = sl.op[which];
-  if (sl.no_room[which]) return false;
-  if (m.ns * m.b < kDigitFp64Bits) {
-    const double need = 4.0 * sl_digits(K, kDigitFp64Bits).ns * (double)M * (double)sl_kp(K);
-    double room = 0.25 * (double)free_device_memory();
-    if (ex.mem_limit > 0) room = std::min(room, (double)(ex.mem_limit - ex.mem_used));
-    if (need > room) {
-      sl.no_room[which] = true;
-      return false;
-    }
-  }
+  const SlUse use(sl);
+  if (!sl_keep(c, sl, which, M, K)) return false;
   try {
     const SlMat &A = sl_op(c, which, kDigitFp64Bits);
     if (ring) sl_pack_B_ring(ex, sl.Bx, c, X, k, A, kDigitFp64Bits);
@@ -350,11 +398,8 @@ void fp64_ops_prepare(adc_ctx *c, int64_t k) {
     if (w == SL_GLAD && ea && c->direct_ladder) continue;
     if (!fp64_digits_usable(c->ex, M[w], Nc[w], K[w])) continue;
     SlCache &sl = sl_cache(c);
-    const double need = 4.0 * sl_digits(K[w], kDigitFp64Bits).ns * (double)M[w] * (double)sl_kp(K[w]);
-    double room = 0.25 * (double)free_device_memory();
-    if (c->ex.mem_limit > 0) room = std::min(room, (double)(c->ex.mem_limit - c->ex.mem_used));
-    if (sl.op[w].ns * sl.op[w].b >= kDigitFp64Bits || sl.no_room[w]) continue;
-    if (need > room) { sl.no_room[w] = true; continue; }
+    const SlUse use(sl);
+    if (sl.op[w].ns * sl.op[w].b >= kDigitFp64Bits || !sl_keep(c, sl, w, M[w], K[w])) continue;
     try {
       sl_op(c, w, kDigitFp64Bits);
     } catch (const Error &e) {

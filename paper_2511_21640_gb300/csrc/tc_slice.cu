@@ -894,8 +894,8 @@ void zgemm_sliced(Exec &ex, int64_t M, int64_t N, int64_t K, int64_t batch, cplx
 // with both operands' slicing, 25 us with the larger one's digits at hand), the slicing's
 // passes over memory at 3 TB/s and the tensor-core kernel's plan; the FP64 units' is their
 // kernel's plan. Measured (GB300, M x N x K, FP64 units / digits, slicing included):
-// 256^3 110 / 150 us, 384^3 320 / 200 us, 200 x 8 x 20000 213 / 250 us,
-// 1000 x 1000 x 64 391 / 104 us, 2500 x 2500 x 40 1760 / 400 us.
+// 256^3 110 / 70 us, 384^3 321 / 82 us, 512^3 756 / 118 us, 200 x 8 x 20000 214 / 224 us,
+// 1000 x 1000 x 64 391 / 95 us.
 static bool digits_pay(int64_t M, int64_t N, int64_t K, int64_t batch, bool kept) {
   if (8.0 * (double)M * (double)N * (double)K * (double)batch < (double)(1 << 24)) return false;
   const double fp64 = zgemm_fp64_clocks(M, N, K, batch);

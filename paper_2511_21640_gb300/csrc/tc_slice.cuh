@@ -59,6 +59,10 @@ struct SlCache {
   bool no_room[SL_NOPS] = {};  // FP64 products: the operator's digits did not fit
   SlWork w;
   DBuf err;
+  int busy = 0;      // a product is being enqueued: its operator's digits stay
+  int dev = 0;
+  int64_t kept = 0;  // bytes of digits kept for FP64 products alone
+  ~SlCache();
 };
 
 // A[m][k] = op(src[m*s_m + k*s_k]); digits for about `bits` significant bits

@@ -83,7 +83,13 @@ size_t free_device_memory() {
 
 void *Exec::alloc(size_t bytes) {
   if (bytes == 0) return nullptr;
-  if (mem_limit > 0 && mem_used + (int64_t)bytes > mem_limit)
+  auto capturing = [&]() {
+    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+    return cudaStreamIsCapturing(stream, &cs) != cudaSuccess || cs != cudaStreamCaptureStatusNone;
+  };
+  auto over = [&]() { return mem_limit > 0 && mem_used + (int64_t)bytes > mem_limit; };
+  if (over() && give_back && !capturing()) give_back(give_back_of);
+  if (over())
     throw Error(ADC_ERR_OOM, "context memory limit exceeded: need " + std::to_string(bytes) +
                                  " bytes, " + std::to_string(mem_used) + " in use of " +
                                  std::to_string(mem_limit));
@@ -93,10 +99,17 @@ void *Exec::alloc(size_t bytes) {
   if (e == cudaErrorMemoryAllocation) {
     // blocks freed on other streams, or kept in sizes that do not fit, go back first
     cudaGetLastError();
-    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
-    if (cudaStreamIsCapturing(stream, &cs) == cudaSuccess && cs == cudaStreamCaptureStatusNone &&
-        cudaStreamSynchronize(stream) == cudaSuccess && cudaMemPoolTrimTo(pool, 0) == cudaSuccess)
-      e = cudaMallocFromPoolAsync(&p, bytes, pool, stream);
+    auto again = [&]() {
+      if (cudaStreamSynchronize(stream) == cudaSuccess && cudaMemPoolTrimTo(pool, 0) == cudaSuccess)
+        e = cudaMallocFromPoolAsync(&p, bytes, pool, stream);
+    };
+    if (!capturing()) {
+      again();
+      if (e == cudaErrorMemoryAllocation && give_back && give_back(give_back_of)) {
+        cudaGetLastError();
+        again();
+      }
+    }
   }
   if (e != cudaSuccess) {
     cudaGetLastError();

@@ -44,6 +44,9 @@ struct Exec {
   int64_t mem_limit = 0;  // 0 = unlimited
   int64_t mem_used = 0;
   int64_t mem_peak = 0;
+  // short of memory, alloc asks once for what is kept for speed alone (false: nothing to give)
+  bool (*give_back)(void *) = nullptr;
+  void *give_back_of = nullptr;
   // per-kernel timing with CUDA events on this stream (off unless enabled)
   bool prof = false;
   std::string tag;

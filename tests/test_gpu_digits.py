@@ -13,6 +13,7 @@ again: 2^(1.5 - bits), and a factor of two in hand. The FP64 reference
 """
 import math
 
+import numpy as np
 import pytest
 
 torch = pytest.importorskip("torch")
@@ -53,3 +54,32 @@ def test_wide_grouped_launch(gpu, which, M, N, K):
     sqrt(2 K) of the largest: 2^-14 covers both."""
     err, _ = gpu.diag_gemm(which, M, N, K, seed=21, reps=1)
     assert err < 2.0 ** -14, err
+
+
+@pytest.mark.parametrize("kind,nocc,nvir", [("EA", 12, 40), ("IP", 36, 20)])
+def test_kept_digits_go_back_when_memory_runs_short(gpu, kind, nocc, nvir):
+    """A memory limit that fits a long block of FP64 products only without the digits kept by an
+    earlier one: the block runs, and equals the unlimited context's to the rounding of either
+    route (56 bits or FP64 sums of K terms: 1e-13 of the largest output)."""
+    from synthetic import make_problem
+    p = make_problem(nocc=nocc, nvir=nvir, naux=60, seed=5)
+    rng = np.random.default_rng(6)
+
+    def context(limit):
+        return gpu.Context(p.B, p.eps_occ, p.eps_vir, kind=kind, order=3, x=0.5, mem_limit=limit)
+
+    with context(0) as c:
+        X = rng.standard_normal((1500, c.N)) + 1j * rng.standard_normal((1500, c.N))
+        held = c.memory()["in_use"]
+        c.sigma(X[:32], "fp64")
+        kept = c.memory()["in_use"] - held
+        setup_peak = c.memory()["peak"]
+        want = c.sigma(X, "fp64")
+        peak = c.memory()["peak"]
+    assert kept > 0 and peak > setup_peak
+    limit = max(peak - kept // 4, setup_peak)
+    with context(limit) as c:
+        c.sigma(X[:32], "fp64")
+        got = c.sigma(X, "fp64")
+        assert c.memory()["peak"] <= limit
+    assert np.abs(got - want).max() < 1e-13 * np.abs(want).max()
