@@ -532,7 +532,7 @@ void adjoint_ee(adc_ctx *c, const cplx *Y, const double *g_host, int64_t k, cplx
   amplitudes_and_integrals_back(c, src, gsrc, G, third, E.t2d, E.t2s, gB, geo, gev);
   double h = 0.0;
   ADC_CUDA(cudaMemcpyAsync(&h, gxp, sizeof(double), cudaMemcpyDeviceToHost, ex.stream));
-  ADC_CUDA(cudaStreamSynchronize(ex.stream));
+  ex.sync();
   *gx += h;
 }
 
@@ -794,7 +794,7 @@ void adjoint_ipea(adc_ctx *c, const cplx *Y, const double *g_host, int64_t k, cp
   amplitudes_and_integrals_back(c, src, gsrc, G, third, t2d, t2s, gB, geo, gev);
   double h = 0.0;
   ADC_CUDA(cudaMemcpyAsync(&h, gxp, sizeof(double), cudaMemcpyDeviceToHost, ex.stream));
-  ADC_CUDA(cudaStreamSynchronize(ex.stream));
+  ex.sync();
   *gx += h;
 }
 

@@ -105,16 +105,24 @@ __global__ void __launch_bounds__(256) k_herm_check(const cplx *B, int64_t Q, in
   atomic_max_nonneg(out + 1, mag);
 }
 
+// A call that fails also reports a wait that gave up in an FP64 product before the failure:
+// left recorded, it would fail the next call instead.
 int fail(adc_ctx *c, const std::exception &e, int code) {
-  if (c) c->err = e.what();
-  g_last_error = e.what();
+  std::string m = e.what();
+  if (c && c->ex.digit_err) {
+    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+    int h = 0;
+    if (cudaStreamIsCapturing(c->ex.stream, &cs) == cudaSuccess && cs == cudaStreamCaptureStatusNone &&
+        cudaStreamSynchronize(c->ex.stream) == cudaSuccess)
+      h = c->ex.take_digits();
+    if (h) {
+      code = ADC_ERR_TIMEOUT;
+      m += "; FP64 product: a tensor-core wait gave up (code " + std::to_string(h) + ")";
+    }
+  }
+  if (c) c->err = m;
+  g_last_error = m;
   return code;
-}
-
-// the stream drained, and no FP64 product's wait given up since the last check
-void sync_check(adc_ctx *c) {
-  ADC_CUDA(cudaStreamSynchronize(c->ex.stream));
-  c->ex.check_digits();
 }
 
 #define ADC_API_TRY try {
@@ -247,7 +255,7 @@ int adc_init(adc_ctx **out, const adc_c128 *B, int64_t naux, const double *eps_o
       else setup_operators(c);
     }
     c->ex.sliced_bits = 0;
-    c->ex.check_digits();
+    c->ex.sync();
     c->setup_n[0] = c->ex.n_sliced;
     c->setup_n[1] = c->ex.n_fp64;
     c->setup_flops[0] = c->ex.flops_sliced;
@@ -289,7 +297,7 @@ int adc_sigma(adc_ctx *c, const adc_c128 *X, adc_c128 *S, int64_t k, int precisi
   DevOut sout(c->ex, S, bytes);
   sigma(c, (const cplx *)xin.p, (cplx *)sout.p, k, precision);
   sout.finish(c->ex);
-  if (sout.host || xin.buf.p) sync_check(c);
+  if (sout.host || xin.buf.p) c->ex.sync();
   return ADC_OK;
   ADC_API_CATCH(c)
 }
@@ -309,7 +317,7 @@ int adc_sigma_share(adc_ctx *c, const adc_c128 *X, adc_c128 *S, int64_t k, int64
   DevOut sout(c->ex, S, (size_t)k * ls * sizeof(cplx));
   sigma_fp64_share(c, (const cplx *)xin.p, (cplx *)sout.p, k, i0, i1, with_main != 0);
   sout.finish(c->ex);
-  if (sout.host || xin.buf.p) sync_check(c);
+  if (sout.host || xin.buf.p) c->ex.sync();
   return ADC_OK;
   ADC_API_CATCH(c)
 }
@@ -319,7 +327,7 @@ int adc_diagonal(adc_ctx *c, double *diag) {
   if (!diag) return ADC_ERR_ARG;
   ADC_API_TRY
   ADC_CUDA(cudaMemcpyAsync(diag, c->diag.p, c->N * sizeof(double), cudaMemcpyDefault, c->ex.stream));
-  sync_check(c);
+  c->ex.sync();
   return ADC_OK;
   ADC_API_CATCH(c)
 }
@@ -329,7 +337,7 @@ int adc_main_block(adc_ctx *c, adc_c128 *M11) {
   if (!M11) return ADC_ERR_ARG;
   ADC_API_TRY
   ADC_CUDA(cudaMemcpyAsync(M11, c->M11.p, c->n1 * c->n1 * sizeof(cplx), cudaMemcpyDefault, c->ex.stream));
-  sync_check(c);
+  c->ex.sync();
   return ADC_OK;
   ADC_API_CATCH(c)
 }
@@ -348,7 +356,7 @@ int adc_davidson(adc_ctx *c, int nroots, double tol, int max_iter, int precision
   yout.finish(c->ex);
   ADC_CUDA(cudaMemcpyAsync(omega, om.data(), nroots * sizeof(double), cudaMemcpyDefault, c->ex.stream));
   if (err64) ADC_CUDA(cudaMemcpyAsync(err64, er.data(), nroots * sizeof(double), cudaMemcpyDefault, c->ex.stream));
-  sync_check(c);
+  c->ex.sync();
   if (rc == ADC_ERR_NOCONV) c->err = "Davidson did not converge within max_iter";
   return rc;
   ADC_API_CATCH(c)
@@ -370,7 +378,7 @@ int adc_fns_density(adc_ctx *c, adc_c128 *D, double *eta, adc_c128 *V, double et
   int64_t nk = 0;
   fns_run(c, (cplx *)dD.p, (double *)dE.p, (cplx *)dV.p, eta_crit, &nk, (cplx *)dU.p, (double *)dN.p);
   dD.finish(c->ex); dE.finish(c->ex); dV.finish(c->ex); dU.finish(c->ex); dN.finish(c->ex);
-  sync_check(c);
+  c->ex.sync();
   *n_keep = nk;
   return ADC_OK;
   ADC_API_CATCH(c)
@@ -385,7 +393,7 @@ int adc_fns_transform(adc_ctx *c, const adc_c128 *U, int64_t ldu, int64_t n_keep
   DevOut bout(c->ex, Bout, (size_t)c->Q * n2 * n2 * sizeof(cplx));
   fns_transform(c, (const cplx *)uin.p, ldu, n_keep, (cplx *)bout.p);
   bout.finish(c->ex);
-  sync_check(c);
+  c->ex.sync();
   return ADC_OK;
   ADC_API_CATCH(c)
 }
@@ -400,7 +408,7 @@ int adc_state_density(adc_ctx *c, const adc_c128 *y, adc_c128 *D) {
   DevOut dD(c->ex, D, (size_t)v * v * sizeof(cplx));
   state_density(c, (const cplx *)yin.p, (cplx *)dD.p);
   dD.finish(c->ex);
-  sync_check(c);
+  c->ex.sync();
   return ADC_OK;
   ADC_API_CATCH(c)
 }
@@ -424,7 +432,7 @@ int adc_ssfns_density(adc_ctx *c, const adc_c128 *y, double eta_crit, adc_c128 *
   int64_t nk = 0;
   fns_run(c, (cplx *)dD.p, (double *)dE.p, nullptr, eta_crit, &nk, (cplx *)dU.p, (double *)dN.p, Dst.c());
   dD.finish(c->ex); dE.finish(c->ex); dU.finish(c->ex); dN.finish(c->ex);
-  sync_check(c);
+  c->ex.sync();
   *n_keep = nk;
   return ADC_OK;
   ADC_API_CATCH(c)
@@ -440,7 +448,7 @@ int adc_fns_vector(adc_ctx *c, const adc_c128 *y, const adc_c128 *U, int64_t ldu
   DevOut gout(c->ex, g, (size_t)fns_dim(c->kind, c->o, n_keep) * sizeof(cplx));
   to_fns_basis(c, (const cplx *)yin.p, (const cplx *)uin.p, ldu, n_keep, (cplx *)gout.p);
   gout.finish(c->ex);
-  sync_check(c);
+  c->ex.sync();
   return ADC_OK;
   ADC_API_CATCH(c)
 }
@@ -457,7 +465,7 @@ int adc_davidson_follow(adc_ctx *c, const adc_c128 *guess, double tol, int max_i
   int rc = davidson_run(c, 1, tol, max_iter, precision, (const cplx *)gin.p, 1, omega, (cplx *)yout.p, &e, st,
                         true);
   yout.finish(c->ex);
-  sync_check(c);
+  c->ex.sync();
   if (err64) *err64 = e;
   if (rc == ADC_ERR_NOCONV) {
     c->err = "davidson: not converged within max_iter";
@@ -497,7 +505,7 @@ int adc_transition_density(adc_ctx *c, const adc_c128 *Y, int64_t k, adc_c128 *r
   DevOut rout(c->ex, rho, (size_t)k * c->nmo * c->nmo * sizeof(cplx));
   transition_density(c, (const cplx *)yin.p, k, (cplx *)rout.p);
   rout.finish(c->ex);
-  sync_check(c);
+  c->ex.sync();
   return ADC_OK;
   ADC_API_CATCH(c)
 }
@@ -511,7 +519,7 @@ int adc_state_pair_density(adc_ctx *c, const adc_c128 *YK, const adc_c128 *YL, i
   DevOut rout(c->ex, rho, (size_t)k * c->nmo * c->nmo * sizeof(cplx));
   state_pair_density(c, (const cplx *)kin.p, (const cplx *)lin.p, k, (cplx *)rout.p);
   rout.finish(c->ex);
-  sync_check(c);
+  c->ex.sync();
   return ADC_OK;
   ADC_API_CATCH(c)
 }
@@ -525,7 +533,7 @@ int adc_spectroscopic_amplitudes(adc_ctx *c, const adc_c128 *Y, int64_t k, adc_c
   DevOut xout(c->ex, x, (size_t)k * c->nmo * sizeof(cplx));
   spectroscopic_amplitudes(c, (const cplx *)yin.p, k, (cplx *)xout.p);
   xout.finish(c->ex);
-  sync_check(c);
+  c->ex.sync();
   return ADC_OK;
   ADC_API_CATCH(c)
 }
@@ -538,7 +546,7 @@ int adc_excited_density(adc_ctx *c, const adc_c128 *Y, int64_t k, adc_c128 *rho)
   DevOut rout(c->ex, rho, (size_t)k * c->nmo * c->nmo * sizeof(cplx));
   excited_density(c, (const cplx *)yin.p, k, (cplx *)rout.p);
   rout.finish(c->ex);
-  sync_check(c);
+  c->ex.sync();
   return ADC_OK;
   ADC_API_CATCH(c)
 }
@@ -621,7 +629,7 @@ int adc_sigma_adjoint(adc_ctx *c, const adc_c128 *Y, const double *gomega, int64
   gbo.finish(c->ex);
   geo.finish(c->ex);
   gev.finish(c->ex);
-  sync_check(c);
+  c->ex.sync();
   *gx = gxh;
   return ADC_OK;
   ADC_API_CATCH(c)

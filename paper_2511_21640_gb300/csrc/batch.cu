@@ -307,7 +307,7 @@ struct BatchCoord {
 };
 
 void batch_submit(adc_ctx *c, const cplx *X, cplx *S, int64_t k) {
-  ADC_CUDA(cudaStreamSynchronize(c->ex.stream));
+  c->ex.sync();
   BatchReq r;
   r.slot = c->batch_slot;
   r.X = X;
@@ -455,8 +455,13 @@ int adc_batch_sigma(adc_batch *b, const adc_c128 *const *X, adc_c128 *const *S, 
     if (precision == ADC_PREC_FP64) {
       for (BatchReq *r : rp) {
         adc_ctx *c = co.ctx[r->slot];
-        sigma(c, r->X, r->S, r->k, ADC_PREC_FP64);
-        ADC_CUDA(cudaStreamSynchronize(c->ex.stream));
+        try {
+          sigma(c, r->X, r->S, r->k, ADC_PREC_FP64);
+          c->ex.sync();
+        } catch (...) {  // nothing of this product is left for the context's next call to report
+          if (cudaStreamSynchronize(c->ex.stream) == cudaSuccess) c->ex.take_digits();
+          throw;
+        }
       }
       return ADC_OK;
     }
@@ -512,6 +517,9 @@ int adc_batch_davidson(adc_batch *b, int nroots, double tol, int max_iter, int p
         rc = ADC_ERR_CUDA;
         msgs[i] = e.what();
       }
+      // (nothing of this solve is left for the context's next call to report)
+      if (rc != ADC_OK && cudaStreamSynchronize(c->ex.stream) == cudaSuccess && c->ex.take_digits())
+        rc = ADC_ERR_TIMEOUT;
       status[i] = rc;
       co.leave();
     });

@@ -261,7 +261,7 @@ struct Davidson {
     if (c->batch) batch_leave(c);
     try {
       sigma(c, X, S, k, prec);
-      ADC_CUDA(cudaStreamSynchronize(ex.stream));
+      ex.sync();
     } catch (...) {
       if (c->batch) batch_rejoin(c);
       throw;
@@ -315,7 +315,7 @@ struct Davidson {
     k_row_norms_fin<<<(k + 127) / 128, 128, 0, ex.stream>>>(part.d(), nseg, k, nrm.d());
     ADC_CHECK_LAUNCH();
     ADC_CUDA(cudaMemcpyAsync(h.data(), nrm.d(), k * sizeof(double), cudaMemcpyDeviceToHost, ex.stream));
-    ADC_CUDA(cudaStreamSynchronize(ex.stream));
+    ex.sync();
     return h;
   }
 
@@ -351,7 +351,7 @@ struct Davidson {
     jacobi_eigh(ex, Gs.c(), nt, nt, w2.d(), Zs.c(), nt, (int *)info.p);
     std::vector<double> lam(nt);
     ADC_CUDA(cudaMemcpyAsync(lam.data(), w2.d(), nt * sizeof(double), cudaMemcpyDeviceToHost, ex.stream));
-    ADC_CUDA(cudaStreamSynchronize(ex.stream));
+    ex.sync();
     const double thr = std::max(1e-28, (1e-8 * nmax) * (1e-8 * nmax));
     std::vector<int> keep;
     for (int j = nt - 1; j >= 0; --j)
@@ -385,7 +385,7 @@ struct Davidson {
     ADC_CUDA(cudaMemcpyAsync(s.data(), ovl.p, m * sizeof(cplx), cudaMemcpyDeviceToHost, ex.stream));
     ADC_CUDA(cudaMemcpy2DAsync(cv.data(), m * sizeof(cplx), Cv.p, mmax * sizeof(cplx), m * sizeof(cplx), m,
                                cudaMemcpyDeviceToHost, ex.stream));
-    ADC_CUDA(cudaStreamSynchronize(ex.stream));
+    ex.sync();
     int best = 0;
     double bo = -1.0;
     for (int r = 0; r < m; ++r) {
@@ -419,7 +419,7 @@ struct Davidson {
     ADC_CHECK_LAUNCH();
     std::vector<double> wh(m);
     ADC_CUDA(cudaMemcpyAsync(wh.data(), w.d(), m * sizeof(double), cudaMemcpyDeviceToHost, ex.stream));
-    ADC_CUDA(cudaStreamSynchronize(ex.stream));
+    ex.sync();
     return wh;
   }
 
@@ -461,7 +461,7 @@ int davidson_run(adc_ctx *c, int nroots, double tol, int max_iter, int precision
       ee_prepare(c, precision == ADC_PREC_FP64 ? 0 : (mixed == ADC_PREC_BF16X6 ? 3 : 2),
                  c->opts.refine == ADC_PREC_SLICED);
     if (precision == ADC_PREC_FP64 || c->opts.refine == ADC_PREC_FP64) fp64_ops_prepare(c, kb);
-    ADC_CUDA(cudaStreamSynchronize(c->ex.stream));
+    c->ex.sync();
     double avail = (double)free_device_memory();
     if (c->ex.mem_limit > 0) avail = std::min(avail, (double)(c->ex.mem_limit - c->ex.mem_used));
     const double vec = (double)N * sizeof(cplx);
@@ -507,7 +507,7 @@ int davidson_run(adc_ctx *c, int nroots, double tol, int max_iter, int precision
     m0 = std::max(m0, std::min<int>((int)N, nroots));
     std::vector<double> dh(N);
     ADC_CUDA(cudaMemcpyAsync(dh.data(), c->diag.d(), N * sizeof(double), cudaMemcpyDeviceToHost, ex.stream));
-    ADC_CUDA(cudaStreamSynchronize(ex.stream));
+    ex.sync();
     std::vector<int64_t> idx(N);
     std::iota(idx.begin(), idx.end(), 0);
     std::partial_sort(idx.begin(), idx.begin() + m0, idx.end(),
@@ -516,7 +516,7 @@ int davidson_run(adc_ctx *c, int nroots, double tol, int max_iter, int precision
     ADC_CUDA(cudaMemcpyAsync(ib.p, idx.data(), m0 * sizeof(int64_t), cudaMemcpyHostToDevice, ex.stream));
     k_unit_vectors<<<m0, 256, 0, ex.stream>>>(d.V.c(), N, (const int64_t *)ib.p, m0);
     ADC_CHECK_LAUNCH();
-    ADC_CUDA(cudaStreamSynchronize(ex.stream));
+    ex.sync();
   }
   if (guess && nguess > 0) {
     // guesses go through the orthonormalisation into V
@@ -647,7 +647,7 @@ int davidson_run(adc_ctx *c, int nroots, double tol, int max_iter, int precision
     wh = d.ritz(nroots);
     rn = d.row_norms(d.R.c(), nroots);
   }
-  ADC_CUDA(cudaStreamSynchronize(ex.stream));
+  ex.sync();
   for (int r = 0; r < nroots; ++r) {
     omega[r] = wh[r];
     if (err64) err64[r] = rn[r];
@@ -655,7 +655,7 @@ int davidson_run(adc_ctx *c, int nroots, double tol, int max_iter, int precision
   if (Yout)
     ADC_CUDA(cudaMemcpyAsync(Yout, d.Y.c(), (int64_t)nroots * N * sizeof(cplx), cudaMemcpyDeviceToDevice,
                              ex.stream));
-  ADC_CUDA(cudaStreamSynchronize(ex.stream));
+  ex.sync();
   d.st.time_total_s = total.s();
   d.st.time_sigma_s = d.tsig;
   d.st.max_residual = *std::max_element(rn.begin(), rn.end());

@@ -381,11 +381,11 @@ void setup_ee(adc_ctx *c) {
     std::vector<double> eo(o), ev(v), d(n1);
     ADC_CUDA(cudaMemcpyAsync(eo.data(), c->eo.p, o * 8, cudaMemcpyDeviceToHost, ex.stream));
     ADC_CUDA(cudaMemcpyAsync(ev.data(), c->ev.p, v * 8, cudaMemcpyDeviceToHost, ex.stream));
-    ADC_CUDA(cudaStreamSynchronize(ex.stream));
+    ex.sync();
     for (int64_t i = 0; i < o; ++i)
       for (int64_t a = 0; a < v; ++a) d[i * v + a] = ev[a] - eo[i];
     ADC_CUDA(cudaMemcpyAsync(E.dS.p, d.data(), n1 * 8, cudaMemcpyHostToDevice, ex.stream));
-    ADC_CUDA(cudaStreamSynchronize(ex.stream));
+    ex.sync();
   }
   add_diag(ex, E.MSS.c(), E.dS.d(), n1, 1.0);
   zaxpby(ex, n1 * n1, C1(), K1.c(), C1(), E.MSS.c());
@@ -427,7 +427,7 @@ void setup_ee(adc_ctx *c) {
                                                         c->diag.d(), c->d2.d());
     ADC_CHECK_LAUNCH();
   }
-  ADC_CUDA(cudaStreamSynchronize(ex.stream));
+  ex.sync();
   // at sizes where the four-virtual terms are chunked, the dense integral
   // blocks of the tables are dropped (they are rebuilt on demand)
   if (chunked) E.eri.clear();

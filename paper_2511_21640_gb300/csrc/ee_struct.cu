@@ -629,13 +629,7 @@ void sigma_ee_split(adc_ctx *c, const cplx *X, cplx *S, int64_t k, int nseg, int
     throw;
   }
   ex.sliced_bits = old_bits;
-  int h = 0;
-  ADC_CUDA(cudaMemcpyAsync(&h, E.tcerr.p, sizeof(int), cudaMemcpyDeviceToHost, ex.stream));
-  ADC_CUDA(cudaStreamSynchronize(ex.stream));
-  if (h != 0) {
-    fill_zero(ex, E.tcerr.p, sizeof(int));
-    throw Error(ADC_ERR_TIMEOUT, "tensor-core GEMM wait gave up (code " + std::to_string(h) + ")");
-  }
+  tc_sync(ex, (int *)E.tcerr.p);
 }
 
 // the operands of the EE products a solve will use, built ahead of its subspace

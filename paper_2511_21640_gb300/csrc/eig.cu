@@ -820,7 +820,7 @@ void eigh_refined(Exec &ex, const cplx *A, int n, int lda, double *w, cplx *V, i
       ADC_CHECK_LAUNCH();
       double st[3];
       ADC_CUDA(cudaMemcpyAsync(st, sc.d() + 1, sizeof(st), cudaMemcpyDeviceToHost, ex.stream));
-      ADC_CUDA(cudaStreamSynchronize(ex.stream));
+      ex.sync();
       last_steps_ = it + 1;
       if (st[0] <= 1e-8 && st[1] == 0.0 && st[2] <= OA_ORTH) { ok = true; break; }
     }

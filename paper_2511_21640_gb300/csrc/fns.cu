@@ -41,7 +41,7 @@ void fns_run(adc_ctx *c, cplx *D, double *eta, cplx *Vout, double eta_crit, int6
   ADC_CHECK_LAUNCH();
   std::vector<double> wh(v);
   ADC_CUDA(cudaMemcpyAsync(wh.data(), wd.d(), v * sizeof(double), cudaMemcpyDeviceToHost, ex.stream));
-  ADC_CUDA(cudaStreamSynchronize(ex.stream));
+  ex.sync();
   int64_t nk = 0;
   while (nk < v && wh[nk] >= eta_crit) ++nk;
   *n_keep = nk;
@@ -67,7 +67,7 @@ void fns_run(adc_ctx *c, cplx *D, double *eta, cplx *Vout, double eta_crit, int6
       zgemm(ex, v, nk, nk, 1, C1(), Vd.c(), 0, v, 1, false, Z.c(), 0, nk, 1, false, C0(), U, 0, v, 1);
     }
   }
-  ADC_CUDA(cudaStreamSynchronize(ex.stream));
+  ex.sync();
 }
 
 // B' in the truncated basis: oo copied, ov = B_ov U, vo = U^H B_vo, vv = U^H B_vv U
@@ -89,7 +89,7 @@ void fns_transform(adc_ctx *c, const cplx *U, int64_t ldu, int64_t nk, cplx *Bou
   DBuf T = cbuf(ex, Q * v * nk);
   zgemm(ex, v, nk, v, Q, C1(), B + o * nmo + o, sQ, nmo, 1, false, U, 0, ldu, 1, false, C0(), T.c(), v * nk, nk, 1);
   zgemm(ex, nk, nk, v, Q, C1(), U, 0, 1, ldu, true, T.c(), v * nk, nk, 1, false, C0(), Bout + o * n2 + o, sQo, n2, 1);
-  ADC_CUDA(cudaStreamSynchronize(ex.stream));
+  ex.sync();
 }
 
 }  // namespace adc

@@ -116,7 +116,7 @@ void transition_density(adc_ctx *c, const cplx *Y, int64_t k, cplx *rho) {
     k_put_block<<<grid1d(v * v, 256), 256, 0, ex.stream>>>(Bvv.c(), v, v, R, nmo, o, o);
     ADC_CHECK_LAUNCH();
   }
-  ADC_CUDA(cudaStreamSynchronize(ex.stream));
+  ex.sync();
 }
 
 namespace {
@@ -234,7 +234,7 @@ void state_pair_density(adc_ctx *c, const cplx *YK, const cplx *YL, int64_t k, c
     k_add_block<<<grid1d(v * o, 256), 256, 0, ex.stream>>>(Bvo.c(), v, o, R, nmo, o, 0);
     ADC_CHECK_LAUNCH();
   }
-  ADC_CUDA(cudaStreamSynchronize(ex.stream));
+  ex.sync();
 }
 
 void excited_density(adc_ctx *c, const cplx *Y, int64_t k, cplx *rho) { state_pair_density(c, Y, Y, k, rho); }
@@ -272,7 +272,7 @@ void spectroscopic_amplitudes(adc_ctx *c, const cplx *Y, int64_t k, cplx *x) {
     einsum(ex, CR(-1.0), y1c, "za", s2, "ka", C0(), xo, "zk");
     einsum(ex, CR(0.5), Y2c, "zjab", t1, "jkab", C1(), xo, "zk");
   }
-  ADC_CUDA(cudaStreamSynchronize(ex.stream));
+  ex.sync();
 }
 
 }  // namespace adc

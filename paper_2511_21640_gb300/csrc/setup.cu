@@ -498,7 +498,7 @@ void setup_operators(adc_ctx *c) {
                                                           c->diag.d(), c->d2.d());
     ADC_CHECK_LAUNCH();
   }
-  ADC_CUDA(cudaStreamSynchronize(ex.stream));
+  ex.sync();
 }
 
 }  // namespace adc

@@ -135,13 +135,7 @@ static void sigma_split_grouped(adc_ctx *c, const cplx *X, cplx *S, int64_t k) {
     else
       pair_pack(ex, T, o * v * o, 0, 1, v * o, o, 1.0, k, 1, o, v, S + n1, N, 0, CR(x), C1());
   }
-  int h = 0;
-  ADC_CUDA(cudaMemcpyAsync(&h, err, sizeof(int), cudaMemcpyDeviceToHost, ex.stream));
-  ADC_CUDA(cudaStreamSynchronize(ex.stream));
-  if (h != 0) {
-    fill_zero(ex, err, sizeof(int));
-    throw Error(ADC_ERR_TIMEOUT, "tensor-core GEMM wait gave up (code " + std::to_string(h) + ")");
-  }
+  tc_sync(ex, err);
 }
 
 void sigma_split(adc_ctx *c, const cplx *X, cplx *S, int64_t k, int nseg) {
@@ -200,13 +194,7 @@ void sigma_split(adc_ctx *c, const cplx *X, cplx *S, int64_t k, int nseg) {
       pair_pack(ex, T, o * v * o, 0, 1, v * o, o, 1.0, k, 1, o, v, S + n1, N, 0, CR(x), C1());
     }
   }
-  int h = 0;
-  ADC_CUDA(cudaMemcpyAsync(&h, err, sizeof(int), cudaMemcpyDeviceToHost, ex.stream));
-  ADC_CUDA(cudaStreamSynchronize(ex.stream));
-  if (h != 0) {
-    fill_zero(ex, err, sizeof(int));
-    throw Error(ADC_ERR_TIMEOUT, "tensor-core GEMM wait gave up (code " + std::to_string(h) + ")");
-  }
+  tc_sync(ex, err);
 }
 
 // ---- products from digits: the same contractions as sliced tensor-core products.
@@ -326,13 +314,7 @@ void sigma_sliced(adc_ctx *c, const cplx *X, cplx *S, int64_t k, int bits) {
       pair_pack(ex, T, o * v * o, 0, 1, v * o, o, 1.0, k, 1, o, v, S + n1, N, 0, CR(x), C1());
     }
   }
-  int h = 0;
-  ADC_CUDA(cudaMemcpyAsync(&h, err, sizeof(int), cudaMemcpyDeviceToHost, ex.stream));
-  ADC_CUDA(cudaStreamSynchronize(ex.stream));
-  if (h != 0) {
-    fill_zero(ex, err, sizeof(int));
-    throw Error(ADC_ERR_TIMEOUT, "tensor-core GEMM wait gave up (code " + std::to_string(h) + ")");
-  }
+  tc_sync(ex, err);
 }
 
 // whether the FP64 digits of an operator are kept, or may be: within a quarter of the

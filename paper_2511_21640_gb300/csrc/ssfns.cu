@@ -93,7 +93,7 @@ void to_fns_basis(adc_ctx *c, const cplx *y, const cplx *U, int64_t ldu, int64_t
       pair_pack(ex, P1.c(), 0, 0, o * pnk, pnk, 1, 0.0, 1, 1, o, pnk, g + o * nk, 0, 0, C1(), C0());
     }
   }
-  ADC_CUDA(cudaStreamSynchronize(ex.stream));
+  ex.sync();
 }
 
 namespace {

@@ -1125,6 +1125,16 @@ void tc_gemm_grouped(Exec &ex, const std::vector<TcJobDesc> &in, TcGroup &grp, i
   ex.prof_end(pr);
 }
 
+void tc_sync(Exec &ex, int *err) {
+  int h = 0;
+  ADC_CUDA(cudaMemcpyAsync(&h, err, sizeof(int), cudaMemcpyDeviceToHost, ex.stream));
+  ADC_CUDA(cudaStreamSynchronize(ex.stream));
+  if (h == 0) return ex.check_digits();
+  ex.take_digits();  // one report for both
+  fill_zero(ex, err, sizeof(int));
+  throw Error(ADC_ERR_TIMEOUT, "tensor-core GEMM wait gave up (code " + std::to_string(h) + ")");
+}
+
 void tc_set_wait_ns(uint64_t ns) {
   const unsigned long long v = ns ? (unsigned long long)ns : (unsigned long long)WAIT_NS;
   ADC_CUDA(cudaMemcpyToSymbol(g_wait_ns, &v, sizeof(v)));

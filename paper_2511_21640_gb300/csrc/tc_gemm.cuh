@@ -106,6 +106,9 @@ struct TcGroup {
 // enqueue all jobs as one persistent launch (plus split-K reductions). With
 // may_tune, jobs with bn == 0 get the autotuned tile width (timing runs need a
 // stream that is not being captured); otherwise a size rule picks it.
+// waits for the stream; a wait that gave up (recorded in *err, device, or by an FP64 product
+// from digits) is cleared and thrown as ADC_ERR_TIMEOUT
+void tc_sync(Exec &ex, int *err);
 // (timing: one of the autotuner's own launches)
 void tc_gemm_grouped(Exec &ex, const std::vector<TcJobDesc> &jobs, TcGroup &grp, int *err, bool may_tune,
                      bool timing = false);

@@ -883,10 +883,7 @@ void zgemm_sliced(Exec &ex, int64_t M, int64_t N, int64_t K, int64_t batch, cplx
   bool begun = false;
   digit_zgemm(ex, M, N, K, batch, alpha, A, sAb, sAm, sAk, conjA, B, sBb, sBk, sBn, conjB, beta, C, sCb, sCm, sCn,
               ex.sliced_bits, (int *)err.p, begun);
-  int h = 0;
-  ADC_CUDA(cudaMemcpyAsync(&h, err.p, sizeof(int), cudaMemcpyDeviceToHost, ex.stream));
-  ADC_CUDA(cudaStreamSynchronize(ex.stream));
-  ADC_REQUIRE(h == 0, ADC_ERR_TIMEOUT, "sliced GEMM: a tensor-core wait gave up (code " + std::to_string(h) + ")");
+  tc_sync(ex, (int *)err.p);
 }
 
 // FP64 products that leave the FP64 units (1.26 TFLOP/s) for the digits: those whose

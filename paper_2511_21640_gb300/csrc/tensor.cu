@@ -132,10 +132,20 @@ void Exec::release(void *p, size_t bytes) {
 
 long long g_launches = 0;
 
-void Exec::check_digits() {
-  if (!digit_err) return;
+int Exec::take_digits() {
+  if (!digit_err) return 0;
   const int h = *(volatile int *)digit_err;
   *digit_err = 0;
+  return h;
+}
+
+void Exec::sync() {
+  ADC_CUDA(cudaStreamSynchronize(stream));
+  check_digits();
+}
+
+void Exec::check_digits() {
+  const int h = take_digits();
   if (h) throw Error(ADC_ERR_TIMEOUT, "FP64 product: a tensor-core wait gave up (code " + std::to_string(h) + ")");
 }
 

@@ -25,8 +25,8 @@ struct Exec {
   // FP64 zgemm on the tensor cores (tc_slice.cu): 0 never (the FP64 units alone),
   // 1 products large enough to pay, 2 every product (a diagnostic's choice)
   int digits = 0;
-  // pinned word in which such a product records a wait that gave up; the host
-  // looks at it after the next synchronisation (check_digits)
+  // pinned word in which such a product records a wait that gave up (the output then holds
+  // NaN). Whoever waits for the stream looks at it: sync() throws ADC_ERR_TIMEOUT
   int *digit_err = nullptr;
   // the FP64 kernel's inner splits: tile counters (zero between launches) and a small
   // buffer of partial products. Held by a context for its life, on its one stream; null
@@ -35,7 +35,9 @@ struct Exec {
     void *p = nullptr;
     size_t bytes = 0;
   } zcount, zpart;
-  void check_digits();
+  int take_digits();    // the recorded code (0: none), cleared; the stream has been waited for
+  void check_digits();  // throws when one was recorded
+  void sync();          // the stream waited for, and check_digits
   // complex GEMMs issued through zgemm since the counters were cleared: how
   // many took the sliced tensor-core route and how many the FP64 kernel, with
   // their algorithmic flops (host-side counts)
