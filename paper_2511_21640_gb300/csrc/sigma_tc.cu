@@ -262,13 +262,32 @@ void sigma_sliced(adc_ctx *c, const cplx *X, cplx *S, int64_t k, int bits) {
   ADC_REQUIRE(c->kind != ADC_EE, ADC_ERR_ARG, "sigma_sliced: IP and EA (EE goes through sigma_ee_split)");
   Exec &ex = c->ex;
   SlCache &sl = sl_cache(c);
-  const SlUse use(sl);
   if (!sl.err.p) {
     sl.err = DBuf(ex, sizeof(int));
     fill_zero(ex, sl.err.p, sizeof(int));
   }
   int *err = (int *)sl.err.p;
-  auto op = [&](int which) -> const SlMat & { return sl_op(c, which, kSlicedBits); };
+  // One term: out = alpha op B^T + beta out, B packed by pack(op). Short of memory it gives back
+  // the digits that FP64 products keep (this product needs three quarters of them) and starts
+  // over: every allocation precedes the launch that writes out
+  auto term = [&](int which, int64_t M, int64_t Nc, auto &&pack, cplx alpha, cplx beta, cplx *out, int64_t s_m,
+                  int64_t s_nh, int64_t s_nl, int64_t n_in) {
+    for (bool again = false;; again = true) {
+      try {
+        const SlUse use(sl);
+        const SlMat &A = sl_op(c, which, kSlicedBits);
+        pack(A);
+        sl_gemm(ex, A, sl.Bx, M, Nc, alpha, beta, out, s_m, s_nh, s_nl, n_in, err, sl.w);
+        return;
+      } catch (const Error &e) {
+        if (again || e.code != ADC_ERR_OOM || !sl_give_back(c)) throw;
+      }
+    }
+  };
+  auto strided = [&](const cplx *src, int64_t Nc, int64_t K, int64_t s_nh, int64_t s_nl, int64_t n_in, int64_t s_k) {
+    return [=, &ex, &sl](const SlMat &A) { sl_pack_B(ex, sl.Bx, src, Nc, K, s_nh, s_nl, n_in, s_k, false, A, bits); };
+  };
+  auto ring = [&](const SlMat &A) { sl_pack_B_ring(ex, sl.Bx, c, X, k, A, bits); };
   const int64_t o = c->o, v = c->v, n1 = c->n1, n2 = c->n2, N = c->N;
   const bool sat = (c->order == 3 && c->x != 0.0);
   const double x = sat ? c->x : 0.0;
@@ -277,11 +296,8 @@ void sigma_sliced(adc_ctx *c, const cplx *X, cplx *S, int64_t k, int bits) {
   zgemm(ex, k, n1, n1, 1, C1(), X, 0, N, 1, false, c->M11.c(), 0, 1, n1, false, C0(), S, 0, N, 1);
   // S1 += Cpl X2, S2 = Cpl^H X1
   ex.tag = "coupling";
-  const SlMat &cpl = op(SL_CPL), &cplt = op(SL_CPLT);
-  sl_pack_B(ex, sl.Bx, X + n1, k, n2, N, 0, 1, 1, false, cpl, bits);
-  sl_gemm(ex, cpl, sl.Bx, n1, k, C1(), C1(), S, 1, N, 0, 1, err, sl.w);
-  sl_pack_B(ex, sl.Bx, X, k, n1, N, 0, 1, 1, false, cplt, bits);
-  sl_gemm(ex, cplt, sl.Bx, n2, k, C1(), C0(), S + n1, 1, N, 0, 1, err, sl.w);
+  term(SL_CPL, n1, k, strided(X + n1, k, n2, N, 0, 1, 1), C1(), C1(), S, 1, N, 0, 1);
+  term(SL_CPLT, n2, k, strided(X, k, n1, N, 0, 1, 1), C1(), C0(), S + n1, 1, N, 0, 1);
   diag_mul_add(ex, k, n2, c->d2.d(), X + n1, N, S + n1, N, 1.0);
   if (sat) {
     if (c->kind == ADC_EA) {
@@ -290,27 +306,19 @@ void sigma_sliced(adc_ctx *c, const cplx *X, cplx *S, int64_t k, int bits) {
       if (c->direct_ladder) {
         ladder_direct(c, X + n1, N, o, S + n1, N, k, x, ADC_LADDER_SLICED, err);
       } else {
-        const SlMat &g = op(SL_GLAD);
-        sl_pack_B(ex, sl.Bx, X + n1, k * o, pv, N, pv, o, 1, false, g, bits);
-        sl_gemm(ex, g, sl.Bx, pv, k * o, CR(x), C1(), S + n1, 1, N, pv, o, err, sl.w);
+        term(SL_GLAD, pv, k * o, strided(X + n1, k * o, pv, N, pv, o, 1), CR(x), C1(), S + n1, 1, N, pv, o);
       }
       ex.tag = "ring";
       cplx *T = scratch(c, k * o * v * v);
-      const SlMat &w = op(SL_W);
-      sl_pack_B_ring(ex, sl.Bx, c, X, k, w, bits);
-      sl_gemm(ex, w, sl.Bx, o * v, k * v, C1(), C0(), T, v, o * v * v, 1, v, err, sl.w);
+      term(SL_W, o * v, k * v, ring, C1(), C0(), T, v, o * v * v, 1, v);
       pair_pack(ex, T, o * v * v, v * v, v, 1, 0, 1.0, k, o, v, 1, S + n1, N, pv, CR(-x), C1());
     } else {
       const int64_t po = npairs(o);
       ex.tag = "ladder";
-      const SlMat &g = op(SL_GLAD);
-      sl_pack_B(ex, sl.Bx, X + n1, k * v, po, N, 1, v, v, false, g, bits);
-      sl_gemm(ex, g, sl.Bx, po, k * v, CR(x), C1(), S + n1, v, N, 1, v, err, sl.w);
+      term(SL_GLAD, po, k * v, strided(X + n1, k * v, po, N, 1, v, v), CR(x), C1(), S + n1, v, N, 1, v);
       ex.tag = "ring";
       cplx *T = scratch(c, k * o * v * o);
-      const SlMat &w = op(SL_W);
-      sl_pack_B_ring(ex, sl.Bx, c, X, k, w, bits);
-      sl_gemm(ex, w, sl.Bx, o * v, k * o, CR(-1.0), C0(), T, o, o * v * o, 1, o, err, sl.w);
+      term(SL_W, o * v, k * o, ring, CR(-1.0), C0(), T, o, o * v * o, 1, o);
       pair_pack(ex, T, o * v * o, 0, 1, v * o, o, 1.0, k, 1, o, v, S + n1, N, 0, CR(x), C1());
     }
   }

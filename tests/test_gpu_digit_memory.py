@@ -1,0 +1,51 @@
+"""Device memory of the digit products: what an earlier FP64 product keeps for speed never makes a
+later call fail that fits without it, and what a limit leaves no room for runs another way."""
+import numpy as np
+import pytest
+
+from synthetic import make_problem
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def gpu():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from conftest import build_library
+    build_library()
+    import paper_2511_21640_gb300 as m
+    return m
+
+
+def _vectors(n, k, seed):
+    rng = np.random.default_rng(seed)
+    return rng.standard_normal((k, n)) + 1j * rng.standard_normal((k, n))
+
+
+@pytest.mark.parametrize("precision", ["sliced", "sliced24"])
+@pytest.mark.parametrize("kind,nocc,nvir", [("EA", 12, 40), ("IP", 36, 20)])
+def test_sliced_product_after_kept_fp64_digits(gpu, kind, nocc, nvir, precision):
+    """A limit that a block of sliced products just fits in: it also fits after an FP64 product has
+    kept its operators' longer digits. Both results carry the product's 40 (24) bits, so they agree
+    to 1e-11 (1e-6) of the largest output."""
+    p = make_problem(nocc=nocc, nvir=nvir, naux=60, seed=5)
+
+    def context(limit):
+        return gpu.Context(p.B, p.eps_occ, p.eps_vir, kind=kind, order=3, x=0.5, mem_limit=limit)
+
+    with context(0) as c:
+        setup_peak = c.memory()["peak"]
+        X = _vectors(c.N, 1500, 6)
+        want = c.sigma(X, precision)
+        peak = c.memory()["peak"]
+    assert peak > setup_peak
+    limit = peak + (1 << 20)
+    with context(limit) as c:
+        held = c.memory()["in_use"]
+        c.sigma(X[:32], "fp64")
+        assert c.memory()["in_use"] > held + (8 << 20)
+        got = c.sigma(X, precision)
+        assert c.memory()["peak"] <= limit
+    assert np.abs(got - want).max() < (1e-11 if precision == "sliced" else 1e-6) * np.abs(want).max()
