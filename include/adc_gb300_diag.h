@@ -82,6 +82,17 @@ int adc_diag_set_setup_chunk(int64_t elems);
  * eighth of the free memory (1 to 16 GiB). Process-wide. Returns ADC_OK. */
 int adc_diag_set_sliced_cap(int64_t bytes);
 
+/* Test hook: device allocations of the library (every context of the process
+ * together) that would take their total past `bytes` fail like the driver's
+ * own out-of-memory; <= 0 takes the limit away. Returns ADC_OK. */
+int adc_diag_set_alloc_limit(int64_t bytes);
+
+/* Bytes of device memory: the total of the library's allocations in this
+ * process, the digits this context keeps for FP64 products, and those kept by
+ * every context on its device. Host-side counters only. ADC_ERR_STATE for a
+ * NULL context, ADC_ERR_ARG for NULL outputs. */
+int adc_diag_memory(const adc_ctx_opaque *ctx, int64_t *total, int64_t *own_digits, int64_t *device_digits);
+
 /* 1 when the context forms its EA ladder integrals inside every product
  * (opts.ladder), else 0. ADC_ERR_STATE for a NULL context. */
 int adc_ladder_mode(const adc_ctx_opaque *ctx, int *direct);

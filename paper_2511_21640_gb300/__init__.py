@@ -123,6 +123,8 @@ def _load():
         "adc_diag_set_wait_ns": (I, [ctypes.c_uint64]),
         "adc_diag_set_setup_chunk": (I, [ctypes.c_int64]),
         "adc_diag_set_sliced_cap": (I, [ctypes.c_int64]),
+        "adc_diag_set_alloc_limit": (I, [ctypes.c_int64]),
+        "adc_diag_memory": (I, [P, P, P, P]),
         "adc_diag_eigh": (I, [I, P, I, P, P, ctypes.POINTER(D), ctypes.POINTER(I)]),
         "adc_sigma_adjoint": (I, [P, P, P, I64, P, P, P, ctypes.POINTER(D)]),
         "adc_state_density": (I, [P, P, P]),
@@ -410,6 +412,13 @@ class Context:
         a, b = ctypes.c_int64(), ctypes.c_int64()
         _check(lib.adc_memory(self._h, ctypes.byref(a), ctypes.byref(b)), self._h)
         return {"in_use": a.value, "peak": b.value}
+
+    def kept_digits(self):
+        """Bytes of the library's device allocations, of the digits this context keeps for FP64
+        products, and of those every context on its device keeps (``adc_diag_memory``)."""
+        v = [ctypes.c_int64() for _ in range(3)]
+        _check(lib.adc_diag_memory(self._h, *(ctypes.byref(x) for x in v)), self._h)
+        return dict(zip(("total", "own", "device"), (x.value for x in v)))
 
     def direct_ladder(self):
         """Whether the context forms its ladder integrals in every product (``adc_ladder_mode``)."""

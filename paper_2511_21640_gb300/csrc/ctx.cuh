@@ -147,6 +147,8 @@ bool fp64_op_product(adc_ctx *c, int which, bool ring, const cplx *X, int64_t k,
                      int64_t b_nh, int64_t b_nl, int64_t b_in, int64_t b_k, cplx alpha, cplx beta, cplx *out,
                      int64_t s_m, int64_t s_nh, int64_t s_nl, int64_t n_in);
 void fp64_ops_prepare(adc_ctx *c, int64_t k);
+// bytes of digits kept for FP64 products: this context's, and those of every context on its device
+void kept_digit_bytes(const adc_ctx *c, int64_t *own, int64_t *device);
 // FP64-accurate sigma with the dense contractions as sliced tensor-core products (IP/EA)
 void sigma_sliced(adc_ctx *c, const cplx *X, cplx *S, int64_t k, int bits = kSlicedBits);
 // estimate of the largest device scratch one sigma call of k vectors allocates (bytes)

@@ -216,6 +216,19 @@ extern "C" int adc_diag_set_sliced_cap(int64_t bytes) {
   return ADC_OK;
 }
 
+extern "C" int adc_diag_set_alloc_limit(int64_t bytes) {
+  set_alloc_limit(bytes);
+  return ADC_OK;
+}
+
+extern "C" int adc_diag_memory(const adc_ctx *c, int64_t *total, int64_t *own, int64_t *device) {
+  if (!c) return ADC_ERR_STATE;
+  if (!total || !own || !device) return ADC_ERR_ARG;
+  *total = alloc_total();
+  kept_digit_bytes(c, own, device);
+  return ADC_OK;
+}
+
 extern "C" int adc_diag_set_setup_chunk(int64_t elems) {
   set_setup_chunk_elems(elems);
   return ADC_OK;

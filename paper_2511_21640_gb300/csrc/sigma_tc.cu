@@ -3,7 +3,7 @@
 // (sigma_sliced, tc_slice.cu). Same terms as sigma.cu (Sec. 2.1 Eqs. 10-12);
 // the coupling, ladder and ring contractions run on the tensor cores, the main
 // block (n1 x n1) and the zeroth-order diagonal stay FP64.
-#include <atomic>
+#include <mutex>
 
 #include "ctx.cuh"
 #include "tc_gemm.cuh"
@@ -198,13 +198,37 @@ void sigma_split(adc_ctx *c, const cplx *X, cplx *S, int64_t k, int nseg) {
 }
 
 // ---- products from digits: the same contractions as sliced tensor-core products.
-// Digits kept for FP64 products, all contexts of a device together: at most an
-// eighth of its memory (an EA problem at o = 40, v = 200 keeps 25 GB).
-static std::atomic<int64_t> sl_kept_total[64];
-SlCache::~SlCache() { sl_kept_total[dev] -= kept; }
+// Digits kept for FP64 products: all contexts of a device together at most an eighth of
+// its memory (an EA problem at o = 40, v = 200 keeps 25 GB), and a context's operators
+// together at most a quarter of what it has left without them.
+static std::mutex kept_mu;
+static double kept_total[64];
+
+static bool kept_reserve(int dev, double bytes, double most) {
+  std::lock_guard<std::mutex> lk(kept_mu);
+  if (kept_total[dev] + bytes > most) return false;
+  kept_total[dev] += bytes;
+  return true;
+}
+static void kept_release(int dev, double bytes) {
+  std::lock_guard<std::mutex> lk(kept_mu);
+  kept_total[dev] -= bytes;
+}
+
+SlCache::~SlCache() { kept_release(dev, kept); }
+
+void kept_digit_bytes(const adc_ctx *c, int64_t *own, int64_t *device) {
+  *own = c->sl ? (int64_t)c->sl->kept : 0;
+  std::lock_guard<std::mutex> lk(kept_mu);
+  *device = (int64_t)kept_total[std::max(0, c->dev) % 64];
+}
+
+// An operator whose digits found no room, or went back, is looked at again after this many
+// of its products (each look asks the driver for the free memory)
+constexpr int kKeepRest = 16;
 
 // The digits kept for FP64 products alone go back when the context runs short of
-// memory, and are not kept again: what fits without them still fits.
+// memory: what fits without them still fits.
 static bool sl_give_back(void *ctx) {
   SlCache *sl = ((adc_ctx *)ctx)->sl.get();
   if (!sl || sl->busy) return false;
@@ -212,11 +236,11 @@ static bool sl_give_back(void *ctx) {
   for (int w = 0; w < SL_NOPS; ++w) {
     if (sl->op[w].ns * sl->op[w].b < kDigitFp64Bits) continue;
     sl->op[w] = SlMat();
-    sl->no_room[w] = true;
+    sl->rest[w] = kKeepRest;
     any = true;
   }
-  sl_kept_total[sl->dev] -= sl->kept;
-  sl->kept = 0;
+  kept_release(sl->dev, sl->kept);
+  sl->kept = 0.0;
   sl->Bx = SlMat();
   sl->w.part.reset();
   return any;
@@ -325,23 +349,32 @@ void sigma_sliced(adc_ctx *c, const cplx *X, cplx *S, int64_t k, int bits) {
   tc_sync(ex, err);
 }
 
-// whether the FP64 digits of an operator are kept, or may be: within a quarter of the
-// context's free memory and the device's share
-static bool sl_keep(adc_ctx *c, SlCache &sl, int which, int64_t M, int64_t K) {
-  if (sl.no_room[which]) return false;
-  if (sl.op[which].ns * sl.op[which].b >= kDigitFp64Bits) return true;
+// the kept FP64 digits of an operator (M x K), built when there is room for them; null: none kept
+static const SlMat *sl_kept_op(adc_ctx *c, SlCache &sl, int which, int64_t M, int64_t K) {
+  SlMat &m = sl.op[which];
+  if (m.ns * m.b >= kDigitFp64Bits) return &m;
+  if (!c->keep_digits) return nullptr;
+  if (sl.rest[which] > 0) {
+    --sl.rest[which];
+    return nullptr;
+  }
   const double need = 4.0 * sl_digits(K, kDigitFp64Bits).ns * (double)M * (double)sl_kp(K);
   double room = (double)free_device_memory();
   if (c->ex.mem_limit > 0) room = std::min(room, (double)(c->ex.mem_limit - c->ex.mem_used));
   size_t fr = 0, tot = 0;
   ADC_CUDA(cudaMemGetInfo(&fr, &tot));
-  if (!c->keep_digits || need > 0.25 * room || (double)sl_kept_total[sl.dev] + need > 0.125 * (double)tot) {
-    sl.no_room[which] = true;
-    return false;
+  sl.rest[which] = kKeepRest;
+  if (sl.kept + need > 0.25 * (room + sl.kept) || !kept_reserve(sl.dev, need, 0.125 * (double)tot)) return nullptr;
+  try {
+    sl_op(c, which, kDigitFp64Bits);
+  } catch (const Error &e) {
+    kept_release(sl.dev, need);
+    if (e.code != ADC_ERR_OOM) throw;
+    return nullptr;
   }
-  sl_kept_total[sl.dev] += (int64_t)need;
-  sl.kept += (int64_t)need;
-  return true;
+  sl.kept += need;
+  sl.rest[which] = 0;
+  return &m;
 }
 
 // ---- one term of the FP64 product with the kept digits of its operator:
@@ -349,8 +382,7 @@ static bool sl_keep(adc_ctx *c, SlCache &sl, int which, int64_t M, int64_t K) {
 // gathered from X2. Slicing the operator again in every product took 6.9 of the
 // 23.6 ms of device time of an EA product at o = 30, v = 150, 8 vectors, and 4.0 of
 // 7.0 ms at second order (o = 25, v = 180, 6 vectors). False (nothing enqueued to out):
-// the term is small, the stream is capturing, or the digits do not fit (they may
-// take a quarter of the free device memory).
+// the term is small, the stream is capturing, or the digits do not fit.
 bool fp64_op_product(adc_ctx *c, int which, bool ring, const cplx *X, int64_t k, const cplx *Bsrc, int64_t Nc,
                      int64_t b_nh, int64_t b_nl, int64_t b_in, int64_t b_k, cplx alpha, cplx beta, cplx *out,
                      int64_t s_m, int64_t s_nh, int64_t s_nl, int64_t n_in) {
@@ -361,15 +393,15 @@ bool fp64_op_product(adc_ctx *c, int which, bool ring, const cplx *X, int64_t k,
   if (!fp64_digits_usable(ex, M, Nc, K)) return false;
   SlCache &sl = sl_cache(c);
   const SlUse use(sl);
-  if (!sl_keep(c, sl, which, M, K)) return false;
+  const SlMat *op = sl_kept_op(c, sl, which, M, K);
+  if (!op) return false;
   try {
-    const SlMat &A = sl_op(c, which, kDigitFp64Bits);
+    const SlMat &A = *op;
     if (ring) sl_pack_B_ring(ex, sl.Bx, c, X, k, A, kDigitFp64Bits);
     else sl_pack_B(ex, sl.Bx, Bsrc, Nc, K, b_nh, b_nl, b_in, b_k, false, A, kDigitFp64Bits);
     sl_gemm(ex, A, sl.Bx, M, Nc, alpha, beta, out, s_m, s_nh, s_nl, n_in, ex.digit_err, sl.w);
   } catch (const Error &e) {
     if (e.code != ADC_ERR_OOM) throw;
-    sl.no_room[which] = true;
     return false;
   }
   return true;
@@ -389,13 +421,7 @@ void fp64_ops_prepare(adc_ctx *c, int64_t k) {
     if (!fp64_digits_usable(c->ex, M[w], Nc[w], K[w])) continue;
     SlCache &sl = sl_cache(c);
     const SlUse use(sl);
-    if (sl.op[w].ns * sl.op[w].b >= kDigitFp64Bits || !sl_keep(c, sl, w, M[w], K[w])) continue;
-    try {
-      sl_op(c, w, kDigitFp64Bits);
-    } catch (const Error &e) {
-      if (e.code != ADC_ERR_OOM) throw;
-      sl.no_room[w] = true;
-    }
+    sl_kept_op(c, sl, w, M[w], K[w]);
   }
 }
 

@@ -56,12 +56,12 @@ struct SlWork {
 enum { SL_CPL = 0, SL_CPLT = 1, SL_GLAD = 2, SL_W = 3, SL_NOPS = 4 };
 struct SlCache {
   SlMat op[SL_NOPS], Bx;
-  bool no_room[SL_NOPS] = {};  // FP64 products: the operator's digits did not fit
+  int rest[SL_NOPS] = {};  // FP64 products of the operator left before its digits may be built again
   SlWork w;
   DBuf err;
   int busy = 0;      // a product is being enqueued: its operator's digits stay
   int dev = 0;
-  int64_t kept = 0;  // bytes of digits kept for FP64 products alone
+  double kept = 0.0;  // bytes of digits kept for FP64 products alone
   ~SlCache();
 };
 

@@ -1,5 +1,6 @@
 // FP64 complex tensor toolkit (see tensor.cuh).
 #include <algorithm>
+#include <atomic>
 #include <cstring>
 #include <map>
 
@@ -81,6 +82,11 @@ size_t free_device_memory() {
   return fr + (size_t)(held > used ? held - used : 0);
 }
 
+// test hook: a device allocation that would take the library's total past the limit fails
+static std::atomic<int64_t> g_alloc_limit{0}, g_alloc_total{0};
+void set_alloc_limit(int64_t bytes) { g_alloc_limit = bytes; }
+int64_t alloc_total() { return g_alloc_total; }
+
 void *Exec::alloc(size_t bytes) {
   if (bytes == 0) return nullptr;
   auto capturing = [&]() {
@@ -95,13 +101,18 @@ void *Exec::alloc(size_t bytes) {
                                  std::to_string(mem_limit));
   void *p = nullptr;
   cudaMemPool_t pool = current_pool();
-  cudaError_t e = cudaMallocFromPoolAsync(&p, bytes, pool, stream);
+  auto take = [&]() {
+    const int64_t lim = g_alloc_limit;
+    return lim > 0 && g_alloc_total + (int64_t)bytes > lim ? cudaErrorMemoryAllocation
+                                                           : cudaMallocFromPoolAsync(&p, bytes, pool, stream);
+  };
+  cudaError_t e = take();
   if (e == cudaErrorMemoryAllocation) {
     // blocks freed on other streams, or kept in sizes that do not fit, go back first
     cudaGetLastError();
     auto again = [&]() {
       if (cudaStreamSynchronize(stream) == cudaSuccess && cudaMemPoolTrimTo(pool, 0) == cudaSuccess)
-        e = cudaMallocFromPoolAsync(&p, bytes, pool, stream);
+        e = take();
     };
     if (!capturing()) {
       again();
@@ -119,6 +130,7 @@ void *Exec::alloc(size_t bytes) {
                     (stage.empty() ? std::string() : ", in " + stage) + (tag.empty() ? std::string() : "/" + tag) +
                     ")");
   }
+  g_alloc_total += (int64_t)bytes;
   mem_used += (int64_t)bytes;
   mem_peak = std::max(mem_peak, mem_used);
   return p;
@@ -127,6 +139,7 @@ void *Exec::alloc(size_t bytes) {
 void Exec::release(void *p, size_t bytes) {
   if (!p) return;
   cudaFreeAsync(p, stream);
+  g_alloc_total -= (int64_t)bytes;
   mem_used -= (int64_t)bytes;
 }
 

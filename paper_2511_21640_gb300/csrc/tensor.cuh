@@ -70,6 +70,10 @@ void pool_release(int dev);
 // free memory of the current device, what the pool holds unused included
 size_t free_device_memory();
 
+// test hook: device allocations of the library fail past this total (<= 0: no limit); the total now
+void set_alloc_limit(int64_t bytes);
+int64_t alloc_total();
+
 // RAII device buffer counted against the context budget.
 struct DBuf {
   Exec *ex = nullptr;

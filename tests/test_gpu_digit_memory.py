@@ -49,3 +49,55 @@ def test_sliced_product_after_kept_fp64_digits(gpu, kind, nocc, nvir, precision)
         got = c.sigma(X, precision)
         assert c.memory()["peak"] <= limit
     assert np.abs(got - want).max() < (1e-11 if precision == "sliced" else 1e-6) * np.abs(want).max()
+
+
+def _problem():
+    return make_problem(nocc=12, nvir=40, naux=60, seed=5)
+
+
+def test_kept_digits_take_a_quarter_together(gpu):
+    """All operators' digits together stay within a quarter of what a limit leaves, also when each
+    alone would fit."""
+    p = _problem()
+    with gpu.Context(p.B, p.eps_occ, p.eps_vir, kind="EA", order=3, x=0.5) as c:
+        held, setup_peak = c.memory()["in_use"], c.memory()["peak"]
+        X = _vectors(c.N, 32, 7)
+        want = c.sigma(X, "fp64")
+        every = c.kept_digits()["own"]
+        assert every > 0
+    left = int(3.6 * every)
+    assert held + left > setup_peak
+    with gpu.Context(p.B, p.eps_occ, p.eps_vir, kind="EA", order=3, x=0.5, mem_limit=held + left) as c:
+        for _ in range(3):
+            got = c.sigma(X, "fp64")
+            assert c.kept_digits()["own"] <= left // 4
+        assert np.abs(got - want).max() < 1e-13 * np.abs(want).max()
+
+
+def test_a_failed_build_is_not_charged_and_not_final(gpu):
+    """Digits whose allocation fails are not counted as kept; once there is memory again, later
+    products keep them; a closed context leaves nothing counted."""
+    p = _problem()
+    with gpu.Context(p.B, p.eps_occ, p.eps_vir, kind="EA", order=3, x=0.5) as c:
+        X = torch.from_numpy(_vectors(c.N, 32, 8)).cuda()
+        want = c.sigma(X, "fp64").cpu().numpy()
+        every = c.kept_digits()
+        assert every["own"] > 0 and every["own"] == every["device"]
+        peak = c.memory()["peak"]
+    with gpu.Context(p.B, p.eps_occ, p.eps_vir, kind="EA", order=3, x=0.5) as c:
+        assert c.kept_digits()["device"] == 0
+        # room for a product on the FP64 units (its scratch), not for the digits
+        scratch = 4 * 16 * 32 * 12 * 40 * 40
+        assert c.memory()["in_use"] + scratch < peak
+        assert gpu.lib.adc_diag_set_alloc_limit(c.kept_digits()["total"] + scratch) == 0
+        try:
+            got = c.sigma(X, "fp64").cpu().numpy()
+            short = c.kept_digits()
+        finally:
+            gpu.lib.adc_diag_set_alloc_limit(0)
+        assert short["own"] == short["device"] < every["own"]
+        for _ in range(40):
+            again = c.sigma(X, "fp64").cpu().numpy()
+        assert c.kept_digits()["own"] == every["own"]
+        for s in (got, again):
+            assert np.abs(s - want).max() < 1e-13 * np.abs(want).max()
