@@ -462,7 +462,7 @@ int davidson_run(adc_ctx *c, int nroots, double tol, int max_iter, int precision
                  c->opts.refine == ADC_PREC_SLICED);
     if (precision == ADC_PREC_FP64 || c->opts.refine == ADC_PREC_FP64) fp64_ops_prepare(c, kb);
     c->ex.sync();
-    double avail = (double)free_device_memory();
+    double avail = (double)free_device_memory(&c->ex);
     if (c->ex.mem_limit > 0) avail = std::min(avail, (double)(c->ex.mem_limit - c->ex.mem_used));
     const double vec = (double)N * sizeof(cplx);
     const double scratch = sigma_scratch_bytes(c, kb);

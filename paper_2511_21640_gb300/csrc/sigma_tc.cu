@@ -3,6 +3,7 @@
 // (sigma_sliced, tc_slice.cu). Same terms as sigma.cu (Sec. 2.1 Eqs. 10-12);
 // the coupling, ladder and ring contractions run on the tensor cores, the main
 // block (n1 x n1) and the zeroth-order diagonal stay FP64.
+#include <algorithm>
 #include <mutex>
 
 #include "ctx.cuh"
@@ -201,8 +202,12 @@ void sigma_split(adc_ctx *c, const cplx *X, cplx *S, int64_t k, int nseg) {
 // Digits kept for FP64 products: all contexts of a device together at most an eighth of
 // its memory (an EA problem at o = 40, v = 200 keeps 25 GB), and a context's operators
 // together at most a quarter of what it has left without them.
+// Any context of the device that runs short of memory takes the digits back (below).
+// The lock guards the list, the totals, and whether a cache is in use: a cache that is
+// not (busy 0) may lose its digits to another thread.
 static std::mutex kept_mu;
 static double kept_total[64];
+static std::vector<SlCache *> kept_caches;
 
 static bool kept_reserve(int dev, double bytes, double most) {
   std::lock_guard<std::mutex> lk(kept_mu);
@@ -215,51 +220,98 @@ static void kept_release(int dev, double bytes) {
   kept_total[dev] -= bytes;
 }
 
-SlCache::~SlCache() { kept_release(dev, kept); }
+SlCache::SlCache(Exec &e, int d) : ex(e), dev(d) {
+  std::lock_guard<std::mutex> lk(kept_mu);
+  kept_caches.push_back(this);
+}
+SlCache::~SlCache() {
+  std::lock_guard<std::mutex> lk(kept_mu);
+  kept_total[dev] -= kept;
+  kept_caches.erase(std::find(kept_caches.begin(), kept_caches.end(), this));
+}
+
+static int kept_dev(int dev) { return std::max(0, dev) % 64; }
 
 void kept_digit_bytes(const adc_ctx *c, int64_t *own, int64_t *device) {
-  *own = c->sl ? (int64_t)c->sl->kept : 0;
   std::lock_guard<std::mutex> lk(kept_mu);
-  *device = (int64_t)kept_total[std::max(0, c->dev) % 64];
+  *own = c->sl ? (int64_t)c->sl->kept : 0;
+  *device = (int64_t)kept_total[kept_dev(c->dev)];
+}
+
+size_t kept_by_others(int dev, const Exec *mine) {
+  std::lock_guard<std::mutex> lk(kept_mu);
+  double b = 0.0;
+  for (const SlCache *sl : kept_caches)
+    if (sl->dev == kept_dev(dev) && &sl->ex != mine) b += sl->kept;
+  return (size_t)b;
 }
 
 // An operator whose digits found no room, or went back, is looked at again after this many
 // of its products (each look asks the driver for the free memory)
 constexpr int kKeepRest = 16;
 
-// The digits kept for FP64 products alone go back when the context runs short of
-// memory: what fits without them still fits.
-static bool sl_give_back(void *ctx) {
-  SlCache *sl = ((adc_ctx *)ctx)->sl.get();
-  if (!sl || sl->busy) return false;
+// The digits kept for FP64 products alone go back (freed in the order of their context's
+// stream). The lock is held; false: none kept, or the cache is in use
+static bool kept_drop(SlCache &sl) {
+  if (sl.busy) return false;
   bool any = false;
   for (int w = 0; w < SL_NOPS; ++w) {
-    if (sl->op[w].ns * sl->op[w].b < kDigitFp64Bits) continue;
-    sl->op[w] = SlMat();
-    sl->rest[w] = kKeepRest;
+    if (sl.op[w].ns * sl.op[w].b < kDigitFp64Bits) continue;
+    sl.op[w] = SlMat();
+    sl.rest[w] = kKeepRest;
     any = true;
   }
-  kept_release(sl->dev, sl->kept);
-  sl->kept = 0.0;
-  sl->Bx = SlMat();
-  sl->w.part.reset();
+  kept_total[sl.dev] -= sl.kept;
+  sl.kept = 0.0;
+  sl.Bx = SlMat();
+  sl.w.part.reset();
+  return any;
+}
+
+// A context over its own limit gives its own digits back; one that finds no device memory
+// takes those of every context that is not in a product: what fits without them still fits.
+static bool sl_give_back(void *ctx) {
+  SlCache *sl = ((adc_ctx *)ctx)->sl.get();
+  if (!sl) return false;
+  std::lock_guard<std::mutex> lk(kept_mu);
+  return kept_drop(*sl);
+}
+
+bool reclaim_kept_digits(int dev) {
+  std::lock_guard<std::mutex> lk(kept_mu);
+  bool any = false;
+  for (SlCache *sl : kept_caches) {
+    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+    if (sl->dev != kept_dev(dev) || sl->busy || sl->kept <= 0.0 ||
+        cudaStreamIsCapturing(sl->ex.stream, &cs) != cudaSuccess || cs != cudaStreamCaptureStatusNone)
+      continue;
+    // the memory is there for another stream once this one has freed it
+    if (kept_drop(*sl)) any = cudaStreamSynchronize(sl->ex.stream) == cudaSuccess || any;
+  }
+  cudaGetLastError();
   return any;
 }
 
 static SlCache &sl_cache(adc_ctx *c) {
   if (!c->sl) {
-    c->sl.reset(new SlCache());
-    c->sl->dev = std::max(0, c->dev) % 64;
+    c->sl.reset(new SlCache(c->ex, kept_dev(c->dev)));
     c->ex.give_back = sl_give_back;
     c->ex.give_back_of = c;
   }
   return *c->sl;
 }
 
+// while it lives the cache's digits and buffers stay
 struct SlUse {
   SlCache &sl;
-  explicit SlUse(SlCache &s) : sl(s) { ++sl.busy; }
-  ~SlUse() { --sl.busy; }
+  explicit SlUse(SlCache &s) : sl(s) {
+    std::lock_guard<std::mutex> lk(kept_mu);
+    ++sl.busy;
+  }
+  ~SlUse() {
+    std::lock_guard<std::mutex> lk(kept_mu);
+    --sl.busy;
+  }
 };
 
 // The digits of a static operator, built when first asked for and rebuilt with
@@ -359,7 +411,7 @@ static const SlMat *sl_kept_op(adc_ctx *c, SlCache &sl, int which, int64_t M, in
     return nullptr;
   }
   const double need = 4.0 * sl_digits(K, kDigitFp64Bits).ns * (double)M * (double)sl_kp(K);
-  double room = (double)free_device_memory();
+  double room = (double)unused_device_memory();
   if (c->ex.mem_limit > 0) room = std::min(room, (double)(c->ex.mem_limit - c->ex.mem_used));
   size_t fr = 0, tot = 0;
   ADC_CUDA(cudaMemGetInfo(&fr, &tot));
@@ -372,7 +424,10 @@ static const SlMat *sl_kept_op(adc_ctx *c, SlCache &sl, int which, int64_t M, in
     if (e.code != ADC_ERR_OOM) throw;
     return nullptr;
   }
-  sl.kept += need;
+  {
+    std::lock_guard<std::mutex> lk(kept_mu);
+    sl.kept += need;
+  }
   sl.rest[which] = 0;
   return &m;
 }

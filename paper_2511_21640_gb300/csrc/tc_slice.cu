@@ -838,7 +838,7 @@ void digit_product(Exec &ex, int64_t M, int64_t N, int64_t K, cplx alpha, const 
 size_t digit_cap(double need) {
   if (g_sliced_cap) return g_sliced_cap;
   if (need <= (double)(1ll << 30)) return (size_t)1 << 30;
-  const size_t fr = free_device_memory();
+  const size_t fr = unused_device_memory();
   return std::min<size_t>((size_t)16 << 30, std::max<size_t>((size_t)1 << 30, fr / 8));
 }
 

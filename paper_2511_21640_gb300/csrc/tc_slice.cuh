@@ -59,9 +59,11 @@ struct SlCache {
   int rest[SL_NOPS] = {};  // FP64 products of the operator left before its digits may be built again
   SlWork w;
   DBuf err;
-  int busy = 0;      // a product is being enqueued: its operator's digits stay
-  int dev = 0;
+  Exec &ex;
+  const int dev;
+  int busy = 0;       // a product is being enqueued: its operator's digits stay
   double kept = 0.0;  // bytes of digits kept for FP64 products alone
+  SlCache(Exec &e, int d);
   ~SlCache();
 };
 

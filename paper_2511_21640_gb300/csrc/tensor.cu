@@ -72,7 +72,7 @@ void pool_release(int dev) {
   cudaMemPoolTrimTo(it->second.pool, 0);
 }
 
-size_t free_device_memory() {
+size_t unused_device_memory() {
   size_t fr = 0, tot = 0;
   ADC_CUDA(cudaMemGetInfo(&fr, &tot));
   uint64_t held = 0, used = 0;
@@ -80,6 +80,12 @@ size_t free_device_memory() {
   ADC_CUDA(cudaMemPoolGetAttribute(p, cudaMemPoolAttrReservedMemCurrent, &held));
   ADC_CUDA(cudaMemPoolGetAttribute(p, cudaMemPoolAttrUsedMemCurrent, &used));
   return fr + (size_t)(held > used ? held - used : 0);
+}
+
+size_t free_device_memory(const Exec *mine) {
+  int dev = 0;
+  ADC_CUDA(cudaGetDevice(&dev));
+  return unused_device_memory() + kept_by_others(dev, mine);
 }
 
 // test hook: a device allocation that would take the library's total past the limit fails
@@ -116,7 +122,8 @@ void *Exec::alloc(size_t bytes) {
     };
     if (!capturing()) {
       again();
-      if (e == cudaErrorMemoryAllocation && give_back && give_back(give_back_of)) {
+      int dev = 0;
+      if (e == cudaErrorMemoryAllocation && cudaGetDevice(&dev) == cudaSuccess && reclaim_kept_digits(dev)) {
         cudaGetLastError();
         again();
       }
@@ -132,7 +139,7 @@ void *Exec::alloc(size_t bytes) {
   }
   g_alloc_total += (int64_t)bytes;
   mem_used += (int64_t)bytes;
-  mem_peak = std::max(mem_peak, mem_used);
+  mem_peak = std::max<int64_t>(mem_peak, mem_used);
   return p;
 }
 

@@ -3,6 +3,8 @@
 // setup of the ADC operators.
 #pragma once
 
+#include <atomic>
+
 #include "common.cuh"
 
 namespace adc {
@@ -44,9 +46,9 @@ struct Exec {
   int64_t n_sliced = 0, n_fp64 = 0;
   double flops_sliced = 0.0, flops_fp64 = 0.0;
   int64_t mem_limit = 0;  // 0 = unlimited
-  int64_t mem_used = 0;
+  std::atomic<int64_t> mem_used{0};  // (another thread may take kept digits back)
   int64_t mem_peak = 0;
-  // short of memory, alloc asks once for what is kept for speed alone (false: nothing to give)
+  // over its limit, alloc asks once for what this context keeps for speed alone (false: nothing to give)
   bool (*give_back)(void *) = nullptr;
   void *give_back_of = nullptr;
   // per-kernel timing with CUDA events on this stream (off unless enabled)
@@ -68,7 +70,12 @@ struct Exec {
 void pool_retain(int dev);
 void pool_release(int dev);
 // free memory of the current device, what the pool holds unused included
-size_t free_device_memory();
+size_t unused_device_memory();
+// the same and the digits that contexts other than `mine` keep for speed alone: an
+// allocation that finds no other memory takes them back
+size_t free_device_memory(const Exec *mine = nullptr);
+size_t kept_by_others(int dev, const Exec *mine);
+bool reclaim_kept_digits(int dev);  // false: nothing to take
 
 // test hook: device allocations of the library fail past this total (<= 0: no limit); the total now
 void set_alloc_limit(int64_t bytes);

@@ -101,3 +101,39 @@ def test_a_failed_build_is_not_charged_and_not_final(gpu):
         assert c.kept_digits()["own"] == every["own"]
         for s in (got, again):
             assert np.abs(s - want).max() < 1e-13 * np.abs(want).max()
+
+
+@pytest.mark.parametrize("other", ["context", "batch"])
+def test_kept_digits_go_back_to_other_contexts(gpu, other):
+    """Device memory that suffices only with the digits another, idle context keeps: a second
+    context's product, and a batch's, take them and run; the first context then works as before."""
+    p = _problem()
+
+    def context():
+        return gpu.Context(p.B, p.eps_occ, p.eps_vir, kind="EA", order=3, x=0.5)
+
+    with context() as a, context() as b:
+        small, X = _vectors(a.N, 32, 9), _vectors(a.N, 300, 10)
+        Xd = torch.from_numpy(X).cuda()
+        need = 16 * (2 * 300 * b.N + 2 * 300 * 12 * 40 * 40)  # host blocks copied in and out, scratch
+        if other == "batch":
+            for _ in range(2):  # operator copies and tile widths first, then what the batch itself holds
+                with gpu.Batch([b]) as batch:
+                    before = b.kept_digits()["total"]
+                    batch.sigma([Xd])
+                    need = b.kept_digits()["total"] - before
+        want = a.sigma(small, "fp64")
+        kept = a.kept_digits()
+        assert kept["own"] == kept["device"] > 0 and need > kept["own"]
+        batch = gpu.Batch([b])
+        assert gpu.lib.adc_diag_set_alloc_limit(a.kept_digits()["total"] + need - kept["own"] // 2) == 0
+        try:
+            got = b.sigma(X, "fp64")[:2] if other == "context" else batch.sigma([Xd])[0][:2].cpu().numpy()
+        finally:
+            gpu.lib.adc_diag_set_alloc_limit(0)
+            batch.close()
+        assert a.kept_digits()["own"] == 0
+        ref = b.sigma(X[:2], "fp64")
+        assert np.abs(got - ref).max() < (1e-13 if other == "context" else 1e-3) * np.abs(ref).max()
+        again = a.sigma(small, "fp64")
+        assert np.abs(again - want).max() < 1e-13 * np.abs(want).max()
