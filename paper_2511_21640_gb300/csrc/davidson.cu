@@ -452,6 +452,13 @@ int davidson_run(adc_ctx *c, int nroots, double tol, int max_iter, int precision
   mmax = (int)std::min<int64_t>(std::min<int64_t>(mmax, N), 1024);
   mmax = std::max(mmax, std::min<int>((int)N, nroots + 1));
   int krmax = std::max(2 * nroots, kb);
+  // no digits are kept while the subspace holds the memory they took
+  struct KeepDigits {
+    bool &flag, was;
+    explicit KeepDigits(bool &f) : flag(f), was(f) {}
+    ~KeepDigits() { flag = was; }
+    void off() { flag = false; }
+  } keep(c->keep_digits);
   if (c->opts.max_subspace <= 0) {
     // the operators of the products first (their transient buffers never meet
     // the subspace); then V and AV take what is left after the Davidson's
@@ -462,8 +469,12 @@ int davidson_run(adc_ctx *c, int nroots, double tol, int max_iter, int precision
                  c->opts.refine == ADC_PREC_SLICED);
     if (precision == ADC_PREC_FP64 || c->opts.refine == ADC_PREC_FP64) fp64_ops_prepare(c, kb);
     c->ex.sync();
-    double avail = (double)free_device_memory(&c->ex);
-    if (c->ex.mem_limit > 0) avail = std::min(avail, (double)(c->ex.mem_limit - c->ex.mem_used));
+    double avail = 0.0;
+    auto look = [&]() {
+      avail = (double)free_device_memory(&c->ex);
+      if (c->ex.mem_limit > 0) avail = std::min(avail, (double)(c->ex.mem_limit - c->ex.mem_used));
+    };
+    look();
     const double vec = (double)N * sizeof(cplx);
     const double scratch = sigma_scratch_bytes(c, kb);
     auto fit_of = [&](int kr) {
@@ -471,6 +482,13 @@ int davidson_run(adc_ctx *c, int nroots, double tol, int max_iter, int precision
     };
     int lo = (int)std::min<int64_t>(N, std::max(2 * nroots, kb) + kb);
     int64_t fit = fit_of(krmax);
+    // the subspace goes before digits kept for speed: a smaller one takes more iterations
+    if (fit < mmax && c->ex.give_back && c->ex.give_back(c->ex.give_back_of)) {
+      keep.off();
+      c->ex.sync();
+      look();
+      fit = fit_of(krmax);
+    }
     // short of memory: keep only the wanted roots at a collapse (thick restart
     // of nroots) and allow a subspace of nroots plus one block
     if (fit < lo) {

@@ -137,3 +137,25 @@ def test_kept_digits_go_back_to_other_contexts(gpu, other):
         assert np.abs(got - ref).max() < (1e-13 if other == "context" else 1e-3) * np.abs(ref).max()
         again = a.sigma(small, "fp64")
         assert np.abs(again - want).max() < 1e-13 * np.abs(want).max()
+
+
+def test_kept_digits_do_not_shrink_the_subspace(gpu, capfd):
+    """An FP64 solve under a limit that just holds its default subspace goes through the same
+    subspace sizes as without a limit (as printed per iteration), and reaches the same roots."""
+    p, nroots, block = _problem(), 16, 32
+
+    def solve(limit):
+        with gpu.Context(p.B, p.eps_occ, p.eps_vir, kind="EA", order=3, x=0.5, mem_limit=limit, block=block,
+                         verbose=True) as c:
+            held, N = c.memory()["in_use"], c.N
+            om = c.davidson(nroots, tol=1e-9, precision="fp64", want_vectors=False)[0]
+        lines = [ln for ln in capfd.readouterr().err.splitlines() if ln.startswith("[davidson] it")]
+        return held, N, om, [int(ln.split(" m ")[1].split()[0]) for ln in lines]
+
+    held, N, want, sizes = solve(0)
+    # 256 vectors and their products, the solve's other vectors and its estimate of one product's scratch, 8% over
+    vec = 16 * N
+    need = (2 * 8 * block + 3 * nroots + 2 * block) * vec + 16 * (2 * block * 12 * 40 * 40 + 8 * block * N)
+    _, _, got, limited = solve(held + int(need / 0.92) + (1 << 20))
+    assert max(sizes) > 160 and limited == sizes
+    assert np.abs(got - want).max() < 1e-9
