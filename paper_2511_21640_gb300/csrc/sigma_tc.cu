@@ -416,6 +416,7 @@ static const SlMat *sl_kept_op(adc_ctx *c, SlCache &sl, int which, int64_t M, in
   size_t fr = 0, tot = 0;
   ADC_CUDA(cudaMemGetInfo(&fr, &tot));
   sl.rest[which] = kKeepRest;
+  const OptionalAlloc opt(c->ex);
   if (sl.kept + need > 0.25 * (room + sl.kept) || !kept_reserve(sl.dev, need, 0.125 * (double)tot)) return nullptr;
   try {
     sl_op(c, which, kDigitFp64Bits);
@@ -450,6 +451,7 @@ bool fp64_op_product(adc_ctx *c, int which, bool ring, const cplx *X, int64_t k,
   const SlUse use(sl);
   const SlMat *op = sl_kept_op(c, sl, which, M, K);
   if (!op) return false;
+  const OptionalAlloc opt(ex);
   try {
     const SlMat &A = *op;
     if (ring) sl_pack_B_ring(ex, sl.Bx, c, X, k, A, kDigitFp64Bits);

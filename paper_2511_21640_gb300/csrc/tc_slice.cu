@@ -632,11 +632,14 @@ void pack_rows(Exec &ex, SlMat &d, const BSrc &s, int64_t rows, int64_t K, bool 
   ex.prof_end(pr);
 }
 
+// spill of one CTA with the widest tile
+constexpr size_t kSpillCta = (size_t)SlTile<128>::VALS * 128 * SlTile<128>::H * sizeof(long long);
+
 template <int BN>
 void launch_sl(Exec &ex, SlArgs &g, SlWork &w, int grid) {
   using L = SlTile<BN>;
   set_smem_limit((const void *)k_sl_gemm<BN>, L::SMEM);
-  const size_t need = (size_t)grid * L::VALS * 128 * L::H * sizeof(long long);
+  const size_t need = (size_t)grid * L::VALS * 128 * L::H * sizeof(long long);  // at most kSpillCta per CTA
   if (g.ns > 4 && w.spill.bytes < need) {
     w.spill.reset();
     w.spill = DBuf(ex, need);
@@ -759,6 +762,7 @@ void sl_gemm(Exec &ex, const SlMat &A, const SlMat &B, int64_t M, int64_t N, cpl
     const size_t need = (size_t)g.ksplit * M * N * sizeof(cplx);
     if (w.part.bytes < need) {
       w.part.reset();
+      const OptionalAlloc opt(ex);
       try {
         w.part = DBuf(ex, need);
       } catch (const Error &e) {
@@ -818,6 +822,12 @@ void digit_product(Exec &ex, int64_t M, int64_t N, int64_t K, cplx alpha, const 
     const int64_t mc = std::min<int64_t>(M, std::max<int64_t>(128, (int64_t)(cap / (4 * ns * kp))));
     int64_t nc = std::min<int64_t>(N, std::max<int64_t>(64, (int64_t)(cap / (8 * ns * kp))));
     if (nc < N && n_in < N) nc = std::max<int64_t>(1, nc / n_in) * n_in;  // whole column groups
+    // several chunks: what a later one could need more of than the first is there before out changes
+    const size_t spill = (size_t)device_sm_count() * kSpillCta;
+    if ((kc < K || mc < M || nc < N) && ns > 4 && w.spill.bytes < spill) {
+      w.spill.reset();
+      w.spill = DBuf(ex, spill);
+    }
     for (int64_t m0 = 0; m0 < M; m0 += mc) {
       const int64_t mm = std::min(mc, M - m0);
       sl_pack_A(ex, Sa, A + m0 * sAm + k0 * sAk, mm, kk, sAm, sAk, conjA, bits);
@@ -833,13 +843,18 @@ void digit_product(Exec &ex, int64_t M, int64_t N, int64_t K, cplx alpha, const 
   }
 }
 
-// bytes per operand chunk: an eighth of the free device memory, between 1 and 16 GiB (need:
-// the larger operand's planes; the free memory is looked up only when they exceed 1 GiB)
-size_t digit_cap(double need) {
+// smallest operand chunk: its inner index is 512 long (digit_product)
+constexpr size_t kDigitCapMin = (size_t)2 << 20;
+
+// bytes per operand chunk: a third of what the context's limit leaves and an eighth of the
+// device's free memory, which other contexts use too, at most 16 GiB (need: the larger
+// operand's planes; the free memory is looked up only when they exceed 1 GiB)
+size_t digit_cap(Exec &ex, double need) {
   if (g_sliced_cap) return g_sliced_cap;
-  if (need <= (double)(1ll << 30)) return (size_t)1 << 30;
-  const size_t fr = unused_device_memory();
-  return std::min<size_t>((size_t)16 << 30, std::max<size_t>((size_t)1 << 30, fr / 8));
+  size_t cap = (size_t)16 << 30;
+  if (ex.mem_limit > 0) cap = std::min(cap, (size_t)std::max<int64_t>(0, ex.mem_limit - ex.mem_used) / 3);
+  if (need > (double)(1ll << 30)) cap = std::min(cap, unused_device_memory() / 8);
+  return std::max(cap, kDigitCapMin);
 }
 
 // zgemm's operands and output (element strides, conj flags, batch). The larger
@@ -848,7 +863,7 @@ size_t digit_cap(double need) {
 void digit_zgemm(Exec &ex, int64_t M, int64_t N, int64_t K, int64_t batch, cplx alpha, const cplx *A, int64_t sAb,
                  int64_t sAm, int64_t sAk, bool conjA, const cplx *B, int64_t sBb, int64_t sBk, int64_t sBn,
                  bool conjB, cplx beta, cplx *C, int64_t sCb, int64_t sCm, int64_t sCn, int bits, int *err,
-                 bool &begun) {
+                 bool &begun, size_t &cap) {
   const bool fold = batch > 1 && (sAb == 0 || sBb == 0);
   if (fold ? sAb != 0 : N > M) {
     std::swap(M, N);
@@ -861,7 +876,8 @@ void digit_zgemm(Exec &ex, int64_t M, int64_t N, int64_t K, int64_t batch, cplx 
   }
   SlMat Sa, Sb;
   SlWork w;
-  const size_t cap = digit_cap(4.0 * sl_digits(K, bits).ns * (double)sl_kp(K) * std::max<double>(M, 2.0 * N * (fold ? batch : 1)));
+  const double need = 4.0 * sl_digits(K, bits).ns * (double)sl_kp(K) * std::max<double>(M, 2.0 * N * (fold ? batch : 1));
+  if (!cap) cap = std::min(digit_cap(ex, need), (size_t)std::max(need, (double)kDigitCapMin));
   if (fold) {
     digit_product(ex, M, N * batch, K, alpha, A, sAm, sAk, conjA, B, sBk, sBb, sBn, N, conjB, beta, C, sCm, sCb, sCn,
                   bits, cap, err, Sa, Sb, w, begun);
@@ -881,8 +897,9 @@ void zgemm_sliced(Exec &ex, int64_t M, int64_t N, int64_t K, int64_t batch, cplx
   DBuf err(ex, sizeof(int));
   fill_zero(ex, err.p, sizeof(int));
   bool begun = false;
+  size_t cap = 0;
   digit_zgemm(ex, M, N, K, batch, alpha, A, sAb, sAm, sAk, conjA, B, sBb, sBk, sBn, conjB, beta, C, sCb, sCm, sCn,
-              ex.sliced_bits, (int *)err.p, begun);
+              ex.sliced_bits, (int *)err.p, begun, cap);
   tc_sync(ex, (int *)err.p);
 }
 
@@ -926,16 +943,19 @@ bool zgemm_fp64_digits(Exec &ex, int64_t M, int64_t N, int64_t K, int64_t batch,
                        int64_t sBn, bool conjB, cplx beta, cplx *C, int64_t sCb, int64_t sCm, int64_t sCn) {
   const int64_t grouped = (batch > 1 && (sAb == 0 || sBb == 0)) ? batch : 1;
   if (ex.digits == 0 || K <= 0 || (ex.digits == 1 && !digits_pay(M, N, K, grouped, false)) || !digits_ready(ex)) return false;
+  const OptionalAlloc opt(ex);
   bool begun = false;
-  try {
-    digit_zgemm(ex, M, N, K, batch, alpha, A, sAb, sAm, sAk, conjA, B, sBb, sBk, sBn, conjB, beta, C, sCb, sCm, sCn,
-                kDigitFp64Bits, ex.digit_err, begun);
-  } catch (const Error &e) {
-    // no room for the digit planes: the FP64 units need none
-    if (e.code != ADC_ERR_OOM || begun) throw;
-    return false;
+  for (size_t cap = 0;; cap /= 4) {
+    try {
+      digit_zgemm(ex, M, N, K, batch, alpha, A, sAb, sAm, sAk, conjA, B, sBb, sBk, sBn, conjB, beta, C, sCb, sCm, sCn,
+                  kDigitFp64Bits, ex.digit_err, begun, cap);
+      return true;
+    } catch (const Error &e) {
+      // no room for the digit planes: smaller chunks, then the FP64 units, which need none
+      if (e.code != ADC_ERR_OOM || begun) throw;
+      if (cap / 4 < kDigitCapMin) return false;
+    }
   }
-  return true;
 }
 
 }  // namespace adc

@@ -100,7 +100,7 @@ void *Exec::alloc(size_t bytes) {
     return cudaStreamIsCapturing(stream, &cs) != cudaSuccess || cs != cudaStreamCaptureStatusNone;
   };
   auto over = [&]() { return mem_limit > 0 && mem_used + (int64_t)bytes > mem_limit; };
-  if (over() && give_back && !capturing()) give_back(give_back_of);
+  if (over() && give_back && !optional && !capturing()) give_back(give_back_of);
   if (over())
     throw Error(ADC_ERR_OOM, "context memory limit exceeded: need " + std::to_string(bytes) +
                                  " bytes, " + std::to_string(mem_used) + " in use of " +
@@ -123,7 +123,7 @@ void *Exec::alloc(size_t bytes) {
     if (!capturing()) {
       again();
       int dev = 0;
-      if (e == cudaErrorMemoryAllocation && cudaGetDevice(&dev) == cudaSuccess && reclaim_kept_digits(dev)) {
+      if (e == cudaErrorMemoryAllocation && !optional && cudaGetDevice(&dev) == cudaSuccess && reclaim_kept_digits(dev)) {
         cudaGetLastError();
         again();
       }

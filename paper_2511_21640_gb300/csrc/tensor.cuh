@@ -51,6 +51,7 @@ struct Exec {
   // over its limit, alloc asks once for what this context keeps for speed alone (false: nothing to give)
   bool (*give_back)(void *) = nullptr;
   void *give_back_of = nullptr;
+  int optional = 0;  // > 0: allocations of something another route does without; they take nothing back
   // per-kernel timing with CUDA events on this stream (off unless enabled)
   bool prof = false;
   std::string tag;
@@ -80,6 +81,12 @@ bool reclaim_kept_digits(int dev);  // false: nothing to take
 // test hook: device allocations of the library fail past this total (<= 0: no limit); the total now
 void set_alloc_limit(int64_t bytes);
 int64_t alloc_total();
+
+struct OptionalAlloc {
+  Exec &ex;
+  explicit OptionalAlloc(Exec &e) : ex(e) { ++ex.optional; }
+  ~OptionalAlloc() { --ex.optional; }
+};
 
 // RAII device buffer counted against the context budget.
 struct DBuf {

@@ -159,3 +159,42 @@ def test_kept_digits_do_not_shrink_the_subspace(gpu, capfd):
     _, _, got, limited = solve(held + int(need / 0.92) + (1 << 20))
     assert max(sizes) > 160 and limited == sizes
     assert np.abs(got - want).max() < 1e-9
+
+
+def _limited(gpu, p, left):
+    """A context with `left` bytes to allocate after its setup."""
+    with gpu.Context(p.B, p.eps_occ, p.eps_vir, kind="EA", order=3, x=0.5) as c:
+        held = c.memory()["in_use"]
+        assert held + left > c.memory()["peak"]
+    return gpu.Context(p.B, p.eps_occ, p.eps_vir, kind="EA", order=3, x=0.5, mem_limit=held + left, profile=True)
+
+
+def test_per_call_planes_leave_kept_digits(gpu):
+    """Digit planes that one product slices and frees never push out those kept for every product."""
+    p = _problem()
+    with gpu.Context(p.B, p.eps_occ, p.eps_vir, kind="EA", order=3, x=0.5) as c:
+        X = _vectors(c.N, 32, 7)
+        want = c.sigma(X, "fp64")
+        left = int(2.5 * c.kept_digits()["own"])
+    with _limited(gpu, p, left) as c:
+        for _ in range(2):
+            got = c.sigma(X, "fp64")
+            assert 0 < c.kept_digits()["own"] <= left // 4
+    assert np.abs(got - want).max() < 1e-13 * np.abs(want).max()
+
+
+def test_a_limit_chunks_the_digits(gpu):
+    """A limit without room for a term's whole digit planes (149 MB for the ladder of 200 vectors):
+    the term runs from digits all the same, in chunks."""
+    p = _problem()
+    with gpu.Context(p.B, p.eps_occ, p.eps_vir, kind="EA", order=3, x=0.5) as c:
+        X = _vectors(c.N, 200, 11)
+        want = c.sigma(X, "fp64")
+    blocks = 16 * (2 * 200 * c.N + 2 * 200 * 12 * 40 * 40)
+    with _limited(gpu, p, blocks + (30 << 20)) as c:
+        c.profile(True)
+        got = c.sigma(X, "fp64")
+        ran = c.profile_read()
+        c.profile(False)
+    assert "tc_digits_fp64/ladder" in ran and "zgemm_fp64/ladder" not in ran, ran
+    assert np.abs(got - want).max() < 1e-13 * np.abs(want).max()
