@@ -88,6 +88,10 @@ int adc_diag_set_sliced_cap(int64_t bytes);
  * own out-of-memory; <= 0 takes the limit away. Returns ADC_OK. */
 int adc_diag_set_alloc_limit(int64_t bytes);
 
+/* The largest total of the library's device allocations in this process since
+ * the last call (or since the process began), bytes; the record starts again. */
+int64_t adc_diag_alloc_peak(void);
+
 /* Bytes of device memory: the total of the library's allocations in this
  * process, the digits this context keeps for FP64 products, and those kept by
  * every context on its device. Host-side counters only. ADC_ERR_STATE for a

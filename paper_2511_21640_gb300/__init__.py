@@ -125,6 +125,7 @@ def _load():
         "adc_diag_set_sliced_cap": (I, [ctypes.c_int64]),
         "adc_diag_set_alloc_limit": (I, [ctypes.c_int64]),
         "adc_diag_memory": (I, [P, P, P, P]),
+        "adc_diag_alloc_peak": (I64, []),
         "adc_diag_eigh": (I, [I, P, I, P, P, ctypes.POINTER(D), ctypes.POINTER(I)]),
         "adc_sigma_adjoint": (I, [P, P, P, I64, P, P, P, ctypes.POINTER(D)]),
         "adc_state_density": (I, [P, P, P]),

@@ -148,20 +148,10 @@ adc_ctx::~adc_ctx() {
   if (pooled) pool_release(dev);
 }
 
-extern "C" {
-
-int adc_opts_default(adc_opts *o) {
-  if (!o) return ADC_ERR_ARG;
-  std::memset(o, 0, sizeof(*o));
-  o->precision = ADC_PREC_FP64;
-  o->herm_tol = 1e-12;
-  o->dd_order = 1;
-  return ADC_OK;
-}
-
-int adc_init(adc_ctx **out, const adc_c128 *B, int64_t naux, const double *eps_occ, int64_t nocc,
-             const double *eps_vir, int64_t nvir, int kind, int order, double x,
-             const adc_opts *opts) {
+namespace adc {
+int context_init(adc_ctx **out, const adc_c128 *B, int64_t naux, const double *eps_occ, int64_t nocc,
+                 const double *eps_vir, int64_t nvir, int kind, int order, double x, const adc_opts *opts,
+                 int64_t digit_limit) {
   if (!out) return ADC_ERR_ARG;
   *out = nullptr;
   adc_ctx *c = nullptr;
@@ -196,6 +186,7 @@ int adc_init(adc_ctx **out, const adc_c128 *B, int64_t naux, const double *eps_o
     c->dd_order = (c->opts.dd_order == 0) ? 0 : 1;
     c->N = c->n1 + c->n2;
     c->ex.mem_limit = c->opts.mem_limit;
+    c->ex.digit_limit = digit_limit;
     ADC_CUDA(cudaGetDevice(&c->dev));
     pool_retain(c->dev);
     c->pooled = true;
@@ -275,6 +266,24 @@ int adc_init(adc_ctx **out, const adc_c128 *B, int64_t naux, const double *eps_o
     delete c;
     return ADC_ERR_CUDA;
   }
+}
+}  // namespace adc
+
+extern "C" {
+
+int adc_opts_default(adc_opts *o) {
+  if (!o) return ADC_ERR_ARG;
+  std::memset(o, 0, sizeof(*o));
+  o->precision = ADC_PREC_FP64;
+  o->herm_tol = 1e-12;
+  o->dd_order = 1;
+  return ADC_OK;
+}
+
+int adc_init(adc_ctx **out, const adc_c128 *B, int64_t naux, const double *eps_occ, int64_t nocc,
+             const double *eps_vir, int64_t nvir, int kind, int order, double x,
+             const adc_opts *opts) {
+  return context_init(out, B, naux, eps_occ, nocc, eps_vir, nvir, kind, order, x, opts, 0);
 }
 
 int adc_dims(const adc_ctx *c, int64_t *n1, int64_t *n2) {

@@ -500,6 +500,21 @@ int adc_batch_davidson(adc_batch *b, int nroots, double tol, int max_iter, int p
     co.ctx[i]->batch = (precision == ADC_PREC_FP64) ? nullptr : &co;
     co.ctx[i]->batch_slot = i;
   }
+  // Products from digits run in every problem's thread at once. Contexts without a share of
+  // their own take, by what they hold, 8% of what is free now: the margin the subspaces leave
+  std::vector<int64_t> own_limit(n);
+  double held = 0.0, margin = 0.0;
+  try {
+    margin = 0.08 * (double)unused_device_memory();
+  } catch (const Error &e) {
+    return bfail(b, e.what(), e.code);
+  }
+  for (int i = 0; i < n; ++i) held += (double)co.ctx[i]->ex.mem_used;
+  for (int i = 0; i < n; ++i) {
+    int64_t &l = co.ctx[i]->ex.digit_limit;
+    own_limit[i] = l;
+    if (n > 1 && l == 0) l = std::max<int64_t>(1, (int64_t)(margin * (double)co.ctx[i]->ex.mem_used / held));
+  }
   std::vector<std::thread> th;
   std::vector<std::string> msgs(n);
   for (int i = 0; i < n; ++i) {
@@ -528,6 +543,7 @@ int adc_batch_davidson(adc_batch *b, int nroots, double tol, int max_iter, int p
   for (int i = 0; i < n; ++i) {
     co.ctx[i]->batch = nullptr;
     co.ctx[i]->batch_slot = -1;
+    co.ctx[i]->ex.digit_limit = own_limit[i];
   }
   int worst = ADC_OK;
   for (int i = 0; i < n; ++i)
@@ -614,16 +630,19 @@ int adc_batch_solve(int n, const adc_problem *p, int nroots, double tol, int max
   const int lanes = o.init_lanes > 0 ? o.init_lanes : 4;
   int dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess) return bfail(nullptr, "adc_batch_solve: no device", ADC_ERR_CUDA);
-  int64_t budget = o.mem_budget;
+  // what the plan may use, and what there is
+  int64_t budget = o.mem_budget, room = o.mem_budget;
   if (budget <= 0) {
     try {
-      budget = (int64_t)(0.85 * (double)free_device_memory());
+      room = (int64_t)free_device_memory();
+      budget = (int64_t)(0.85 * (double)room);
     } catch (const Error &e) {
       return bfail(nullptr, e.what(), e.code);
     }
   }
   std::vector<int> order(n), wave(n);
-  int nw = plan_waves(n, p, nroots, budget, order.data(), wave.data(), nullptr, nullptr, o.refine == ADC_PREC_SLICED);
+  std::vector<int64_t> est(n);
+  int nw = plan_waves(n, p, nroots, budget, order.data(), wave.data(), est.data(), nullptr, o.refine == ADC_PREC_SLICED);
   if (nw < 0) return bfail(nullptr, "adc_batch_solve: invalid problem sizes", nw);
   adc_batch_info acc{};
   int worst = ADC_OK;
@@ -634,6 +653,21 @@ int adc_batch_solve(int n, const adc_problem *p, int nroots, double tol, int max
       if (wave[order[t]] == w) ids.push_back(order[t]);
     std::vector<adc_ctx *> ctxs(ids.size(), nullptr);
     std::vector<int> irc(ids.size(), ADC_OK);
+    // The plan does not count the digit planes that FP64 products take while they run (the setup
+    // of EA o = 18, v = 90 peaks at 1.7 GB, its estimate is 0.9): the problems share what the plan
+    // leaves by their estimates, those set up at the same time among themselves. A problem
+    // alone in its wave takes what it finds
+    std::vector<int64_t> by(ids.size());
+    for (size_t j = 0; j < ids.size(); ++j) by[j] = est[ids[j]];
+    std::sort(by.rbegin(), by.rend());
+    double all = 0.0, at_once = 0.0;
+    for (size_t j = 0; j < by.size(); ++j) {
+      all += (double)by[j];
+      if (j < (size_t)lanes) at_once += (double)by[j];
+    }
+    auto share = [&](int id, double among) -> int64_t {
+      return ids.size() < 2 ? 0 : std::max<int64_t>(1, (int64_t)(((double)room - all) * (double)est[id] / among));
+    };
     // initialise the wave on a few lanes, largest problems first
     const double t0 = now_s();
     std::atomic<int> next{0};
@@ -649,9 +683,11 @@ int adc_batch_solve(int n, const adc_problem *p, int nroots, double tol, int max
           adc_opts_default(&op);
           op.setup = o.setup;
           op.refine = o.refine;
-          irc[j] = adc_init(&ctxs[j], q.B, q.naux, q.eps_occ, q.nocc, q.eps_vir, q.nvir, q.kind, q.order, q.x, &op);
+          irc[j] = context_init(&ctxs[j], q.B, q.naux, q.eps_occ, q.nocc, q.eps_vir, q.nvir, q.kind, q.order, q.x,
+                                &op, share(ids[j], at_once));
           if (irc[j] == ADC_OK) {
             ctxs[j]->keep_digits = false;  // the plan's memory has no room for them
+            ctxs[j]->ex.digit_limit = share(ids[j], all);
             irc[j] = adc_sync(ctxs[j]);
           }
         }

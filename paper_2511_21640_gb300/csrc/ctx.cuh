@@ -66,6 +66,10 @@ struct adc_ctx {
 };
 
 namespace adc {
+// adc_init; digit_limit: Exec::digit_limit, 1 for none of the products from digits (api.cu)
+int context_init(adc_ctx **out, const adc_c128 *B, int64_t naux, const double *eps_occ, int64_t nocc,
+                 const double *eps_vir, int64_t nvir, int kind, int order, double x, const adc_opts *opts,
+                 int64_t digit_limit);
 TV Bview(adc_ctx *c, char p, char q);               // B^Q block view [Q][p][q]
 DBuf eri_block(adc_ctx *c, const char *spec);       // dense <pq||rs> of a 4-letter o/v spec
 DBuf build_vvvv_packed(adc_ctx *c);                 // [Pv][Pv] <ab||cd>, a<b, c<d

@@ -221,6 +221,8 @@ extern "C" int adc_diag_set_alloc_limit(int64_t bytes) {
   return ADC_OK;
 }
 
+extern "C" int64_t adc_diag_alloc_peak(void) { return alloc_peak_reset(); }
+
 extern "C" int adc_diag_memory(const adc_ctx *c, int64_t *total, int64_t *own, int64_t *device) {
   if (!c) return ADC_ERR_STATE;
   if (!total || !own || !device) return ADC_ERR_ARG;

@@ -449,6 +449,9 @@ bool fp64_op_product(adc_ctx *c, int which, bool ring, const cplx *X, int64_t k,
   if (!fp64_digits_usable(ex, M, Nc, K)) return false;
   SlCache &sl = sl_cache(c);
   const SlUse use(sl);
+  // (the whole block is sliced at once)
+  const double bx = 8.0 * sl_digits(K, kDigitFp64Bits).ns * (double)Nc * (double)sl_kp(K);
+  if (ex.digit_limit > 0 && bx > 0.375 * (double)ex.digit_limit) return false;
   const SlMat *op = sl_kept_op(c, sl, which, M, K);
   if (!op) return false;
   const OptionalAlloc opt(ex);

@@ -690,6 +690,13 @@ void sl_pack_B_ring(Exec &ex, SlMat &dst, const adc_ctx *c, const cplx *X, int64
   sl_pack_B_impl(ex, dst, s, Nc, c->o * c->v, false, like, bits);
 }
 
+// a product within Exec::digit_limit: two operand chunks of three eighths, a quarter of
+// partial sums, and the spill
+constexpr int64_t kDigitLimitMin = (int64_t)64 << 20;
+static size_t digit_share(Exec &ex, double part) {
+  return (size_t)std::max(0.0, part * ((double)ex.digit_limit - (double)kSpillCta * device_sm_count()));
+}
+
 // Tile width and inner split of a product: the ones that leave the SM with the most
 // work the least of it, in units of an inner block of a 128-column tile (ns (ns + 1) / 2
 // block products of 256 clocks). A 64-column block takes 0.75 and a 32-column one 0.6
@@ -700,7 +707,8 @@ struct SlPlan {
   int bn = 128, ksplit = 1;
   double clocks = 0.0;
 };
-static SlPlan sl_plan(int64_t M, int64_t N, int64_t kps, int ns) {
+constexpr size_t kMaxPartBytes = (size_t)1 << 30;
+static SlPlan sl_plan(int64_t M, int64_t N, int64_t kps, int ns, size_t max_part = kMaxPartBytes) {
   const double sms = device_sm_count(), block = 128.0 * ns * (ns + 1);
   const int64_t N2 = 2 * N, tm = (M + 127) / 128;
   SlPlan best;
@@ -710,8 +718,7 @@ static SlPlan sl_plan(int64_t M, int64_t N, int64_t kps, int ns) {
     const int64_t tiles = tm * ((N2 + bn - 1) / bn);
     const double per = block * (bn == 128 ? 1.0 : bn == 64 ? 0.75 : 0.6), fixed = bn == 128 ? 28e3 : 16e3;
     for (int s = 1; s <= 64 && (s == 1 || kps / s >= 2); ++s) {
-      // partial products within 1 GiB
-      if (s > 1 && (double)s * M * N * sizeof(cplx) > (double)(1ll << 30)) break;
+      if (s > 1 && (double)s * M * N * sizeof(cplx) > (double)max_part) break;
       const double red = s > 1 ? 2e4 + (double)(s + 1) * M * N * 0.01 : 0.0;
       const double c = std::ceil(tiles * s / sms) * ((double)((kps + s - 1) / s) * per + fixed) + red;
       if (c < best.clocks) { best.clocks = c; best.bn = bn; best.ksplit = s; }
@@ -732,7 +739,8 @@ void sl_gemm(Exec &ex, const SlMat &A, const SlMat &B, int64_t M, int64_t N, cpl
   g.b = A.b;
   g.ns = std::min(A.ns, B.ns);  // the common leading slices
   const int64_t N2 = 2 * N, kp2 = 2 * A.kp;
-  const SlPlan plan = sl_plan(M, N, kp2 / 64, g.ns);
+  const SlPlan plan = sl_plan(M, N, kp2 / 64, g.ns,
+                              ex.digit_limit > 0 ? std::min(kMaxPartBytes, digit_share(ex, 0.25)) : kMaxPartBytes);
   const int bn = plan.bn;
   tc_make_map3(&g.mA, A.planes.p, A.rows, kp2, A.ns, A.rows * kp2, 128);
   tc_make_map3(&g.mB, B.planes.p, B.rows, kp2, B.ns, B.rows * kp2, bn);
@@ -852,6 +860,7 @@ constexpr size_t kDigitCapMin = (size_t)2 << 20;
 size_t digit_cap(Exec &ex, double need) {
   if (g_sliced_cap) return g_sliced_cap;
   size_t cap = (size_t)16 << 30;
+  if (ex.digit_limit > 0) cap = std::min(cap, digit_share(ex, 3.0 / 8));
   if (ex.mem_limit > 0) cap = std::min(cap, (size_t)std::max<int64_t>(0, ex.mem_limit - ex.mem_used) / 3);
   if (need > (double)(1ll << 30)) cap = std::min(cap, unused_device_memory() / 8);
   return std::max(cap, kDigitCapMin);
@@ -922,11 +931,13 @@ static bool digits_pay(int64_t M, int64_t N, int64_t K, int64_t batch, bool kept
   return digits < fp64;
 }
 
-// a stream under capture keeps the FP64 units (the digit route allocates and may look up free memory)
+// a stream under capture keeps the FP64 units (the digit route allocates and may look up free
+// memory), and so does a context with next to no memory for it
 static bool digits_ready(Exec &ex) {
   cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
   ADC_CUDA(cudaStreamIsCapturing(ex.stream, &cs));
   if (cs != cudaStreamCaptureStatusNone) return false;
+  if (ex.digit_limit && ex.digit_limit < kDigitLimitMin) return false;
   if (!ex.digit_err) {
     ADC_CUDA(cudaHostAlloc((void **)&ex.digit_err, sizeof(int), cudaHostAllocMapped));
     *ex.digit_err = 0;

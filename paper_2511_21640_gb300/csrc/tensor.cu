@@ -89,9 +89,10 @@ size_t free_device_memory(const Exec *mine) {
 }
 
 // test hook: a device allocation that would take the library's total past the limit fails
-static std::atomic<int64_t> g_alloc_limit{0}, g_alloc_total{0};
+static std::atomic<int64_t> g_alloc_limit{0}, g_alloc_total{0}, g_alloc_peak{0};
 void set_alloc_limit(int64_t bytes) { g_alloc_limit = bytes; }
 int64_t alloc_total() { return g_alloc_total; }
+int64_t alloc_peak_reset() { return g_alloc_peak.exchange(g_alloc_total); }
 
 void *Exec::alloc(size_t bytes) {
   if (bytes == 0) return nullptr;
@@ -137,7 +138,9 @@ void *Exec::alloc(size_t bytes) {
                     (stage.empty() ? std::string() : ", in " + stage) + (tag.empty() ? std::string() : "/" + tag) +
                     ")");
   }
-  g_alloc_total += (int64_t)bytes;
+  const int64_t now = g_alloc_total += (int64_t)bytes;
+  for (int64_t top = g_alloc_peak; now > top && !g_alloc_peak.compare_exchange_weak(top, now);) {
+  }
   mem_used += (int64_t)bytes;
   mem_peak = std::max<int64_t>(mem_peak, mem_used);
   return p;

@@ -27,6 +27,9 @@ struct Exec {
   // FP64 zgemm on the tensor cores (tc_slice.cu): 0 never (the FP64 units alone),
   // 1 products large enough to pay, 2 every product (a diagnostic's choice)
   int digits = 0;
+  // bytes that one such product may take for digit planes, partial sums and its spill
+  // (0: by what is free): the share of a context that others run beside, whose memory is planned
+  int64_t digit_limit = 0;
   // pinned word in which such a product records a wait that gave up (the output then holds
   // NaN). Whoever waits for the stream looks at it: sync() throws ADC_ERR_TIMEOUT
   int *digit_err = nullptr;
@@ -81,6 +84,7 @@ bool reclaim_kept_digits(int dev);  // false: nothing to take
 // test hook: device allocations of the library fail past this total (<= 0: no limit); the total now
 void set_alloc_limit(int64_t bytes);
 int64_t alloc_total();
+int64_t alloc_peak_reset();  // the largest total since the last call
 
 struct OptionalAlloc {
   Exec &ex;

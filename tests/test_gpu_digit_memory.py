@@ -198,3 +198,27 @@ def test_a_limit_chunks_the_digits(gpu):
         c.profile(False)
     assert "tc_digits_fp64/ladder" in ran and "zgemm_fp64/ladder" not in ran, ran
     assert np.abs(got - want).max() < 1e-13 * np.abs(want).max()
+
+
+def test_batch_solve_stays_within_its_plan(gpu):
+    """Two problems in a wave whose budget is just the plan's estimate, set up one after the other
+    (the estimate does not count the intermediates of setups at the same time): the digit planes
+    of their FP64 setup and products, which it does not count either, stay out of it. The roots are those
+    of the problems solved alone, to the solves' tolerance."""
+    probs = []
+    for i in range(2):
+        p = make_problem(nocc=18, nvir=90, naux=60, seed=12 + i)
+        p.kind, p.order, p.x = "EA", 3, 0.5
+        probs.append(p)
+    sizes = [dict(nocc=18, nvir=90, naux=60, kind="EA", order=3, x=0.5)] * 2
+    budget = int(gpu.batch_plan(sizes, 2, 1 << 60)[3].sum())
+    gpu.lib.adc_diag_alloc_peak()
+    before = gpu.lib.adc_diag_alloc_peak()  # the record starts at the total now
+    om, _, status, info, rc = gpu.batch_solve(probs, 2, tol=1e-6, precision="fp64", mem_budget=budget,
+                                              init_lanes=1)
+    peak = gpu.lib.adc_diag_alloc_peak() - before
+    assert rc == 0 and info["waves"] == 1
+    assert peak <= budget, (peak, budget)
+    for p, w in zip(probs, om):
+        with gpu.Context(p.B, p.eps_occ, p.eps_vir, kind="EA", order=3, x=0.5) as c:
+            assert np.abs(c.davidson(2, tol=1e-6, precision="fp64", want_vectors=False)[0] - w).max() < 1e-8
