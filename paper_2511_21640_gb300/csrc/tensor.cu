@@ -566,8 +566,20 @@ void zgemm(Exec &ex, int64_t M, int64_t N, int64_t K, int64_t batch, cplx alpha,
     const int64_t tiles = (M + p.t->bm - 1) / p.t->bm * ((N + p.t->bn - 1) / p.t->bn) * slice;
     if (tiles <= (int64_t)(ex.zcount.bytes / sizeof(unsigned))) cnt = (unsigned *)ex.zcount.p;
     // the partial products: the context's own small buffer, or one of the call
-    if (cnt && (size_t)p.ksplit * slice * M * N * sizeof(cplx) <= ex.zpart.bytes) pp = (cplx *)ex.zpart.p;
-    else { part = cbuf(ex, (int64_t)p.ksplit * slice * M * N); pp = part.c(); }
+    if (cnt && (size_t)p.ksplit * slice * M * N * sizeof(cplx) <= ex.zpart.bytes) {
+      pp = (cplx *)ex.zpart.p;
+    } else {
+      const OptionalAlloc opt(ex);
+      try {
+        part = cbuf(ex, (int64_t)p.ksplit * slice * M * N);
+        pp = part.c();
+      } catch (const Error &e) {  // no room for them: whole inner sums
+        if (e.code != ADC_ERR_OOM) throw;
+        p = z_plan(M, N, K, batch, 1, 0, false);
+        ADC_REQUIRE(p.t, ADC_ERR_UNSUPPORTED, "zgemm: shape too large");
+        cnt = nullptr;
+      }
+    }
   }
   int pr = ex.prof_begin("zgemm_fp64", 8.0 * (double)M * N * K * batch,
                          16.0 * (double)batch * ((double)M * K + (double)K * N + (double)M * N));

@@ -222,3 +222,17 @@ def test_batch_solve_stays_within_its_plan(gpu):
     for p, w in zip(probs, om):
         with gpu.Context(p.B, p.eps_occ, p.eps_vir, kind="EA", order=3, x=0.5) as c:
             assert np.abs(c.davidson(2, tol=1e-6, precision="fp64", want_vectors=False)[0] - w).max() < 1e-8
+
+
+@pytest.mark.parametrize("M,N,K", [(1300, 1300, 2000), (300, 36, 12600), (700, 650, 3000)])
+def test_fp64_units_without_room_for_partial_sums(gpu, M, N, K):
+    """A product on the FP64 units with memory for its operands alone runs with whole inner sums.
+    Reference and product are the same computation there: equal."""
+    with gpu.Context(*(lambda p: (p.B, p.eps_occ, p.eps_vir))(make_problem(4, 6, 8, seed=1)), kind="IP") as c:
+        operands = 16 * (M * K + N * K + 2 * M * N)
+        assert gpu.lib.adc_diag_set_alloc_limit(c.kept_digits()["total"] + operands + 65536) == 0
+        try:
+            err, _ = gpu.diag_gemm(0, M, N, K, seed=3, reps=1)
+        finally:
+            gpu.lib.adc_diag_set_alloc_limit(0)
+    assert err == 0.0
