@@ -233,11 +233,13 @@ int context_init(adc_ctx **out, const adc_c128 *B, int64_t naux, const double *e
     // the setup's large contractions as the sliced tensor-core product when asked for
     c->ex.sliced_bits = (c->opts.setup == ADC_PREC_SLICED) ? 48 : 0;
     c->ex.digits = 1;
-    ex.zcount.p = ex.alloc(4096 * sizeof(unsigned));
-    ex.zcount.bytes = 4096 * sizeof(unsigned);
-    fill_zero(ex, ex.zcount.p, ex.zcount.bytes);
-    ex.zpart.p = ex.alloc((size_t)4 << 20);
-    ex.zpart.bytes = (size_t)4 << 20;
+    if (c->ex.mem_limit <= 0) {  // (a limit is for what the problem needs)
+      ex.zcount.p = ex.alloc(4096 * sizeof(unsigned));
+      ex.zcount.bytes = 4096 * sizeof(unsigned);
+      fill_zero(ex, ex.zcount.p, ex.zcount.bytes);
+      ex.zpart.p = ex.alloc((size_t)4 << 20);
+      ex.zpart.bytes = (size_t)4 << 20;
+    }
     c->ex.n_sliced = c->ex.n_fp64 = 0;
     c->ex.flops_sliced = c->ex.flops_fp64 = 0.0;
     {

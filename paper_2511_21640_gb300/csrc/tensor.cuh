@@ -34,8 +34,8 @@ struct Exec {
   // NaN). Whoever waits for the stream looks at it: sync() throws ADC_ERR_TIMEOUT
   int *digit_err = nullptr;
   // the FP64 kernel's inner splits: tile counters (zero between launches) and a small
-  // buffer of partial products. Held by a context for its life, on its one stream; null
-  // elsewhere: a second kernel then sums the splits
+  // buffer of partial products. Held by a context without a memory limit for its life, on its
+  // one stream; null elsewhere: a second kernel then sums the splits
   struct Held {
     void *p = nullptr;
     size_t bytes = 0;

@@ -236,3 +236,18 @@ def test_fp64_units_without_room_for_partial_sums(gpu, M, N, K):
         finally:
             gpu.lib.adc_diag_set_alloc_limit(0)
     assert err == 0.0
+
+
+def test_a_limit_equal_to_what_a_context_holds(gpu):
+    """Nothing is held for speed alone under a limit: a product of device operands too small for
+    digits needs no more than its scratch."""
+    p = make_problem(4, 10, 12, seed=2)
+    with gpu.Context(p.B, p.eps_occ, p.eps_vir, kind="EA", order=3, x=0.5) as c:
+        peak = c.memory()["peak"]
+    free = peak - (4 << 20) - (16 << 10)  # what the partial sums' buffers of an unlimited context take
+    with gpu.Context(p.B, p.eps_occ, p.eps_vir, kind="EA", order=3, x=0.5, mem_limit=free + (1 << 18)) as c:
+        X = torch.from_numpy(_vectors(c.N, 2, 3)).cuda()
+        got = c.sigma(X, "fp64").cpu().numpy()
+    with gpu.Context(p.B, p.eps_occ, p.eps_vir, kind="EA", order=3, x=0.5) as c:
+        want = c.sigma(X, "fp64").cpu().numpy()
+    assert np.abs(got - want).max() < 1e-13 * np.abs(want).max()
