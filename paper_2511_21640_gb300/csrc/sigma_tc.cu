@@ -316,7 +316,9 @@ struct SlUse {
 
 // The digits of a static operator, built when first asked for and rebuilt with
 // more digits when asked for more; a product with fewer bits uses the leading
-// digits of the trial vectors and the same leading digits of the operator.
+// digits of the trial vectors and the same leading digits of the operator. The shorter
+// digits are cut from the longer ones' integers, so that a sliced product is the
+// same whether or not an FP64 product has built these before it.
 static const SlMat &sl_op(adc_ctx *c, int which, int bits) {
   Exec &ex = c->ex;
   SlMat &m = sl_cache(c).op[which];
@@ -326,10 +328,10 @@ static const SlMat &sl_op(adc_ctx *c, int which, int bits) {
   SlMat t;
   std::swap(t.planes, m.planes);
   std::swap(t.exps, m.exps);
-  if (which == SL_CPL) sl_pack_A(ex, t, c->Cpl.c(), n1, n2, n2, 1, false, bits);
-  else if (which == SL_CPLT) sl_pack_A(ex, t, c->Cpl.c(), n2, n1, 1, n2, true, bits);
-  else if (which == SL_GLAD) sl_pack_A(ex, t, c->Glad.c(), P, P, P, 1, false, bits);
-  else sl_pack_A(ex, t, c->W.c(), o * v, o * v, o * v, 1, false, bits);
+  if (which == SL_CPL) sl_pack_A(ex, t, c->Cpl.c(), n1, n2, n2, 1, false, bits, kDigitFp64Bits);
+  else if (which == SL_CPLT) sl_pack_A(ex, t, c->Cpl.c(), n2, n1, 1, n2, true, bits, kDigitFp64Bits);
+  else if (which == SL_GLAD) sl_pack_A(ex, t, c->Glad.c(), P, P, P, 1, false, bits, kDigitFp64Bits);
+  else sl_pack_A(ex, t, c->W.c(), o * v, o * v, o * v, 1, false, bits, kDigitFp64Bits);
   m = std::move(t);
   return m;
 }

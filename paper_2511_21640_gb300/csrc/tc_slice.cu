@@ -110,13 +110,13 @@ __device__ __forceinline__ uint32_t bf16x2_of(int a, int b) {
 // The digits come from the top, each the remainder rounded to nearest, so that
 // they are centred on zero: digits cut from the bottom, in [-2^(b-1), 2^(b-1) - 1],
 // have a mean of -1/2, and the dropped classes would leave an error that grows with K.
+// bits: of the integer they are cut from, b ns or more (then these are its leading digits).
 template <int EMB>
 __global__ void __launch_bounds__(256)
 k_sl_pack(BSrc src, int64_t rows, int64_t K, int conj, int64_t kp, int kfast, const unsigned *__restrict__ W, int b, int ns,
-          __nv_bfloat16 *base, int64_t pe) {
+          int bits, __nv_bfloat16 *base, int64_t pe) {
   __shared__ cplx tile[PK_R * PK_LD];
   __shared__ PkRow row[PK_R];
-  const int bits = b * ns;
   for (int64_t n0 = (int64_t)blockIdx.x * PK_R; n0 < rows; n0 += (int64_t)gridDim.x * PK_R) {
     if (threadIdx.x < PK_R) row[threadIdx.x] = pk_row(src, min(n0 + (int64_t)threadIdx.x, rows - 1));
     __syncthreads();
@@ -137,7 +137,7 @@ k_sl_pack(BSrc src, int64_t rows, int64_t K, int conj, int64_t kp, int kfast, co
           im[j] = dead ? 0 : fixed_of(conj ? -x.y : x.y, e, bits);
         }
         for (int i = 0; i < ns; ++i) {
-          const int sh = b * (ns - 1 - i);
+          const int sh = bits - b * (i + 1);
           const long long rnd = (1ll << sh) >> 1;
           int dr[8], di[8];
 #pragma unroll
@@ -600,8 +600,8 @@ void alloc_sl(Exec &ex, SlMat &d, int64_t rows, int64_t nscale) {
   d.rows = rows;
 }
 
-// scales and digits of `rows` complex rows (emb 1: A rows, 2: B rows)
-void pack_rows(Exec &ex, SlMat &d, const BSrc &s, int64_t rows, int64_t K, bool conj, int emb) {
+// scales and digits of `rows` complex rows (emb 1: A rows, 2: B rows; cut_from: see sl_pack_A)
+void pack_rows(Exec &ex, SlMat &d, const BSrc &s, int64_t rows, int64_t K, bool conj, int emb, int cut_from = 0) {
   alloc_sl(ex, d, emb * rows, rows);
   if (rows <= 0) return;
   ADC_REQUIRE(s.mode == 0 || K < (1ll << 31), ADC_ERR_UNSUPPORTED, "sliced product: ring size");
@@ -621,12 +621,13 @@ void pack_rows(Exec &ex, SlMat &d, const BSrc &s, int64_t rows, int64_t K, bool 
   k_sl_scale<<<dim3(gx, gy), 256, 0, ex.stream>>>(s, rows, K, krange, kfast, W);
   ADC_CHECK_LAUNCH();
   const dim3 grid(gx, (unsigned)std::min<int64_t>(d.kp / PK_K, 65535));
+  const int bits = std::max(d.b * d.ns, cut_from);
   const int64_t pe = (int64_t)emb * rows * 2 * d.kp;
   if (emb == 1)
-    k_sl_pack<1><<<grid, 256, 0, ex.stream>>>(s, rows, K, conj ? 1 : 0, d.kp, kfast, W, d.b, d.ns,
+    k_sl_pack<1><<<grid, 256, 0, ex.stream>>>(s, rows, K, conj ? 1 : 0, d.kp, kfast, W, d.b, d.ns, bits,
                                               (__nv_bfloat16 *)d.planes.p, pe);
   else
-    k_sl_pack<2><<<grid, 256, 0, ex.stream>>>(s, rows, K, conj ? 1 : 0, d.kp, kfast, W, d.b, d.ns,
+    k_sl_pack<2><<<grid, 256, 0, ex.stream>>>(s, rows, K, conj ? 1 : 0, d.kp, kfast, W, d.b, d.ns, bits,
                                               (__nv_bfloat16 *)d.planes.p, pe);
   ADC_CHECK_LAUNCH();
   ex.prof_end(pr);
@@ -654,14 +655,14 @@ void launch_sl(Exec &ex, SlArgs &g, SlWork &w, int grid) {
 void sl_set_wait_ns(unsigned long long ns) { ADC_CUDA(cudaMemcpyToSymbol(g_wait_ns, &ns, sizeof(ns))); }
 
 void sl_pack_A(Exec &ex, SlMat &dst, const cplx *src, int64_t M, int64_t K, int64_t s_m, int64_t s_k, bool conj,
-               int bits) {
+               int bits, int cut_from) {
   const SlDigits dg = sl_digits(K, bits);
   dst.kp = sl_kp(K);
   dst.kreal = K;
   dst.b = dg.b;
   dst.ns = dg.ns;
   const BSrc s{src, 0, 0, s_m, std::max<int64_t>(M, 1), s_k, 0, 0, 0, 0};
-  pack_rows(ex, dst, s, M, K, conj, 1);
+  pack_rows(ex, dst, s, M, K, conj, 1, cut_from);
 }
 
 static void sl_pack_B_impl(Exec &ex, SlMat &dst, const BSrc &s, int64_t Nc, int64_t K, bool conj, const SlMat &like,

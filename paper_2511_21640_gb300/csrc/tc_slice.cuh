@@ -67,9 +67,10 @@ struct SlCache {
   ~SlCache();
 };
 
-// A[m][k] = op(src[m*s_m + k*s_k]); digits for about `bits` significant bits
+// A[m][k] = op(src[m*s_m + k*s_k]); digits for about `bits` significant bits, with cut_from
+// the leading digits of the slicing to that many bits
 void sl_pack_A(Exec &ex, SlMat &dst, const cplx *src, int64_t M, int64_t K, int64_t s_m, int64_t s_k, bool conj,
-               int bits);
+               int bits, int cut_from = 0);
 // B[n][k] = op(src[(n / n_in)*s_nh + (n % n_in)*s_nl + k*s_k]), sliced like the A operand `like`
 // bits > 0: only the leading digits for about that many significant bits (the
 // product then uses the same leading slices of A)

@@ -251,3 +251,16 @@ def test_a_limit_equal_to_what_a_context_holds(gpu):
     with gpu.Context(p.B, p.eps_occ, p.eps_vir, kind="EA", order=3, x=0.5) as c:
         want = c.sigma(X, "fp64").cpu().numpy()
     assert np.abs(got - want).max() < 1e-13 * np.abs(want).max()
+
+
+@pytest.mark.parametrize("precision", ["sliced", "sliced24"])
+@pytest.mark.parametrize("kind,nocc,nvir", [("EA", 12, 40), ("IP", 36, 20)])
+def test_sliced_product_does_not_depend_on_earlier_calls(gpu, kind, nocc, nvir, precision):
+    """The same sliced product before and after an FP64 product of the context: the same bits."""
+    p = make_problem(nocc=nocc, nvir=nvir, naux=60, seed=13)
+    with gpu.Context(p.B, p.eps_occ, p.eps_vir, kind=kind, order=3, x=0.5) as c:
+        X = _vectors(c.N, 32, 14)
+        first = c.sigma(X, precision)
+        c.sigma(X, "fp64")
+        assert c.kept_digits()["own"] > 0
+        assert np.array_equal(c.sigma(X, precision), first)
