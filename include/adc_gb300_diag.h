@@ -34,6 +34,17 @@ typedef struct adc_ctx adc_ctx_opaque;
 int adc_diag_gemm(int which, int64_t M, int64_t N, int64_t K, uint64_t seed, int reps,
                   double *rel_err, double *ms);
 
+/* One FP64 product of host arrays: C[b] = alpha op(A[b]) op(B[b]) + beta C[b],
+ * on the FP64 units (digits 0) or from 56-bit digits on the tensor cores
+ * (digits 1, whatever the size). size: M, N, K, batch (each at least 1).
+ * factors: alpha (re, im), beta (re, im). A, B, C hold nA, nB, nC elements;
+ * sA, sB, sC are element strides (batch, m, k), (batch, k, n), (batch, m, n),
+ * not negative, every element inside its array, else ADC_ERR_ARG; conjA, conjB:
+ * the operand conjugated. Allocates and frees its own device memory. */
+int adc_diag_zgemm(int digits, const int64_t *size, const double *factors, const adc_c128 *A, int64_t nA,
+                   const int64_t *sA, int conjA, const adc_c128 *B, int64_t nB, const int64_t *sB, int conjB,
+                   adc_c128 *C, int64_t nC, const int64_t *sC);
+
 /* Per-kernel timing of one context. adc_profile_enable(ctx, 1) clears the
  * record and starts recording a CUDA event pair around every GEMM launch on
  * the context's stream (0 stops). adc_profile_read() synchronises the stream

@@ -118,6 +118,7 @@ def _load():
         "adc_strerror": (ctypes.c_char_p, [I]),
         "adc_last_error": (ctypes.c_char_p, [P]),
         "adc_diag_gemm": (I, [I, I64, I64, I64, ctypes.c_uint64, I, ctypes.POINTER(D), ctypes.POINTER(D)]),
+        "adc_diag_zgemm": (I, [I, P, P, P, I64, P, I, P, I64, P, I, P, I64, P]),
         "adc_diag_blockops": (I, [I, I64, I64, I64, ctypes.c_uint64, I, ctypes.POINTER(D), ctypes.POINTER(D)]),
         "adc_diag_fp64_peak": (I, [I, I64, ctypes.POINTER(D), ctypes.POINTER(D)]),
         "adc_diag_set_wait_ns": (I, [ctypes.c_uint64]),
@@ -685,6 +686,19 @@ def diag_gemm(which, M, N, K, seed=1, reps=3):
                            ctypes.byref(t))
     _check(rc)
     return e.value, t.value
+
+
+def diag_zgemm(digits, size, A, sA, B, sB, C, sC, alpha=1.0, beta=0.0, conjA=False, conjB=False):
+    """C[b] = alpha op(A[b]) op(B[b]) + beta C[b] (``adc_diag_zgemm``) for flat complex128 arrays A, B and C
+    (returned, C itself is not changed); size (M, N, K, batch), strides (batch, m, k), (batch, k, n), (batch, m, n)."""
+    A, B = (np.ascontiguousarray(v, dtype=np.complex128) for v in (A, B))
+    out = np.array(C, dtype=np.complex128, order="C")
+    ints = [np.array(v, dtype=np.int64) for v in (size, sA, sB, sC)]
+    f = np.array([complex(alpha).real, complex(alpha).imag, complex(beta).real, complex(beta).imag])
+    _check(lib.adc_diag_zgemm(1 if digits else 0, ints[0].ctypes.data, f.ctypes.data, A.ctypes.data, A.size,
+                              ints[1].ctypes.data, int(bool(conjA)), B.ctypes.data, B.size, ints[2].ctypes.data,
+                              int(bool(conjB)), out.ctypes.data, out.size, ints[3].ctypes.data))
+    return out
 
 
 def diag_blockops(which, m, nb, n, seed=1, reps=3):

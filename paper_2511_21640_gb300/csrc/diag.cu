@@ -199,6 +199,39 @@ extern "C" int adc_diag_gemm(int which, int64_t M, int64_t N, int64_t K, uint64_
   }
 }
 
+// C[b] = alpha opA(A[b]) opB(B[b]) + beta C[b] of host arrays through zgemm; strides in elements
+extern "C" int adc_diag_zgemm(int digits, const int64_t *size, const double *factors, const adc_c128 *A, int64_t nA,
+                              const int64_t *sA, int conjA, const adc_c128 *B, int64_t nB, const int64_t *sB,
+                              int conjB, adc_c128 *C, int64_t nC, const int64_t *sC) {
+  if (!size || !factors || !A || !B || !C || !sA || !sB || !sC) return ADC_ERR_ARG;
+  const int64_t M = size[0], N = size[1], K = size[2], batch = size[3];
+  auto inside = [&](const int64_t *s, int64_t e1, int64_t e2, int64_t n) {
+    return s[0] >= 0 && s[1] >= 0 && s[2] >= 0 && (batch - 1) * s[0] + (e1 - 1) * s[1] + (e2 - 1) * s[2] < n;
+  };
+  if (M < 1 || N < 1 || K < 1 || batch < 1 || !inside(sA, M, K, nA) || !inside(sB, K, N, nB) || !inside(sC, M, N, nC))
+    return ADC_ERR_ARG;
+  Exec ex;
+  int rc = ADC_OK;
+  try {
+    ADC_CUDA(cudaStreamCreateWithFlags(&ex.stream, cudaStreamNonBlocking));
+    ex.digits = digits ? 2 : 0;
+    DBuf a = cbuf(ex, nA), b = cbuf(ex, nB), c = cbuf(ex, nC);
+    ADC_CUDA(cudaMemcpyAsync(a.p, A, a.bytes, cudaMemcpyHostToDevice, ex.stream));
+    ADC_CUDA(cudaMemcpyAsync(b.p, B, b.bytes, cudaMemcpyHostToDevice, ex.stream));
+    ADC_CUDA(cudaMemcpyAsync(c.p, C, c.bytes, cudaMemcpyHostToDevice, ex.stream));
+    zgemm(ex, M, N, K, batch, cmake(factors[0], factors[1]), a.c(), sA[0], sA[1], sA[2], conjA != 0, b.c(), sB[0], sB[1],
+          sB[2], conjB != 0, cmake(factors[2], factors[3]), c.c(), sC[0], sC[1], sC[2]);
+    ADC_CUDA(cudaMemcpyAsync(C, c.p, c.bytes, cudaMemcpyDeviceToHost, ex.stream));
+    ex.sync();
+  } catch (const Error &e) {
+    fprintf(stderr, "adc_diag_zgemm: %s\n", e.what());
+    rc = e.code;
+  }
+  if (ex.stream) { cudaStreamSynchronize(ex.stream); cudaStreamDestroy(ex.stream); }
+  if (ex.digit_err) cudaFreeHost(ex.digit_err);
+  return rc;
+}
+
 extern "C" int adc_profile_enable(adc_ctx *c, int on) {
   if (!c) return ADC_ERR_STATE;
   try {
