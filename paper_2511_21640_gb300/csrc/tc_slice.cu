@@ -39,18 +39,19 @@ namespace adc {
 namespace {
 
 // ---------------------------------------------------------------- row scales
-// The scale of a row is kept as its largest magnitude word: the high 31 bits
-// of |x| (the lowest bit set too when only the low word is nonzero), so that
-// an integer maximum finds it. 0: a row of zeros; exponent field 2047: the row
-// holds an infinity or a NaN.
+// The scale of a row is kept as its largest magnitude word: the high 31 bits of |x| (the
+// lowest bit set too when only the low word is nonzero), so that an integer maximum
+// finds it; of a subnormal |x| the number of its significant bits. 0: a row of zeros;
+// exponent field 2047: the row holds an infinity or a NaN.
 __device__ __forceinline__ unsigned mag_word(double x) {
   const unsigned hi = (unsigned)__double2hiint(x) & 0x7fffffffu;
+  if (hi < 0x100000u) return 64u - (unsigned)__clzll(__double_as_longlong(x) & 0x7fffffffffffffffll);
   return hi | (__double2loint(x) != 0 ? 1u : 0u);
 }
 __device__ __forceinline__ unsigned mag_word(cplx x) { return max(mag_word(x.x), mag_word(x.y)); }
 __device__ __forceinline__ bool not_finite(unsigned w) { return (w >> 20) == 0x7ffu; }
-// E with every |x| of the row below 2^E
-__device__ __forceinline__ int scale_exp(unsigned w) { return (w >> 20) ? (int)(w >> 20) - 1022 : -1021; }
+// E with every |x| of the row below 2^E, and 2^E at most twice the largest
+__device__ __forceinline__ int scale_exp(unsigned w) { return (w >> 20) ? (int)(w >> 20) - 1022 : (int)w - 1074; }
 
 // round(x 2^(bits - E)) as an integer (|x| < 2^E, so at most 2^bits; ties to even)
 __device__ __forceinline__ long long fixed_of(double x, int E, int bits) {

@@ -69,7 +69,7 @@ def bound(A, B, alpha, beta, C0):
     top = lambda x, ax: np.ldexp(1.0, np.frexp(np.maximum(np.abs(x.real), np.abs(x.imag)).max(axis=ax))[1])
     ea, eb = top(A, 1)[:, None], top(B, 0)[None, :]
     sa, sb = _mag(A).sum(axis=1)[:, None], _mag(B).sum(axis=0)[None, :]
-    t = 1.01 * 2.0 ** -57 * (ea * sb + eb * sa) + 1.8 * 2.0 ** -56 * 2 * A.shape[1] * ea * eb
+    t = 1.01 * 2.0 ** -57 * (ea * sb + eb * sa) + 1.8 * 2.0 ** -56 * 2 * A.shape[1] * (ea * eb)
     fa = abs(complex(alpha).real) + abs(complex(alpha).imag)
     fb = abs(complex(beta).real) + abs(complex(beta).imag)
     return fa * t + 2.0 ** -51 * (fa * (_mag(A) @ _mag(B)) + fb * _mag(C0)) + 5e-324
@@ -157,7 +157,7 @@ def test_operand_chunks(gpu, M, N, K, share, batch):
         gpu.lib.adc_diag_set_sliced_cap(0)
 
 
-@pytest.mark.parametrize("what", ["spikes", "tails", "opposed", "zero rows", "huge and tiny", "one term"])
+@pytest.mark.parametrize("what", ["spikes", "tails", "opposed", "zero rows", "huge and tiny", "subnormal", "one term"])
 @pytest.mark.parametrize("M,N,K", [(31, 9, 80), (9, 31, 80)])
 def test_graded_rows(gpu, M, N, K, what):
     """Rows whose elements differ by many orders of magnitude, maxima at different inner indices."""
@@ -179,6 +179,9 @@ def test_graded_rows(gpu, M, N, K, what):
     elif what == "huge and tiny":
         A *= 1e290
         B *= 1e-300
+    elif what == "subnormal":
+        A = np.ldexp(A.real, -1050) + 1j * np.ldexp(A.imag, -1050)
+        B = B * 2.0 ** 900
     else:
         A[0, :, 1:] = 0.0
     check(gpu, A, B, order_b="k")
