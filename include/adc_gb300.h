@@ -53,9 +53,16 @@ enum { ADC_IP = 0, ADC_EA = 1, ADC_EE = 2 };
 
 /* Arithmetic of a sigma product.
  * ADC_PREC_FP64:   FP64 throughout: small contractions on the CUDA cores, large
- *   ones on the tensor cores from 56-bit integer digits (below): 56 bits
- *   relative to the row and column maxima, measured no further from exact sums
- *   than FP64 multiply-adds.
+ *   ones on the tensor cores from 56-bit integer digits (below). The error of
+ *   those is relative to the row and column maxima: at most 2^-51 K max|A_m|
+ *   max|B_n| for the element (m, n) of a product over K terms, in practice
+ *   about 2^-57 sqrt(K) of them, no more than FP64 multiply-adds leave where
+ *   rows and columns are of one order of magnitude. Where the large elements
+ *   of a row meet small ones of the column, an element far below that product
+ *   has fewer correct digits than multiply-adds give; opts.fp64_units keeps
+ *   every contraction on the CUDA cores. Which contractions run from digits
+ *   depends on their sizes and on the memory there is for the digits; none do
+ *   while the stream is being captured.
  * ADC_PREC_BF16X3: the dense contractions on the tensor cores (tcgen05) with
  *   each FP64 operand split into two BF16 parts (hi + lo) and the three
  *   products hi*hi + hi*lo + lo*hi accumulated in FP32; complex arithmetic by
@@ -152,6 +159,12 @@ typedef struct {
                            0 = every tensor-core term (both coupling
                            directions, ladder, ring) as jobs of one grouped
                            persistent launch (default); -1 = one launch per term */
+  int fp64_units;       /* 1 = every FP64 contraction (setup, products,
+                           gradients, densities) by multiply-adds on the CUDA
+                           cores, whatever its size: rounding relative to each
+                           term; 0 = large ones from digits (default, see
+                           ADC_PREC_FP64). Explicit sliced and split precisions
+                           are not affected */
 } adc_opts;
 
 typedef struct {
@@ -546,6 +559,7 @@ typedef struct {
   int setup;           /* adc_opts.setup of every problem's adc_init (ADC_PREC_FP64 or ADC_PREC_SLICED) */
   int refine;          /* adc_opts.refine of every problem (ADC_PREC_FP64 or ADC_PREC_SLICED;
                           the waves then leave room for the sliced operator copies) */
+  int fp64_units;      /* adc_opts.fp64_units of every problem */
 } adc_batch_opts;
 
 /* Host-only planner (no GPU needed): estimated device bytes mem_est[i] and

@@ -41,7 +41,7 @@ class adc_opts(ctypes.Structure):
                 ("mem_limit", ctypes.c_int64), ("verbose", ctypes.c_int), ("dd_order", ctypes.c_int),
                 ("refine", ctypes.c_int), ("setup", ctypes.c_int), ("ee_vvvv", ctypes.c_int),
                 ("correction", ctypes.c_int), ("ladder", ctypes.c_int), ("profile", ctypes.c_int),
-                ("grouped_sigma", ctypes.c_int)]
+                ("grouped_sigma", ctypes.c_int), ("fp64_units", ctypes.c_int)]
 
 
 class adc_stats(ctypes.Structure):
@@ -89,7 +89,7 @@ class adc_problem(ctypes.Structure):
 
 class adc_batch_opts(ctypes.Structure):
     _fields_ = [("mem_budget", ctypes.c_int64), ("init_lanes", ctypes.c_int), ("verbose", ctypes.c_int),
-                ("setup", ctypes.c_int), ("refine", ctypes.c_int)]
+                ("setup", ctypes.c_int), ("refine", ctypes.c_int), ("fp64_units", ctypes.c_int)]
 
 
 def _load():
@@ -212,7 +212,7 @@ class Context:
     def __init__(self, B, eps_occ, eps_vir, kind="IP", order=3, x=1.0, precision="fp64", stream=None,
                  block=0, max_subspace=0, herm_tol=1e-12, mem_limit=0, verbose=False, dd_order=1,
                  refine="fp64", setup="fp64", vvvv="auto", correction="davidson", ladder="auto",
-                 profile=False, grouped_sigma=True):
+                 profile=False, grouped_sigma=True, fp64_units=False):
         o = adc_opts()
         lib.adc_opts_default(ctypes.byref(o))
         o.precision = PRECISIONS[precision] if isinstance(precision, str) else int(precision)
@@ -234,6 +234,7 @@ class Context:
         o.ladder = {"auto": 0, "direct": 1, "stored": -1}[ladder]
         o.profile = 1 if profile else 0
         o.grouped_sigma = 0 if grouped_sigma else -1
+        o.fp64_units = 1 if fp64_units else 0
         naux, nmo, nmo2 = B.shape
         nocc, nvir = eps_occ.shape[0], eps_vir.shape[0]
         if nmo != nmo2 or nmo != nocc + nvir:
@@ -618,11 +619,12 @@ def batch_plan(problems, nroots, mem_budget):
 
 
 def batch_solve(problems, nroots, tol=1e-6, max_iter=300, precision="bf16x3", mem_budget=0, init_lanes=0,
-                setup="fp64", refine="fp64"):
+                setup="fp64", refine="fp64", fp64_units=False):
     """Solve many problems given as host arrays (``adc_batch_solve``): (omega, err64, status, info, rc)."""
     n = len(problems)
     arr, keep = _problems(problems)
-    o = adc_batch_opts(int(mem_budget), int(init_lanes), 0, PRECISIONS[setup], PRECISIONS[refine])
+    o = adc_batch_opts(int(mem_budget), int(init_lanes), 0, PRECISIONS[setup], PRECISIONS[refine],
+                       1 if fp64_units else 0)
     omega = np.empty((n, nroots), dtype=np.float64)
     err = np.empty((n, nroots), dtype=np.float64)
     status = np.empty(n, dtype=np.int32)
@@ -638,7 +640,7 @@ def batch_solve(problems, nroots, tol=1e-6, max_iter=300, precision="bf16x3", me
 
 
 def ssfns(B, eps_occ, eps_vir, kind="EA", order=3, x=1.0, nroots=1, eta_crit=1e-5, tol=1e-8, max_iter=300,
-          precision="fp64", refine="fp64"):
+          precision="fp64", refine="fp64", fp64_units=False):
     """State-specific natural-spinor energies of the nroots lowest EA/EE roots (``adc_ssfns``,
     Sec. 2.4, Eqs. 31-32): a list of dicts (omega_corrected, omega_fns, omega2_canonical, omega2_fns,
     err64, n_keep, status)."""
@@ -648,6 +650,7 @@ def ssfns(B, eps_occ, eps_vir, kind="EA", order=3, x=1.0, nroots=1, eta_crit=1e-
     o = adc_opts()
     lib.adc_opts_default(ctypes.byref(o))
     o.refine = PRECISIONS[refine] if isinstance(refine, str) else int(refine)
+    o.fp64_units = 1 if fp64_units else 0
     out = (adc_ssfns_root * int(nroots))()
     p = PRECISIONS[precision] if isinstance(precision, str) else int(precision)
     rc = lib.adc_ssfns(B.ctypes.data, B.shape[0], eo.ctypes.data, eo.shape[0], ev.ctypes.data, ev.shape[0],

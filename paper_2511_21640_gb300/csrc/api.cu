@@ -176,6 +176,7 @@ int context_init(adc_ctx **out, const adc_c128 *B, int64_t naux, const double *e
     ADC_REQUIRE(c->opts.ladder >= -1 && c->opts.ladder <= 1, ADC_ERR_ARG, "opts.ladder: -1, 0 or 1");
     ADC_REQUIRE(c->opts.grouped_sigma == 0 || c->opts.grouped_sigma == -1, ADC_ERR_ARG,
                 "opts.grouped_sigma: 0 or -1");
+    ADC_REQUIRE(c->opts.fp64_units == 0 || c->opts.fp64_units == 1, ADC_ERR_ARG, "opts.fp64_units: 0 or 1");
     c->kind = kind;
     c->order = order;
     c->x = (order == 3) ? x : 0.0;
@@ -232,7 +233,7 @@ int context_init(adc_ctx **out, const adc_c128 *B, int64_t naux, const double *e
     }
     // the setup's large contractions as the sliced tensor-core product when asked for
     c->ex.sliced_bits = (c->opts.setup == ADC_PREC_SLICED) ? 48 : 0;
-    c->ex.digits = 1;
+    c->ex.digits = c->opts.fp64_units ? 0 : 1;
     if (c->ex.mem_limit <= 0) {  // (a limit is for what the problem needs)
       ex.zcount.p = ex.alloc(4096 * sizeof(unsigned));
       ex.zcount.bytes = 4096 * sizeof(unsigned);

@@ -683,6 +683,7 @@ int adc_batch_solve(int n, const adc_problem *p, int nroots, double tol, int max
           adc_opts_default(&op);
           op.setup = o.setup;
           op.refine = o.refine;
+          op.fp64_units = o.fp64_units;
           irc[j] = context_init(&ctxs[j], q.B, q.naux, q.eps_occ, q.nocc, q.eps_vir, q.nvir, q.kind, q.order, q.x,
                                 &op, share(ids[j], at_once));
           if (irc[j] == ADC_OK) {
