@@ -887,7 +887,8 @@ void digit_zgemm(Exec &ex, int64_t M, int64_t N, int64_t K, int64_t batch, cplx 
   }
   SlMat Sa, Sb;
   SlWork w;
-  const double need = 4.0 * sl_digits(K, bits).ns * (double)sl_kp(K) * std::max<double>(M, 2.0 * N * (fold ? batch : 1));
+  const double need = 4.0 * sl_digits(K, bits).ns * (double)sl_kp(K) *
+                      std::max<double>(128, std::max<double>(M, 2.0 * N * (fold ? batch : 1)));
   if (!cap) cap = std::min(digit_cap(ex, need), (size_t)std::max(need, (double)kDigitCapMin));
   if (fold) {
     digit_product(ex, M, N * batch, K, alpha, A, sAm, sAk, conjA, B, sBk, sBb, sBn, N, conjB, beta, C, sCm, sCb, sCn,

@@ -157,6 +157,15 @@ def test_operand_chunks(gpu, M, N, K, share, batch):
         gpu.lib.adc_diag_set_sliced_cap(0)
 
 
+def test_few_rows_are_one_chunk(gpu):
+    """Operands of less than a row tile whose memory there is room for: sliced and multiplied at once
+    (two launches per operand, the product, and the sum of its inner splits)."""
+    A, B = _ops(20, 10, 5000)
+    n0 = gpu.launch_count()
+    gpu.diag_zgemm(1, (20, 10, 5000, 1), A.ravel(), (0, 5000, 1), B.ravel(), (0, 10, 1), np.zeros(200), (0, 10, 1))
+    assert gpu.launch_count() - n0 <= 6
+
+
 @pytest.mark.parametrize("what", ["spikes", "tails", "opposed", "zero rows", "huge and tiny", "subnormal", "one term"])
 @pytest.mark.parametrize("M,N,K", [(31, 9, 80), (9, 31, 80)])
 def test_graded_rows(gpu, M, N, K, what):
