@@ -39,19 +39,26 @@ namespace adc {
 namespace {
 
 // ---------------------------------------------------------------- row scales
-// The scale of a row is kept as its largest magnitude word: the high 31 bits of |x| (the
-// lowest bit set too when only the low word is nonzero), so that an integer maximum
-// finds it; of a subnormal |x| the number of its significant bits. 0: a row of zeros;
-// exponent field 2047: the row holds an infinity or a NaN.
+// The scale of a row is kept as one word: the high 31 bits of its largest |x| with 64 added to
+// the exponent field; b + 12 in that field when it is subnormal and has b significant bits.
+// 0: a row of zeros; the field kWordInf: the row holds an infinity or a NaN. The exponent
+// E follows by one subtraction (the product's results take it per column).
+constexpr unsigned kWordInf = 0x7ffu + 64u;
+// high 31 bits of |x|, the lowest bit set too when only the low word is nonzero: an integer
+// maximum finds the largest but among subnormal numbers (below 0x100000)
 __device__ __forceinline__ unsigned mag_word(double x) {
   const unsigned hi = (unsigned)__double2hiint(x) & 0x7fffffffu;
-  if (hi < 0x100000u) return 64u - (unsigned)__clzll(__double_as_longlong(x) & 0x7fffffffffffffffll);
   return hi | (__double2loint(x) != 0 ? 1u : 0u);
 }
 __device__ __forceinline__ unsigned mag_word(cplx x) { return max(mag_word(x.x), mag_word(x.y)); }
-__device__ __forceinline__ bool not_finite(unsigned w) { return (w >> 20) == 0x7ffu; }
-// E with every |x| of the row below 2^E, and 2^E at most twice the largest
-__device__ __forceinline__ int scale_exp(unsigned w) { return (w >> 20) ? (int)(w >> 20) - 1022 : (int)w - 1074; }
+// the row's word for a subnormal x (zero: 0)
+__device__ __forceinline__ unsigned subnormal_word(double x) {
+  const long long m = __double_as_longlong(x) & 0x7fffffffffffffffll;
+  return m ? (unsigned)(64 - __clzll(m) + 12) << 20 : 0u;
+}
+__device__ __forceinline__ bool not_finite(unsigned w) { return (w >> 20) == kWordInf; }
+// E with every |x| of the row below 2^E, and 2^E at most twice the largest (any E for zeros)
+__device__ __forceinline__ int scale_exp(unsigned w) { return (int)(w >> 20) - 1086; }
 
 // round(x 2^(bits - E)) as an integer (|x| < 2^E, so at most 2^bits; ties to even)
 __device__ __forceinline__ long long fixed_of(double x, int E, int bits) {
@@ -59,7 +66,7 @@ __device__ __forceinline__ long long fixed_of(double x, int E, int bits) {
   const int field = (int)((u >> 52) & 0x7ff);
   long long m = u & 0xfffffffffffffll;
   if (field) m |= 1ll << 52;
-  const int s = (field ? field : 1) - 1075 + bits - E;  // value = m 2^(s + E - bits); s <= bits - 53
+  const int s = (field ? field : 1) - 1075 + bits - E;  // value = m 2^(s + E - bits), m 2^s < 2^bits
   long long r;
   if (s >= 0) r = m << s;
   else if (s >= -54) r = (m + ((1ll << (-s - 1)) - 1) + ((m >> -s) & 1)) >> -s;
@@ -93,7 +100,21 @@ k_sl_scale(BSrc src, int64_t rows, int64_t K, int64_t krange, int kfast, unsigne
       });
     if (!kfast) atomicMax(&mx[threadIdx.x & 31], own);
     __syncthreads();
-    if (threadIdx.x < PK_R && n0 + threadIdx.x < rows) atomicMax(&W[n0 + threadIdx.x], mx[threadIdx.x]);
+    const unsigned top = threadIdx.x < PK_R ? mx[threadIdx.x] : 0;
+    unsigned word = top >= 0x100000u ? top + (64u << 20) : 0;
+    // rows of subnormal numbers here: once more, by their significant bits (a branch among the
+    // loads above would keep them from overlapping)
+    if (__syncthreads_or(top != 0 && top < 0x100000u)) {
+      if (threadIdx.x < PK_R) mx[threadIdx.x] = 0;
+      __syncthreads();
+      for (int64_t k0 = kb; k0 < ke; k0 += PK_K)
+        pk_load(src, n0, rows, k0, ke, kfast != 0, row, [&](int r, int, cplx x) {
+          if (mag_word(x) < 0x100000u) atomicMax(&mx[r], max(subnormal_word(x.x), subnormal_word(x.y)));
+        });
+      __syncthreads();
+      if (threadIdx.x < PK_R && top < 0x100000u) word = mx[threadIdx.x];
+    }
+    if (threadIdx.x < PK_R && n0 + threadIdx.x < rows) atomicMax(&W[n0 + threadIdx.x], word);
     __syncthreads();
   }
 }
@@ -129,7 +150,7 @@ k_sl_pack(BSrc src, int64_t rows, int64_t K, int conj, int64_t kp, int kfast, co
       if (n < rows) {
         const unsigned w = W[n];
         const int e = scale_exp(w);
-        const bool dead = not_finite(w);
+        const bool dead = w == 0 || not_finite(w);
         long long re[8], im[8];
 #pragma unroll
         for (int j = 0; j < 8; ++j) {

@@ -168,7 +168,8 @@ def test_few_rows_are_one_chunk(gpu):
 
 @pytest.mark.parametrize("what", ["spikes", "tails", "opposed", "zero rows", "huge and tiny", "subnormal", "one term"])
 @pytest.mark.parametrize("M,N,K", [(31, 9, 80), (9, 31, 80)])
-def test_graded_rows(gpu, M, N, K, what):
+@pytest.mark.parametrize("order", ["k", "m"])
+def test_graded_rows(gpu, M, N, K, what, order):
     """Rows whose elements differ by many orders of magnitude, maxima at different inner indices."""
     A, B = _ops(M, N, K)
     if what == "spikes":
@@ -193,7 +194,7 @@ def test_graded_rows(gpu, M, N, K, what):
         B = B * 2.0 ** 900
     else:
         A[0, :, 1:] = 0.0
-    check(gpu, A, B, order_b="k")
+    check(gpu, A, B, order_a=order, order_b="k" if order == "k" else "n")
 
 
 @pytest.mark.parametrize("bad", [np.nan, np.inf, -np.inf])
