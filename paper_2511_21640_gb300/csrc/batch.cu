@@ -500,16 +500,27 @@ int adc_batch_davidson(adc_batch *b, int nroots, double tol, int max_iter, int p
     co.ctx[i]->batch = (precision == ADC_PREC_FP64) ? nullptr : &co;
     co.ctx[i]->batch_slot = i;
   }
-  // Products from digits run in every problem's thread at once. Contexts without a share of
-  // their own take, by what they hold, 8% of what is free now: the margin the subspaces leave
+  // Products from digits run in every problem's thread at once. Contexts without a share of their
+  // own take, by what they hold, half of the memory the solves will leave (the plan's estimate of
+  // each problem less what it holds), at least 8% of what is free: the subspaces' own margin
   std::vector<int64_t> own_limit(n);
   double held = 0.0, margin = 0.0;
   try {
-    margin = 0.08 * (double)unused_device_memory();
+    const double unused = (double)unused_device_memory();
+    margin = unused;
+    for (int i = 0; i < n; ++i) {
+      const adc_ctx *c = co.ctx[i];
+      adc_problem q{};
+      q.nocc = c->o; q.nvir = c->v; q.naux = c->Q;
+      q.kind = c->kind; q.order = c->order; q.x = c->x;
+      const double used = (double)c->ex.mem_used;
+      held += used;
+      margin -= std::max(0.0, (double)mem_estimate(q, nroots, c->opts.refine == ADC_PREC_SLICED) - used);
+    }
+    margin = std::max(0.08 * unused, 0.5 * margin);
   } catch (const Error &e) {
     return bfail(b, e.what(), e.code);
   }
-  for (int i = 0; i < n; ++i) held += (double)co.ctx[i]->ex.mem_used;
   for (int i = 0; i < n; ++i) {
     int64_t &l = co.ctx[i]->ex.digit_limit;
     own_limit[i] = l;
