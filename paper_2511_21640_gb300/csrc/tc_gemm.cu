@@ -485,7 +485,7 @@ __device__ __forceinline__ TgTile tg_decode(const TcJob *__restrict__ jobs, int 
   d.m0 = tm * TC_BM;
   d.n0 = tn * J.bn;
   d.kb_beg = d.split * J.kb_per_split;
-  d.nkb = min(TC_SEG * J.kps, d.kb_beg + J.kb_per_split) - d.kb_beg;
+  d.nkb = min(J.nseg * J.kps, d.kb_beg + J.kb_per_split) - d.kb_beg;
   return d;
 }
 
@@ -607,8 +607,8 @@ k_tc_grouped(const TcJob *__restrict__ jobs, int njobs, int total_tiles, int *co
         // the products of one k-block (hi hi, hi lo, lo hi) back to back, so
         // that the second read of an operand block comes from L2
         const int kg = d.kb_beg + i;
-        const int seg = kg % TC_SEG;
-        const int kx = (kg / TC_SEG) * TC_BK;
+        const int seg = kg % J.nseg;
+        const int kx = (kg / J.nseg) * TC_BK;
         const uint32_t fb = smem_u32(&full[s]);
         mbar_expect_tx(fb, bytes);
         uint8_t *sa = smem + s * TgLayout::STAGE;
@@ -978,7 +978,7 @@ void tc_gemm_grouped(Exec &ex, const std::vector<TcJobDesc> &in, TcGroup &grp, i
   const bool capturing = (cs != cudaStreamCaptureStatusNone);
   if (capturing) may_tune = false;
   struct Plan {
-    int idx, bn, kps, tiles_m, tiles_n, ksplit, kbps;
+    int idx, bn, kps, tiles_m, tiles_n, ksplit, kbps, nseg;
     int64_t N2;
   };
   std::vector<Plan> pl;
@@ -999,9 +999,10 @@ void tc_gemm_grouped(Exec &ex, const std::vector<TcJobDesc> &in, TcGroup &grp, i
     if (p.bn <= 0) p.bn = bn_rule(p.N2);
     ADC_REQUIRE(p.bn >= 32 && p.bn <= TC_BNMAX && p.bn % 32 == 0, ADC_ERR_ARG, "tc_gemm_grouped: tile width");
     p.kps = (int)(2 * d.A->kp / TC_BK);
+    p.nseg = 3;  // hi hi, hi lo, lo hi
     p.tiles_m = (int)((d.M + TC_BM - 1) / TC_BM);
     p.tiles_n = (int)((p.N2 + p.bn - 1) / p.bn);
-    const double job_work = (double)p.tiles_m * p.tiles_n * (double)TC_SEG * p.kps;
+    const double job_work = (double)p.tiles_m * p.tiles_n * (double)p.nseg * p.kps;
     work += job_work;
     cols += job_work * p.bn;
     if (p.bn >= 192) wide_cols += job_work * p.bn;
@@ -1016,7 +1017,7 @@ void tc_gemm_grouped(Exec &ex, const std::vector<TcJobDesc> &in, TcGroup &grp, i
   const double target = std::max(16.0, work / (4.0 * sms));
   size_t part_need = 0;
   for (auto &p : pl) {
-    const int total_kb = TC_SEG * p.kps;
+    const int total_kb = p.nseg * p.kps;
     int ks = 1;
     if (total_kb > target) ks = (int)std::min<double>(128.0, std::ceil(total_kb / target));
     p.kbps = (total_kb + ks - 1) / ks;
@@ -1056,6 +1057,7 @@ void tc_gemm_grouped(Exec &ex, const std::vector<TcJobDesc> &in, TcGroup &grp, i
     make_map(&J.mBh, d.B->hi.p, d.B->rows, kp2, p.bn);
     make_map(&J.mBl, d.B->lo.p, d.B->rows, kp2, p.bn);
     J.out = d.out;
+    J.nseg = p.nseg;
     J.part = p.ksplit > 1 ? (float *)grp.part.p + poff : nullptr;
     if (p.ksplit > 1) poff += (size_t)p.ksplit * d.M * p.N2;
     J.s_m = d.s_m;

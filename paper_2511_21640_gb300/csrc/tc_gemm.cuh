@@ -61,7 +61,6 @@ void tc_gemm(Exec &ex, const TcView &A, const TcView &B, int64_t M, int64_t N, c
 
 // ---- grouped persistent launch (several problems and terms in one kernel)
 constexpr int TC_BNMAX = 256;
-constexpr int TC_SEG = 3;  // products of an inner block: hi hi, hi lo, lo hi
 
 // one job as the kernel reads it (device memory, 128-byte aligned tensor maps)
 struct alignas(128) TcJob {
@@ -70,7 +69,7 @@ struct alignas(128) TcJob {
   float *part;  // split-K partials [ksplit][M][N2] or null
   int64_t s_m, s_nh, s_nl, n_in;
   cplx alpha, beta;
-  int M, N2, kps, bn, tiles_n, tiles_m, ksplit, kb_per_split, tile_begin;
+  int M, N2, kps, bn, tiles_n, tiles_m, ksplit, kb_per_split, tile_begin, nseg;
   int l2keepB;  // 1: the B operand (re-read by every row block) loaded with an L2 evict-last
                 // policy and A with evict-first, so that B stays in L2 while A streams
   int panel;    // column blocks per panel: tiles run panel by panel, row blocks inside a

@@ -3,6 +3,8 @@
 #include <atomic>
 #include <cstring>
 #include <map>
+
+#include <map>
 #include <mutex>
 #include <set>
 #include <tuple>
