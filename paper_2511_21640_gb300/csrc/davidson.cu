@@ -482,8 +482,10 @@ int davidson_run(adc_ctx *c, int nroots, double tol, int max_iter, int precision
     };
     int lo = (int)std::min<int64_t>(N, std::max(2 * nroots, kb) + kb);
     int64_t fit = fit_of(krmax);
-    // the subspace goes before digits kept for speed: a smaller one takes more iterations
-    if (fit < mmax && c->ex.give_back && c->ex.give_back(c->ex.give_back_of)) {
+    // the subspace goes before digits kept for speed: a smaller one takes more iterations (a
+    // sliced refinement reads them, and would have to build its own in what is left)
+    const bool sliced_refine = precision != ADC_PREC_FP64 && c->opts.refine == ADC_PREC_SLICED;
+    if (fit < mmax && !sliced_refine && c->ex.give_back && c->ex.give_back(c->ex.give_back_of)) {
       keep.off();
       c->ex.sync();
       look();
