@@ -79,7 +79,8 @@ __device__ __forceinline__ cplx axpby(int ka, cplx alpha, cplx v, int kb, cplx b
   return r;
 }
 
-// Division of n < 2^31 by a constant found at run time: two multiplies' worth instead of
+// Division of n < 2^31 by a constant found at run time (Granlund and Montgomery, "Division by
+// invariant integers using multiplication", 1994): two multiplies' worth instead of
 // the tens of instructions of an integer division
 struct FastDiv {
   uint32_t d, mul, sh;

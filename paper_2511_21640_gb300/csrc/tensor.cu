@@ -3,8 +3,6 @@
 #include <atomic>
 #include <cstring>
 #include <map>
-
-#include <map>
 #include <mutex>
 #include <set>
 #include <tuple>
