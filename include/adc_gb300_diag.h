@@ -89,9 +89,9 @@ int adc_diag_set_setup_chunk(int64_t elems);
 /* Test hook: bytes of one operand chunk of the sliced product behind the
  * setup's large contractions (the digit planes of A row blocks and B column
  * blocks; when one 128-row tile would exceed it, the inner index is split and
- * the FP64-accurate partial products add up). <= 0 restores the rule of a
- * third of what the context's mem_limit leaves and an eighth of the device's
- * free memory, at most 16 GiB. Process-wide. Returns ADC_OK. */
+ * the FP64-accurate partial products add up). <= 0 restores the rule of an
+ * eighth of the free memory (1 to 16 GiB), at most a third of what the
+ * context's mem_limit leaves. Process-wide. Returns ADC_OK. */
 int adc_diag_set_sliced_cap(int64_t bytes);
 
 /* Test hook: device allocations of the library (every context of the process

@@ -877,17 +877,22 @@ void digit_product(Exec &ex, int64_t M, int64_t N, int64_t K, cplx alpha, const 
 // smallest operand chunk: its inner index is 512 long (digit_product)
 constexpr size_t kDigitCapMin = (size_t)2 << 20;
 
-// bytes per operand chunk: a third of what the context's limit leaves and an eighth of the
-// device's free memory, which other contexts use too, at most 16 GiB (need: the larger
-// operand's planes; the free memory is looked up only when they exceed 1 GiB)
+// Bytes per operand chunk: an eighth of the free device memory, between 1 and 16 GiB (need:
+// the larger operand's planes; the free memory is looked up only when they exceed 1 GiB),
+// and no more than a third of what the context's limit leaves or its share
 size_t digit_cap(Exec &ex, double need) {
   if (g_sliced_cap) return g_sliced_cap;
-  size_t cap = (size_t)16 << 30;
-  if (ex.digit_limit > 0) cap = std::min(cap, digit_share(ex, 3.0 / 8));
+  size_t cap = (size_t)1 << 30;
+  if (need > (double)cap) cap = std::min<size_t>((size_t)16 << 30, std::max(cap, unused_device_memory() / 8));
   if (ex.mem_limit > 0) cap = std::min(cap, (size_t)std::max<int64_t>(0, ex.mem_limit - ex.mem_used) / 3);
-  if (need > (double)(1ll << 30)) cap = std::min(cap, unused_device_memory() / 8);
+  if (ex.digit_limit > 0) cap = std::min(cap, digit_share(ex, 3.0 / 8));
   return std::max(cap, kDigitCapMin);
 }
+
+// operand chunks of a product: bytes allowed (0: by digit_cap), bytes of its whole planes
+struct DigitChunks {
+  size_t cap = 0, whole = 0;
+};
 
 // zgemm's operands and output (element strides, conj flags, batch). The larger
 // of M and N becomes the A side (half the bytes per digit); a batch whose A
@@ -895,7 +900,7 @@ size_t digit_cap(Exec &ex, double need) {
 void digit_zgemm(Exec &ex, int64_t M, int64_t N, int64_t K, int64_t batch, cplx alpha, const cplx *A, int64_t sAb,
                  int64_t sAm, int64_t sAk, bool conjA, const cplx *B, int64_t sBb, int64_t sBk, int64_t sBn,
                  bool conjB, cplx beta, cplx *C, int64_t sCb, int64_t sCm, int64_t sCn, int bits, int *err,
-                 bool &begun, size_t &cap) {
+                 bool &begun, DigitChunks &ch) {
   const bool fold = batch > 1 && (sAb == 0 || sBb == 0);
   if (fold ? sAb != 0 : N > M) {
     std::swap(M, N);
@@ -908,9 +913,10 @@ void digit_zgemm(Exec &ex, int64_t M, int64_t N, int64_t K, int64_t batch, cplx 
   }
   SlMat Sa, Sb;
   SlWork w;
-  const double need = 4.0 * sl_digits(K, bits).ns * (double)sl_kp(K) *
-                      std::max<double>(128, std::max<double>(M, 2.0 * N * (fold ? batch : 1)));
-  if (!cap) cap = std::min(digit_cap(ex, need), (size_t)std::max(need, (double)kDigitCapMin));
+  const double need = 4.0 * sl_digits(K, bits).ns * (double)sl_kp(K) * std::max<double>(M, 2.0 * N * (fold ? batch : 1));
+  if (!ch.cap) ch.cap = digit_cap(ex, need);
+  ch.whole = (size_t)need;
+  const size_t cap = ch.cap;
   if (fold) {
     digit_product(ex, M, N * batch, K, alpha, A, sAm, sAk, conjA, B, sBk, sBb, sBn, N, conjB, beta, C, sCm, sCb, sCn,
                   bits, cap, err, Sa, Sb, w, begun);
@@ -930,9 +936,9 @@ void zgemm_sliced(Exec &ex, int64_t M, int64_t N, int64_t K, int64_t batch, cplx
   DBuf err(ex, sizeof(int));
   fill_zero(ex, err.p, sizeof(int));
   bool begun = false;
-  size_t cap = 0;
+  DigitChunks ch;
   digit_zgemm(ex, M, N, K, batch, alpha, A, sAb, sAm, sAk, conjA, B, sBb, sBk, sBn, conjB, beta, C, sCb, sCm, sCn,
-              ex.sliced_bits, (int *)err.p, begun, cap);
+              ex.sliced_bits, (int *)err.p, begun, ch);
   tc_sync(ex, (int *)err.p);
 }
 
@@ -980,15 +986,15 @@ bool zgemm_fp64_digits(Exec &ex, int64_t M, int64_t N, int64_t K, int64_t batch,
   if (ex.digits == 0 || K <= 0 || (ex.digits == 1 && !digits_pay(M, N, K, grouped, false)) || !digits_ready(ex)) return false;
   const OptionalAlloc opt(ex);
   bool begun = false;
-  for (size_t cap = 0;; cap /= 4) {
+  for (DigitChunks ch;; ch.cap = std::min(ch.cap, ch.whole) / 4) {
     try {
       digit_zgemm(ex, M, N, K, batch, alpha, A, sAb, sAm, sAk, conjA, B, sBb, sBk, sBn, conjB, beta, C, sCb, sCm, sCn,
-                  kDigitFp64Bits, ex.digit_err, begun, cap);
+                  kDigitFp64Bits, ex.digit_err, begun, ch);
       return true;
     } catch (const Error &e) {
       // no room for the digit planes: smaller chunks, then the FP64 units, which need none
       if (e.code != ADC_ERR_OOM || begun) throw;
-      if (cap / 4 < kDigitCapMin) return false;
+      if (std::min(ch.cap, ch.whole) / 4 < kDigitCapMin) return false;
     }
   }
 }
