@@ -7,8 +7,8 @@ A step is one complete Davidson solve of those roots with tensor-core (BF16x3)
 sigma products refined by FP64-accurate sigma products until every residual
 norm of those is below tol; the setup of the operators (adc_init) is timed
 separately. The refinement products are, by default, the sliced tensor-core
-product (integer BF16 digits summed exactly in FP32, combined in FP64, about
-1e-12 relative); --refine fp64 uses the FP64 CUDA-core product instead.
+product (integer BF16 digits summed exactly in FP32, then in integers, about
+1e-12 relative); --refine fp64 uses the FP64 product instead.
 
 Metric: Davidson seconds per root (lower is better); the line also carries
 the sigma TFLOP/s of the mixed and FP64 products, the FP64 Davidson s/root,
