@@ -471,7 +471,8 @@ int davidson_run(adc_ctx *c, int nroots, double tol, int max_iter, int precision
     c->ex.sync();
     double avail = 0.0;
     auto look = [&]() {
-      avail = (double)free_device_memory(&c->ex);
+      // (beside other solves the others' digits are in use)
+      avail = (double)(c->ex.digit_limit ? unused_device_memory() : free_device_memory(&c->ex));
       if (c->ex.mem_limit > 0) avail = std::min(avail, (double)(c->ex.mem_limit - c->ex.mem_used));
     };
     look();

@@ -1,10 +1,12 @@
 // FP64 complex tensor toolkit (see tensor.cuh).
 #include <algorithm>
 #include <atomic>
+#include <chrono>
 #include <cstring>
 #include <map>
 #include <mutex>
 #include <set>
+#include <thread>
 #include <tuple>
 
 #include "tensor.cuh"
@@ -70,6 +72,12 @@ void pool_release(int dev) {
   cudaMemPoolTrimTo(it->second.pool, 0);
 }
 
+static int pool_contexts(int dev) {
+  std::lock_guard<std::mutex> lk(g_pool_mu);
+  auto it = g_pools.find(dev);
+  return it == g_pools.end() ? 0 : it->second.contexts;
+}
+
 size_t unused_device_memory() {
   size_t fr = 0, tot = 0;
   ADC_CUDA(cudaMemGetInfo(&fr, &tot));
@@ -121,10 +129,15 @@ void *Exec::alloc(size_t bytes) {
     };
     if (!capturing()) {
       again();
+      // Then what every context of the device keeps for speed. A context inside a product keeps
+      // its digits and holds that product's planes until it is enqueued: with others
+      // there, look again for a tenth of a second
       int dev = 0;
-      if (e == cudaErrorMemoryAllocation && !optional && cudaGetDevice(&dev) == cudaSuccess && reclaim_kept_digits(dev)) {
+      const int looks = !optional && cudaGetDevice(&dev) == cudaSuccess ? (pool_contexts(dev) > 1 ? 50 : 1) : 0;
+      for (int t = 0; e == cudaErrorMemoryAllocation && t < looks; ++t) {
+        if (t) std::this_thread::sleep_for(std::chrono::milliseconds(2));
         cudaGetLastError();
-        again();
+        if (reclaim_kept_digits(dev) || t) again();
       }
     }
   }

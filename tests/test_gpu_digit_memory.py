@@ -264,3 +264,46 @@ def test_sliced_product_does_not_depend_on_earlier_calls(gpu, kind, nocc, nvir, 
         c.sigma(X, "fp64")
         assert c.kept_digits()["own"] > 0
         assert np.array_equal(c.sigma(X, precision), first)
+
+
+def test_memory_comes_back_beside_running_products(gpu):
+    """The same while the other context, in a thread of its own, runs FP64 products all the time: its
+    digits are in use and its products' planes come and go, and the second context's products all
+    find their memory."""
+    import threading
+    p = _problem()
+
+    def context():
+        return gpu.Context(p.B, p.eps_occ, p.eps_vir, kind="EA", order=3, x=0.5)
+
+    with context() as a, context() as b:
+        small, X = _vectors(a.N, 32, 9), _vectors(a.N, 300, 10)
+        Xa = torch.from_numpy(small).cuda()
+        Sa = torch.empty_like(Xa)
+        torch.cuda.synchronize()
+        want, ref = a.sigma(small, "fp64"), b.sigma(X, "sliced")[:2]
+        need = 16 * 2 * 300 * b.N
+        stop, failed = threading.Event(), []
+
+        def products():
+            while not stop.is_set():
+                rc = [gpu.lib.adc_sigma(a._h, Xa.data_ptr(), Sa.data_ptr(), 32, 0) for _ in range(50)]
+                rc.append(gpu.lib.adc_sync(a._h))
+                if any(rc):
+                    failed.append(rc)
+                    return
+
+        own = a.kept_digits()["own"]
+        assert gpu.lib.adc_diag_set_alloc_limit(a.kept_digits()["total"] + need - own // 2) == 0
+        t = threading.Thread(target=products)
+        t.start()
+        try:
+            for _ in range(100):
+                got = b.sigma(X, "sliced")[:2]
+        finally:
+            stop.set()
+            t.join()
+            gpu.lib.adc_diag_set_alloc_limit(0)
+        assert not failed
+        assert np.abs(got - ref).max() < 1e-11 * np.abs(ref).max()
+        assert np.abs(a.sigma(small, "fp64") - want).max() < 1e-13 * np.abs(want).max()
